@@ -58,6 +58,9 @@ constexpr int kPartial = kExtraUnits - 32 * (kExtraSlots - 1);  // lanes of the 
 constexpr int kPairSmemWords = kRing * 2 * kWin + kRing * kSharedWords + kRow * kPairThreads;
 constexpr int kPairSmemBytes = kPairSmemWords * (int)sizeof(uint32_t) + 3 * kRing * 8;
 constexpr int kMinPairsPerItem = 16;
+constexpr int kListCap = 4096;             // pairs of one block of the listed form
+constexpr int kListedSmemBytes = kPairSmemBytes + kListCap * (int)sizeof(uint32_t);
+static_assert(kListedSmemBytes <= 227 * 1024, "the listed pair kernel fits one SM");
 constexpr int kTileThreads = 512;
 constexpr int kMaxTileBits = 12;
 
@@ -328,10 +331,24 @@ __device__ __forceinline__ bool fold_pair(uint32_t jj, uint32_t Ta_jj, uint32_t*
 // bounded; one that gives up sets kErrTimeout in *flags and the thread stops
 // (after waiting, bounded again, for the copies it started), so the launch
 // ends with its results marked invalid.
+//
+// kListed (pruned recurrence, k_dp_pruned.cu): the pairs are the Ta's within T
+// that have a long list, found by the block before the pair loop: from the
+// members of T's lowest request or, when those are fewer, from the proper
+// parts of T, either way in increasing Ta.  A tile's pairs are cut into
+// at most items_per_tile ranges of at least kMinPairsPerItem.
+struct ListedPairs {
+  const uint32_t* info;     // row list of each Ta (kListLong)
+  const uint32_t* long_ta;  // Ta's with a long list, by lowest request
+  const uint32_t* member_n;
+  unsigned int* pairs_run;  // total, for the profile
+};
+
+template <bool kListed>
 __global__ void __launch_bounds__(kPairThreads, 1)
 k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, unsigned long long* __restrict__ partial,
            int L, int kh, uint32_t pairs_per_tile, uint32_t items_per_tile, uint32_t pairs_per_item,
-           int32_t* __restrict__ flags) {
+           int32_t* __restrict__ flags, ListedPairs listed) {
   extern __shared__ __align__(16) uint32_t smem[];
   // ring slot c: X at smem + 2c * kWin, Y right after it; then one per-pair
   // minimum array of the shared rows per slot; then the running-best Ta of
@@ -347,11 +364,50 @@ k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, uns
   const uint32_t T = colex_unrank(tile, kh, L);
   const uint32_t low = T & (~T + 1u);
   const uint32_t R = T ^ low;
-  const uint32_t q0 = item * pairs_per_item;
-  const uint32_t q1 = min(q0 + pairs_per_item, pairs_per_tile);
-  const uint32_t npairs = q1 > q0 ? q1 - q0 : 0u;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+  uint32_t q0 = item * pairs_per_item;
+  uint32_t q1 = min(q0 + pairs_per_item, pairs_per_tile);
+  uint32_t* lst = reinterpret_cast<uint32_t*>(folded + kRing);  // kListed: this block's Ta's
+  if constexpr (kListed) {
+    __shared__ uint32_t wn[kPairThreads / 32];
+    const int l = __ffs(T) - 1;
+    const uint32_t nm = listed.member_n[kMaxMembersL + l];
+    const bool by_parts = pairs_per_tile < nm;
+    const uint32_t total = by_parts ? pairs_per_tile : nm;
+    const uint32_t* mem = listed.long_ta + ((1u << L) - (1u << (L - l)));
+    auto candidate = [&](uint32_t i) -> uint32_t {  // Ta, or 0
+      if (i >= total) return 0u;
+      const uint32_t Ta = by_parts ? (low | deposit_bits(i, R)) : mem[i];
+      if ((Ta & ~T) != 0 || Ta == T) return 0u;
+      return by_parts && !(listed.info[Ta] & kListLong) ? 0u : Ta;
+    };
+    uint32_t n = 0;
+    for (uint32_t base = 0; base < total; base += kPairThreads)
+      n += (uint32_t)__syncthreads_count(candidate(base + threadIdx.x) != 0);
+    const uint32_t parts = min(items_per_tile, (n + kMinPairsPerItem - 1) / kMinPairsPerItem);
+    if (item >= parts) return;  // the same decision in every thread
+    q0 = (uint32_t)((unsigned long long)n * item / parts);
+    q1 = (uint32_t)((unsigned long long)n * (item + 1) / parts);
+    if (threadIdx.x == 0) atomicAdd(listed.pairs_run, q1 - q0);
+    uint32_t at = 0;
+    for (uint32_t base = 0; base < total && at < q1; base += kPairThreads) {
+      const uint32_t Ta = candidate(base + threadIdx.x);
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, Ta != 0);
+      if (lane == 0) wn[warp] = __popc(bal);
+      __syncthreads();
+      uint32_t o = at + __popc(bal & ((1u << lane) - 1u));
+      for (uint32_t w = 0; w < kPairThreads / 32; ++w) {
+        o += w < warp ? wn[w] : 0u;
+        at += wn[w];
+      }
+      if (Ta != 0 && o >= q0 && o < q1 && o - q0 < (uint32_t)kListCap) lst[o - q0] = Ta;
+      __syncthreads();
+    }
+    if (MPT_BAD(flags, q1 - q0 <= (uint32_t)kListCap)) return;
+  }
+  const uint32_t npairs = q1 > q0 ? q1 - q0 : 0u;
 #ifdef MPT_BOUNDS
+  if constexpr (!kListed)
   {
     // the tile, and every pair's Ta: a part of T holding its lowest request,
     // so both windows lie inside the 2^(L + kB)-entry tables
@@ -407,7 +463,7 @@ k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, uns
   __syncthreads();
 
   // the first pair, into slot 0
-  uint32_t sub = deposit_bits(q0, R);
+  uint32_t sub = kListed ? (npairs >= 1 ? lst[0] ^ low : 0u) : deposit_bits(q0, R);
   if (npairs >= 1) copy_pair(smem, smem + kWin, Gp + ((size_t)(low | sub) << kB), Gc + ((size_t)(R ^ sub) << kB), &full[0]);
 
   bool ok = true;
@@ -415,7 +471,7 @@ k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, uns
   for (uint32_t j = 0; j < npairs; ++j) {
     const uint32_t c = j % kRing;
     const uint32_t Ta = low | sub;
-    const uint32_t next = (sub - R) & R;
+    const uint32_t next = kListed ? (j + 1 < npairs ? lst[j + 1] ^ low : 0u) : (sub - R) & R;
     // copies of pair j + 1, into the slot pair j + 1 - kRing has left
     if (j + 1 < npairs) {
       const uint32_t cn = (j + 1) % kRing;
@@ -546,7 +602,7 @@ template <typename Tab>
 __global__ void __launch_bounds__(kTileThreads)
 k_dp_tile(int L, int b, int kh, const Tab* __restrict__ wIr, const unsigned long long* __restrict__ partial,
           uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot,
-          int32_t* __restrict__ flags) {
+          int32_t* __restrict__ flags, InnerPerm perm) {
   __shared__ uint32_t cur_p[1 << kMaxTileBits];   // this tile, F << b
   __shared__ uint32_t other_c[1 << kMaxTileBits]; // complement form: this tile (kh = 0) or tile 0 (kh >= 1)
   __shared__ uint16_t order[1 << kMaxTileBits];   // inner subsets sorted by size, then colex
@@ -618,7 +674,7 @@ k_dp_tile(int L, int b, int kh, const Tab* __restrict__ wIr, const unsigned long
         best = o < best ? o : best;
       }
       if (active && r == 0) {
-        const size_t idx = ((size_t)T << b) | U;
+        const size_t idx = ((size_t)T << b) | perm.stored(U);
         int64_t f;
         uint32_t A;
         if (U == 0 && T == 0) {
@@ -699,7 +755,7 @@ template <typename Tab, bool kZcGlobal>
 __global__ void __launch_bounds__(kRowsThreads)
 k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long long* __restrict__ partial,
                uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot,
-               int32_t* __restrict__ flags) {
+               int32_t* __restrict__ flags, const uint32_t* __restrict__ info, InnerPerm perm) {
   extern __shared__ __align__(16) uint32_t smem[];
   uint32_t* cur = smem;                                   // this tile, F << kB, padded rows
   uint32_t* zc = smem + kWin;                             // tile 0, complement form, padded rows (shared copy)
@@ -711,6 +767,7 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
   const uint32_t T = colex_unrank(tile, kh, L);
   const size_t tbase = (size_t)T << kB;
   if (MPT_BAD(flags, tile < c_binom.v[L][kh] && T < (1u << L) && __popc(T) == kh)) return;
+  if (info && !(info[T] & kTileLong)) return;  // finished by k_dp_pruned
 
   if constexpr (!kZcGlobal) {
     for (int c = threadIdx.x; c < (1 << (kB - 2)); c += kRowsThreads) {
@@ -789,6 +846,7 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
     }
     if (finisher) {
       const uint32_t s1 = s1f;
+      const uint32_t nat_s1 = info ? perm.nat(s1 << kB2) : s1 << kB2;  // stored order undone (pruned recurrence)
       uint32_t z[kRow], c[kRow];
       load_zrow<kZcGlobal>(z, zc, Gc, 0);
 #pragma unroll
@@ -809,7 +867,7 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
           f = wv[s2];
           A = 0;
         } else {
-          const uint32_t Ua = (bk & kMask) + U - kMask;
+          const uint32_t Ua = (bk & kMask) + (nat_s1 | (info ? perm.nat((uint32_t)s2) : (uint32_t)s2)) - kMask;
           f = (bk >> kB) - wv[s2];
           A = (Ua << L) | bt;
         }
@@ -826,9 +884,10 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
   for (int u = threadIdx.x; u < (1 << kB); u += kRowsThreads) {
     const uint32_t gp = cur[row_pos((uint32_t)u >> kB2) * kRowStride + (u & (kRow - 1))];
     const uint32_t A = bsplit[best_word((uint32_t)u)];
-    if (MPT_BAD(flags, valid_split(T | ((uint32_t)u << L), A))) continue;
+    const uint32_t nat = info ? perm.nat((uint32_t)u) : (uint32_t)u;
+    if (MPT_BAD(flags, valid_split(T | (nat << L), A))) continue;
     Gp[tbase | (uint32_t)u] = gp;
-    Gc[tbase | (uint32_t)u] = gp | (~(uint32_t)u & kMask);
+    Gc[tbase | (uint32_t)u] = gp | (~nat & kMask);
     split_rot[tbase | (uint32_t)u] = A;
   }
 }
@@ -880,24 +939,59 @@ int64_t blocked_partial_entries(int m, int b) {
 
 int blocked_max_launches(const Shape& s) { return 2 * (s.L + 1); }
 
+namespace {
+
+// The kernels' shared-memory attributes belong to the current device: set them
+// on every call (a host-side call, negligible against a solve), so that any
+// device works.
+cudaError_t blocked_attributes(bool listed) {
+  cudaError_t e = listed ? cudaFuncSetAttribute(k_dp_pairs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                kListedSmemBytes)
+                         : cudaFuncSetAttribute(k_dp_pairs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                kPairSmemBytes);
+  auto rows = [&](auto kernel, bool zc_global) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem_bytes(zc_global));
+  };
+  rows(k_dp_tile_rows<int64_t, false>, false);
+  rows(k_dp_tile_rows<int32_t, false>, false);
+  rows(k_dp_tile_rows<int64_t, true>, true);
+  rows(k_dp_tile_rows<int32_t, true>, true);
+  return e;
+}
+
+// The tile kernel of step kh (info: the pruned recurrence's lists, or null).
+void launch_tiles(const Shape& s, const Workspace& ws, int kh, const uint32_t* info, cudaStream_t stream) {
+  const unsigned long long tiles = h_binom.v[s.L][kh];
+  if (kh == 0) {
+    if (s.lean)
+      k_dp_tile<<<1, kTileThreads, 0, stream>>>(s.L, s.b, 0, ws.fw_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
+                                                ws.counters + 1, s.perm);
+    else
+      k_dp_tile<<<1, kTileThreads, 0, stream>>>(s.L, s.b, 0, ws.wI_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
+                                                ws.counters + 1, s.perm);
+    return;
+  }
+  const unsigned long long* part = kh >= 2 ? ws.partial : nullptr;
+  const bool zg = s.L >= kZcGlobalMinL;
+  const int sm_bytes = rows_smem_bytes(zg);
+  if (s.lean) {
+    auto k = zg ? k_dp_tile_rows<int32_t, true> : k_dp_tile_rows<int32_t, false>;
+    k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(s.L, kh, ws.fw_rot, part, ws.Gp, ws.Gc, ws.split_rot,
+                                                           ws.counters + 1, info, s.perm);
+  } else {
+    auto k = zg ? k_dp_tile_rows<int64_t, true> : k_dp_tile_rows<int64_t, false>;
+    k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(s.L, kh, ws.wI_rot, part, ws.Gp, ws.Gc, ws.split_rot,
+                                                           ws.counters + 1, info, s.perm);
+  }
+}
+
+}  // namespace
+
 cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                               BlockedTiming* timing, int step_begin, int step_end) {
   {
-    // the attributes belong to the current device: set them on every call (a
-    // host-side call, negligible against a solve), so that any device works
-    cudaError_t e = cudaFuncSetAttribute(k_dp_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_tile_rows<int64_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             rows_smem_bytes(false));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_tile_rows<int32_t, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             rows_smem_bytes(false));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_tile_rows<int64_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             rows_smem_bytes(true));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_dp_tile_rows<int32_t, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             rows_smem_bytes(true));
+    cudaError_t e = blocked_attributes(false);
     if (e != cudaSuccess) return e;
   }
   const int b = s.b, L = s.L;
@@ -919,8 +1013,8 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
       cudaError_t e = cudaMemsetAsync(ws.partial, 0xFF, (size_t)(tiles << b) * sizeof(unsigned long long), stream);
       if (e != cudaSuccess) return e;
       if (timing && timing->pair_ev) cudaEventRecord(timing->pair_ev[2 * timing->pair_launches], stream);
-      k_dp_pairs<<<(unsigned)(tiles * items), kPairThreads, kPairSmemBytes, stream>>>(
-          ws.Gp, ws.Gc, ws.partial, L, kh, P, (uint32_t)items, ppi, ws.counters + 1);
+      k_dp_pairs<false><<<(unsigned)(tiles * items), kPairThreads, kPairSmemBytes, stream>>>(
+          ws.Gp, ws.Gc, ws.partial, L, kh, P, (uint32_t)items, ppi, ws.counters + 1, ListedPairs{});
       if (timing && timing->pair_ev) cudaEventRecord(timing->pair_ev[2 * timing->pair_launches + 1], stream);
       if (timing) {
         timing->pair_launches++;
@@ -931,32 +1025,63 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
       if (e != cudaSuccess) return e;
     }
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches], stream);
-    if (kh == 0) {
-      if (s.lean)
-        k_dp_tile<<<1, kTileThreads, 0, stream>>>(L, b, 0, ws.fw_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
-                                                  ws.counters + 1);
-      else
-        k_dp_tile<<<1, kTileThreads, 0, stream>>>(L, b, 0, ws.wI_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
-                                                  ws.counters + 1);
-    } else {
-      const unsigned long long* part = kh >= 2 ? ws.partial : nullptr;
-      const bool zg = L >= kZcGlobalMinL;
-      const int sm_bytes = rows_smem_bytes(zg);
-      if (s.lean) {
-        auto k = zg ? k_dp_tile_rows<int32_t, true> : k_dp_tile_rows<int32_t, false>;
-        k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(L, kh, ws.fw_rot, part, ws.Gp, ws.Gc, ws.split_rot,
-                                                               ws.counters + 1);
-      } else {
-        auto k = zg ? k_dp_tile_rows<int64_t, true> : k_dp_tile_rows<int64_t, false>;
-        k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(L, kh, ws.wI_rot, part, ws.Gp, ws.Gc, ws.split_rot,
-                                                               ws.counters + 1);
-      }
-    }
+    launch_tiles(s, ws, kh, nullptr, stream);
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches + 1], stream);
     if (timing) timing->tile_launches++;
     ++*launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// The pruned recurrence (k_dp_pruned.cu): each layer in k_dp_pruned; only when
+// the host's bound says that a long list is possible does the pair kernel run
+// before it, over the long lists, and the row kernel after it.
+cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
+                             BlockedTiming* timing) {
+  cudaError_t e = blocked_attributes(true);
+  if (e != cudaSuccess) return e;
+  const int L = s.L;
+  const unsigned long long sms = (unsigned long long)sm_count();
+  if ((e = launch_prune_lists(s, ws, stream, launches)) != cudaSuccess) return e;
+  auto mark = [&](cudaEvent_t* ev, int i) {
+    if (timing && ev) cudaEventRecord(ev[i], stream);
+  };
+  for (int kh = 0; kh <= L; ++kh) {
+    const unsigned long long tiles = h_binom.v[L][kh];
+    const uint32_t blocks = kh >= 2 ? pruned_items(s, kh) : 1u;  // per tile, in k_dp_pruned
+    const bool meet = pruned_meet(s, kh, blocks);
+    if (meet) {
+      e = cudaMemsetAsync(ws.partial, 0xFF, (size_t)(tiles << kB) * sizeof(unsigned long long), stream);
+      if (e != cudaSuccess) return e;
+    }
+    if (kh >= 2 && s.prune_long) {
+      const uint32_t P = (1u << (kh - 1)) - 1u;
+      // blocks for about four waves, and enough that a block's pairs fit its list
+      unsigned long long items = (4 * sms + tiles - 1) / tiles;
+      const unsigned long long most = (P + kMinPairsPerItem - 1) / kMinPairsPerItem;
+      const unsigned long long least = (P + kListCap - 1) / kListCap;
+      if (items > most) items = most;
+      if (items < least) items = least;
+      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches);
+      const ListedPairs lp{ws.prune_info, ws.prune_long, ws.prune_n,
+                           reinterpret_cast<unsigned int*>(ws.counters + 2)};
+      k_dp_pairs<true><<<(unsigned)(tiles * items), kPairThreads, kListedSmemBytes, stream>>>(
+          ws.Gp, ws.Gc, ws.partial, L, kh, P, (uint32_t)items, 0u, ws.counters + 1, lp);
+      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches++ + 1);
+      ++*launches;
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches);
+    if (kh >= 1) e = launch_pruned_layer(s, ws, kh, blocks, meet ? ws.partial : nullptr, stream, launches);
+    if (e != cudaSuccess) return e;
+    if (kh == 0 || s.prune_long) {
+      launch_tiles(s, ws, kh, kh == 0 ? nullptr : ws.prune_info, stream);
+      ++*launches;
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches++ + 1);
   }
   return cudaSuccess;
 }

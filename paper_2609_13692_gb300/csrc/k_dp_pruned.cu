@@ -1,0 +1,743 @@
+// K3 (pruned form): the Sec. 3.1 recurrence on the tiles of k_dp_blocked.cu,
+// over the splits that can be reported instead of all of them.
+//
+// Which splits can be reported.  Let A | B be the reported split of S (the
+// smallest optimal A among those holding S's lowest request) and |A| >= 2,
+// with A1 | A2 the split of A, A1 holding that request.  A1 | (A2 + B) is a
+// split of S too, A1 is a proper subset of A and so the smaller integer, and
+//     F(A1) + F(A2 + B) <= F(A1) + F(A2) + F(B) - w(I(A2 + B))
+//                        = F(A) + F(B) + w(I(A)) - w(I(A2 + B)).
+// If w(I(A)) <= w(I(A2 + B)) it would be at least as good, against the choice
+// of A.  So w(I(A)) > w(I(A2 + B)) >= w(I(S)): on the tables less the
+// universal weight u (k_scatter_zeta.cu), where every w(I(.)) >= 0,
+//     the reported A is a single request or has w(I(A)) > 0.
+// Leaving every other A out changes no F(S) and no split(S).  Requests that
+// share few chunks leave few such A ("members").
+//
+// Members are downward closed (A' within A keeps I(A)), so a member
+// A = (Ta, Ua) has (Ta, {}) a member or a single request.  With the inner bits
+// Ua = (a1, a2), a2 the low kRB bits, the members of one Ta are a list of
+// rows (a1, mask of the a2's):
+//   k_prune_lists    per Ta the row list, and whether it is short (at most
+//                    kPruneRows rows);
+//   k_prune_members  per lowest request the Ta's with a short and those with
+//                    a long list, each in increasing order;
+//   k_dp_pruned      per tile T every short Ta within T, then, where T's own
+//                    list is short too, the self pair and the tile's final
+//                    entries.  Where T has no list, w(I(T, U)) = 0 for all U.
+// Long lists go through the pair kernel of the full recurrence on just those
+// Ta, and tiles with a long list through its row kernel (k_dp_blocked.cu).
+//
+// Measured on one GB300 (whole solve with layout and tables, full recurrence
+// before, pruned after): 28 requests of 20 passages 673 -> 7.6 .. 23 ms by
+// seed (a passage held by 12 to 17 of the 28 decides it), 24 requests of 10
+// passages 11.1 -> 1.3 ms, 26 requests of 40 passages 81 -> 19 .. 29 ms.
+// k_dp_pruned is bound by the integer ALU pipe where a popular passage gives
+// long a1 lists: 55 % of the pipe busy in the heaviest layers of the first 26
+// of the 28 requests, a sixth of it on the bookkeeping per pair, the rest of
+// the time lost to the barrier per pair (the warps of a block have 1, 2 or 4
+// rows of work each).  Also measured there (tile stage at m = 28, seed 1,
+// 15.6 ms): three slots and three blocks per SM 16.8 ms, two slots and three
+// blocks 16.7, two blocks 21.9; the members evaluated one by one instead of by
+// rows 242 ms; the inner bits in natural order 69.9 ms; the warps' row groups
+// dealt in turn per SM instead of by a hash 16.2 ms.
+#include "mpt_internal.cuh"
+
+namespace mpt {
+namespace {
+
+constexpr int kPB = 12;  // inner bits of a tile
+constexpr uint32_t kPMask = (1u << kPB) - 1u;
+constexpr int kPQueue = 512;     // pairs queued between two rounds of evaluation
+constexpr int kQueueShift = 20;  // queue entries: Ta below (L <= 20), rows above
+static_assert(kPruneRows < 1 << (32 - kQueueShift), "queue entries hold the row count");
+constexpr int kRowBytes = 128;
+constexpr uint32_t kUnitSteps = 60;
+constexpr uint32_t kLongSteps = 9000;  // a pair of the full recurrence runs 2,187 units of 243 steps on 8 warps
+constexpr int kPruneMinPairs = 16;     // pairs that a further block of a tile has to have
+
+// Shape of the kernel for 32-bit keys (rows of 32) and 64-bit keys (rows of
+// 16): one thread per row.
+template <typename Key>
+struct PrunedCfg {
+  static constexpr int kRB = sizeof(Key) == 4 ? 5 : 4;
+  static constexpr int kRow = 1 << kRB;
+  static constexpr int kRows = 1 << (kPB - kRB);  // = threads per block
+  static constexpr int kLogWarps = kPB - kRB - 5;
+  static constexpr int kBlocks = sizeof(Key) == 4 ? 4 : 2;  // per SM
+  static constexpr int kSlots = 2;
+  static constexpr int kSlotBytes = (kRows + kPruneRows) * kRowBytes;  // Y window, X rows
+  static constexpr int kTileBytes = kRows * (kRow + 1) * (int)sizeof(Key);  // a tile's keys, rows kRow + 1 apart
+  static constexpr int kSeqStride = kRows + 2;  // so that a row's entries lie in different banks
+  static constexpr int kSeqBytes = kRow * kSeqStride * 2;
+  static constexpr int kSmem = kSlots * kSlotBytes + kSeqBytes + kPQueue * 4;
+  static_assert(kSlotBytes >= kTileBytes, "a tile's keys fit a slot");
+  static_assert((kSmem + 3072) * kBlocks <= 228 * 1024, "blocks per SM");
+};
+
+// Row list of every Ta.  A warp reads 32 entries of w(I(Ta, .)) at a time;
+// the ballot of the non-zero ones is the mask of one row of 32, or of two
+// rows of 16.  info: 0 when Ta has no member, else rows | members << 8 |
+// kListLong when they are more than kPruneRows or, where the pair kernel runs
+// (long_ok), cost more than a pair there | kTileLong when the tile T = Ta is
+// left to the row kernel (a long list, or more than kPruneSelf members).
+// Cost: a row takes as many warps as have a lane whose row holds a1, each for
+// its steps and the loads, here kUnitSteps steps' worth.
+template <typename Key, typename Tab>
+__global__ void __launch_bounds__(256)
+k_prune_lists(int L, bool long_ok, const Tab* __restrict__ wIr, uint32_t* __restrict__ info, uint2* __restrict__ rows) {
+  constexpr int kRB = PrunedCfg<Key>::kRB;
+  constexpr int kHalves = 32 >> kRB;
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t Ta = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; Ta < (1u << L); Ta += warps) {
+    const Tab* win = wIr + ((size_t)Ta << kPB);
+    if (Ta == 0 || ((Ta & (Ta - 1u)) != 0 && win[0] == 0)) {
+      if (lane == 0) info[Ta] = 0;
+      continue;
+    }
+    uint2* out = rows + (size_t)Ta * kPruneRows;
+    uint32_t n = 0, members = 0, cost = 0;
+    for (uint32_t base = 0; base <= kPMask; base += 256) {
+      bool nz[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) nz[k] = win[base + 32u * k + lane] != 0;
+      if (base == 0 && lane == 0) nz[0] = true;  // (Ta, {}): a member, or a single request
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, nz[k]);
+        members += (uint32_t)__popc(bal);
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h) {
+          const uint32_t mask = kHalves == 1 ? bal : (bal >> (16 * h)) & 0xFFFFu;
+          if (mask) {
+            const uint32_t a1 = (base + 32u * k) / (1u << kRB) + h;
+            const uint32_t steps =
+                __reduce_add_sync(0xFFFFFFFFu, (mask >> lane & 1u) ? (1u << kRB) >> __popc(lane) : 0u);
+            cost += (steps + kUnitSteps) << (PrunedCfg<Key>::kLogWarps - __popc(a1 >> 5));
+            if (lane == 0 && n < (uint32_t)kPruneRows) out[n] = make_uint2(a1, mask);
+            ++n;
+          }
+        }
+      }
+    }
+    if (lane == 0) {
+      const bool is_long = n > (uint32_t)kPruneRows || (long_ok && cost > kLongSteps);
+      info[Ta] = min(n, 255u) | (members << 8) | (is_long ? kListLong : 0u) |
+                 (is_long || members > (uint32_t)kPruneSelf ? kTileLong : 0u);
+    }
+  }
+}
+
+// Ta's with lowest request l: 2^(L-1-l) of them, kept in this region of the
+// two member arrays.
+__host__ __device__ __forceinline__ uint32_t member_base(int L, int l) { return (1u << L) - (1u << (L - l)); }
+
+// One block per lowest request: the Ta's with short and with long lists, each
+// in increasing order (kPer consecutive candidates per thread and round).
+__global__ void __launch_bounds__(1024)
+k_prune_members(int L, const uint32_t* __restrict__ info, uint32_t* __restrict__ short_ta,
+                uint32_t* __restrict__ long_ta, uint32_t* __restrict__ member_n) {
+  constexpr int kPer = 8;
+  __shared__ uint32_t ws[32], wl[32];
+  const int l = blockIdx.x;
+  const uint32_t total = 1u << (L - 1 - l);
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t* so = short_ta + member_base(L, l);
+  uint32_t* lo = long_ta + member_base(L, l);
+  uint32_t ns = 0, nl = 0;
+  for (uint32_t base = 0; base < total; base += 1024 * kPer) {
+    uint32_t c[kPer];
+    uint32_t ks = 0, kl = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t h = base + threadIdx.x * kPer + (uint32_t)k;
+      c[k] = h < total ? info[(h << (l + 1)) | (1u << l)] : 0u;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      ks += c[k] != 0 && !(c[k] & kListLong);
+      kl += (c[k] & kListLong) != 0;
+    }
+    uint32_t is = ks, il = kl;
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t a = __shfl_up_sync(0xFFFFFFFFu, is, off), b = __shfl_up_sync(0xFFFFFFFFu, il, off);
+      if (lane >= (uint32_t)off) {
+        is += a;
+        il += b;
+      }
+    }
+    if (lane == 31) {
+      ws[warp] = is;
+      wl[warp] = il;
+    }
+    __syncthreads();
+    uint32_t ts = 0, tl = 0, bs = 0, bl = 0;
+    for (uint32_t q = 0; q < 32; ++q) {
+      bs += q < warp ? ws[q] : 0u;
+      bl += q < warp ? wl[q] : 0u;
+      ts += ws[q];
+      tl += wl[q];
+    }
+    uint32_t ps = ns + bs + is - ks, pl = nl + bl + il - kl;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t Ta = ((base + threadIdx.x * kPer + (uint32_t)k) << (l + 1)) | (1u << l);
+      if (c[k] & kListLong)
+        lo[pl++] = Ta;
+      else if (c[k] != 0)
+        so[ps++] = Ta;
+    }
+    ns += ts;
+    nl += tl;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    member_n[l] = ns;
+    member_n[kMaxMembersL + l] = nl;
+  }
+}
+
+__device__ __forceinline__ uint32_t min_keep(uint32_t a, uint32_t b, bool* keep) { return __vibmin_u32(a, b, keep); }
+__device__ __forceinline__ unsigned long long min_keep(unsigned long long a, unsigned long long b, bool* keep) {
+  *keep = a <= b;
+  return *keep ? a : b;
+}
+__device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_sync(0xFFFFFFFFu, v); }
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
+  for (int off = 16; off > 0; off >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, v, off);
+    v = o < v ? o : v;
+  }
+  return v;
+}
+
+__device__ __forceinline__ void pcopy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// One 128-byte window row; `swz` (a multiple of 16) is XOR-ed into the offsets of
+// its 16-byte chunks.  Window rows are kept with swz = (row mod 8) * 16, so
+// that lanes reading the same chunk of consecutive rows hit different banks.
+template <typename Key, int kRow>
+__device__ __forceinline__ void pload_row(Key (&v)[kRow], const char* p, uint32_t swz) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint4 t = *reinterpret_cast<const uint4*>(p + (((uint32_t)c << 4) ^ swz));
+    if constexpr (sizeof(Key) == 4) {
+      v[4 * c] = t.x;
+      v[4 * c + 1] = t.y;
+      v[4 * c + 2] = t.z;
+      v[4 * c + 3] = t.w;
+    } else {
+      v[2 * c] = ((Key)t.y << 32) | t.x;
+      v[2 * c + 1] = ((Key)t.w << 32) | t.z;
+    }
+  }
+}
+
+// acc[s2] = min over the a2 of `mask` within s2 of x[a2] + y[s2 ^ a2]; with
+// kAll the mask is full.  The mask is the same in every lane: each a2, and
+// each 16 bytes of x, is one uniform branch around its steps.  x is read as it
+// is needed, which keeps the kernel within 128 registers.
+template <typename Key, int kRow, bool kAll>
+__device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key (&y)[kRow], uint32_t mask) {
+  constexpr int kPer = 16 / (int)sizeof(Key);
+#pragma unroll
+  for (int g = 0; g < kRow; g += kPer) {
+    if (kAll || (mask >> g & ((1u << kPer) - 1u))) {
+      const uint4 t = *reinterpret_cast<const uint4*>(x + g * (int)sizeof(Key));
+      Key v[kPer];
+      if constexpr (sizeof(Key) == 4) {
+        v[0] = t.x;
+        v[1] = t.y;
+        v[2] = t.z;
+        v[3] = t.w;
+      } else {
+        v[0] = ((Key)t.y << 32) | t.x;
+        v[1] = ((Key)t.w << 32) | t.z;
+      }
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const int a2 = g + q;
+        if (kAll || (mask >> a2 & 1u)) {
+#pragma unroll
+          for (int s2 = 0; s2 < kRow; ++s2) {
+            if ((a2 & s2) == a2) {
+              const Key k = v[q] + y[s2 ^ a2];
+              acc[s2] = k < acc[s2] ? k : acc[s2];
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+// One tile T with |T| = kh >= 1 per block, or `items` blocks per tile that
+// each take every items-th pair.  Thread = row s1 of the tile, with its
+// kRow outputs' best keys in registers and, in shared memory, the numbers of
+// their pairs in the queue (written only on a strict improvement, the pairs
+// coming in increasing Ta).  Per pair the complement window Y and the listed
+// rows of X are copied to shared memory, kSlots - 1 pairs ahead of the steps;
+// one barrier per pair.  Every lane of a warp runs the same (a1, mask) at a
+// time, with those lanes idle whose row does not hold a1, so that X is read
+// by broadcast.
+// The inner bits are stored in an order (perm) that puts those of the request
+// sets that cost most first into a2, where a listed row is then one register
+// convolution without idle lanes, and next into the bits that tell the warps
+// apart.  The warps are dealt the row groups in an order that varies with
+// the block: rows with more of a list's a1 bits take longer, and the blocks
+// of one SM then load its four sub-partitions about alike.
+// Blocks of one tile, rounds of one block beyond the queue and, with
+// long_lists, the pair kernel's minima meet in `partial`: (key << 32 | Ta),
+// 32-bit keys only.  The block that finishes last (done[]) goes on to the
+// tile's entries.
+template <typename Key, typename Tab>
+__global__ void __launch_bounds__(PrunedCfg<Key>::kRows, PrunedCfg<Key>::kBlocks)
+k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
+            const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
+            const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* __restrict__ done, Key* Gp,
+            Key* Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
+  using C = PrunedCfg<Key>;
+  constexpr int kRB = C::kRB, kRow = C::kRow, NT = C::kRows, kWarps = NT / 32;
+  constexpr uint32_t kFull = 0xFFFFFFFFu >> (32 - kRow);
+  constexpr Key kNone = ~(Key)0;
+  constexpr uint32_t kSelf = 0xFFFFu, kListed = 0x8000u;  // pair numbers of the self pair and of listed entries
+  static_assert(kPQueue <= 0x8000, "pair numbers fit beside the two marks");
+  extern __shared__ __align__(16) char psm[];
+  Key* skey = reinterpret_cast<Key*>(psm + C::kSlotBytes);  // after the pairs: keys, rows kRow + 1 apart
+  uint16_t* seq = reinterpret_cast<uint16_t*>(psm + C::kSlots * C::kSlotBytes);  // [in-row entry][thread]
+  uint32_t* queue = reinterpret_cast<uint32_t*>(psm + C::kSlots * C::kSlotBytes + C::kSeqBytes);
+  __shared__ uint32_t warp_n[kWarps];
+  __shared__ uint2 s_rows[C::kSlots][kPruneRows];  // (a1 | rows << 16, mask)
+  // listed entries of T: F << b, split, Ua, row of the list; by level, levels' sizes
+  __shared__ Key s_f[kPruneSelf];
+  __shared__ uint32_t s_sp[kPruneSelf], s_start[kPB + 2];
+  __shared__ uint16_t s_u[kPruneSelf];
+  __shared__ uint8_t s_k[kPruneSelf], s_order[kPruneSelf];
+  __shared__ uint32_t s_last;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t tiles = gridDim.x / items, tile = blockIdx.x % tiles, item = blockIdx.x / tiles;
+  const uint32_t T = colex_unrank((unsigned long long)tile, kh, L);
+  if (MPT_BAD(flags, T < (1u << L) && __popc(T) == kh)) return;
+  const uint32_t iT = info[T];
+  const bool long_tile = (iT & kTileLong) != 0;
+  if (long_tile && kh == 1) return;  // no pairs: the row kernel does it all
+  const uint32_t cT = (iT >> 8) & 0x1FFFu;
+  const int l = __ffs(T) - 1;
+  const uint32_t low = 1u << l, rest = T ^ low;
+  // (the blocks of one SM differ by a multiple of 4, hence the hash)
+  const uint32_t rot = (blockIdx.x * 2654435761u) >> (32 - C::kLogWarps);
+  const uint32_t s1 = lane | (((warp + rot) & (kWarps - 1)) << 5);
+  auto key_at = [&](uint32_t U) -> Key& { return skey[U + (U >> kRB)]; };
+  auto seq_at = [&](uint32_t U) -> uint16_t& {  // in the column of the thread that has the row
+    const uint32_t r = U >> kRB;
+    return seq[(U & (kRow - 1)) * C::kSeqStride + ((r & 31u) | ((((r >> 5) + kWarps - rot) & (kWarps - 1)) << 5))];
+  };
+
+  Key bk[kRow];
+#pragma unroll
+  for (int i = 0; i < kRow; ++i) {
+    bk[i] = kNone;
+    seq[i * C::kSeqStride + tid] = 0;
+  }
+
+  auto stage_window = [&](char* slot, const Key* win) {
+    const char* y = reinterpret_cast<const char*>(win);
+    const uint32_t c0 = tid >> 3, col = (tid & 7u) * 16u, swz = col ^ ((c0 & 7u) * 16u);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t r = c0 + (uint32_t)(j * (NT / 8));
+      pcopy16(slot + r * kRowBytes + swz, y + r * kRowBytes + col);
+    }
+  };
+  // The row list of queued pair p: rows tid / 8 and tid / 8 + NT / 8 (at most
+  // kPruneRows in all) of this thread's copies, read one pair ahead of them.
+  constexpr int kHeld = (kPruneRows * 8 + NT - 1) / NT;
+  uint2 held[kHeld];
+  auto hold = [&](uint32_t p) {
+    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = queue[p] >> kQueueShift;
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j) {
+      const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
+      if (r < n) held[j] = rows[(size_t)Tp * kPruneRows + r];
+    }
+  };
+  auto stage = [&](uint32_t p, uint32_t s) {
+    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = queue[p] >> kQueueShift;
+    char* slot = psm + s * C::kSlotBytes;
+    const uint32_t col = (tid & 7u) * 16u;
+    const char* x = reinterpret_cast<const char*>(Gp + ((size_t)Tp << kPB));
+    stage_window(slot, Gc + ((size_t)(T ^ Tp) << kPB));
+#pragma unroll
+    for (int j = 0; j < kHeld; ++j) {
+      const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
+      if (r < n) {
+        if (col == 0) s_rows[s][r] = make_uint2(held[j].x | (n << 16), held[j].y);
+        pcopy16(slot + (NT + r) * kRowBytes + col, x + held[j].x * kRowBytes + col);
+      }
+    }
+  };
+  // Candidates: the short lists of lowest request l, or the proper parts of T
+  // holding it when those are fewer; both in increasing order.  A queue entry,
+  // or 0.
+  const uint32_t nm = member_n[l], np = (1u << (kh - 1)) - 1u;
+  const bool by_parts = np < nm;
+  const uint32_t total = by_parts ? np : nm;
+  const uint32_t* mem = short_ta + member_base(L, l);
+  auto candidate = [&](uint32_t i) -> uint32_t {
+    if (i >= total) return 0u;
+    const uint32_t Ta = by_parts ? (low | deposit_bits(i, rest)) : mem[i];
+    if ((Ta & ~T) != 0 || Ta == T) return 0u;
+    const uint32_t c = info[Ta];
+    return c == 0 || (c & kListLong) ? 0u : Ta | ((c & 255u) << kQueueShift);
+  };
+  // Blocks of this tile that take part: as many as there are kPruneMinPairs
+  // pairs for (the same number in each of them).
+  constexpr int kScan = kPQueue / NT;  // runs of 32 candidates that a warp looks at together: one round's finds fit
+  uint32_t parts = 1;
+  if (items > 1) {
+    uint32_t n = 0;
+    for (uint32_t base = tid; base < total; base += kScan * NT) {
+#pragma unroll
+      for (int k = 0; k < kScan; ++k) n += candidate(base + (uint32_t)(k * NT)) != 0;
+    }
+    n = __reduce_add_sync(0xFFFFFFFFu, n);
+    if (lane == 0) warp_n[warp] = n;
+    __syncthreads();
+    n = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) n += warp_n[w];
+    parts = min(items, max(1u, n / (uint32_t)kPruneMinPairs));
+    if (item >= parts) return;
+    __syncthreads();
+  }
+
+  // Keys and Ta's of the round to shared memory; from here thread tid has the
+  // outputs tid, tid + NT, ..
+  auto dump = [&]() {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kRow; ++i) skey[s1 * (kRow + 1) + i] = bk[i];
+    __syncthreads();
+  };
+  unsigned long long* pt = partial + ((size_t)tile << kPB);  // 32-bit keys
+  // the Ta of an output's best pair, before the self pair: from the queue, or
+  // where the minima have met
+  bool met = parts > 1;  // minima in `partial`
+  auto ta_at = [&](uint32_t U) -> uint32_t {
+    return met ? (uint32_t)__ldcg(&pt[U]) : queue[seq_at(U)] & ((1u << kQueueShift) - 1u);
+  };
+  auto to_partial = [&]() {
+    for (uint32_t U = tid; U <= kPMask; U += NT) {
+      const unsigned long long own =
+          ((unsigned long long)key_at(U) << 32) | (queue[seq_at(U)] & ((1u << kQueueShift) - 1u));
+      if (own < __ldcg(&pt[U])) atomicMin(&pt[U], own);
+    }
+  };
+
+  // The pairs, a queue of them at a time.
+  uint32_t found = 0, base = 0;
+  if (long_lists && kh >= 2) {
+    // has T a part with a long list?
+    const uint32_t nl = member_n[kMaxMembersL + l];
+    bool any = false;
+    if (np < nl) {
+      for (uint32_t i = tid; i < np; i += NT) any = any || (info[low | deposit_bits(i, rest)] & kListLong) != 0;
+    } else {
+      for (uint32_t i = tid; i < nl; i += NT) {
+        const uint32_t Ta = long_ta[member_base(L, l) + i];
+        any = any || ((Ta & ~T) == 0 && Ta != T);
+      }
+    }
+    met = __syncthreads_or(any) || met || long_tile;
+  }
+  // phase 0: the pairs; phase 1: the self pair, Ta = T over the tile's own
+  // members, B = (0, U \ Ua) in tile 0
+  for (int phase = kh >= 2 ? 0 : 1; phase < 2;) {
+    uint32_t qn = 1;
+    if (phase == 0) {
+      for (qn = 0; base < total; base += kScan * NT) {
+        uint32_t Ta[kScan], bal[kScan], mine = 0;
+#pragma unroll
+        for (int k = 0; k < kScan; ++k) Ta[k] = candidate(base + (warp * kScan + (uint32_t)k) * 32u + lane);
+#pragma unroll
+        for (int k = 0; k < kScan; ++k) {
+          bal[k] = __ballot_sync(0xFFFFFFFFu, Ta[k] != 0);
+          mine += (uint32_t)__popc(bal[k]);
+        }
+        __syncthreads();
+        if (lane == 0) warp_n[warp] = mine;
+        __syncthreads();
+        uint32_t at = found, sum = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+          at += (uint32_t)w < warp ? warp_n[w] : 0u;
+          sum += warp_n[w];
+        }
+        // this block's pairs are the found ones numbered item, item + parts, ..
+        const uint32_t q0 = (found + parts - 1 - item) / parts, q1 = (found + sum + parts - 1 - item) / parts;
+        if (qn + q1 - q0 > (uint32_t)kPQueue) break;  // next round
+#pragma unroll
+        for (int k = 0; k < kScan; ++k) {
+          const uint32_t o = at + __popc(bal[k] & ((1u << lane) - 1u));
+          if (Ta[k] != 0 && o % parts == item) queue[qn + o / parts - q0] = Ta[k];
+          at += (uint32_t)__popc(bal[k]);
+        }
+        found += sum;
+        qn += q1 - q0;
+      }
+      __syncthreads();
+      // the first kSlots - 1 pairs; a group is committed for each slot, also
+      // without a pair, so that the waits below can count them
+#pragma unroll
+      for (int p = 0; p < C::kSlots - 1; ++p) {
+        if ((uint32_t)p < qn) {
+          hold(p);
+          stage(p, p);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+      if ((uint32_t)(C::kSlots - 1) < qn) hold(C::kSlots - 1);
+    } else {
+      if (cT == 0) break;
+      // The listed entries themselves first, one thread each, level by level
+      // in |Ua| (a member Ua' within Ua has a lower level): a level's entries
+      // are finished, then offered to the later ones.  Then X = their rows.
+      stage_window(psm, Gc);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      const uint32_t n = iT & 255u;
+      if (tid <= (uint32_t)kPB + 1) s_start[tid] = 0;
+      if (warp == 0) {
+        static_assert(kPruneRows <= 32, "one list row per lane");
+        const uint2 own = lane < n ? rows[(size_t)T * kPruneRows + lane] : make_uint2(0u, 0u);
+        uint32_t at = 0;
+        for (uint32_t k = 0; k < n; ++k) {
+          const uint2 e = make_uint2(__shfl_sync(0xFFFFFFFFu, own.x, k), __shfl_sync(0xFFFFFFFFu, own.y, k));
+          if (e.y >> lane & 1u) {
+            const uint32_t i = at + __popc(e.y & ((1u << lane) - 1u));
+            s_u[i] = (uint16_t)((e.x << kRB) | lane);
+            s_k[i] = (uint8_t)k;
+          }
+          if (lane == 0) s_rows[0][k] = make_uint2(e.x | (n << 16), e.y);
+          at += __popc(e.y);
+        }
+      }
+      __syncthreads();
+      static_assert(kPruneSelf <= NT, "one thread per listed entry");
+      const bool mine = tid < cT;
+      const uint32_t u = mine ? s_u[tid] : 0u;
+      const uint32_t level = mine ? (uint32_t)__popc(u) : 32u;
+      const Key w = mine ? (Key)wIr[((size_t)T << kPB) | u] : (Key)0;
+      uint32_t rank = 0;
+      for (uint32_t j = 0; j < cT; ++j) {
+        const uint32_t lj = (uint32_t)__popc(s_u[j]);
+        rank += lj < level || (lj == level && j < tid);
+      }
+      if (mine) {
+        s_order[rank] = (uint8_t)tid;
+        atomicAdd(&s_start[level + 1], 1u);
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      Key best = mine && kh >= 2 ? key_at(u) : kNone;
+      uint32_t ta = mine && kh >= 2 ? ta_at(u) : 0u;
+      for (uint32_t lv = 0, k = 0; k < cT; ++lv) {
+        if (level == lv) {
+          Key f = w;
+          uint32_t A = 0;
+          if (!(kh == 1 && u == 0)) {
+            f = (best >> kPB) - w;
+            A = (((uint32_t)(best & kPMask) + perm.nat(u) - kPMask) << L) | ta;
+          }
+          s_f[tid] = f << kPB;
+          s_sp[tid] = A;
+          *reinterpret_cast<Key*>(psm + (NT + s_k[tid]) * kRowBytes + (u & (kRow - 1)) * sizeof(Key)) = f << kPB;
+        }
+        __syncthreads();
+        for (const uint32_t end = k + s_start[lv + 1]; k < end; ++k) {
+          const uint32_t j = s_order[k], uj = s_u[j], v = u ^ uj;
+          if (mine && level > lv && (uj & ~u) == 0) {
+            const uint32_t r = v >> kRB, off = (v & (kRow - 1)) * (uint32_t)sizeof(Key);
+            const Key c = s_f[j] + *reinterpret_cast<const Key*>(psm + r * kRowBytes + (off ^ ((r & 7u) * 16u)));
+            if (c < best) {  // equal: the smaller Ta stays
+              best = c;
+              ta = T;
+            }
+          }
+        }
+      }
+    }
+    for (uint32_t p = 0, s = 0; p < qn; ++p, s = s + 1 == (uint32_t)C::kSlots ? 0 : s + 1) {
+      // pair p's copies have landed; behind the barrier every thread is done
+      // with pair p - 1, whose slot takes the next pair to be copied
+      asm volatile("cp.async.wait_group %0;" ::"n"(C::kSlots - 2) : "memory");
+      __syncthreads();
+      if (phase == 0) {
+        const uint32_t q = p + (uint32_t)(C::kSlots - 1);
+        if (q < qn) stage(q, s == 0 ? C::kSlots - 1 : s - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (q + 1 < qn) hold(q + 1);
+      }
+      const char* slot = psm + s * C::kSlotBytes;
+      const uint2* list = s_rows[s];
+      const uint32_t n = list[0].x >> 16;
+      Key acc[kRow];
+#pragma unroll
+      for (int i = 0; i < kRow; ++i) acc[i] = kNone;
+      for (uint32_t k = 0; k < n; ++k) {
+        const uint32_t a1 = list[k].x & 0xFFFFu, mask = list[k].y;
+        if ((a1 & ~s1) != 0) continue;
+        Key y[kRow];
+        const uint32_t r = s1 ^ a1;
+        const char* x = slot + (NT + k) * kRowBytes;
+        pload_row<Key, kRow>(y, slot + r * kRowBytes, (r & 7u) * 16u);
+        if (mask == kFull)
+          pconv<Key, kRow, true>(acc, x, y, mask);
+        else
+          pconv<Key, kRow, false>(acc, x, y, mask);
+      }
+      __syncwarp();
+      const uint16_t number = (uint16_t)(phase == 0 ? p : kSelf);
+#pragma unroll
+      for (int i = 0; i < kRow; ++i) {
+        bool keep;  // true when the running best is <= this pair's minimum
+        bk[i] = min_keep(bk[i], acc[i], &keep);
+        if (!keep) seq[i * C::kSeqStride + tid] = number;
+      }
+    }
+    dump();
+    if (phase == 1) break;
+    if constexpr (sizeof(Key) == 4) {
+      if (met || base < total) {
+        to_partial();
+        if (base < total) {  // a further round
+          met = true;
+          __syncthreads();
+#pragma unroll
+          for (int i = 0; i < kRow; ++i) {
+            bk[i] = kNone;
+            seq[i * C::kSeqStride + tid] = 0;
+          }
+          continue;
+        }
+        if (long_tile) return;  // the row kernel goes on from there
+        __threadfence();
+        __syncthreads();
+        if (parts > 1) {
+          if (tid == 0) {
+            const uint32_t before = atomicAdd(&done[tile], 1u);
+            s_last = before == parts - 1;
+            if (s_last) done[tile] = 0;  // for the next layer
+          }
+          __syncthreads();
+          if (!s_last) return;
+          __threadfence();
+        }
+        for (uint32_t U = tid; U <= kPMask; U += NT) {
+          const unsigned long long v = __ldcg(&pt[U]);
+          key_at(U) = (Key)(v >> 32);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kRow; ++i) bk[i] = skey[s1 * (kRow + 1) + i];
+      }
+    }
+    if (long_tile) {
+      // only with the pair and row kernels around (the host's bound)
+      if (tid == 0) atomicOr(flags, kErrWorkspace);
+      return;
+    }
+    phase = 1;
+  }
+
+  // w(I(T, U)) = 0 outside the tile's list; the listed entries replace theirs
+  if (cT != 0) {
+    for (uint32_t i = tid; i < cT; i += NT) {
+      key_at(s_u[i]) = s_f[i];
+      seq_at(s_u[i]) = (uint16_t)(kListed | i);
+    }
+    __syncthreads();
+  }
+  const size_t tbase = (size_t)T << kPB;
+  const uint32_t nat_lo = perm.nat(tid);
+  for (uint32_t U0 = 0; U0 <= kPMask; U0 += NT) {
+    const uint32_t U = U0 | tid, nat = nat_lo | perm.nat(U0);
+    Key key = key_at(U);
+    const uint32_t number = cT != 0 ? seq_at(U) : 0u;
+    uint32_t A;
+    if ((number & kListed) && number != kSelf) {
+      A = s_sp[number & ~kListed];
+    } else {
+      A = (((uint32_t)(key & kPMask) + nat - kPMask) << L) | (number == kSelf ? T : ta_at(U));
+      key &= ~(Key)kPMask;  // F << b
+    }
+    if (MPT_BAD(flags, valid_split(T | (nat << L), A))) continue;
+    Gp[tbase | U] = key;
+    Gc[tbase | U] = key | (Key)(~nat & kPMask);
+    split_rot[tbase | U] = A;
+  }
+}
+
+template <typename Key, typename Tab>
+cudaError_t lists(const Shape& s, const Workspace& ws, const Tab* wIr, cudaStream_t stream, int* launches) {
+  const int64_t warps = (int64_t)1 << s.L;
+  int64_t blocks = (warps + 7) / 8;
+  const int64_t most = sm_count() * 8;
+  if (blocks > most) blocks = most;
+  k_prune_lists<Key><<<(unsigned)blocks, 256, 0, stream>>>(s.L, s.prune_long, wIr, ws.prune_info, ws.prune_rows);
+  k_prune_members<<<(unsigned)s.L, 1024, 0, stream>>>(s.L, ws.prune_info, ws.prune_short, ws.prune_long, ws.prune_n);
+  *launches += 2;
+  return cudaGetLastError();
+}
+
+template <typename Key, typename Tab>
+cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, uint32_t items,
+                  unsigned long long* partial, Key* Gp, Key* Gc, cudaStream_t stream, int* launches) {
+  using C = PrunedCfg<Key>;
+  auto k = k_dp_pruned<Key, Tab>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)(h_binom.v[s.L][kh] * items), C::kRows, C::kSmem, stream>>>(
+      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long, ws.prune_n, partial, ws.prune_done, Gp, Gc,
+      ws.split_rot, ws.counters + 1);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_prune_lists(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
+  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, kPruneSplitTiles * 4, stream);
+  if (e != cudaSuccess) return e;
+  if (s.lean) return lists<uint32_t>(s, ws, ws.fw_rot, stream, launches);
+  return lists<uint32_t>(s, ws, ws.wI_rot, stream, launches);
+}
+
+// Blocks per tile of a layer with 32-bit keys.  The pairs of a tile vary from
+// one to the bound, so a layer is cut so that its longest tile gives blocks of
+// about kPartPairs pairs, as far as kMostBlocks blocks go round; blocks that
+// find no part of theirs leave after counting the tile's pairs.
+uint32_t pruned_items(const Shape& s, int kh) {
+  constexpr double kPartPairs = 48, kMostBlocks = 16384;
+  const double tiles = (double)h_binom.v[s.L][kh];
+  if (tiles > kPruneSplitTiles) return 1;
+  const double P = (double)((1ull << (kh - 1)) - 1ull), most = P < s.prune_most ? P : s.prune_most;
+  const double items = most / kPartPairs < kMostBlocks / tiles ? most / kPartPairs : kMostBlocks / tiles;
+  return items < 1.0 ? 1u : (uint32_t)items;
+}
+
+// Whether the blocks of a layer meet in `partial`.
+bool pruned_meet(const Shape& s, int kh, uint32_t items) {
+  if (kh < 2) return false;
+  const double P = (double)((1ull << (kh - 1)) - 1ull);
+  return s.prune_long || items > 1 || (P < s.prune_most ? P : s.prune_most) > (double)kPQueue;
+}
+
+cudaError_t launch_pruned_layer(const Shape& s, const Workspace& ws, int kh, uint32_t items,
+                                unsigned long long* partial, cudaStream_t stream, int* launches) {
+  if (s.lean) return layer<uint32_t>(s, ws, ws.fw_rot, kh, items, partial, ws.Gp, ws.Gc, stream, launches);
+  return layer<uint32_t>(s, ws, ws.wI_rot, kh, items, partial, ws.Gp, ws.Gc, stream, launches);
+}
+
+}  // namespace mpt

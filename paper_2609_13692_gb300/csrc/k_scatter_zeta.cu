@@ -43,7 +43,8 @@ template <typename G>
 __global__ void __launch_bounds__(kScatterThreads)
 k_scatter(const int64_t* __restrict__ w, const uint64_t* __restrict__ bits, int64_t n, int m, int64_t words,
           G* __restrict__ g, unsigned long long* __restrict__ priv, uint32_t* __restrict__ used_N,
-          int32_t* __restrict__ used_x, int32_t* __restrict__ counters, int64_t slots, bool rotated, int L, int b) {
+          int32_t* __restrict__ used_x, int32_t* __restrict__ counters, int64_t slots, bool rotated, int L, int b,
+          InnerPerm perm) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const uint32_t full = m >= 32 ? 0xFFFFFFFFu : (1u << m) - 1u;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
@@ -56,8 +57,8 @@ k_scatter(const int64_t* __restrict__ w, const uint64_t* __restrict__ bits, int6
         atomicAdd(&priv[__ffs(N) - 1], (unsigned long long)w[x]);
       else if (priv && N == full)  // m >= 2 here: for m = 1 the full set is a singleton
         atomicAdd(&priv[kUniversalSlot], (unsigned long long)w[x]);
-      else if (!MPT_BAD(&counters[1], (rotated ? rot_index(N, L, b) : (size_t)N) < ((size_t)1 << m)))
-        atomicAdd(&g[rotated ? rot_index(N, L, b) : (size_t)N], (G)w[x]);
+      else if (!MPT_BAD(&counters[1], (rotated ? rot_index(N, L, b, perm) : (size_t)N) < ((size_t)1 << m)))
+        atomicAdd(&g[rotated ? rot_index(N, L, b, perm) : (size_t)N], (G)w[x]);
       const int k = atomicAdd(&counters[0], 1);
       if (k < slots) {
         used_N[k] = N;
@@ -260,11 +261,11 @@ cudaError_t launch_scatter(const Shape& s, const Workspace& ws, cudaStream_t str
   if (s.lean)
     k_scatter<<<(unsigned)blocks, kScatterThreads, 0, stream>>>(
         ws.weights, ws.bits, s.n, s.m, s.words, static_cast<unsigned int*>(g), s.blocked ? ws.priv : nullptr,
-        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b);
+        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm);
   else
     k_scatter<<<(unsigned)blocks, kScatterThreads, 0, stream>>>(
         ws.weights, ws.bits, s.n, s.m, s.words, static_cast<unsigned long long*>(g), s.blocked ? ws.priv : nullptr,
-        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b);
+        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm);
   ++*launches;
   return cudaGetLastError();
 }

@@ -38,18 +38,20 @@ enum Offset { kNone, kPiOfS, kPiOfSingletons };
 template <typename Src, typename Dst, typename Op, Offset Off>
 __global__ void __launch_bounds__(kTile * kRowsPerPass)
 k_unrotate(const Src* __restrict__ src, Dst* __restrict__ dst, int L, int b,
-           const unsigned long long* __restrict__ priv, int m) {
+           const unsigned long long* __restrict__ priv, int m, InnerPerm perm) {
   __shared__ Dst t[kTile][kTile + 1];
   __shared__ long long piT[kTile], piU[kTile], pi_all, univ;
+  __shared__ uint32_t nat_of[kTile];  // the stored order of the block's U values undone
   const size_t nT = (size_t)1 << L, nU = (size_t)1 << b;
   const size_t T0 = (size_t)blockIdx.x * kTile, U0 = (size_t)blockIdx.y * kTile;
   const int tx = threadIdx.x, ty = threadIdx.y;
+  if (ty == kRowsPerPass - 1) nat_of[tx] = perm.nat((uint32_t)U0 + tx);
   if (Off != kNone && ty < 3) {
     // row 0: pi of the block's T values (requests 0..L-1), row 1: of its U
     // values (requests L..m-1), row 2, lane 0: of all requests
     long long v = 0;
-    const size_t x = (ty == 0 ? T0 : U0) + tx;
-    if (priv && ty < 2 && x < (ty == 0 ? nT : nU)) {
+    const size_t x = ty == 0 ? T0 + tx : (size_t)perm.nat((uint32_t)U0 + tx);
+    if (priv && ty < 2 && (ty == 0 ? T0 : U0) + tx < (ty == 0 ? nT : nU)) {
       for (uint32_t r = (uint32_t)x; r; r &= r - 1) v += (long long)priv[(ty == 0 ? 0 : L) + __ffs(r) - 1];
     }
     if (ty == 0) piT[tx] = v;
@@ -73,7 +75,8 @@ k_unrotate(const Src* __restrict__ src, Dst* __restrict__ dst, int L, int b,
     const size_t U = U0 + ty + j, T = T0 + tx;
     if (T < nT && U < nU) {
       Dst v = t[tx][ty + j];
-      const uint32_t S = ((uint32_t)U << L) | (uint32_t)T;
+      const size_t nat = nat_of[ty + j];
+      const uint32_t S = ((uint32_t)nat << L) | (uint32_t)T;
       if (Off == kPiOfS) {
         if (S != 0) v += (Dst)(piT[tx] + piU[ty + j] + univ);
       } else if (Off == kPiOfSingletons) {
@@ -83,7 +86,7 @@ k_unrotate(const Src* __restrict__ src, Dst* __restrict__ dst, int L, int b,
         else if ((S & (S - 1)) == 0)
           v += (Dst)(T ? piT[tx] : piU[ty + j]);
       }
-      dst[(U << L) | T] = v;
+      dst[(nat << L) | T] = v;
     }
   }
 }
@@ -92,7 +95,7 @@ template <typename Src, typename Dst, typename Op, Offset Off>
 cudaError_t unrotate(const Src* src, Dst* dst, const Shape& s, const unsigned long long* priv, cudaStream_t stream) {
   const dim3 grid((unsigned)((((size_t)1 << s.L) + kTile - 1) / kTile),
                   (unsigned)((((size_t)1 << s.b) + kTile - 1) / kTile));
-  k_unrotate<Src, Dst, Op, Off><<<grid, dim3(kTile, kRowsPerPass), 0, stream>>>(src, dst, s.L, s.b, priv, s.m);
+  k_unrotate<Src, Dst, Op, Off><<<grid, dim3(kTile, kRowsPerPass), 0, stream>>>(src, dst, s.L, s.b, priv, s.m, s.perm);
   return cudaGetLastError();
 }
 

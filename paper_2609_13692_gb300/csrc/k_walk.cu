@@ -27,7 +27,7 @@ constexpr int kMaxM = 32;
 __global__ void __launch_bounds__(kWalkThreads)
 k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F, const int32_t* __restrict__ F32,
        const uint32_t* __restrict__ Gp, const unsigned long long* __restrict__ Gp64,
-       const unsigned long long* __restrict__ priv, int L, int b, const uint32_t* __restrict__ used_N,
+       const unsigned long long* __restrict__ priv, int L, int b, InnerPerm perm, const uint32_t* __restrict__ used_N,
        const int32_t* __restrict__ used_x, int32_t* __restrict__ counters, int64_t slots,
        unsigned long long* __restrict__ keys, int64_t* __restrict__ perm_offsets, int64_t* __restrict__ perm_chunks,
        int32_t* __restrict__ dfs, int64_t* __restrict__ opt) {
@@ -65,7 +65,7 @@ k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F,
         continue;
       }
       // blocked path: split and F (as F << b in Gp) in rotated order
-      const uint32_t A = (Gp || Gp64) ? split[rot_index(S, L, b)] : split[S];
+      const uint32_t A = (Gp || Gp64) ? split[rot_index(S, L, b, perm)] : split[S];
       if (A == 0 || (A & ~S) != 0 || A == S || sp + 2 > 2 * kMaxM) {
         bad = 1;
         break;
@@ -83,8 +83,8 @@ k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F,
       for (int i = 0; i < m; ++i) pi_all += (int64_t)priv[i];
       pi_all += (int64_t)priv[kUniversalSlot];
     }
-    *opt = Gp64 ? (int64_t)(Gp64[rot_index(full, L, b)] >> b) + pi_all
-           : Gp ? (int64_t)(Gp[rot_index(full, L, b)] >> b) + pi_all
+    *opt = Gp64 ? (int64_t)(Gp64[rot_index(full, L, b, perm)] >> b) + pi_all
+           : Gp ? (int64_t)(Gp[rot_index(full, L, b, perm)] >> b) + pi_all
                 : (F ? F[full] : (int64_t)F32[full]);
   }
   __syncthreads();
@@ -168,7 +168,7 @@ cudaError_t launch_walk(const Shape& s, const Workspace& ws, cudaStream_t stream
   k_walk<<<1, kWalkThreads, 0, stream>>>(s.m, s.blocked ? ws.split_rot : ws.split, s.lean ? nullptr : ws.F,
                                          s.lean ? ws.fw : nullptr, s.blocked && !s.wide ? ws.Gp : nullptr,
                                          s.blocked && s.wide ? ws.Gp64 : nullptr, s.blocked ? ws.priv : nullptr,
-                                         s.L, s.b, ws.used_N,
+                                         s.L, s.b, s.perm, ws.used_N,
                                          ws.used_x, ws.counters, s.slots, ws.keys,
                                          ws.perm_offsets, ws.perm_chunks, ws.dfs, ws.opt);
   ++*launches;

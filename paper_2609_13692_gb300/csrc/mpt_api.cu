@@ -2,6 +2,7 @@
 // carve-up and the order of launches.  Every step of the solve itself runs in
 // the kernels of k_scatter_zeta.cu, k_dp_blocked.cu / k_dp_general.cu and
 // k_walk.cu, all on the caller's stream.
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 #include <cstring>
@@ -18,6 +19,12 @@ struct mpt_ctx {
   std::vector<uint64_t> bits;
   int64_t sum_w = 0;     // sum_i w(R_i)
   int64_t shared_w = 0;  // the same less the chunks one or every request needs
+  // distinct request sets N_x of the other chunks, when there are at most
+  // kMaxSupports of those chunks (many_supports otherwise)
+  std::vector<uint32_t> supports;
+  bool many_supports = false;
+  mpt::InnerPerm perm;          // stored order of the inner bits in the pruned recurrence
+  mpt::Shape solved_shape{};    // of the last solve: as `shape`, with the order its tables have
   int32_t mode = MPT_DP_AUTO;
   int32_t tables = MPT_TABLES_INT64;
   void* own_ws = nullptr;
@@ -70,6 +77,89 @@ bool use_wide(const mpt_ctx* c) {
   return c->mode == MPT_DP_AUTO && !blocked_feasible(c) && wide_feasible(c);
 }
 
+constexpr size_t kMaxSupports = 8192;
+
+// Whether a one-shot AUTO solve takes the pruned recurrence
+// (k_dp_pruned.cu), from the sets N_x alone.  Its members are the parts of
+// some N_x, so with N = (N_T, N_U) the tile and inner bits of N_x:
+//   * the members (Ta, Ua) of one Ta number at most sum over N_T containing
+//     Ta of 2^|N_U|, their rows at most the sum of 2^|row bits of N_U|, and no
+//     Ta has more than the single request in it.  When no request's sums
+//     exceed the limits of a short list, there is no long one and the pair
+//     and row kernels are not launched at all;
+//   * the pairs with a member Ta are, over all tiles T, at most
+//     sum over N of sum over Ta within N_T of 2^(L - 1 - lowest(Ta) - (|Ta| - 1)),
+//     plus one per T for the single request.  A Ta whose lowest request is the
+//     j-th of N_T contributes 2^(L - 1 - e_j) (3/2)^(requests of N_T above it)
+//     over all choices of the others.
+// A pair whose list lies in N_U alone takes 3^|N_U| 2^(b - |N_U|) of the 3^b
+// splits of a full pair, at about a third of its rate.  The pruned form is
+// taken when the pairs' times so estimated are below 0.6 of the full
+// recurrence's, or when there is no long list.  Leave-one-out requests (every
+// N_x all but one) stay with the full form.
+void prune_shape(mpt_ctx* c) {
+  mpt::Shape& s = c->shape;
+  c->perm = mpt::InnerPerm{};
+  s.pruned = s.prune_long = false;
+  if (c->mode != MPT_DP_AUTO || !s.blocked || s.wide || s.L < 1 || c->many_supports) return;
+  double members[32], rows[32], tas[32];
+  for (int l = 0; l < s.L; ++l) members[l] = rows[l] = tas[l] = 1.0;
+  double time = 0.05 * (double)(1ull << s.L);
+  double full = 0.5;
+  for (int l = 0; l < s.L; ++l) full *= 3.0;
+  for (uint32_t N : c->supports) {
+    const uint32_t T = N & ((1u << s.L) - 1u), U = N >> s.L;
+    double above = 1.0, above2 = 1.0, here = 0.0;
+    for (int l = s.L - 1; l >= 0; --l) {
+      if (!((T >> l) & 1u)) continue;
+      members[l] += (double)(1ull << __builtin_popcount(U));
+      rows[l] += (double)(1ull << __builtin_popcount(U >> 5));
+      here += (double)(1ull << (s.L - 1 - l)) * above;
+      tas[l] += above2;
+      above *= 1.5;
+      above2 *= 2.0;
+    }
+    // of a full pair's time: the inner splits, at a third of its rate
+    double inner = 3.0;
+    for (int u = __builtin_popcount(U); u < s.b; ++u) inner *= 2.0 / 3.0;
+    time += here * (inner + 0.05 < 1.0 ? inner + 0.05 : 1.0);
+  }
+  for (int l = 0; l < s.L; ++l)
+    s.prune_long = s.prune_long || members[l] > (double)mpt::kPruneSelf || rows[l] > (double)mpt::kPruneRows;
+  s.prune_most = *std::max_element(tas, tas + s.L);
+  s.pruned = !s.prune_long || time < 0.6 * full;
+  if (!s.pruned) return;
+  // Stored order of the inner bits: those of the N_x whose members cost most
+  // (pairs times inner splits) first.  The first five are the in-row bits,
+  // the next two tell the warps of a block apart, the last five its lanes.
+  std::vector<std::pair<double, uint32_t>> cost;
+  try {
+    for (uint32_t N : c->supports) {
+      const uint32_t T = N & ((1u << s.L) - 1u), U = N >> s.L;
+      double sum = 0.0, above = 1.0;
+      for (int l = s.L - 1; l >= 0; --l)
+        if ((T >> l) & 1u) {
+          sum += (double)(1ull << (s.L - 1 - l)) * above;
+          above *= 1.5;
+        }
+      for (int u = __builtin_popcount(U); u > 0; --u) sum *= 1.5;
+      cost.emplace_back(-sum, U);
+    }
+  } catch (...) {
+    return;  // the natural order
+  }
+  std::sort(cost.begin(), cost.end());
+  static const uint8_t place[12] = {0, 1, 2, 3, 4, 11, 10, 9, 8, 7, 6, 5};
+  uint32_t left = (1u << s.b) - 1u;
+  int n = 0;
+  cost.emplace_back(0.0, left);
+  for (const auto& e : cost)
+    for (uint32_t r = e.second & left; r; r &= r - 1) {
+      c->perm.to_nat[place[n++]] = (uint8_t)__builtin_ctz(r);
+      left &= ~(r & (~r + 1u));
+    }
+}
+
 void refresh_shape(mpt_ctx* c) {
   mpt::Shape& s = c->shape;
   s.blocked = use_blocked(c);
@@ -80,6 +170,7 @@ void refresh_shape(mpt_ctx* c) {
   s.partial_entries = !s.blocked ? 0
                       : s.wide   ? (mpt::wide_partial_slots(s.m, s.b) << s.b)
                                  : mpt::blocked_partial_entries(s.m, s.b);
+  prune_shape(c);
 }
 
 mpt_status cuda_fail(mpt_ctx* c, cudaError_t e, const char* what) {
@@ -158,6 +249,18 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
   ws->perm_chunks = reinterpret_cast<int64_t*>(take(slots * 8));
   ws->dfs = reinterpret_cast<int32_t*>(take((size_t)s.m * 4));
   ws->opt = reinterpret_cast<int64_t*>(take(8));
+  // after everything else, so that the rest sits where it does without them
+  ws->prune_info = ws->prune_short = ws->prune_long = ws->prune_n = ws->prune_done = nullptr;
+  ws->prune_rows = nullptr;
+  if (s.pruned) {
+    const size_t P = (size_t)1 << s.L;
+    ws->prune_info = reinterpret_cast<uint32_t*>(take(P * 4));
+    ws->prune_rows = reinterpret_cast<uint2*>(take(P * mpt::kPruneRows * sizeof(uint2)));
+    ws->prune_short = reinterpret_cast<uint32_t*>(take(P * 4));
+    ws->prune_long = reinterpret_cast<uint32_t*>(take(P * 4));
+    ws->prune_n = reinterpret_cast<uint32_t*>(take(2 * mpt::kMaxMembersL * 4));
+    ws->prune_done = reinterpret_cast<uint32_t*>(take(mpt::kPruneSplitTiles * 4));
+  }
   return off;
 }
 
@@ -214,6 +317,8 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
   // exactly one request needs (per word, the bits seen once, s1, but not
   // twice, s2) and, for m >= 2, m times those that every request needs
   int64_t private_w = 0;
+  std::vector<uint32_t> supports;
+  bool many_supports = false;
   for (int64_t j = 0; j < words; ++j) {
     uint64_t s1 = 0, s2 = 0, all = ~0ull;
     for (int i = 0; i < m; ++i) {
@@ -225,7 +330,22 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
     for (uint64_t v = s1 & ~s2; v; v &= v - 1) private_w += weights[j * 64 + __builtin_ctzll(v)];
     if (m >= 2)
       for (uint64_t v = all; v; v &= v - 1) private_w += (int64_t)m * weights[j * 64 + __builtin_ctzll(v)];
+    // the other shared chunks' request sets (only instances with tile bits use them)
+    for (uint64_t v = s2 & ~all; v && m > mpt::blocked_tile_bits(m) && !many_supports; v &= v - 1) {
+      const int bit = __builtin_ctzll(v);
+      uint32_t N = 0;
+      for (int i = 0; i < m; ++i)
+        N |= (uint32_t)((req_bits[(size_t)i * (size_t)words + (size_t)j] >> bit) & 1u) << i;
+      try {
+        supports.push_back(N);
+      } catch (...) {
+        return MPT_ERR_OUT_OF_MEMORY;
+      }
+      many_supports = supports.size() > kMaxSupports;
+    }
   }
+  std::sort(supports.begin(), supports.end());
+  supports.erase(std::unique(supports.begin(), supports.end()), supports.end());
   mpt_ctx* c = new (std::nothrow) mpt_ctx();
   if (!c) return MPT_ERR_OUT_OF_MEMORY;
   try {
@@ -241,6 +361,8 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
   c->shape.slots = slots;
   c->sum_w = sum;
   c->shared_w = sum - private_w;
+  c->supports = std::move(supports);
+  c->many_supports = many_supports;
   refresh_shape(c);
   *out = c;
   return MPT_OK;
@@ -322,9 +444,8 @@ mpt_status bind_workspace(mpt_ctx* c, void* d_workspace, size_t workspace_bytes,
 }
 
 // Input copies (unless this workspace already holds them), K1 and K2.
-mpt_status run_front(mpt_ctx* c, const mpt::Workspace& ws, char* base, cudaStream_t stream, int* launches,
+mpt_status run_front(mpt_ctx* c, const mpt::Shape& s, const mpt::Workspace& ws, char* base, cudaStream_t stream, int* launches,
                      cudaEvent_t* ev) {
-  const mpt::Shape& s = c->shape;
   auto mark = [&](int i) {
     if (ev) cudaEventRecord(ev[i], stream);
   };
@@ -361,9 +482,8 @@ mpt_status run_steps(mpt_ctx* c, const mpt::Workspace& ws, cudaStream_t stream, 
 }
 
 // The walk, the copies of its results and the consistency flags.
-mpt_status run_back(mpt_ctx* c, const mpt::Workspace& ws, cudaStream_t stream, int* launches, cudaEvent_t* ev,
-                    int64_t* opt_out) {
-  const mpt::Shape& s = c->shape;
+mpt_status run_back(mpt_ctx* c, const mpt::Shape& s, const mpt::Workspace& ws, cudaStream_t stream, int* launches,
+                    cudaEvent_t* ev, int64_t* opt_out, uint32_t* pairs_run = nullptr) {
   auto mark = [&](int i) {
     if (ev) cudaEventRecord(ev[i], stream);
   };
@@ -396,6 +516,7 @@ mpt_status run_back(mpt_ctx* c, const mpt::Workspace& ws, cudaStream_t stream, i
     return (counters[1] & mpt::kErrTimeout) ? MPT_ERR_TIMEOUT : MPT_ERR_INTERNAL;
   }
   *opt_out = opt;
+  if (pairs_run) *pairs_run = (uint32_t)counters[2];
   return MPT_OK;
 }
 
@@ -405,7 +526,8 @@ mpt_status mpt_solve(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes, vo
   mpt_ctx* c = ctx;
   if (!c || !opt_cost) return MPT_ERR_INVALID_ARG;
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_ptr);
-  const mpt::Shape& s = c->shape;
+  mpt::Shape s = c->shape;
+  if (s.pruned) s.perm = c->perm;
   c->solved = false;
   c->staged_next = -1;
   c->err.clear();
@@ -429,17 +551,23 @@ mpt_status mpt_solve(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes, vo
 
   int launches = 0;
   const size_t N = (size_t)1 << s.m;
-  if ((st = run_front(c, ws, base, stream, &launches, ev)) != MPT_OK) return st;
+  if ((st = run_front(c, s, ws, base, stream, &launches, ev)) != MPT_OK) return st;
   mpt::BlockedTiming timing{};
   if (s.blocked) {
     timing.pair_ev = ev ? ev + 7 : nullptr;
     timing.tile_ev = ev ? ev + 7 + 2 * dp_launches : nullptr;
   }
-  if ((st = run_steps(c, ws, stream, &launches, &timing, 0, -1)) != MPT_OK) return st;
+  if (s.pruned)
+    MPT_CK(mpt::launch_dp_pruned(s, ws, stream, &launches, &timing), "pruned DP kernels");
+  else if ((st = run_steps(c, ws, stream, &launches, &timing, 0, -1)) != MPT_OK)
+    return st;
   if (ev) cudaEventRecord(ev[4], stream);
   int64_t opt = 0;
-  if ((st = run_back(c, ws, stream, &launches, ev, &opt)) != MPT_OK) return st;
+  uint32_t pairs_run = 0;
+  if ((st = run_back(c, s, ws, stream, &launches, ev, &opt, &pairs_run)) != MPT_OK) return st;
+  if (s.pruned) timing.pair_splits = (double)pairs_run * 531441.0;  // 3^12 splits per pair of windows
   c->ws = ws;
+  c->solved_shape = s;
   c->opt = opt;
   c->resident = base;
 
@@ -494,7 +622,7 @@ mpt_status mpt_solve_begin(mpt_ctx* ctx, void* d_workspace, size_t workspace_byt
   mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   int launches = 0;
-  if ((st = run_front(c, ws, base, stream, &launches, nullptr)) != MPT_OK) return st;
+  if ((st = run_front(c, c->shape, ws, base, stream, &launches, nullptr)) != MPT_OK) return st;
   if ((st = run_steps(c, ws, stream, &launches, nullptr, 0, 1)) != MPT_OK) return st;
   c->resident = base;
   c->staged_base = base;
@@ -549,8 +677,9 @@ mpt_status mpt_solve_end(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes
   if (base != c->staged_base) return MPT_ERR_INVALID_ARG;
   int launches = 0;
   int64_t opt = 0;
-  if ((st = run_back(c, ws, reinterpret_cast<cudaStream_t>(stream_ptr), &launches, nullptr, &opt)) != MPT_OK) return st;
+  if ((st = run_back(c, c->shape, ws, reinterpret_cast<cudaStream_t>(stream_ptr), &launches, nullptr, &opt)) != MPT_OK) return st;
   c->ws = ws;
+  c->solved_shape = c->shape;
   c->opt = opt;
   c->staged_next = -1;
   std::memset(&c->prof, 0, sizeof(c->prof));
@@ -568,7 +697,7 @@ namespace {
 // Fill the natural-order views of a blocked solve's tables (once per solve).
 mpt_status ensure_natural(mpt_ctx* c) {
   if (c->natural) return MPT_OK;
-  const mpt::Shape& s = c->shape;
+  const mpt::Shape& s = c->solved_shape;
   const mpt::Workspace& ws = c->ws;
   int prev = 0;
   MPT_CK(cudaGetDevice(&prev), "cudaGetDevice");

@@ -232,12 +232,38 @@ struct Workspace {
   // instead of to g, and the rotated tables hold w(I) and F less them (see
   // the scatter in k_scatter_zeta.cu)
   unsigned long long* priv;  // [kOffsetSlots] or nullptr
+  // pruned recurrence (k_dp_pruned.cu), at the end of the workspace, or nullptr
+  uint32_t* prune_info;   // [2^L] row list of each Ta: rows, members, kListLong, kTileLong
+  uint2* prune_rows;      // [2^L * kPruneRows] (a1, mask of a2)
+  uint32_t* prune_short;  // [2^L] Ta's with a short list, by lowest request
+  uint32_t* prune_long;   // [2^L] Ta's with a long list, by lowest request
+  uint32_t* prune_n;      // [2 * kMaxMembersL] their numbers per lowest request
+  uint32_t* prune_done;   // [kPruneSplitTiles] finished blocks of each tile of a layer
   // layout
   unsigned long long* keys;  // [slots]
   int64_t* perm_offsets;     // [m + 1]
   int64_t* perm_chunks;      // [slots]
   int32_t* dfs;              // [m]
   int64_t* opt;              // [1]
+};
+
+// Order in which the blocked tables keep the inner bits U of a subset: bit j
+// of the stored index is inner bit to_nat[j] (requests L..m-1).  The pruned
+// recurrence chooses it by cost; every other path keeps the natural order.
+struct InnerPerm {
+  uint8_t to_nat[12] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11};
+  __host__ __device__ __forceinline__ uint32_t nat(uint32_t v) const {
+    uint32_t u = 0;
+#pragma unroll
+    for (int j = 0; j < 12; ++j) u |= (v >> j & 1u) << to_nat[j];
+    return u;
+  }
+  __host__ __device__ __forceinline__ uint32_t stored(uint32_t u) const {
+    uint32_t v = 0;
+#pragma unroll
+    for (int j = 0; j < 12; ++j) v |= (u >> to_nat[j] & 1u) << j;
+    return v;
+  }
 };
 
 struct Shape {
@@ -251,13 +277,27 @@ struct Shape {
   int b;            // tile bits (blocked)
   int L;            // m - b
   int64_t partial_entries;
+  InnerPerm perm;   // of the tables of this solve
+  bool pruned;      // one-shot solves run the pruned recurrence (k_dp_pruned.cu)
+  double prune_most;  // the host's bound on the pairs of one tile
+  bool prune_long;  // some list may be long
 };
+
+// Pruned recurrence (k_dp_pruned.cu): rows of a short list, members of a tile
+// that the pruned kernel finishes itself, the most tiles of a layer that is
+// cut into several blocks per tile, and the flags of a list.
+constexpr int kPruneRows = 32;
+constexpr int kPruneSelf = 128;
+constexpr int kPruneSplitTiles = 16384;
+constexpr int kMaxMembersL = 32;
+constexpr uint32_t kListLong = 1u << 30;
+constexpr uint32_t kTileLong = 1u << 31;
 
 size_t carve_workspace(const Shape& s, char* base, Workspace* ws);
 
 // Rotated position of subset S in the blocked path's tables.
-__host__ __device__ __forceinline__ size_t rot_index(uint32_t S, int L, int b) {
-  return ((size_t)(S & ((1u << L) - 1u)) << b) | (size_t)(S >> L);
+__host__ __device__ __forceinline__ size_t rot_index(uint32_t S, int L, int b, const InnerPerm& perm) {
+  return ((size_t)(S & ((1u << L) - 1u)) << b) | (size_t)perm.stored(S >> L);
 }
 
 // The table K1 scatters into and K2 transforms: w(I) in rotated order for the
@@ -291,6 +331,14 @@ struct BlockedTiming {
 int blocked_max_launches(const Shape& s);  // upper bound on pair + tile launches
 cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                               BlockedTiming* timing, int step_begin = 0, int step_end = -1);
+// The same over the members only (k_dp_pruned.cu): lists, then every step.
+cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
+                             BlockedTiming* timing);
+cudaError_t launch_prune_lists(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
+uint32_t pruned_items(const Shape& s, int kh);
+bool pruned_meet(const Shape& s, int kh, uint32_t items);
+cudaError_t launch_pruned_layer(const Shape& s, const Workspace& ws, int kh, uint32_t items,
+                                unsigned long long* partial, cudaStream_t stream, int* launches);
 int64_t blocked_partial_entries(int m, int b);
 int blocked_tile_bits(int m);
 

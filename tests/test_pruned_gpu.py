@@ -1,0 +1,104 @@
+"""The pruned recurrence (AUTO) against the full one (BLOCKED), table for table.
+
+AUTO leaves out splits whose named part has more than one request and no
+common weight; by the exchange argument in k_dp_pruned.cu that changes no
+F(S) and no split(S).  The cases sit where the rule or its kernels could go
+wrong: one tile bit, list lengths around the short/long limit (128), both
+tile widths of the sparse kernel, requests without chunks, identical
+requests, ties, a universal chunk, instances that must stay with the full
+recurrence.
+"""
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2609_13692_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def mpt():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_13692_gb300 import build as B
+
+    B.build()
+    O.build()
+    from paper_2609_13692_gb300 import mpt as M
+
+    M.load()
+    return M
+
+
+def _from_supports(m, supports, seed, wmax=9):
+    """One chunk per request set in `supports` (bit masks), weights 1..wmax."""
+    w = np.random.default_rng(seed).integers(1, wmax + 1, size=len(supports)).astype(np.int64)
+    reqs = [[x for x, N in enumerate(supports) if N >> i & 1] for i in range(m)]
+    return I.Instance(w, I.pack_requests(reqs, len(supports)), f"supports m={m}")
+
+
+def _mask(*bits):
+    return sum(1 << b for b in bits)
+
+
+def _cases():
+    rng = np.random.default_rng(5)
+    for m in range(13, 23):
+        yield I.rag_pools(m, 3000, 5, 40, 8, 1.1, seed=m)
+    for m in (13, 14, 17, 19):
+        yield I.zipf_small(m, 60, 5, 1.0, seed=m)
+        yield I.random_instance(m, 40, (0, 9), seed=m, wmin=1, wmax=3, allow_empty=True)
+    yield I.leave_one_out(15)
+    m = 18
+    # inner parts of 6, 7 and 8 requests (2^6 .. 2^8 listed sets), alone and
+    # nested in tile parts of several sizes
+    for inner in (6, 7, 8):
+        top = _mask(*range(6, 6 + inner))
+        yield _from_supports(m, [top | _mask(0, 2, 5)], inner)
+        yield _from_supports(m, [top | _mask(1), top | _mask(1, 3), _mask(0, 1, 2, 3, 4, 5), _mask(2, 17)], inner)
+    # all requests inside one tile part; no shared chunk at all; identical requests
+    yield _from_supports(m, [_mask(0, 1, 2), _mask(3, 4, 5), _mask(0, 5)], 1)
+    yield _from_supports(m, [1 << i for i in range(m)], 2)
+    yield I.Instance(np.ones(3, dtype=np.int64), I.pack_requests([[0, 1]] * 9 + [[2]] * 8, 3), "identical")
+    yield I.with_common_prefix(_from_supports(m, [int(x) for x in rng.integers(1, 1 << m, 12) & rng.integers(1, 1 << m, 12)], 3, 1), 77)
+    # many small sets: every tile has short lists
+    pairs = [_mask(i, j) for i in range(16) for j in range(i)]
+    yield _from_supports(16, pairs, 4, 2)
+    # one large set among small ones: long lists beside short ones
+    yield _from_supports(20, [_mask(*range(0, 20, 2)), _mask(*range(3, 20)), _mask(0, 1), _mask(1, 19)], 6)
+    yield _from_supports(20, [(1 << 20) - 2, _mask(0, 1), _mask(4, 12, 13)], 7)
+
+
+@pytest.mark.parametrize("inst", list(_cases()), ids=lambda inst: inst.name.replace(" ", "_")[:40])
+def test_equals_the_full_recurrence(mpt, inst):
+    a = mpt.solve(inst.weights, inst.bits, mode="auto")
+    b = mpt.solve(inst.weights, inst.bits, mode="blocked")
+    assert a.opt == b.opt
+    for x, y in zip(mpt.mpt_tables(a.ctx), mpt.mpt_tables(b.ctx)):
+        assert torch.equal(x, y)
+    assert a.perm_chunks.tolist() == b.perm_chunks.tolist() and a.dfs_order.tolist() == b.dfs_order.tolist()
+    lean = mpt.solve(inst.weights, inst.bits, tables="lean")
+    F, split = mpt.mpt_tables32(lean.ctx)
+    assert lean.opt == b.opt and torch.equal(split, mpt.mpt_tables(b.ctx)[2])
+    assert torch.equal(F.long(), mpt.mpt_tables(b.ctx)[0])
+
+
+def test_route(mpt):
+    """Few shared chunks: no pair kernel.  Leave-one-out: the full one."""
+    few = I.rag_pools(18, 3000, 5, 40, 8, 1.2, seed=3)
+    assert mpt.mpt_get_profile(mpt.solve(few.weights, few.bits).ctx)["launches_pairs"] == 0
+    loo = I.leave_one_out(16)
+    p = mpt.mpt_get_profile(mpt.solve(loo.weights, loo.bits).ctx)
+    assert p["launches_pairs"] == 3 and p["splits_pairs"] > 0
+
+
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_m24_equals_the_full_recurrence(mpt, seed):
+    inst = I.config(3, seed=seed)
+    a = mpt.solve(inst.weights, inst.bits)
+    b = mpt.solve(inst.weights, inst.bits, mode="blocked")
+    assert all(torch.equal(x, y) for x, y in zip(mpt.mpt_tables(a.ctx), mpt.mpt_tables(b.ctx)))
