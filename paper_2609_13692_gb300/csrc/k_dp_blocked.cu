@@ -61,8 +61,6 @@ constexpr int kMinPairsPerItem = 16;
 constexpr int kListCap = 4096;             // pairs of one block of the listed form
 constexpr int kListedSmemBytes = kPairSmemBytes + kListCap * (int)sizeof(uint32_t);
 static_assert(kListedSmemBytes <= 227 * 1024, "the listed pair kernel fits one SM");
-constexpr int kTileThreads = 512;
-constexpr int kMaxTileBits = 12;
 
 static_assert(kRing * 2 * kWin * (int)sizeof(uint32_t) >= (1 << kB) * 8, "merge buffer must fit in the windows");
 static_assert((kRing * 2 * kWin + kRing * kSharedWords + kRow * kPairThreads) % 2 == 0, "8-byte aligned barriers");
@@ -586,123 +584,200 @@ k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, uns
   for (int i = threadIdx.x; i < (1 << kB); i += kPairThreads) atomicMin(&out[i], merged[i]);
 }
 
-// Generic tile kernel: finishes every entry of the tiles with |T| = kh, level
-// by level in |U|, folding in the self pair (kh >= 1) or running the whole
-// recurrence on the inner bits (kh = 0).  One block per tile.  Used for tile 0
-// (any b <= 12); the tiles with kh >= 1 go to k_dp_tile_rows.
-// Both tile kernels read w(I) and write split in rotated order, one tile's
-// entries contiguous; F itself stays in Gp (F << b).
+// Tile 0: the whole recurrence on the b inner bits, one block.  The tile
+// kernels read w(I) and write split in stored order (perm; the natural one
+// outside the pruned recurrence); F itself stays in Gp (F << b).
 // Tab: int64 w(I) table, or the int32 one of the lean layout.
 template <typename Tab>
 __device__ __forceinline__ int64_t load_wI(const Tab* p) {
   return (int64_t)__ldg(p);
 }
 
+// One finished entry of tile 0 to the tables: f = F(U), A = split(U).
+__device__ __forceinline__ void put_tile0(int L, int b, const InnerPerm& perm, uint32_t U, uint32_t gp, uint32_t A,
+                                          uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc,
+                                          uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
+  const uint32_t idx = perm.stored(U);
+  if (MPT_BAD(flags, idx < (1u << b) && valid_split(U << L, A << L))) return;
+  Gp[idx] = gp;
+  Gc[idx] = gp | (~U & ((1u << b) - 1u));
+  split_rot[idx] = A << L;
+}
+
+// b <= 5: one warp, lane = U, level by level in |U|.
 template <typename Tab>
-__global__ void __launch_bounds__(kTileThreads)
-k_dp_tile(int L, int b, int kh, const Tab* __restrict__ wIr, const unsigned long long* __restrict__ partial,
-          uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot,
-          int32_t* __restrict__ flags, InnerPerm perm) {
-  __shared__ uint32_t cur_p[1 << kMaxTileBits];   // this tile, F << b
-  __shared__ uint32_t other_c[1 << kMaxTileBits]; // complement form: this tile (kh = 0) or tile 0 (kh >= 1)
-  __shared__ uint16_t order[1 << kMaxTileBits];   // inner subsets sorted by size, then colex
+__global__ void __launch_bounds__(32)
+k_dp_tile0_small(int L, int b, InnerPerm perm, const Tab* __restrict__ wIr, uint32_t* __restrict__ Gp,
+                 uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
+  __shared__ uint32_t cur[32];
+  const uint32_t U = threadIdx.x, mask = (1u << b) - 1u, low = U & (~U + 1u);
+  const bool has = U <= mask;
+  const uint32_t w = has ? (uint32_t)load_wI(wIr + U) : 0u;
+  uint32_t gp = 0, A = 0;
+  for (int p = 0; p <= b; ++p) {
+    if (has && __popc(U) == p) {
+      if (p == 1) gp = w << b;
+      if (p >= 2) {
+        uint32_t best = 0xFFFFFFFFu;
+        const uint32_t rest = U ^ low;
+        for (uint32_t sub = 0; sub != rest; sub = (sub - rest) & rest) {
+          const uint32_t a = low | sub;
+          best = min(best, cur[a] + cur[U ^ a] + a);  // (value << b) + A
+        }
+        gp = ((best >> b) - w) << b;
+        A = best & mask;
+      }
+      cur[U] = gp;
+    }
+    __syncwarp();
+  }
+  if (has) put_tile0(L, b, perm, U, gp, A, Gp, Gc, split_rot, flags);
+}
 
-  const uint32_t tile = blockIdx.x;
-  const uint32_t T = kh == 0 ? 0u : colex_unrank(tile, kh, L);
-  const int size = 1 << b;
-  const uint32_t mask = (uint32_t)size - 1u;
+// acc[s2] = min over a2 within s2 holding lowbit(s2) of x[a2] + y[s2 ^ a2], s2 = 1..31
+__device__ __forceinline__ void conv_rows_low(uint32_t (&acc)[kRow], const uint32_t (&x)[kRow],
+                                              const uint32_t (&y)[kRow]) {
+#pragma unroll
+  for (int a2 = 1; a2 < kRow; ++a2) {
+#pragma unroll
+    for (int s2 = 1; s2 < kRow; ++s2)
+      if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0) acc[s2] = min(acc[s2], x[a2] + y[s2 ^ a2]);
+  }
+}
 
-  for (int u = threadIdx.x; u < size; u += kTileThreads) {
-    const int p = __popc(u);
-    uint32_t start = 0;
-    for (int j = 0; j < p; ++j) start += (uint32_t)c_binom.v[b][j];
-    order[start + colex_rank((uint32_t)u)] = (uint16_t)u;
-    if (kh >= 1) other_c[u] = Gc[u];
+// b >= 6, row-blocked: U = (s1, s2), rows s1 of 32 entries, level by level in
+// |s1|.  A split of U names its part A = (a1, a2) holding lowbit(U):
+//   * s2 != 0: a2 holds lowbit(s2), any a1 within s1; a1 not in {0, s1}: rows
+//     of earlier levels, a register convolution of two rows (phase A); a1 = 0
+//     and a1 = s1: the in-row recurrence, in increasing s2, in registers
+//     (phase B, one thread per row);
+//   * s2 = 0: a1 holds lowbit(s1), the entry-0 column of the same row pairs.
+// cur holds F << b; the key of A | B is cur[A] + cur[B] + A = (value << b) + A.
+// One block is all there is to run, so its chains bound it: phase A spreads a
+// row's 2^p1 - 2 row pairs over 2^(p1 - 1) lanes (at most 32), and the 32
+// minima of a row then reduce by shuffles.  m = 12: 275 us with one subset per
+// lane group and a block barrier per size of U (a lane per few submasks, each
+// two dependent shared loads), TILE0US us in this form.
+constexpr int kT0Threads = 384;
+constexpr int kT0LevelRows = 35;  // C(7, 3)
+
+template <typename Tab>
+__global__ void __launch_bounds__(kT0Threads)
+k_dp_tile0(int L, int b, InnerPerm perm, const Tab* __restrict__ wIr, uint32_t* __restrict__ Gp,
+           uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
+  __shared__ __align__(16) uint32_t cur[kWin];
+  __shared__ uint32_t ws[kRows * (kRow + 1)];            // w(I), then split
+  __shared__ uint32_t amin[kT0LevelRows * (kRow + 1)];   // phase A minima of a level's rows
+  const int t = threadIdx.x, nb = b - kB2;
+  const uint32_t mask = (1u << b) - 1u;
+  for (uint32_t v = t; v <= mask; v += kT0Threads) {
+    const uint32_t U = perm.nat(v);
+    ws[U + (U >> kB2)] = (uint32_t)load_wI(wIr + v);
   }
   __syncthreads();
-
-  uint32_t start = 0;
-  for (int p = 0; p <= b; ++p) {
-    const int cnt = (int)c_binom.v[b][p];
-    const int g = p > 3 ? min(p - 3, 5) : 0;  // log2(lanes per output)
-    const int G = 1 << g;
-    const int groups = kTileThreads >> g;
-    for (int base = 0; base < cnt; base += groups) {
-      const int gi = base + (int)(threadIdx.x >> g);
-      const uint32_t r = threadIdx.x & (uint32_t)(G - 1);
-      const bool active = gi < cnt;
-      unsigned long long best = ~0ull;
-      uint32_t U = 0;
-      bool single = false;
-      if (active) {
-        U = order[start + gi];
-        const uint32_t nreq = (uint32_t)p + (uint32_t)kh;
-        single = nreq == 1;
-        if (nreq >= 2 && !(kh >= 1 && U == 0)) {
-          // kh = 0: Ua = lowbit(U) | part, part a proper subset of U \ lowbit(U).
-          // kh >= 1: Ua = part, a proper subset of U (Ta = T).
-          const uint32_t lowU = kh == 0 ? (U & (~U + 1u)) : 0u;
-          const uint32_t emask = U ^ lowU;
-          uint32_t hi = 0, rr = emask;
-          for (int t = 0; t < g; ++t) {
-            const uint32_t top = 1u << (31 - __clz(rr));
-            hi |= top;
-            rr ^= top;
+  // level 0: row 0, the recurrence on the five lowest inner requests
+  if (t == 0) {
+    uint32_t c[kRow];
+#pragma unroll
+    for (int s2 = 0; s2 < kRow; ++s2) {
+      uint32_t f = 0, A = 0;
+      if ((s2 & (s2 - 1)) == 0) {
+        f = s2 ? ws[s2] : 0u;
+      } else {
+        uint32_t key = 0xFFFFFFFFu;
+#pragma unroll
+        for (int a2 = 1; a2 < kRow; ++a2)
+          if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0 && a2 != s2) key = min(key, c[a2] + c[s2 ^ a2] + (uint32_t)a2);
+        f = (key >> b) - ws[s2];
+        A = key & mask;
+      }
+      c[s2] = f << b;
+      ws[s2] = A;
+    }
+#pragma unroll
+    for (int i = 0; i < kRow; ++i) cur[i] = c[i];  // row 0 is at position 0
+  }
+  __syncthreads();
+  for (int p1 = 1; p1 <= nb; ++p1) {
+    const int rows = (int)c_binom.v[nb][p1];
+    if (p1 >= 2) {
+      const int g = p1 - 1 < 5 ? p1 - 1 : 5, G = 1 << g;  // lanes per row: at most 35 x 8 = 280, 21 x 16 = 336
+      const int ri = t >> g;
+      const uint32_t r = (uint32_t)t & (uint32_t)(G - 1);
+      uint32_t acc[kRow];
+#pragma unroll
+      for (int i = 0; i < kRow; ++i) acc[i] = 0xFFFFFFFFu;
+      if (ri < rows) {
+        const uint32_t s1 = colex_unrank((unsigned long long)ri, p1, nb);
+        const uint32_t lowb = s1 & (~s1 + 1u);
+        uint32_t hi = 0, rr = s1;
+        for (int q = 0; q < g; ++q) {
+          const uint32_t top = 1u << (31 - __clz(rr));
+          hi |= top;
+          rr ^= top;
+        }
+        const uint32_t freem = s1 ^ hi;
+        const uint32_t fixed = deposit_bits(r, hi);
+        uint32_t sub = 0;
+        do {
+          const uint32_t a1 = fixed | sub;
+          if (a1 != 0 && a1 != s1) {
+            uint32_t x[kRow], y[kRow];
+            load_row(x, cur + row_pos(a1) * kRowStride);
+            load_row(y, cur + row_pos(s1 ^ a1) * kRowStride);
+#pragma unroll
+            for (int i = 0; i < kRow; ++i) x[i] += (a1 << kB2) | (uint32_t)i;
+            conv_rows_low(acc, x, y);
+            if (a1 & lowb) acc[0] = min(acc[0], x[0] + y[0]);
           }
-          const uint32_t freem = emask ^ hi;
-          const uint32_t fixed = deposit_bits(r, hi);
-          const unsigned long long ta = kh == 0 ? 0ull : (unsigned long long)T;
-          uint32_t s = 0;
-          do {
-            const uint32_t part = fixed | s;
-            if (part != emask) {
-              const uint32_t Ua = lowU | part;
-              const uint32_t key = cur_p[Ua] + other_c[U ^ Ua];
-              const unsigned long long c = ((unsigned long long)key << 32) | ta;
-              best = c < best ? c : best;
-            }
-            s = (s - freem) & freem;
-          } while (s != 0);
-        }
-        if (kh >= 2 && r == 0) {
-          const unsigned long long pv = partial[((size_t)tile << b) | U];
-          best = pv < best ? pv : best;
-        }
+          sub = (sub - freem) & freem;
+        } while (sub != 0);
       }
       for (int off = G >> 1; off > 0; off >>= 1) {
-        const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-        best = o < best ? o : best;
+#pragma unroll
+        for (int i = 0; i < kRow; ++i) acc[i] = min(acc[i], __shfl_xor_sync(0xFFFFFFFFu, acc[i], off));
       }
-      if (active && r == 0) {
-        const size_t idx = ((size_t)T << b) | perm.stored(U);
-        int64_t f;
-        uint32_t A;
-        if (U == 0 && T == 0) {
-          f = 0;
-          A = 0;
-        } else if (single) {
-          f = load_wI(wIr + idx);
-          A = 0;
-        } else {
-          const uint32_t key = (uint32_t)(best >> 32);
-          const uint32_t Ua = (key & mask) + U - mask;
-          f = (int64_t)(key >> b) - load_wI(wIr + idx);
-          A = (Ua << L) | (uint32_t)best;
-        }
-        const uint32_t gp = (uint32_t)f << b;
-        const uint32_t gc = gp | (~U & mask);
-        cur_p[U] = gp;
-        if (kh == 0) other_c[U] = gc;
-        if (!MPT_BAD(flags, idx < ((size_t)1 << (L + b)) && valid_split(T | (U << L), A))) {
-          Gp[idx] = gp;
-          Gc[idx] = gc;
-          split_rot[idx] = A;
-        }
+      if (ri < rows && r == 0) {
+#pragma unroll
+        for (int i = 0; i < kRow; ++i) amin[ri * (kRow + 1) + i] = acc[i];
       }
+      __syncthreads();
     }
-    start += (uint32_t)cnt;
+    if (t < rows) {
+      const uint32_t s1 = colex_unrank((unsigned long long)t, p1, nb), S1 = s1 << kB2;
+      uint32_t* own = ws + s1 * (kRow + 1);
+      uint32_t z[kRow], c[kRow];
+      load_row(z, cur);
+#pragma unroll
+      for (int s2 = 0; s2 < kRow; ++s2) {
+        const uint32_t w = own[s2];
+        uint32_t f = w, A = 0;
+        if (!(s2 == 0 && p1 == 1)) {  // else U = (s1, 0) is a single request
+          // two independent minima (a1 = 0 and a1 = s1) shorten the chains
+          uint32_t k0 = p1 >= 2 ? amin[t * (kRow + 1) + s2] : 0xFFFFFFFFu, k1 = 0xFFFFFFFFu;
+#pragma unroll
+          for (int a2 = 1; a2 < kRow; ++a2) {
+            if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0) {
+              k0 = min(k0, z[a2] + c[s2 ^ a2] + (uint32_t)a2);
+              if (a2 != s2) k1 = min(k1, c[a2] + z[s2 ^ a2] + (S1 | (uint32_t)a2));
+            }
+          }
+          const uint32_t key = min(k0, k1);
+          f = (key >> b) - w;
+          A = key & mask;
+        }
+        c[s2] = f << b;
+        own[s2] = A;
+      }
+      uint4* dst = reinterpret_cast<uint4*>(cur + row_pos(s1) * kRowStride);
+#pragma unroll
+      for (int q = 0; q < kRow / 4; ++q) dst[q] = make_uint4(c[4 * q], c[4 * q + 1], c[4 * q + 2], c[4 * q + 3]);
+    }
     __syncthreads();
   }
+  for (uint32_t U = t; U <= mask; U += kT0Threads)
+    put_tile0(L, b, perm, U, cur[row_pos(U >> kB2) * kRowStride + (U & (kRow - 1))], ws[U + (U >> kB2)], Gp, Gc,
+              split_rot, flags);
 }
 
 // Row-blocked tile kernel for |T| = kh >= 1 (inner bits b = kB).  The self
@@ -964,12 +1039,16 @@ cudaError_t blocked_attributes(bool listed) {
 void launch_tiles(const Shape& s, const Workspace& ws, int kh, const uint32_t* info, cudaStream_t stream) {
   const unsigned long long tiles = h_binom.v[s.L][kh];
   if (kh == 0) {
+    auto go = [&](const auto* wIr) {
+      if (s.b <= kB2)
+        k_dp_tile0_small<<<1, 32, 0, stream>>>(s.L, s.b, s.perm, wIr, ws.Gp, ws.Gc, ws.split_rot, ws.counters + 1);
+      else
+        k_dp_tile0<<<1, kT0Threads, 0, stream>>>(s.L, s.b, s.perm, wIr, ws.Gp, ws.Gc, ws.split_rot, ws.counters + 1);
+    };
     if (s.lean)
-      k_dp_tile<<<1, kTileThreads, 0, stream>>>(s.L, s.b, 0, ws.fw_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
-                                                ws.counters + 1, s.perm);
+      go(ws.fw_rot);
     else
-      k_dp_tile<<<1, kTileThreads, 0, stream>>>(s.L, s.b, 0, ws.wI_rot, nullptr, ws.Gp, ws.Gc, ws.split_rot,
-                                                ws.counters + 1, s.perm);
+      go(ws.wI_rot);
     return;
   }
   const unsigned long long* part = kh >= 2 ? ws.partial : nullptr;
