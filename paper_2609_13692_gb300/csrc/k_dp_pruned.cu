@@ -18,8 +18,8 @@
 // A = (Ta, Ua) has (Ta, {}) a member or a single request.  With the inner bits
 // Ua = (a1, a2), a2 the low kRB bits, the members of one Ta are a list of
 // rows (a1, mask of the a2's):
-//   k_prune_lists    per Ta the row list, and whether it is short (at most
-//                    kPruneRows rows);
+//   k_prune_tiles    w(I), and per Ta the row list and whether it is short (at
+//                    most kPruneRows rows);
 //   k_prune_members  per lowest request the Ta's with a short and those with
 //                    a long list, each in increasing order;
 //   k_dp_pruned      per tile T every short Ta within T, then, where T's own
@@ -75,56 +75,104 @@ struct PrunedCfg {
   static_assert((kSmem + 3072) * kBlocks <= 228 * 1024, "blocks per SM");
 };
 
-// Row list of every Ta.  A warp reads 32 entries of w(I(Ta, .)) at a time;
-// the ballot of the non-zero ones is the mask of one row of 32, or of two
-// rows of 16.  info: 0 when Ta has no member, else rows | members << 8 |
-// kListLong when they are more than kPruneRows or, where the pair kernel runs
-// (long_ok), cost more than a pair there | kTileLong when the tile T = Ta is
-// left to the row kernel (a long list, or more than kPruneSelf members).
-// Cost: a row takes as many warps as have a lane whose row holds a1, each for
-// its steps and the loads, here kUnitSteps steps' worth.
-template <typename Key, typename Tab>
+// w(I(T, .)) and the row list of every T, one block per tile at a time, from
+// the sets N_x of the chunks that some but not all requests share (N: stored
+// rotated index, w: weight; K1's list): w(I(S)) = sum of w over N containing
+// S.  Few tiles lie within any N_x, so most are a write of zeros, and the
+// others a superset sum over the 2^12 inner sets in shared memory: the table
+// is written once and never read, where the general transform (K2) reads and
+// writes it once per 8 to 12 request bits after a clear.
+// m = 28: 0.29 + 2.0 ms of clear and transform (HBM-bound) -> 0.29 ms (7.5 TB/s written).
+// The row list: threads = rows, the mask of a row from its non-zero entries.
+// info: 0 when T has no member, else rows | members << 8 | kListLong when
+// they are more than kPruneRows or, where the pair kernel runs (long_ok), cost
+// more than a pair there | kTileLong when the tile is left to the row kernel (a
+// long list, or more than kPruneSelf members).  Cost: a row takes as many
+// warps as have a lane whose row holds a1, each for its steps and the loads,
+// here kUnitSteps steps' worth.
+template <typename Key, typename G>
 __global__ void __launch_bounds__(256)
-k_prune_lists(int L, bool long_ok, const Tab* __restrict__ wIr, uint32_t* __restrict__ info, uint2* __restrict__ rows) {
-  constexpr int kRB = PrunedCfg<Key>::kRB;
-  constexpr int kHalves = 32 >> kRB;
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t Ta = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; Ta < (1u << L); Ta += warps) {
-    const Tab* win = wIr + ((size_t)Ta << kPB);
-    if (Ta == 0 || ((Ta & (Ta - 1u)) != 0 && win[0] == 0)) {
-      if (lane == 0) info[Ta] = 0;
+k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N, const unsigned long long* __restrict__ w,
+              G* __restrict__ wIr, uint32_t* __restrict__ info, uint2* __restrict__ rows,
+              const int32_t* __restrict__ counters) {
+  using C = PrunedCfg<Key>;
+  constexpr int kThreads = 256, kPer = 16 / (int)sizeof(G);
+  __shared__ __align__(16) G s[1 << kPB];
+  __shared__ uint32_t warp_n[8], warp_m[8], warp_c[8];
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const int n = min(counters[3], n_shared);
+  for (uint32_t T = blockIdx.x; T < (1u << L); T += gridDim.x) {
+    const bool single = T != 0 && (T & (T - 1u)) == 0;
+    bool clear = false;  // s holds the tile
+    for (int base = 0; base < n; base += kThreads) {
+      const int i = base + (int)tid;
+      const uint32_t Ni = i < n ? N[i] : 0u;
+      const bool hit = i < n && (T & ~(Ni >> kPB)) == 0;
+      if (!__syncthreads_or(hit)) continue;
+      if (!clear) {
+        for (uint32_t v = tid; v <= kPMask; v += kThreads) s[v] = 0;
+        clear = true;
+        __syncthreads();
+      }
+      if (hit) atomicAdd(&s[Ni & kPMask], (G)w[i]);
+    }
+    G* out = wIr + ((size_t)T << kPB);
+    if (!clear) {
+      for (uint32_t v = tid; v < (1u << kPB) / kPer; v += kThreads) reinterpret_cast<uint4*>(out)[v] = make_uint4(0, 0, 0, 0);
+      if (tid == 0) {
+        info[T] = single ? 1u | (1u << 8) : 0u;  // a single request is always listed
+        if (single) rows[(size_t)T * kPruneRows] = make_uint2(0u, 1u);
+      }
       continue;
     }
-    uint2* out = rows + (size_t)Ta * kPruneRows;
-    uint32_t n = 0, members = 0, cost = 0;
-    for (uint32_t base = 0; base <= kPMask; base += 256) {
-      bool nz[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) nz[k] = win[base + 32u * k + lane] != 0;
-      if (base == 0 && lane == 0) nz[0] = true;  // (Ta, {}): a member, or a single request
+    for (int j = 0; j < kPB; ++j) {
+      __syncthreads();
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, nz[k]);
-        members += (uint32_t)__popc(bal);
-#pragma unroll
-        for (int h = 0; h < kHalves; ++h) {
-          const uint32_t mask = kHalves == 1 ? bal : (bal >> (16 * h)) & 0xFFFFu;
-          if (mask) {
-            const uint32_t a1 = (base + 32u * k) / (1u << kRB) + h;
-            const uint32_t steps =
-                __reduce_add_sync(0xFFFFFFFFu, (mask >> lane & 1u) ? (1u << kRB) >> __popc(lane) : 0u);
-            cost += (steps + kUnitSteps) << (PrunedCfg<Key>::kLogWarps - __popc(a1 >> 5));
-            if (lane == 0 && n < (uint32_t)kPruneRows) out[n] = make_uint2(a1, mask);
-            ++n;
-          }
-        }
+      for (int q = 0; q < (1 << (kPB - 1)) / kThreads; ++q) {
+        const uint32_t p = tid + (uint32_t)(q * kThreads);
+        const uint32_t v = ((p >> j) << (j + 1)) | (p & ((1u << j) - 1u));
+        s[v] += s[v | (1u << j)];
       }
     }
+    __syncthreads();
+    for (uint32_t v = tid; v < (1u << kPB) / kPer; v += kThreads)
+      reinterpret_cast<uint4*>(out)[v] = reinterpret_cast<const uint4*>(s)[v];
+    uint32_t mask = 0;
+    if (T != 0 && tid < (uint32_t)C::kRows) {
+      // entry i + row of the row at a time, so that a warp reads different banks
+      for (uint32_t i = 0; i < (uint32_t)C::kRow; ++i) {
+        const uint32_t a2 = (i + tid) & (C::kRow - 1);
+        if (s[tid * C::kRow + a2] != 0) mask |= 1u << a2;
+      }
+      if (single && tid == 0) mask |= 1u;
+    }
+    uint32_t steps = 0;
+    for (uint32_t r = mask; r; r &= r - 1) steps += (uint32_t)C::kRow >> __popc(__ffs(r) - 1);
+    const uint32_t cost = mask ? (steps + kUnitSteps) << (C::kLogWarps - __popc(tid >> 5)) : 0u;
+    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, mask != 0);
+    const uint32_t members = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)__popc(mask));
+    const uint32_t costs = __reduce_add_sync(0xFFFFFFFFu, cost);
     if (lane == 0) {
-      const bool is_long = n > (uint32_t)kPruneRows || (long_ok && cost > kLongSteps);
-      info[Ta] = min(n, 255u) | (members << 8) | (is_long ? kListLong : 0u) |
-                 (is_long || members > (uint32_t)kPruneSelf ? kTileLong : 0u);
+      warp_n[warp] = (uint32_t)__popc(bal);
+      warp_m[warp] = members;
+      warp_c[warp] = costs;
+    }
+    __syncthreads();
+    uint32_t at = (uint32_t)__popc(bal & ((1u << lane) - 1u)), nr = 0, nm = 0, nc = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      at += (uint32_t)q < warp ? warp_n[q] : 0u;
+      nr += warp_n[q];
+      nm += warp_m[q];
+      nc += warp_c[q];
+    }
+    if (mask && at < (uint32_t)kPruneRows) rows[(size_t)T * kPruneRows + at] = make_uint2(tid, mask);
+    if (tid == 0) {
+      const bool is_long = nr > (uint32_t)kPruneRows || (long_ok && nc > kLongSteps);
+      info[T] = nr == 0 ? 0u
+                        : min(nr, 255u) | (nm << 8) | (is_long ? kListLong : 0u) |
+                              (is_long || nm > (uint32_t)kPruneSelf ? kTileLong : 0u);
     }
   }
 }
@@ -679,13 +727,11 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   }
 }
 
-template <typename Key, typename Tab>
-cudaError_t lists(const Shape& s, const Workspace& ws, const Tab* wIr, cudaStream_t stream, int* launches) {
-  const int64_t warps = (int64_t)1 << s.L;
-  int64_t blocks = (warps + 7) / 8;
-  const int64_t most = sm_count() * 8;
-  if (blocks > most) blocks = most;
-  k_prune_lists<Key><<<(unsigned)blocks, 256, 0, stream>>>(s.L, s.prune_long, wIr, ws.prune_info, ws.prune_rows);
+template <typename Key, typename G>
+cudaError_t tables(const Shape& s, const Workspace& ws, G* wIr, cudaStream_t stream, int* launches) {
+  const int64_t tiles = (int64_t)1 << s.L, most = sm_count() * 8 * 8;
+  k_prune_tiles<Key><<<(unsigned)(tiles < most ? tiles : most), 256, 0, stream>>>(
+      s.L, s.prune_long, s.n_shared, ws.shared_N, ws.shared_w, wIr, ws.prune_info, ws.prune_rows, ws.counters);
   k_prune_members<<<(unsigned)s.L, 1024, 0, stream>>>(s.L, ws.prune_info, ws.prune_short, ws.prune_long, ws.prune_n);
   *launches += 2;
   return cudaGetLastError();
@@ -707,11 +753,11 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
 
 }  // namespace
 
-cudaError_t launch_prune_lists(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
+cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
   cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, kPruneSplitTiles * 4, stream);
   if (e != cudaSuccess) return e;
-  if (s.lean) return lists<uint32_t>(s, ws, ws.fw_rot, stream, launches);
-  return lists<uint32_t>(s, ws, ws.wI_rot, stream, launches);
+  if (s.lean) return tables<uint32_t>(s, ws, reinterpret_cast<unsigned int*>(ws.fw_rot), stream, launches);
+  return tables<uint32_t>(s, ws, reinterpret_cast<unsigned long long*>(ws.wI_rot), stream, launches);
 }
 
 // Blocks per tile of a layer with 32-bit keys.  The pairs of a tile vary from

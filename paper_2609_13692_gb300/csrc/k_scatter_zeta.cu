@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kScatterThreads)
 k_scatter(const int64_t* __restrict__ w, const uint64_t* __restrict__ bits, int64_t n, int m, int64_t words,
           G* __restrict__ g, unsigned long long* __restrict__ priv, uint32_t* __restrict__ used_N,
           int32_t* __restrict__ used_x, int32_t* __restrict__ counters, int64_t slots, bool rotated, int L, int b,
-          InnerPerm perm) {
+          InnerPerm perm, uint32_t* __restrict__ shared_N, unsigned long long* __restrict__ shared_w, int n_shared) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const uint32_t full = m >= 32 ? 0xFFFFFFFFu : (1u << m) - 1u;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
@@ -57,7 +57,16 @@ k_scatter(const int64_t* __restrict__ w, const uint64_t* __restrict__ bits, int6
         atomicAdd(&priv[__ffs(N) - 1], (unsigned long long)w[x]);
       else if (priv && N == full)  // m >= 2 here: for m = 1 the full set is a singleton
         atomicAdd(&priv[kUniversalSlot], (unsigned long long)w[x]);
-      else if (!MPT_BAD(&counters[1], (rotated ? rot_index(N, L, b, perm) : (size_t)N) < ((size_t)1 << m)))
+      else if (shared_N) {
+        // pruned recurrence: listed for k_prune_tiles
+        const int k = atomicAdd(&counters[3], 1);
+        if (k < n_shared) {
+          shared_N[k] = (uint32_t)rot_index(N, L, b, perm);
+          shared_w[k] = (unsigned long long)w[x];
+        } else {
+          atomicOr(&counters[1], kErrWorkspace);
+        }
+      } else if (!MPT_BAD(&counters[1], (rotated ? rot_index(N, L, b, perm) : (size_t)N) < ((size_t)1 << m)))
         atomicAdd(&g[rotated ? rot_index(N, L, b, perm) : (size_t)N], (G)w[x]);
       const int k = atomicAdd(&counters[0], 1);
       if (k < slots) {
@@ -252,7 +261,7 @@ __global__ void __launch_bounds__(kZetaThreads) k_zeta_high8(G* __restrict__ g, 
 
 }  // namespace
 
-cudaError_t launch_scatter(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
+cudaError_t launch_scatter(const Shape& s, const Workspace& ws, bool pruned, cudaStream_t stream, int* launches) {
   int64_t blocks = (s.n + kScatterThreads - 1) / kScatterThreads;
   const int64_t cap = sm_count() * 16;
   if (blocks > cap) blocks = cap;
@@ -261,11 +270,13 @@ cudaError_t launch_scatter(const Shape& s, const Workspace& ws, cudaStream_t str
   if (s.lean)
     k_scatter<<<(unsigned)blocks, kScatterThreads, 0, stream>>>(
         ws.weights, ws.bits, s.n, s.m, s.words, static_cast<unsigned int*>(g), s.blocked ? ws.priv : nullptr,
-        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm);
+        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm,
+        pruned ? ws.shared_N : nullptr, ws.shared_w, s.n_shared);
   else
     k_scatter<<<(unsigned)blocks, kScatterThreads, 0, stream>>>(
         ws.weights, ws.bits, s.n, s.m, s.words, static_cast<unsigned long long*>(g), s.blocked ? ws.priv : nullptr,
-        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm);
+        ws.used_N, ws.used_x, ws.counters, s.slots, s.blocked, s.L, s.b, s.perm,
+        pruned ? ws.shared_N : nullptr, ws.shared_w, s.n_shared);
   ++*launches;
   return cudaGetLastError();
 }

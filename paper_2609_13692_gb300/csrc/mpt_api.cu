@@ -252,8 +252,13 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
   // after everything else, so that the rest sits where it does without them
   ws->prune_info = ws->prune_short = ws->prune_long = ws->prune_n = ws->prune_done = nullptr;
   ws->prune_rows = nullptr;
+  ws->shared_N = nullptr;
+  ws->shared_w = nullptr;
   if (s.pruned) {
     const size_t P = (size_t)1 << s.L;
+    const size_t ns = (size_t)(s.n_shared > 0 ? s.n_shared : 1);
+    ws->shared_N = reinterpret_cast<uint32_t*>(take(ns * 4));
+    ws->shared_w = reinterpret_cast<unsigned long long*>(take(ns * 8));
     ws->prune_info = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_rows = reinterpret_cast<uint2*>(take(P * mpt::kPruneRows * sizeof(uint2)));
     ws->prune_short = reinterpret_cast<uint32_t*>(take(P * 4));
@@ -344,6 +349,7 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
       many_supports = supports.size() > kMaxSupports;
     }
   }
+  const int n_shared = (int)supports.size();  // (when not too many)
   std::sort(supports.begin(), supports.end());
   supports.erase(std::unique(supports.begin(), supports.end()), supports.end());
   mpt_ctx* c = new (std::nothrow) mpt_ctx();
@@ -361,6 +367,7 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
   c->shape.slots = slots;
   c->sum_w = sum;
   c->shared_w = sum - private_w;
+  c->shape.n_shared = n_shared;
   c->supports = std::move(supports);
   c->many_supports = many_supports;
   refresh_shape(c);
@@ -443,9 +450,10 @@ mpt_status bind_workspace(mpt_ctx* c, void* d_workspace, size_t workspace_bytes,
   return MPT_OK;
 }
 
-// Input copies (unless this workspace already holds them), K1 and K2.
-mpt_status run_front(mpt_ctx* c, const mpt::Shape& s, const mpt::Workspace& ws, char* base, cudaStream_t stream, int* launches,
-                     cudaEvent_t* ev) {
+// Input copies (unless this workspace already holds them), K1 and K2 (or
+// what the pruned recurrence has in its place).
+mpt_status run_front(mpt_ctx* c, const mpt::Shape& s, const mpt::Workspace& ws, bool pruned, char* base,
+                     cudaStream_t stream, int* launches, cudaEvent_t* ev) {
   auto mark = [&](int i) {
     if (ev) cudaEventRecord(ev[i], stream);
   };
@@ -458,11 +466,14 @@ mpt_status run_front(mpt_ctx* c, const mpt::Shape& s, const mpt::Workspace& ws, 
   }
   MPT_CK(cudaMemsetAsync(ws.counters, 0, 8 * 4, stream), "memset counters");
   if (ws.priv) MPT_CK(cudaMemsetAsync(ws.priv, 0, mpt::kOffsetSlots * 8, stream), "memset offsets");
-  MPT_CK(cudaMemsetAsync(mpt::g_table(s, ws), 0, N * (s.lean ? 4 : 8), stream), "memset g");
+  if (!pruned) MPT_CK(cudaMemsetAsync(mpt::g_table(s, ws), 0, N * (s.lean ? 4 : 8), stream), "memset g");
   mark(1);
-  MPT_CK(mpt::launch_scatter(s, ws, stream, launches), "scatter kernel");
+  MPT_CK(mpt::launch_scatter(s, ws, pruned, stream, launches), "scatter kernel");
   mark(2);
-  MPT_CK(mpt::launch_zeta(s, ws, stream, launches), "zeta kernels");
+  if (pruned)
+    MPT_CK(mpt::launch_prune_tables(s, ws, stream, launches), "pruned table kernels");
+  else
+    MPT_CK(mpt::launch_zeta(s, ws, stream, launches), "zeta kernels");
   mark(3);
   return MPT_OK;
 }
@@ -551,7 +562,7 @@ mpt_status mpt_solve(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes, vo
 
   int launches = 0;
   const size_t N = (size_t)1 << s.m;
-  if ((st = run_front(c, s, ws, base, stream, &launches, ev)) != MPT_OK) return st;
+  if ((st = run_front(c, s, ws, s.pruned, base, stream, &launches, ev)) != MPT_OK) return st;
   mpt::BlockedTiming timing{};
   if (s.blocked) {
     timing.pair_ev = ev ? ev + 7 : nullptr;
@@ -622,7 +633,7 @@ mpt_status mpt_solve_begin(mpt_ctx* ctx, void* d_workspace, size_t workspace_byt
   mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   int launches = 0;
-  if ((st = run_front(c, c->shape, ws, base, stream, &launches, nullptr)) != MPT_OK) return st;
+  if ((st = run_front(c, c->shape, ws, false, base, stream, &launches, nullptr)) != MPT_OK) return st;
   if ((st = run_steps(c, ws, stream, &launches, nullptr, 0, 1)) != MPT_OK) return st;
   c->resident = base;
   c->staged_base = base;

@@ -204,7 +204,7 @@ struct Workspace {
   // scatter outputs
   uint32_t* used_N;   // [slots]  request set N_x of each used chunk
   int32_t* used_x;    // [slots]  chunk id
-  int32_t* counters;  // [8]      0: number of used chunks, 1: device error flags
+  int32_t* counters;  // [8]      0: number of used chunks, 1: device error flags, 2: pairs run, 3: shared chunks listed
   // tables, natural subset order (int64 tables: wI and F; lean: fw alone,
   // w(I(S)) until the recurrence writes F(S) over it).  The blocked path
   // leaves them in rotated order (below) and fills the natural views only
@@ -233,6 +233,8 @@ struct Workspace {
   // the scatter in k_scatter_zeta.cu)
   unsigned long long* priv;  // [kOffsetSlots] or nullptr
   // pruned recurrence (k_dp_pruned.cu), at the end of the workspace, or nullptr
+  uint32_t* shared_N;     // [n_shared] rotated index of N_x of each chunk that some but not all requests share
+  unsigned long long* shared_w;  // [n_shared] its weight
   uint32_t* prune_info;   // [2^L] row list of each Ta: rows, members, kListLong, kTileLong
   uint2* prune_rows;      // [2^L * kPruneRows] (a1, mask of a2)
   uint32_t* prune_short;  // [2^L] Ta's with a short list, by lowest request
@@ -279,6 +281,7 @@ struct Shape {
   int64_t partial_entries;
   InnerPerm perm;   // of the tables of this solve
   bool pruned;      // one-shot solves run the pruned recurrence (k_dp_pruned.cu)
+  int n_shared;       // chunks that some (two or more) but not all requests share
   double prune_most;  // the host's bound on the pairs of one tile
   bool prune_long;  // some list may be long
 };
@@ -310,7 +313,9 @@ inline void* g_table(const Shape& s, const Workspace& ws) {
 // ---------------------------------------------------------------------------
 // Launchers.  All enqueue on `stream` and return the launch error (if any).
 // ---------------------------------------------------------------------------
-cudaError_t launch_scatter(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
+// pruned: chunks that some but not all requests share are listed (shared_N,
+// shared_w) instead of added to g.
+cudaError_t launch_scatter(const Shape& s, const Workspace& ws, bool pruned, cudaStream_t stream, int* launches);
 cudaError_t launch_zeta(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
 
 // The recurrence runs in steps that depend only on earlier steps: the blocked
@@ -334,7 +339,8 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
 // The same over the members only (k_dp_pruned.cu): lists, then every step.
 cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                              BlockedTiming* timing);
-cudaError_t launch_prune_lists(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
+// w(I) (instead of K2) and the lists; needs K1's list of shared chunks.
+cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
 uint32_t pruned_items(const Shape& s, int kh);
 bool pruned_meet(const Shape& s, int kh, uint32_t items);
 cudaError_t launch_pruned_layer(const Shape& s, const Workspace& ws, int kh, uint32_t items,

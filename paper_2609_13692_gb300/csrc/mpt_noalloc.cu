@@ -197,7 +197,7 @@ extern "C" mpt_status mpt_solve_noalloc(const int64_t* d_weights, int64_t n_chun
       (ws.priv && cudaMemsetAsync(ws.priv, 0, mpt::kOffsetSlots * sizeof(unsigned long long), stream) !=
                       cudaSuccess))
     return MPT_ERR_CUDA;
-  if (mpt::launch_scatter(s, ws, stream, &launches) != cudaSuccess) return MPT_ERR_CUDA;
+  if (mpt::launch_scatter(s, ws, false, stream, &launches) != cudaSuccess) return MPT_ERR_CUDA;
   if (mpt::launch_zeta(s, ws, stream, &launches) != cudaSuccess) return MPT_ERR_CUDA;
   cudaError_t e = s.blocked ? mpt::launch_dp_blocked(s, ws, stream, &launches, nullptr)
                             : mpt::launch_dp_general(s, ws, stream, &launches);
