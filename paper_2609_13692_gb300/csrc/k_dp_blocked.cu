@@ -584,200 +584,13 @@ k_dp_pairs(const uint32_t* __restrict__ Gp, const uint32_t* __restrict__ Gc, uns
   for (int i = threadIdx.x; i < (1 << kB); i += kPairThreads) atomicMin(&out[i], merged[i]);
 }
 
-// Tile 0: the whole recurrence on the b inner bits, one block.  The tile
-// kernels read w(I) and write split in stored order (perm; the natural one
-// outside the pruned recurrence); F itself stays in Gp (F << b).
+// The tile kernels read w(I) and write split in stored order (perm; the
+// natural one outside the pruned recurrence); F itself stays in Gp (F << b).
+// Tile 0 is k_dp_tile0.cu's.
 // Tab: int64 w(I) table, or the int32 one of the lean layout.
 template <typename Tab>
 __device__ __forceinline__ int64_t load_wI(const Tab* p) {
   return (int64_t)__ldg(p);
-}
-
-// One finished entry of tile 0 to the tables: f = F(U), A = split(U).
-__device__ __forceinline__ void put_tile0(int L, int b, const InnerPerm& perm, uint32_t U, uint32_t gp, uint32_t A,
-                                          uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc,
-                                          uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
-  const uint32_t idx = perm.stored(U);
-  if (MPT_BAD(flags, idx < (1u << b) && valid_split(U << L, A << L))) return;
-  Gp[idx] = gp;
-  Gc[idx] = gp | (~U & ((1u << b) - 1u));
-  split_rot[idx] = A << L;
-}
-
-// b <= 5: one warp, lane = U, level by level in |U|.
-template <typename Tab>
-__global__ void __launch_bounds__(32)
-k_dp_tile0_small(int L, int b, InnerPerm perm, const Tab* __restrict__ wIr, uint32_t* __restrict__ Gp,
-                 uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
-  __shared__ uint32_t cur[32];
-  const uint32_t U = threadIdx.x, mask = (1u << b) - 1u, low = U & (~U + 1u);
-  const bool has = U <= mask;
-  const uint32_t w = has ? (uint32_t)load_wI(wIr + U) : 0u;
-  uint32_t gp = 0, A = 0;
-  for (int p = 0; p <= b; ++p) {
-    if (has && __popc(U) == p) {
-      if (p == 1) gp = w << b;
-      if (p >= 2) {
-        uint32_t best = 0xFFFFFFFFu;
-        const uint32_t rest = U ^ low;
-        for (uint32_t sub = 0; sub != rest; sub = (sub - rest) & rest) {
-          const uint32_t a = low | sub;
-          best = min(best, cur[a] + cur[U ^ a] + a);  // (value << b) + A
-        }
-        gp = ((best >> b) - w) << b;
-        A = best & mask;
-      }
-      cur[U] = gp;
-    }
-    __syncwarp();
-  }
-  if (has) put_tile0(L, b, perm, U, gp, A, Gp, Gc, split_rot, flags);
-}
-
-// acc[s2] = min over a2 within s2 holding lowbit(s2) of x[a2] + y[s2 ^ a2], s2 = 1..31
-__device__ __forceinline__ void conv_rows_low(uint32_t (&acc)[kRow], const uint32_t (&x)[kRow],
-                                              const uint32_t (&y)[kRow]) {
-#pragma unroll
-  for (int a2 = 1; a2 < kRow; ++a2) {
-#pragma unroll
-    for (int s2 = 1; s2 < kRow; ++s2)
-      if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0) acc[s2] = min(acc[s2], x[a2] + y[s2 ^ a2]);
-  }
-}
-
-// b >= 6, row-blocked: U = (s1, s2), rows s1 of 32 entries, level by level in
-// |s1|.  A split of U names its part A = (a1, a2) holding lowbit(U):
-//   * s2 != 0: a2 holds lowbit(s2), any a1 within s1; a1 not in {0, s1}: rows
-//     of earlier levels, a register convolution of two rows (phase A); a1 = 0
-//     and a1 = s1: the in-row recurrence, in increasing s2, in registers
-//     (phase B, one thread per row);
-//   * s2 = 0: a1 holds lowbit(s1), the entry-0 column of the same row pairs.
-// cur holds F << b; the key of A | B is cur[A] + cur[B] + A = (value << b) + A.
-// One block is all there is to run, so its chains bound it: phase A spreads a
-// row's 2^p1 - 2 row pairs over 2^(p1 - 1) lanes (at most 32), and the 32
-// minima of a row then reduce by shuffles.  m = 12: 275 us with one subset per
-// lane group and a block barrier per size of U (a lane per few submasks, each
-// two dependent shared loads), 34 us in this form.
-constexpr int kT0Threads = 384;
-constexpr int kT0LevelRows = 35;  // C(7, 3)
-
-template <typename Tab>
-__global__ void __launch_bounds__(kT0Threads)
-k_dp_tile0(int L, int b, InnerPerm perm, const Tab* __restrict__ wIr, uint32_t* __restrict__ Gp,
-           uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
-  __shared__ __align__(16) uint32_t cur[kWin];
-  __shared__ uint32_t ws[kRows * (kRow + 1)];            // w(I), then split
-  __shared__ uint32_t amin[kT0LevelRows * (kRow + 1)];   // phase A minima of a level's rows
-  const int t = threadIdx.x, nb = b - kB2;
-  const uint32_t mask = (1u << b) - 1u;
-  for (uint32_t v = t; v <= mask; v += kT0Threads) {
-    const uint32_t U = perm.nat(v);
-    ws[U + (U >> kB2)] = (uint32_t)load_wI(wIr + v);
-  }
-  __syncthreads();
-  // level 0: row 0, the recurrence on the five lowest inner requests
-  if (t == 0) {
-    uint32_t c[kRow];
-#pragma unroll
-    for (int s2 = 0; s2 < kRow; ++s2) {
-      uint32_t f = 0, A = 0;
-      if ((s2 & (s2 - 1)) == 0) {
-        f = s2 ? ws[s2] : 0u;
-      } else {
-        uint32_t key = 0xFFFFFFFFu;
-#pragma unroll
-        for (int a2 = 1; a2 < kRow; ++a2)
-          if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0 && a2 != s2) key = min(key, c[a2] + c[s2 ^ a2] + (uint32_t)a2);
-        f = (key >> b) - ws[s2];
-        A = key & mask;
-      }
-      c[s2] = f << b;
-      ws[s2] = A;
-    }
-#pragma unroll
-    for (int i = 0; i < kRow; ++i) cur[i] = c[i];  // row 0 is at position 0
-  }
-  __syncthreads();
-  for (int p1 = 1; p1 <= nb; ++p1) {
-    const int rows = (int)c_binom.v[nb][p1];
-    if (p1 >= 2) {
-      const int g = p1 - 1 < 5 ? p1 - 1 : 5, G = 1 << g;  // lanes per row: at most 35 x 8 = 280, 21 x 16 = 336
-      const int ri = t >> g;
-      const uint32_t r = (uint32_t)t & (uint32_t)(G - 1);
-      uint32_t acc[kRow];
-#pragma unroll
-      for (int i = 0; i < kRow; ++i) acc[i] = 0xFFFFFFFFu;
-      if (ri < rows) {
-        const uint32_t s1 = colex_unrank((unsigned long long)ri, p1, nb);
-        const uint32_t lowb = s1 & (~s1 + 1u);
-        uint32_t hi = 0, rr = s1;
-        for (int q = 0; q < g; ++q) {
-          const uint32_t top = 1u << (31 - __clz(rr));
-          hi |= top;
-          rr ^= top;
-        }
-        const uint32_t freem = s1 ^ hi;
-        const uint32_t fixed = deposit_bits(r, hi);
-        uint32_t sub = 0;
-        do {
-          const uint32_t a1 = fixed | sub;
-          if (a1 != 0 && a1 != s1) {
-            uint32_t x[kRow], y[kRow];
-            load_row(x, cur + row_pos(a1) * kRowStride);
-            load_row(y, cur + row_pos(s1 ^ a1) * kRowStride);
-#pragma unroll
-            for (int i = 0; i < kRow; ++i) x[i] += (a1 << kB2) | (uint32_t)i;
-            conv_rows_low(acc, x, y);
-            if (a1 & lowb) acc[0] = min(acc[0], x[0] + y[0]);
-          }
-          sub = (sub - freem) & freem;
-        } while (sub != 0);
-      }
-      for (int off = G >> 1; off > 0; off >>= 1) {
-#pragma unroll
-        for (int i = 0; i < kRow; ++i) acc[i] = min(acc[i], __shfl_xor_sync(0xFFFFFFFFu, acc[i], off));
-      }
-      if (ri < rows && r == 0) {
-#pragma unroll
-        for (int i = 0; i < kRow; ++i) amin[ri * (kRow + 1) + i] = acc[i];
-      }
-      __syncthreads();
-    }
-    if (t < rows) {
-      const uint32_t s1 = colex_unrank((unsigned long long)t, p1, nb), S1 = s1 << kB2;
-      uint32_t* own = ws + s1 * (kRow + 1);
-      uint32_t z[kRow], c[kRow];
-      load_row(z, cur);
-#pragma unroll
-      for (int s2 = 0; s2 < kRow; ++s2) {
-        const uint32_t w = own[s2];
-        uint32_t f = w, A = 0;
-        if (!(s2 == 0 && p1 == 1)) {  // else U = (s1, 0) is a single request
-          // two independent minima (a1 = 0 and a1 = s1) shorten the chains
-          uint32_t k0 = p1 >= 2 ? amin[t * (kRow + 1) + s2] : 0xFFFFFFFFu, k1 = 0xFFFFFFFFu;
-#pragma unroll
-          for (int a2 = 1; a2 < kRow; ++a2) {
-            if ((a2 & s2) == a2 && (a2 & (s2 & -s2)) != 0) {
-              k0 = min(k0, z[a2] + c[s2 ^ a2] + (uint32_t)a2);
-              if (a2 != s2) k1 = min(k1, c[a2] + z[s2 ^ a2] + (S1 | (uint32_t)a2));
-            }
-          }
-          const uint32_t key = min(k0, k1);
-          f = (key >> b) - w;
-          A = key & mask;
-        }
-        c[s2] = f << b;
-        own[s2] = A;
-      }
-      uint4* dst = reinterpret_cast<uint4*>(cur + row_pos(s1) * kRowStride);
-#pragma unroll
-      for (int q = 0; q < kRow / 4; ++q) dst[q] = make_uint4(c[4 * q], c[4 * q + 1], c[4 * q + 2], c[4 * q + 3]);
-    }
-    __syncthreads();
-  }
-  for (uint32_t U = t; U <= mask; U += kT0Threads)
-    put_tile0(L, b, perm, U, cur[row_pos(U >> kB2) * kRowStride + (U & (kRow - 1))], ws[U + (U >> kB2)], Gp, Gc,
-              split_rot, flags);
 }
 
 // Row-blocked tile kernel for |T| = kh >= 1 (inner bits b = kB).  The self
@@ -1035,22 +848,9 @@ cudaError_t blocked_attributes(bool listed) {
   return e;
 }
 
-// The tile kernel of step kh (info: the pruned recurrence's lists, or null).
+// The tiles of step kh >= 1 (info: the pruned recurrence's lists, or null).
 void launch_tiles(const Shape& s, const Workspace& ws, int kh, const uint32_t* info, cudaStream_t stream) {
   const unsigned long long tiles = h_binom.v[s.L][kh];
-  if (kh == 0) {
-    auto go = [&](const auto* wIr) {
-      if (s.b <= kB2)
-        k_dp_tile0_small<<<1, 32, 0, stream>>>(s.L, s.b, s.perm, wIr, ws.Gp, ws.Gc, ws.split_rot, ws.counters + 1);
-      else
-        k_dp_tile0<<<1, kT0Threads, 0, stream>>>(s.L, s.b, s.perm, wIr, ws.Gp, ws.Gc, ws.split_rot, ws.counters + 1);
-    };
-    if (s.lean)
-      go(ws.fw_rot);
-    else
-      go(ws.wI_rot);
-    return;
-  }
   const unsigned long long* part = kh >= 2 ? ws.partial : nullptr;
   const bool zg = s.L >= kZcGlobalMinL;
   const int sm_bytes = rows_smem_bytes(zg);
@@ -1104,7 +904,10 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
       if (e != cudaSuccess) return e;
     }
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches], stream);
-    launch_tiles(s, ws, kh, nullptr, stream);
+    if (kh == 0)
+      launch_tile0(s, ws, stream);
+    else
+      launch_tiles(s, ws, kh, nullptr, stream);
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches + 1], stream);
     if (timing) timing->tile_launches++;
     ++*launches;
@@ -1114,54 +917,28 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
   return cudaSuccess;
 }
 
-// The pruned recurrence (k_dp_pruned.cu): each layer in k_dp_pruned; only when
-// the host's bound says that a long list is possible does the pair kernel run
-// before it, over the long lists, and the row kernel after it.
-cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
-                             BlockedTiming* timing) {
+cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
   cudaError_t e = blocked_attributes(true);
   if (e != cudaSuccess) return e;
-  const int L = s.L;
-  const unsigned long long sms = (unsigned long long)sm_count();
-  auto mark = [&](cudaEvent_t* ev, int i) {
-    if (timing && ev) cudaEventRecord(ev[i], stream);
-  };
-  for (int kh = 0; kh <= L; ++kh) {
-    const unsigned long long tiles = h_binom.v[L][kh];
-    const uint32_t blocks = kh >= 2 ? pruned_items(s, kh) : 1u;  // per tile, in k_dp_pruned
-    const bool meet = pruned_meet(s, kh, blocks);
-    if (meet) {
-      e = cudaMemsetAsync(ws.partial, 0xFF, (size_t)(tiles << kB) * sizeof(unsigned long long), stream);
-      if (e != cudaSuccess) return e;
-    }
-    if (kh >= 2 && s.prune_long) {
-      const uint32_t P = (1u << (kh - 1)) - 1u;
-      // blocks for about four waves, and enough that a block's pairs fit its list
-      unsigned long long items = (4 * sms + tiles - 1) / tiles;
-      const unsigned long long most = (P + kMinPairsPerItem - 1) / kMinPairsPerItem;
-      const unsigned long long least = (P + kListCap - 1) / kListCap;
-      if (items > most) items = most;
-      if (items < least) items = least;
-      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches);
-      const ListedPairs lp{ws.prune_info, ws.prune_long, ws.prune_n,
-                           reinterpret_cast<unsigned int*>(ws.counters + 2)};
-      k_dp_pairs<true><<<(unsigned)(tiles * items), kPairThreads, kListedSmemBytes, stream>>>(
-          ws.Gp, ws.Gc, ws.partial, L, kh, P, (uint32_t)items, 0u, ws.counters + 1, lp);
-      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches++ + 1);
-      ++*launches;
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches);
-    if (kh >= 1) e = launch_pruned_layer(s, ws, kh, blocks, meet ? ws.partial : nullptr, stream, launches);
-    if (e != cudaSuccess) return e;
-    if (kh == 0 || s.prune_long) {
-      launch_tiles(s, ws, kh, kh == 0 ? nullptr : ws.prune_info, stream);
-      ++*launches;
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches++ + 1);
-  }
-  return cudaSuccess;
+  const unsigned long long tiles = h_binom.v[s.L][kh], sms = (unsigned long long)sm_count();
+  const uint32_t P = (1u << (kh - 1)) - 1u;
+  // blocks for about four waves, and enough that a block's pairs fit its list
+  unsigned long long items = (4 * sms + tiles - 1) / tiles;
+  const unsigned long long most = (P + kMinPairsPerItem - 1) / kMinPairsPerItem;
+  const unsigned long long least = (P + kListCap - 1) / kListCap;
+  if (items > most) items = most;
+  if (items < least) items = least;
+  const ListedPairs lp{ws.prune_info, ws.prune_long, ws.prune_n, reinterpret_cast<unsigned int*>(ws.counters + 2)};
+  k_dp_pairs<true><<<(unsigned)(tiles * items), kPairThreads, kListedSmemBytes, stream>>>(
+      ws.Gp, ws.Gc, ws.partial, s.L, kh, P, (uint32_t)items, 0u, ws.counters + 1, lp);
+  ++*launches;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
+  launch_tiles(s, ws, kh, ws.prune_info, stream);
+  ++*launches;
+  return cudaGetLastError();
 }
 
 }  // namespace mpt

@@ -28,10 +28,14 @@
 // Long lists go through the pair kernel of the full recurrence on just those
 // Ta, and tiles with a long list through its row kernel (k_dp_blocked.cu).
 //
+// 64-bit keys have no pair kernel for long lists: their rows beyond the first
+// kPruneRows are read from the table as they come.
+//
 // Measured on one GB300 (whole solve with layout and tables, full recurrence
 // before, pruned after): 28 requests of 20 passages 673 -> 7.6 .. 23 ms by
 // seed (a passage held by 12 to 17 of the 28 decides it), 24 requests of 10
-// passages 11.1 -> 1.3 ms, 26 requests of 40 passages 81 -> 19 .. 29 ms.
+// passages 11.1 -> 0.9 ms and with 64-bit keys 80 -> 1.0 ms, 26 requests of 40
+// passages 81 -> 17 .. 29 ms.
 // k_dp_pruned is bound by the integer ALU pipe where a popular passage gives
 // long a1 lists: 55 % of the pipe busy in the heaviest layers of the first 26
 // of the 28 requests, a sixth of it on the bookkeeping per pair, the rest of
@@ -50,8 +54,10 @@ constexpr int kPB = 12;  // inner bits of a tile
 constexpr uint32_t kPMask = (1u << kPB) - 1u;
 constexpr int kPQueue = 512;     // pairs queued between two rounds of evaluation
 constexpr int kQueueShift = 20;  // queue entries: Ta below (L <= 20), rows above
-static_assert(kPruneRows < 1 << (32 - kQueueShift), "queue entries hold the row count");
+static_assert(256 < 1 << (32 - kQueueShift), "queue entries hold the row count");
 constexpr int kRowBytes = 128;
+constexpr int kMembersShift = 9;  // info: rows below, members above
+constexpr uint32_t kRowsMask = (1u << kMembersShift) - 1u;
 constexpr uint32_t kUnitSteps = 60;
 constexpr uint32_t kLongSteps = 9000;  // a pair of the full recurrence runs 2,187 units of 243 steps on 8 warps
 constexpr int kPruneMinPairs = 16;     // pairs that a further block of a tile has to have
@@ -64,6 +70,8 @@ struct PrunedCfg {
   static constexpr int kRow = 1 << kRB;
   static constexpr int kRows = 1 << (kPB - kRB);  // = threads per block
   static constexpr int kLogWarps = kPB - kRB - 5;
+  // rows kept per Ta: those of a short list, or all (64-bit keys have no other kernel for a long one)
+  static constexpr int kKept = sizeof(Key) == 4 ? kPruneRows : kRows;
   static constexpr int kBlocks = sizeof(Key) == 4 ? 4 : 2;  // per SM
   static constexpr int kSlots = 2;
   static constexpr int kSlotBytes = (kRows + kPruneRows) * kRowBytes;  // Y window, X rows
@@ -84,10 +92,11 @@ struct PrunedCfg {
 // writes it once per 8 to 12 request bits after a clear.
 // m = 28: 0.29 + 2.0 ms of clear and transform (HBM-bound) -> 0.29 ms (7.5 TB/s written).
 // The row list: threads = rows, the mask of a row from its non-zero entries.
-// info: 0 when T has no member, else rows | members << 8 | kListLong when
-// they are more than kPruneRows or, where the pair kernel runs (long_ok), cost
-// more than a pair there | kTileLong when the tile is left to the row kernel (a
-// long list, or more than kPruneSelf members).  Cost: a row takes as many
+// info: 0 when T has no member, else rows | members << kMembersShift |
+// kListLong (32-bit keys) when they are more than kPruneRows or, where the pair
+// kernel runs (long_ok), cost more than a pair there | kTileLong when the tile
+// is left to the row kernel (a long list, or more than kPruneRows rows or
+// kPruneSelf members).  Cost: a row takes as many
 // warps as have a lane whose row holds a1, each for its steps and the loads,
 // here kUnitSteps steps' worth.
 template <typename Key, typename G>
@@ -120,8 +129,8 @@ k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N,
     if (!clear) {
       for (uint32_t v = tid; v < (1u << kPB) / kPer; v += kThreads) reinterpret_cast<uint4*>(out)[v] = make_uint4(0, 0, 0, 0);
       if (tid == 0) {
-        info[T] = single ? 1u | (1u << 8) : 0u;  // a single request is always listed
-        if (single) rows[(size_t)T * kPruneRows] = make_uint2(0u, 1u);
+        info[T] = single ? 1u | (1u << kMembersShift) : 0u;  // a single request is always listed
+        if (single) rows[(size_t)T * C::kKept] = make_uint2(0u, 1u);
       }
       continue;
     }
@@ -167,12 +176,13 @@ k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N,
       nm += warp_m[q];
       nc += warp_c[q];
     }
-    if (mask && at < (uint32_t)kPruneRows) rows[(size_t)T * kPruneRows + at] = make_uint2(tid, mask);
+    if (mask && at < (uint32_t)C::kKept) rows[(size_t)T * C::kKept + at] = make_uint2(tid, mask);
     if (tid == 0) {
-      const bool is_long = nr > (uint32_t)kPruneRows || (long_ok && nc > kLongSteps);
+      const bool many = nr > (uint32_t)kPruneRows;
+      const bool is_long = sizeof(Key) == 4 && (many || (long_ok && nc > kLongSteps));
       info[T] = nr == 0 ? 0u
-                        : min(nr, 255u) | (nm << 8) | (is_long ? kListLong : 0u) |
-                              (is_long || nm > (uint32_t)kPruneSelf ? kTileLong : 0u);
+                        : nr | (nm << kMembersShift) | (is_long ? kListLong : 0u) |
+                              (is_long || many || nm > (uint32_t)kPruneSelf ? kTileLong : 0u);
     }
   }
 }
@@ -338,14 +348,16 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 // the block: rows with more of a list's a1 bits take longer, and the blocks
 // of one SM then load its four sub-partitions about alike.
 // Blocks of one tile, rounds of one block beyond the queue and, with
-// long_lists, the pair kernel's minima meet in `partial`: (key << 32 | Ta),
-// 32-bit keys only.  The block that finishes last (done[]) goes on to the
-// tile's entries.
+// long_lists, the pair kernel's minima meet in `partial` ((key << 32 | Ta); for
+// 64-bit keys, one block per tile and no pair kernel, the key, and Ta in
+// partial_ta).  The block that finishes last (done[]) goes on to the tile's
+// entries.
 template <typename Key, typename Tab>
 __global__ void __launch_bounds__(PrunedCfg<Key>::kRows, PrunedCfg<Key>::kBlocks)
 k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
             const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
-            const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* __restrict__ done, Key* Gp,
+            const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* partial_ta,
+            uint32_t* __restrict__ done, Key* Gp,
             Key* Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
   using C = PrunedCfg<Key>;
   constexpr int kRB = C::kRB, kRow = C::kRow, NT = C::kRows, kWarps = NT / 32;
@@ -371,8 +383,11 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   if (MPT_BAD(flags, T < (1u << L) && __popc(T) == kh)) return;
   const uint32_t iT = info[T];
   const bool long_tile = (iT & kTileLong) != 0;
-  if (long_tile && kh == 1) return;  // no pairs: the row kernel does it all
-  const uint32_t cT = (iT >> 8) & 0x1FFFu;
+  if (long_tile && kh == 1) {  // no pairs: the row kernel does it all
+    if (!long_lists && tid == 0) atomicOr(flags, kErrWorkspace);
+    return;
+  }
+  const uint32_t cT = (iT >> kMembersShift) & 0x1FFFu;
   const int l = __ffs(T) - 1;
   const uint32_t low = 1u << l, rest = T ^ low;
   // (the blocks of one SM differ by a multiple of 4, hence the hash)
@@ -409,7 +424,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
 #pragma unroll
     for (int j = 0; j < kHeld; ++j) {
       const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
-      if (r < n) held[j] = rows[(size_t)Tp * kPruneRows + r];
+      if (r < n && r < (uint32_t)kPruneRows) held[j] = rows[(size_t)Tp * C::kKept + r];
     }
   };
   auto stage = [&](uint32_t p, uint32_t s) {
@@ -421,7 +436,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
 #pragma unroll
     for (int j = 0; j < kHeld; ++j) {
       const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
-      if (r < n) {
+      if (r < n && r < (uint32_t)kPruneRows) {
         if (col == 0) s_rows[s][r] = make_uint2(held[j].x | (n << 16), held[j].y);
         pcopy16(slot + (NT + r) * kRowBytes + col, x + held[j].x * kRowBytes + col);
       }
@@ -439,7 +454,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     const uint32_t Ta = by_parts ? (low | deposit_bits(i, rest)) : mem[i];
     if ((Ta & ~T) != 0 || Ta == T) return 0u;
     const uint32_t c = info[Ta];
-    return c == 0 || (c & kListLong) ? 0u : Ta | ((c & 255u) << kQueueShift);
+    return c == 0 || (c & kListLong) ? 0u : Ta | ((c & kRowsMask) << kQueueShift);
   };
   // Blocks of this tile that take part: as many as there are kPruneMinPairs
   // pairs for (the same number in each of them).
@@ -470,12 +485,14 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     for (int i = 0; i < kRow; ++i) skey[s1 * (kRow + 1) + i] = bk[i];
     __syncthreads();
   };
-  unsigned long long* pt = partial + ((size_t)tile << kPB);  // 32-bit keys
+  unsigned long long* pt = partial + ((size_t)tile << kPB);
+  uint32_t* pt_ta = partial_ta + ((size_t)tile << kPB);  // 64-bit keys
   // the Ta of an output's best pair, before the self pair: from the queue, or
   // where the minima have met
   bool met = parts > 1;  // minima in `partial`
   auto ta_at = [&](uint32_t U) -> uint32_t {
-    return met ? (uint32_t)__ldcg(&pt[U]) : queue[seq_at(U)] & ((1u << kQueueShift) - 1u);
+    if (!met) return queue[seq_at(U)] & ((1u << kQueueShift) - 1u);
+    return sizeof(Key) == 4 ? (uint32_t)__ldcg(&pt[U]) : pt_ta[U];
   };
   auto to_partial = [&]() {
     for (uint32_t U = tid; U <= kPMask; U += NT) {
@@ -487,7 +504,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
 
   // The pairs, a queue of them at a time.
   uint32_t found = 0, base = 0;
-  if (long_lists && kh >= 2) {
+  if (sizeof(Key) == 4 && long_lists && kh >= 2) {
     // has T a part with a long list?
     const uint32_t nl = member_n[kMaxMembersL + l];
     bool any = false;
@@ -555,11 +572,11 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       // are finished, then offered to the later ones.  Then X = their rows.
       stage_window(psm, Gc);
       asm volatile("cp.async.commit_group;" ::: "memory");
-      const uint32_t n = iT & 255u;
+      const uint32_t n = iT & kRowsMask;  // at most kPruneRows
       if (tid <= (uint32_t)kPB + 1) s_start[tid] = 0;
       if (warp == 0) {
         static_assert(kPruneRows <= 32, "one list row per lane");
-        const uint2 own = lane < n ? rows[(size_t)T * kPruneRows + lane] : make_uint2(0u, 0u);
+        const uint2 own = lane < n ? rows[(size_t)T * C::kKept + lane] : make_uint2(0u, 0u);
         uint32_t at = 0;
         for (uint32_t k = 0; k < n; ++k) {
           const uint2 e = make_uint2(__shfl_sync(0xFFFFFFFFu, own.x, k), __shfl_sync(0xFFFFFFFFu, own.y, k));
@@ -633,7 +650,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       Key acc[kRow];
 #pragma unroll
       for (int i = 0; i < kRow; ++i) acc[i] = kNone;
-      for (uint32_t k = 0; k < n; ++k) {
+      for (uint32_t k = 0; k < min(n, (uint32_t)kPruneRows); ++k) {
         const uint32_t a1 = list[k].x & 0xFFFFu, mask = list[k].y;
         if ((a1 & ~s1) != 0) continue;
         Key y[kRow];
@@ -644,6 +661,18 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           pconv<Key, kRow, true>(acc, x, y, mask);
         else
           pconv<Key, kRow, false>(acc, x, y, mask);
+      }
+      if constexpr (C::kKept > kPruneRows) {
+        // the rest of a long list, its rows of X straight from the table
+        const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u);
+        for (uint32_t k = kPruneRows; k < n; ++k) {
+          const uint2 e = rows[(size_t)Tp * C::kKept + k];
+          if ((e.x & ~s1) != 0) continue;
+          Key y[kRow];
+          const uint32_t r = s1 ^ e.x;
+          pload_row<Key, kRow>(y, slot + r * kRowBytes, (r & 7u) * 16u);
+          pconv<Key, kRow, false>(acc, reinterpret_cast<const char*>(Gp + (((size_t)Tp << kPB) | (e.x << kRB))), y, e.y);
+        }
       }
       __syncwarp();
       const uint16_t number = (uint16_t)(phase == 0 ? p : kSelf);
@@ -686,6 +715,35 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           const unsigned long long v = __ldcg(&pt[U]);
           key_at(U) = (Key)(v >> 32);
         }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kRow; ++i) bk[i] = skey[s1 * (kRow + 1) + i];
+      }
+    }
+    if constexpr (sizeof(Key) == 8) {
+      // one block per tile, its rounds one after the other: plain merges; a
+      // tile left to the row kernel has its minima in its slot there
+      if (met || base < total || long_tile) {
+        for (uint32_t U = tid; U <= kPMask; U += NT) {
+          const Key k = key_at(U);
+          const uint32_t ta = queue[seq_at(U)] & ((1u << kQueueShift) - 1u);
+          if (!met || k < pt[U] || (k == pt[U] && ta < pt_ta[U])) {
+            pt[U] = k;
+            pt_ta[U] = ta;
+          }
+        }
+        met = true;
+        __syncthreads();
+        if (base < total) {
+#pragma unroll
+          for (int i = 0; i < kRow; ++i) {
+            bk[i] = kNone;
+            seq[i * C::kSeqStride + tid] = 0;
+          }
+          continue;
+        }
+        if (long_tile && long_lists) return;
+        for (uint32_t U = tid; U <= kPMask; U += NT) key_at(U) = pt[U];
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kRow; ++i) bk[i] = skey[s1 * (kRow + 1) + i];
@@ -745,7 +803,7 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
   if (e != cudaSuccess) return e;
   k<<<(unsigned)(h_binom.v[s.L][kh] * items), C::kRows, C::kSmem, stream>>>(
-      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long, ws.prune_n, partial, ws.prune_done, Gp, Gc,
+      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long, ws.prune_n, partial, ws.partial_ta, ws.prune_done, Gp, Gc,
       ws.split_rot, ws.counters + 1);
   ++*launches;
   return cudaGetLastError();
@@ -756,8 +814,12 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
 cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
   cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, kPruneSplitTiles * 4, stream);
   if (e != cudaSuccess) return e;
-  if (s.lean) return tables<uint32_t>(s, ws, reinterpret_cast<unsigned int*>(ws.fw_rot), stream, launches);
-  return tables<uint32_t>(s, ws, reinterpret_cast<unsigned long long*>(ws.wI_rot), stream, launches);
+  auto* lean = reinterpret_cast<unsigned int*>(ws.fw_rot);
+  auto* full = reinterpret_cast<unsigned long long*>(ws.wI_rot);
+  if (s.wide)
+    return s.lean ? tables<unsigned long long>(s, ws, lean, stream, launches)
+                  : tables<unsigned long long>(s, ws, full, stream, launches);
+  return s.lean ? tables<uint32_t>(s, ws, lean, stream, launches) : tables<uint32_t>(s, ws, full, stream, launches);
 }
 
 // Blocks per tile of a layer with 32-bit keys.  The pairs of a tile vary from
@@ -767,7 +829,7 @@ cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_
 uint32_t pruned_items(const Shape& s, int kh) {
   constexpr double kPartPairs = 48, kMostBlocks = 16384;
   const double tiles = (double)h_binom.v[s.L][kh];
-  if (tiles > kPruneSplitTiles) return 1;
+  if (s.wide || kh < 2 || tiles > kPruneSplitTiles) return 1;
   const double P = (double)((1ull << (kh - 1)) - 1ull), most = P < s.prune_most ? P : s.prune_most;
   const double items = most / kPartPairs < kMostBlocks / tiles ? most / kPartPairs : kMostBlocks / tiles;
   return items < 1.0 ? 1u : (uint32_t)items;
@@ -775,15 +837,44 @@ uint32_t pruned_items(const Shape& s, int kh) {
 
 // Whether the blocks of a layer meet in `partial`.
 bool pruned_meet(const Shape& s, int kh, uint32_t items) {
-  if (kh < 2) return false;
+  if (s.wide || kh < 2) return false;
   const double P = (double)((1ull << (kh - 1)) - 1ull);
   return s.prune_long || items > 1 || (P < s.prune_most ? P : s.prune_most) > (double)kPQueue;
 }
 
-cudaError_t launch_pruned_layer(const Shape& s, const Workspace& ws, int kh, uint32_t items,
-                                unsigned long long* partial, cudaStream_t stream, int* launches) {
-  if (s.lean) return layer<uint32_t>(s, ws, ws.fw_rot, kh, items, partial, ws.Gp, ws.Gc, stream, launches);
-  return layer<uint32_t>(s, ws, ws.wI_rot, kh, items, partial, ws.Gp, ws.Gc, stream, launches);
+cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
+                             BlockedTiming* timing) {
+  cudaError_t e = cudaSuccess;
+  auto mark = [&](cudaEvent_t* ev, int i) {
+    if (timing && ev) cudaEventRecord(ev[i], stream);
+  };
+  for (int kh = 0; kh <= s.L && e == cudaSuccess; ++kh) {
+    const uint32_t items = pruned_items(s, kh);
+    if (pruned_meet(s, kh, items))
+      e = cudaMemsetAsync(ws.partial, 0xFF, (size_t)(h_binom.v[s.L][kh] << kPB) * sizeof(unsigned long long), stream);
+    if (e == cudaSuccess && kh >= 2 && s.prune_long && !s.wide) {
+      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches);
+      e = launch_listed_pairs(s, ws, kh, stream, launches);
+      if (timing) mark(timing->pair_ev, 2 * timing->pair_launches++ + 1);
+    }
+    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches);
+    if (e == cudaSuccess && kh == 0) {
+      e = launch_tile0(s, ws, stream);
+      ++*launches;
+    } else if (e == cudaSuccess) {
+      if (s.wide)
+        e = s.lean ? layer(s, ws, ws.fw_rot, kh, items, ws.partial, ws.Gp64, ws.Gc64, stream, launches)
+                   : layer(s, ws, ws.wI_rot, kh, items, ws.partial, ws.Gp64, ws.Gc64, stream, launches);
+      else
+        e = s.lean ? layer(s, ws, ws.fw_rot, kh, items, ws.partial, ws.Gp, ws.Gc, stream, launches)
+                   : layer(s, ws, ws.wI_rot, kh, items, ws.partial, ws.Gp, ws.Gc, stream, launches);
+      if (e == cudaSuccess && s.prune_long)
+        e = s.wide ? launch_wide_listed_tiles(s, ws, kh, stream, launches)
+                   : launch_listed_tiles(s, ws, kh, stream, launches);
+    }
+    if (timing) mark(timing->tile_ev, 2 * timing->tile_launches++ + 1);
+  }
+  return e;
 }
 
 }  // namespace mpt

@@ -24,10 +24,10 @@
 // every pair (pairs in increasing Ta, strict improvement), and each block
 // writes its 4096 bests to a slot of its own: no atomics in global memory.
 //
-// Tile kernel.  One block per tile finishes all 4096 entries level by level
-// in |U|: the self pair (A = (T, Ua), B = (0, U \ Ua)) or, for tile 0, the
-// whole recurrence over the inner bits, by lanes per subset, then the
-// lexicographic (key, Ta) minimum with the tile's pair slots.
+// Tile kernel (|T| >= 1; tile 0 is k_dp_tile0.cu's).  One block per tile
+// finishes all 4096 entries level by level in |U|: the self pair
+// (A = (T, Ua), B = (0, U \ Ua)) by lanes per subset, then the lexicographic
+// (key, Ta) minimum with the tile's pair slots.
 #include "mpt_internal.cuh"
 
 namespace mpt {
@@ -354,27 +354,21 @@ template <typename Tab>
 __global__ void __launch_bounds__(kWTileThreads)
 k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __restrict__ pkey,
             const uint32_t* __restrict__ pta, uint32_t items, u64* __restrict__ Gp, u64* __restrict__ Gc,
-            uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
+            uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags, const uint32_t* __restrict__ info, InnerPerm perm) {
   extern __shared__ __align__(16) u64 tsm[];
   u64* cur = tsm;                       // this tile, F << b
-  u64* oc = tsm + (1 << kWB);           // complement form: this tile (kh = 0) or tile 0 (kh >= 1)
+  u64* oc = tsm + (1 << kWB);           // complement form of tile 0
   uint16_t* order = reinterpret_cast<uint16_t*>(tsm + 2 * (1 << kWB));  // subsets by size, then colex
 
   const uint32_t tile = blockIdx.x;
-  const uint32_t T = kh == 0 ? 0u : colex_unrank(tile, kh, L);
+  const uint32_t T = colex_unrank(tile, kh, L);
+  if (info && !(info[T] & kTileLong)) return;  // finished by k_dp_pruned
   const int size = 1 << b;
   const uint32_t mask = (uint32_t)size - 1u;
 
   for (int u = threadIdx.x; u < size; u += kWTileThreads) {
-    if (b == kWB) {
-      order[u] = g_order12.v[u];
-    } else {  // fewer than 12 requests: tile 0 only, one block
-      const int p = __popc(u);
-      uint32_t start = 0;
-      for (int j = 0; j < p; ++j) start += (uint32_t)c_binom.v[b][j];
-      order[start + colex_rank((uint32_t)u)] = (uint16_t)u;
-    }
-    if (kh >= 1) oc[u] = Gc[u];
+    order[u] = g_order12.v[u];
+    oc[u] = Gc[u];
   }
   __syncthreads();
 
@@ -395,11 +389,9 @@ k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __rest
         U = order[start + gi];
         const uint32_t nreq = (uint32_t)p + (uint32_t)kh;
         single = nreq == 1;
-        if (nreq >= 2 && !(kh >= 1 && U == 0)) {
-          // kh = 0: Ua = lowbit(U) | part, part a proper subset of U \ lowbit(U).
-          // kh >= 1: Ua = part, a proper subset of U (Ta = T).
-          const uint32_t lowU = kh == 0 ? (U & (~U + 1u)) : 0u;
-          const uint32_t emask = U ^ lowU;
+        if (nreq >= 2 && U != 0) {
+          // Ua: a proper subset of U (Ta = T)
+          const uint32_t emask = U;
           uint32_t hi = 0, rr = emask;
           for (int t = 0; t < g; ++t) {
             const uint32_t top = 1u << (31 - __clz(rr));
@@ -412,7 +404,7 @@ k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __rest
           do {
             const uint32_t part = fixed | s;
             if (part != emask) {
-              const uint32_t Ua = lowU | part;
+              const uint32_t Ua = part;
               const u64 key = cur[Ua] + oc[U ^ Ua];
               best = key < best ? key : best;
             }
@@ -420,11 +412,11 @@ k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __rest
           } while (s != 0);
         }
       }
-      // the self pair's candidates carry Ta = T (kh = 0: none); the pair
+      // the self pair's candidates carry Ta = T; the pair
       // kernel's slots of this tile, one per block, are spread over the G
       // lanes of the output; then the lexicographic (key, Ta) minimum of the
       // group, in which the self pair wins ties only against larger Ta
-      uint32_t ta = kh == 0 ? 0u : T;
+      uint32_t ta = T;
       if (active && kh >= 2) {
         for (uint32_t it = r; it < items; it += (uint32_t)G) {
           const size_t w = ((size_t)(tile * items + it) << b) | U;
@@ -448,22 +440,19 @@ k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __rest
         const size_t idx = ((size_t)T << b) | U;
         int64_t f;
         uint32_t A;
-        if (U == 0 && T == 0) {
-          f = 0;
-          A = 0;
-        } else if (single) {
+        const uint32_t nat = info ? perm.nat(U) : U;  // stored order undone (pruned recurrence)
+        if (single) {
           f = load_wI_w(wIr + idx);
           A = 0;
         } else {
-          const uint32_t Ua = (uint32_t)(best & mask) + U - mask;
+          const uint32_t Ua = (uint32_t)(best & mask) + nat - mask;
           f = (int64_t)(best >> b) - load_wI_w(wIr + idx);
           A = (Ua << L) | ta;
         }
         const u64 gp = (u64)f << b;
-        const u64 gc = gp | (u64)(~U & mask);
+        const u64 gc = gp | (u64)(~nat & mask);
         cur[U] = gp;
-        if (kh == 0) oc[U] = gc;
-        if (!MPT_BAD(flags, idx < ((size_t)1 << (L + b)) && valid_split(T | (U << L), A))) {
+        if (!MPT_BAD(flags, idx < ((size_t)1 << (L + b)) && valid_split(T | (nat << L), A))) {
           Gp[idx] = gp;
           Gc[idx] = gc;
           split_rot[idx] = A;
@@ -485,14 +474,45 @@ int64_t wide_partial_slots(int m, int b) {
   return most > 0 ? (int64_t)(2 * most) : 1;
 }
 
+namespace {
+
+// The tiles of step kh >= 1, with `items` slots each (info: the pruned
+// recurrence's lists, or null).
+void launch_wide_tiles(const Shape& s, const Workspace& ws, int kh, uint32_t items, const uint32_t* info,
+                       cudaStream_t stream) {
+  const unsigned tiles = (unsigned)h_binom.v[s.L][kh];
+  if (s.lean)
+    k_dp_tile_w<<<tiles, kWTileThreads, kWTileSmemBytes, stream>>>(s.L, s.b, kh, ws.fw_rot, ws.partial, ws.partial_ta,
+                                                                   items, ws.Gp64, ws.Gc64, ws.split_rot,
+                                                                   ws.counters + 1, info, s.perm);
+  else
+    k_dp_tile_w<<<tiles, kWTileThreads, kWTileSmemBytes, stream>>>(s.L, s.b, kh, ws.wI_rot, ws.partial, ws.partial_ta,
+                                                                   items, ws.Gp64, ws.Gc64, ws.split_rot,
+                                                                   ws.counters + 1, info, s.perm);
+}
+
+cudaError_t wide_tile_attributes() {
+  cudaError_t e = cudaFuncSetAttribute(k_dp_tile_w<int64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWTileSmemBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_dp_tile_w<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWTileSmemBytes);
+  return e;
+}
+
+}  // namespace
+
+cudaError_t launch_wide_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
+  const cudaError_t e = wide_tile_attributes();
+  if (e != cudaSuccess) return e;
+  launch_wide_tiles(s, ws, kh, 1u, ws.prune_info, stream);
+  ++*launches;
+  return cudaGetLastError();
+}
+
 cudaError_t launch_dp_wide(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                            BlockedTiming* timing, int step_begin, int step_end) {
   cudaError_t e = cudaFuncSetAttribute(k_dp_pairs_w, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmemBytes);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_dp_tile_w<int64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWTileSmemBytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_dp_tile_w<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWTileSmemBytes);
-  if (e != cudaSuccess) return e;
+  if ((e = wide_tile_attributes()) != cudaSuccess) return e;
   int sms = 0, dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -521,15 +541,11 @@ cudaError_t launch_dp_wide(const Shape& s, const Workspace& ws, cudaStream_t str
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches], stream);
-    const unsigned grid = kh == 0 ? 1u : (unsigned)tiles;
-    if (s.lean)
-      k_dp_tile_w<<<grid, kWTileThreads, kWTileSmemBytes, stream>>>(L, b, kh, ws.fw_rot, ws.partial, ws.partial_ta,
-                                                                     (uint32_t)items, ws.Gp64, ws.Gc64, ws.split_rot,
-                                                                     ws.counters + 1);
+    if (kh == 0)
+      e = launch_tile0(s, ws, stream);
     else
-      k_dp_tile_w<<<grid, kWTileThreads, kWTileSmemBytes, stream>>>(L, b, kh, ws.wI_rot, ws.partial, ws.partial_ta,
-                                                                     (uint32_t)items, ws.Gp64, ws.Gc64, ws.split_rot,
-                                                                     ws.counters + 1);
+      launch_wide_tiles(s, ws, kh, (uint32_t)items, nullptr, stream);
+    if (e != cudaSuccess) return e;
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches + 1], stream);
     if (timing) timing->tile_launches++;
     ++*launches;

@@ -101,7 +101,7 @@ void prune_shape(mpt_ctx* c) {
   mpt::Shape& s = c->shape;
   c->perm = mpt::InnerPerm{};
   s.pruned = s.prune_long = false;
-  if (c->mode != MPT_DP_AUTO || !s.blocked || s.wide || s.L < 1 || c->many_supports) return;
+  if (c->mode != MPT_DP_AUTO || !s.blocked || s.L < 1 || c->many_supports) return;
   double members[32], rows[32], tas[32];
   for (int l = 0; l < s.L; ++l) members[l] = rows[l] = tas[l] = 1.0;
   double time = 0.05 * (double)(1ull << s.L);
@@ -113,7 +113,7 @@ void prune_shape(mpt_ctx* c) {
     for (int l = s.L - 1; l >= 0; --l) {
       if (!((T >> l) & 1u)) continue;
       members[l] += (double)(1ull << __builtin_popcount(U));
-      rows[l] += (double)(1ull << __builtin_popcount(U >> 5));
+      rows[l] += (double)(1ull << __builtin_popcount(U >> (s.wide ? 4 : 5)));
       here += (double)(1ull << (s.L - 1 - l)) * above;
       tas[l] += above2;
       above *= 1.5;
@@ -149,7 +149,10 @@ void prune_shape(mpt_ctx* c) {
     return;  // the natural order
   }
   std::sort(cost.begin(), cost.end());
-  static const uint8_t place[12] = {0, 1, 2, 3, 4, 11, 10, 9, 8, 7, 6, 5};
+  // (64-bit keys: rows of 16, so four, three and five)
+  static const uint8_t place32[12] = {0, 1, 2, 3, 4, 11, 10, 9, 8, 7, 6, 5};
+  static const uint8_t place64[12] = {0, 1, 2, 3, 11, 10, 9, 8, 7, 6, 5, 4};
+  const uint8_t* place = s.wide ? place64 : place32;
   uint32_t left = (1u << s.b) - 1u;
   int n = 0;
   cost.emplace_back(0.0, left);
@@ -260,7 +263,7 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
     ws->shared_N = reinterpret_cast<uint32_t*>(take(ns * 4));
     ws->shared_w = reinterpret_cast<unsigned long long*>(take(ns * 8));
     ws->prune_info = reinterpret_cast<uint32_t*>(take(P * 4));
-    ws->prune_rows = reinterpret_cast<uint2*>(take(P * mpt::kPruneRows * sizeof(uint2)));
+    ws->prune_rows = reinterpret_cast<uint2*>(take(P * (s.wide ? 256 : mpt::kPruneRows) * sizeof(uint2)));
     ws->prune_short = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_long = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_n = reinterpret_cast<uint32_t*>(take(2 * mpt::kMaxMembersL * 4));

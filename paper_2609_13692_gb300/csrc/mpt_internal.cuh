@@ -236,7 +236,7 @@ struct Workspace {
   uint32_t* shared_N;     // [n_shared] rotated index of N_x of each chunk that some but not all requests share
   unsigned long long* shared_w;  // [n_shared] its weight
   uint32_t* prune_info;   // [2^L] row list of each Ta: rows, members, kListLong, kTileLong
-  uint2* prune_rows;      // [2^L * kPruneRows] (a1, mask of a2)
+  uint2* prune_rows;      // [2^L * kPruneRows, or 256 with 64-bit keys] (a1, mask of a2)
   uint32_t* prune_short;  // [2^L] Ta's with a short list, by lowest request
   uint32_t* prune_long;   // [2^L] Ta's with a long list, by lowest request
   uint32_t* prune_n;      // [2 * kMaxMembersL] their numbers per lowest request
@@ -341,10 +341,13 @@ cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t s
                              BlockedTiming* timing);
 // w(I) (instead of K2) and the lists; needs K1's list of shared chunks.
 cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
-uint32_t pruned_items(const Shape& s, int kh);
-bool pruned_meet(const Shape& s, int kh, uint32_t items);
-cudaError_t launch_pruned_layer(const Shape& s, const Workspace& ws, int kh, uint32_t items,
-                                unsigned long long* partial, cudaStream_t stream, int* launches);
+// Step kh over its long lists only: the 32-bit pair kernel, and the row kernels
+// of either key width on tiles with a long list.
+cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
+cudaError_t launch_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
+cudaError_t launch_wide_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
+// Tile 0 with either key width (k_dp_tile0.cu).
+cudaError_t launch_tile0(const Shape& s, const Workspace& ws, cudaStream_t stream);
 int64_t blocked_partial_entries(int m, int b);
 int blocked_tile_bits(int m);
 

@@ -87,6 +87,31 @@ def test_equals_the_full_recurrence(mpt, inst):
     assert torch.equal(F.long(), mpt.mpt_tables(b.ctx)[0])
 
 
+@pytest.mark.parametrize("inst", [c for c in _cases() if c.m <= 20], ids=lambda inst: inst.name.replace(" ", "_")[:40])
+def test_wide_equals_the_full_recurrence(mpt, inst):
+    """The same with weights too heavy for the 32-bit keys."""
+    w = inst.weights << 21
+    a = mpt.solve(w, inst.bits, mode="auto")
+    b = mpt.solve(w, inst.bits, mode="wide")
+    assert a.opt == b.opt
+    for x, y in zip(mpt.mpt_tables(a.ctx), mpt.mpt_tables(b.ctx)):
+        assert torch.equal(x, y)
+    assert a.perm_chunks.tolist() == b.perm_chunks.tolist() and a.dfs_order.tolist() == b.dfs_order.tolist()
+
+
+def test_wide_many_members(mpt):
+    """64-bit keys beyond one queue of pairs (more than 512 members per
+    lowest request) and lists of more than 32 rows."""
+    inst = _from_supports(24, [_mask(*range(0, 24, 2)) | _mask(1, 3, 5, 7, 9), _mask(*range(0, 12)), _mask(2, 13),
+                               _mask(0, *range(12, 24)), _mask(3, 20)], 8)
+    a = mpt.solve(inst.weights << 21, inst.bits)
+    b = mpt.solve(inst.weights, inst.bits, mode="blocked")
+    assert a.opt == b.opt << 21
+    Fa, wa, sa = mpt.mpt_tables(a.ctx)
+    Fb, wb, sb = mpt.mpt_tables(b.ctx)
+    assert torch.equal(Fa, Fb << 21) and torch.equal(wa, wb << 21) and torch.equal(sa, sb)
+
+
 def test_route(mpt):
     """Few shared chunks: no pair kernel.  Leave-one-out: the full one."""
     few = I.rag_pools(18, 3000, 5, 40, 8, 1.2, seed=3)
