@@ -518,6 +518,112 @@ __device__ __forceinline__ void bconv_restricted(uint32_t (&acc)[kBRow], const u
   }
 }
 
+// The recurrence over the splits that can be reported (k_dp_pruned.cu), for an
+// instance with few of them: the reported part A of S has one request or
+// w(I(A)) > w(I(S)) >= w(I(all)), so with w* = w(I(all)) every other A can be
+// left out, and a set that is no such "member" has w(I(S)) = w*.  Gp holds
+// w(I) on entry and (F << m) + X afterwards, as in the row form.  Members
+// are closed under taking parts (of two requests or more), so they are
+// finished first, size by size, each over its own parts; then the other sets,
+// by lowest request from the highest down (B = S \ A has a higher one), each
+// over the members of its lowest request.  list: the members by lowest
+// request, the single request first, as (A, Gp(A)); keys hold A, so the
+// order in a list does not matter.
+// False, with Gp untouched, when there is no room for the list or its tests
+// (sum over S of its list's length) are more than half of the row form's
+// 3^m / 2 splits.  1,000 groups of 14-16 requests: 5.7 -> 2.0 ms per solve;
+// 20,000 groups of 8-13: 1.49 -> 1.30 ms, most of it copies.  With the line at
+// a quarter of the splits 2.0 and 1.42 ms, at an eighth 2.8 and 1.53, at all
+// of them 2.0 and 1.27; a test costs two to four row steps, so half is where
+// an instance near the line loses least.
+template <int TPI, typename Put>
+__device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put) {
+  __shared__ int cnt[kBMaxRowsM], start[kBMaxRowsM + 1], most, use;
+  const int t = threadIdx.x;
+  const uint32_t N = 1u << m, mask = N - 1u;
+  if (t < kBMaxRowsM) cnt[t] = 1;
+  if (t == 0) most = 1;
+  __syncthreads();
+  const uint32_t wall = Gp[bidx(mask)];
+  for (uint32_t U = t; U < N; U += TPI)
+    if ((U & (U - 1u)) != 0 && Gp[bidx(U)] > wall) {
+      atomicAdd(&cnt[__ffs(U) - 1], 1);
+      atomicMax(&most, __popc(U));
+    }
+  __syncthreads();
+  if (t == 0) {
+    unsigned long long tests = 0, splits = 1;
+    int at = 0;
+    for (int l = 0; l < m; ++l) {
+      start[l] = at;
+      at += cnt[l];
+      tests += (unsigned long long)cnt[l] << (m - 1 - l);
+      splits *= 3;
+      cnt[l] = 1;
+    }
+    start[m] = at;
+    use = at <= cap && 2 * tests < splits / 2;
+  }
+  __syncthreads();
+  if (!use) return false;
+  for (uint32_t U = t; U < N; U += TPI) {
+    const uint32_t v = Gp[bidx(U)];
+    if ((U & (U - 1u)) == 0) {
+      const uint32_t gp = U ? (v << m) + U : 0u;
+      Gp[bidx(U)] = gp;
+      put(U, 0u);
+      if (U) list[start[__ffs(U) - 1]] = make_uint2(U, gp);
+    } else if (v > wall) {
+      const int l = __ffs(U) - 1;
+      list[start[l] + atomicAdd(&cnt[l], 1)] = make_uint2(U, 0u);
+    }
+  }
+  const int total = start[m];
+  for (int p = 2; p <= most; ++p) {
+    __syncthreads();
+    for (int e = t; e < total; e += TPI) {
+      const uint32_t A = list[e].x;
+      if (__popc(A) != p) continue;
+      const uint32_t low = A & (~A + 1u), rest = A ^ low;
+      uint32_t key = 0xFFFFFFFFu;
+      for (uint32_t sub = 0; sub != rest; sub = (sub - rest) & rest) {
+        const uint32_t a = low | sub, b = A ^ a;
+        key = min(key, Gp[bidx(a)] + Gp[bidx(b)] - b);
+      }
+      const uint32_t gp = (((key >> m) - Gp[bidx(A)]) << m) + A;
+      Gp[bidx(A)] = gp;
+      list[e].y = gp;
+      put(A, key & mask);
+    }
+  }
+  for (int l = m - 2; l >= 0; --l) {
+    __syncthreads();
+    const int b0 = start[l], b1 = start[l + 1];
+    for (uint32_t h = t; h < (1u << (m - 1 - l)); h += TPI) {
+      const uint32_t S = (h << (l + 1)) | (1u << l);
+      uint32_t* own = &Gp[bidx(S)];
+      // only an unfinished set still has w* here: a finished one has F >= w*,
+      // and F > 0 when w* = 0 (a member shares weight)
+      if (h == 0 || *own != wall) continue;
+      const uint32_t warp_all = S | (31u << (l + 1));  // holds every S of the warp
+      const int pos = brow_pos(S >> 5);
+      uint32_t key = 0xFFFFFFFFu;
+      for (int e = b0; e < b1; ++e) {
+        const uint2 a = list[e];
+        if ((a.x & ~warp_all) != 0) continue;
+        if ((a.x & ~S) == 0) {
+          const uint32_t b = S ^ a.x;
+          key = min(key, a.y + Gp[(pos ^ brow_pos(a.x >> 5)) * kBRowStride + (int)(b & 31u)] - b);
+        }
+      }
+      *own = (((key >> m) - wall) << m) + S;
+      put(S, key & mask);
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
 template <int TPI, bool kGRows = false>
 __global__ void __launch_bounds__(TPI, TPI >= 256 ? 3 : (TPI == 128 ? 6 : 12))  // 12 warps or more per SM
 k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
@@ -613,6 +719,8 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
     __syncthreads();
   }
 
+  if (!batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
+                          [&](uint32_t U, uint32_t A) { put_split(U, A, &bflags); })) {
   // level 0: row 0, the recurrence on the five low requests
   if (t == 0) {
     uint32_t zp[kBRow], zc[kBRow];
@@ -749,6 +857,7 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
       }
     }
     __syncthreads();
+  }
   }
 
   // outputs: tables and OPT

@@ -127,3 +127,37 @@ def test_m24_equals_the_full_recurrence(mpt, seed):
     a = mpt.solve(inst.weights, inst.bits)
     b = mpt.solve(inst.weights, inst.bits, mode="blocked")
     assert all(torch.equal(x, y) for x, y in zip(mpt.mpt_tables(a.ctx), mpt.mpt_tables(b.ctx)))
+
+
+def _groups(seed):
+    """Groups of 6..16 requests: pooled passages (few members), one chunk in
+    every request, no shared chunk, identical requests, and nearly everything
+    shared (too many members for the list)."""
+    rng = np.random.default_rng(seed)
+    n = 400
+    out = []
+    for m in list(range(6, 17)) * 2:
+        pool = rng.choice(n - 20, size=40, replace=False)
+        base = [[int(x) for x in rng.choice(pool, size=6, replace=False)] for _ in range(m)]
+        out.append(base)
+        out.append([r + [n - 1] for r in base])
+        out.append([[(17 * i + j) % (n - 20) for j in range(3)] for i in range(m)])
+        out.append([[1, 2, 3]] * m)
+        out.append([[n - 20 + j for j in range(min(m, 12)) if j != i] for i in range(m)])
+        out.append([[int(x)] if x % 3 else [] for x in rng.integers(0, 9, size=m)])
+    return rng.integers(1, 30, size=n).astype(np.int64), out
+
+
+@pytest.mark.parametrize("scale", [1, 1 << 12])
+def test_batch_equals_single_solves(mpt, scale):
+    w, groups = _groups(3)
+    w = w * scale
+    if scale > 1:  # 16 requests need packed keys
+        groups = [g for g in groups if len(g) <= 14]
+    opt, perms, orders, b = mpt.solve_batch(w, groups)
+    F, split, offs = mpt.mpt_batch_tables(b)
+    for i, g in enumerate(groups):
+        one = mpt.solve(w, I.pack_requests(g, len(w)), mode="wide" if scale > 1 else "blocked")
+        tF, _, ts = mpt.mpt_tables(one.ctx)
+        assert opt[i] == one.opt and perms[i] == one.permutations() and orders[i] == one.dfs_order.tolist(), i
+        assert torch.equal(F[offs[i]:offs[i + 1]], tF) and torch.equal(split[offs[i]:offs[i + 1]], ts), i
