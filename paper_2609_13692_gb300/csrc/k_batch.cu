@@ -84,7 +84,7 @@ __device__ __forceinline__ int64_t batch_offset(uint32_t S, int64_t lo, const lo
 // as many slots as occurrences, so every insertion ends within `size` probes.
 template <int TPI>
 __device__ int batch_gather(int m, int64_t r0, int64_t o0, int occ, int occ_cap, const int64_t* __restrict__ req_off,
-                            const int64_t* __restrict__ chunks, int32_t* tkey, uint32_t* tmask, int32_t* cx,
+                            const int32_t* __restrict__ chunks, int32_t* tkey, uint32_t* tmask, int32_t* cx,
                             uint32_t* cN, int* roff, int* ndistinct_s, int32_t* bflags) {
   int& ndistinct = *ndistinct_s;
   const int t = threadIdx.x;
@@ -100,7 +100,7 @@ __device__ int batch_gather(int m, int64_t r0, int64_t o0, int occ, int occ_cap,
   for (int j = t; j < occ; j += TPI) {
     int i = 0;
     while (roff[i + 1] <= j) ++i;  // the request whose slot range holds j
-    const int32_t x = (int32_t)chunks[o0 + j];
+    const int32_t x = chunks[o0 + j];
     uint32_t h = lg > 0 ? ((uint32_t)x * 2654435761u) >> (32 - lg) : 0u;
     for (int probe = 0; probe < size; ++probe) {
       const int32_t old = atomicCAS(&tkey[h], -1, x);
@@ -133,7 +133,7 @@ __device__ int batch_gather(int m, int64_t r0, int64_t o0, int occ, int occ_cap,
 template <int TPI, typename SplitT>
 __device__ void batch_walk(int inst, int m, int64_t r0, int64_t o0, const int* roff, const SplitT* split,
                            unsigned long long* keys, const int32_t* cx, const uint32_t* cN, int nd,
-                           int64_t* __restrict__ perm_out, int32_t* __restrict__ dfs_out,
+                           int32_t* __restrict__ perm_out, int32_t* __restrict__ dfs_out,
                            int32_t* __restrict__ status) {
   __shared__ uint32_t anc[16][16];
   __shared__ int leaf_depth[16], fill[16], dfs_s[16];
@@ -202,7 +202,7 @@ __device__ void batch_walk(int inst, int m, int64_t r0, int64_t o0, const int* r
       const unsigned long long kj = keys[base + j];
       int rank = 0;
       for (int q = 0; q < len; ++q) rank += keys[base + q] < kj;
-      perm_out[o0 + base + rank] = (int64_t)(kj & 0xFFFFFFFFull);
+      perm_out[o0 + base + rank] = (int32_t)(kj & 0xFFFFFFFFull);
     }
   }
   if (t == 0) status[inst] = 0;
@@ -210,10 +210,10 @@ __device__ void batch_walk(int inst, int m, int64_t r0, int64_t o0, const int* r
 
 __global__ void __launch_bounds__(kBatchThreads)
 k_batch_solve(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
-              const int64_t* __restrict__ req_off, const int64_t* __restrict__ chunks,
+              const int64_t* __restrict__ req_off, const int32_t* __restrict__ chunks,
               const int64_t* __restrict__ tab_off, const int32_t* __restrict__ inst_list,
               const uint8_t* __restrict__ flags, int occ_cap, int max_m, int64_t* __restrict__ opt_out,
-              int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int64_t* __restrict__ perm_out,
+              int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
               int32_t* __restrict__ dfs_out, int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int inst = inst_list[blockIdx.x];
@@ -627,10 +627,10 @@ __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put
 template <int TPI, bool kGRows = false>
 __global__ void __launch_bounds__(TPI, TPI >= 256 ? 3 : (TPI == 128 ? 6 : 12))  // 12 warps or more per SM
 k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
-             const int64_t* __restrict__ req_off, const int64_t* __restrict__ chunks,
+             const int64_t* __restrict__ req_off, const int32_t* __restrict__ chunks,
              const int64_t* __restrict__ tab_off, const int32_t* __restrict__ inst_list,
              const uint8_t* __restrict__ flags, int occ_cap, int mm, int64_t* __restrict__ opt_out,
-             int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int64_t* __restrict__ perm_out,
+             int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
              int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int inst = inst_list[blockIdx.x];
@@ -900,9 +900,9 @@ size_t batch_smem_bytes(int max_m, int occ_cap) {
 
 // One grid over `count` instances of size m (ids inst_list[0..count)).
 cudaError_t launch_batch(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
-                         const int64_t* req_off, const int64_t* chunks, const int64_t* tab_off,
+                         const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
                          const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
-                         uint32_t* split, int64_t* perm, int32_t* dfs, int32_t* status, cudaStream_t stream) {
+                         uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status, cudaStream_t stream) {
   const size_t smem = batch_smem_bytes(m, occ_cap);
   cudaError_t e = cudaFuncSetAttribute(k_batch_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -927,9 +927,9 @@ size_t batch_rows_scratch_words(int m) {
 // One grid of the row-blocked kernel over `count` instances of size m >= 6
 // whose request weights allow packed keys.
 cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
-                              const int64_t* req_off, const int64_t* chunks, const int64_t* tab_off,
+                              const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
                               const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
-                              uint32_t* split, int64_t* perm, int32_t* dfs, int32_t* status, uint32_t* rows_scratch,
+                              uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status, uint32_t* rows_scratch,
                               cudaStream_t stream) {
   if (m < 6 || m > kBMaxRowsM || (m >= kBGlobalRowsM && !rows_scratch)) return cudaErrorInvalidValue;
   const size_t smem = batch_rows_smem_bytes(m, occ_cap);

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <thread>
@@ -17,13 +18,13 @@ size_t batch_smem_bytes(int max_m, int occ_cap);
 size_t batch_rows_smem_bytes(int m, int occ_cap);
 size_t batch_rows_scratch_words(int m);
 cudaError_t launch_batch(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
-                         const int64_t* req_off, const int64_t* chunks, const int64_t* tab_off,
+                         const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
                          const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
-                         uint32_t* split, int64_t* perm, int32_t* dfs, int32_t* status, cudaStream_t stream);
+                         uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status, cudaStream_t stream);
 cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
-                              const int64_t* req_off, const int64_t* chunks, const int64_t* tab_off,
+                              const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
                               const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
-                              uint32_t* split, int64_t* perm, int32_t* dfs, int32_t* status, uint32_t* rows_scratch,
+                              uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status, uint32_t* rows_scratch,
                               cudaStream_t stream);
 }  // namespace mpt
 
@@ -31,7 +32,9 @@ struct mpt_batch {
   int32_t batch = 0;
   int64_t n = 0, requests = 0, occurrences = 0, table_entries = 0;
   int max_m = 0, occ_cap = 1;
-  std::vector<int64_t> w, inst_req, req_off, chunks, tab_off;
+  std::vector<int64_t> w, inst_req, req_off, tab_off;
+  // chunk ids fit 32 bits (n < 2^31); not initialised, written by mpt_batch_create's threads
+  std::unique_ptr<int32_t[]> chunks;
   // instances grouped by size m: inst_list[group_start[m] .. group_start[m+1]),
   // those for the row-blocked kernel (m >= 6, packed keys) first, up to
   // group_rows_end[m]; each part with its own occurrence cap
@@ -44,7 +47,8 @@ struct mpt_batch {
   std::vector<uint8_t> flags;
   // results of the last solve
   bool solved = false;
-  std::vector<int64_t> opt, perm;
+  std::vector<int64_t> opt;
+  std::unique_ptr<int32_t[]> perm;
   std::vector<int32_t> dfs, status;
   const int64_t* d_F = nullptr;
   const uint32_t* d_split = nullptr;
@@ -127,7 +131,8 @@ struct ChunkSlot {
 };
 
 mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, int64_t r0, int64_t r1,
-                          const int64_t* req_offsets, const int64_t* chunk_ids, ChunkSlot* table, uint8_t* flags) {
+                          const int64_t* req_offsets, const int64_t* chunk_ids, ChunkSlot* table, int32_t* ids32,
+                          uint8_t* flags) {
   const int m = (int)(r1 - r0);
   const int64_t occ = req_offsets[r1] - req_offsets[r0];
   if (occ > kBatchMaxOcc) return MPT_ERR_TOO_LARGE;
@@ -140,6 +145,7 @@ mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, i
     for (int64_t j = req_offsets[r]; j < req_offsets[r + 1]; ++j) {
       const int64_t x = chunk_ids[j];
       if (x < 0 || x >= n_chunks) return MPT_ERR_INVALID_ARG;
+      ids32[j] = (int32_t)x;
       uint32_t h = ((uint32_t)x * 2654435761u) >> (32 - lg);
       while (table[h].inst == b && table[h].chunk != (int32_t)x) h = (h + 1u) & mask;
       ChunkSlot& e = table[h];
@@ -183,19 +189,18 @@ mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, i
   return MPT_OK;
 }
 
-// Every instance; *bad and *bad_at: the status and number of the first one
-// that fails.  Ranges of instances run on up to eight threads (one per 2^15
+// Every instance, and its chunk ids as 32-bit numbers; *bad: the status of
+// the first one that fails.  Ranges of instances run on up to eight threads (one per 2^15
 // occurrences); a thread that cannot be started has its range done here.
 void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, const int64_t* inst_requests,
-                     const int64_t* req_offsets, const int64_t* chunk_ids, uint8_t* flags, mpt_status* bad,
-                     int32_t* bad_at) {
+                     const int64_t* req_offsets, const int64_t* chunk_ids, int32_t* ids32, uint8_t* flags,
+                     mpt_status* bad) {
   const int64_t occ = req_offsets[inst_requests[batch]];
   const int64_t cores = std::max<int64_t>(1, (int64_t)std::thread::hardware_concurrency());
   const int64_t ranges = std::min<int64_t>({8, cores, 1 + (occ >> 15), batch});
   struct Range {
     std::vector<ChunkSlot> table;
     mpt_status status = MPT_OK;
-    int32_t at = 0;
   };
   std::vector<Range> out((size_t)ranges);
   for (Range& r : out) r.table.resize(2 * kBatchMaxOcc);  // here, so that a thread has nothing that throws
@@ -204,8 +209,7 @@ void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, co
     const int32_t end = (int32_t)(batch * (k + 1) / ranges);
     for (int32_t b = (int32_t)(batch * k / ranges); b < end && r.status == MPT_OK; ++b) {
       r.status = check_instance(weights, n_chunks, b, inst_requests[b], inst_requests[b + 1], req_offsets, chunk_ids,
-                                r.table.data(), flags + b);
-      r.at = b;
+                                r.table.data(), ids32, flags + b);
     }
   };
   std::vector<std::thread> threads;
@@ -222,13 +226,13 @@ void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, co
   for (const Range& r : out)
     if (r.status != MPT_OK) {
       *bad = r.status;
-      *bad_at = r.at;
       return;
     }
 }
 
 struct BatchCarve {
-  int64_t *weights, *inst_req, *req_off, *chunks, *tab_off, *opt, *F, *perm;
+  int64_t *weights, *inst_req, *req_off, *tab_off, *opt, *F;
+  int32_t *chunks, *perm;
   uint32_t *split, *rows_scratch;
   int32_t *dfs, *status, *inst_list;
   uint8_t* flags;
@@ -244,12 +248,12 @@ size_t carve(const mpt_batch* b, char* base, BatchCarve* c) {
   c->weights = reinterpret_cast<int64_t*>(take((size_t)b->n * 8));
   c->inst_req = reinterpret_cast<int64_t*>(take(((size_t)b->batch + 1) * 8));
   c->req_off = reinterpret_cast<int64_t*>(take(((size_t)b->requests + 1) * 8));
-  c->chunks = reinterpret_cast<int64_t*>(take((size_t)std::max<int64_t>(b->occurrences, 1) * 8));
+  c->chunks = reinterpret_cast<int32_t*>(take((size_t)std::max<int64_t>(b->occurrences, 1) * 4));
   c->tab_off = reinterpret_cast<int64_t*>(take(((size_t)b->batch + 1) * 8));
   c->opt = reinterpret_cast<int64_t*>(take((size_t)b->batch * 8));
   c->F = reinterpret_cast<int64_t*>(take((size_t)b->table_entries * 8));
   c->split = reinterpret_cast<uint32_t*>(take((size_t)b->table_entries * 4));
-  c->perm = reinterpret_cast<int64_t*>(take((size_t)std::max<int64_t>(b->occurrences, 1) * 8));
+  c->perm = reinterpret_cast<int32_t*>(take((size_t)std::max<int64_t>(b->occurrences, 1) * 4));
   c->dfs = reinterpret_cast<int32_t*>(take((size_t)b->requests * 4));
   c->status = reinterpret_cast<int32_t*>(take((size_t)b->batch * 4));
   c->inst_list = reinterpret_cast<int32_t*>(take((size_t)b->batch * 4));
@@ -296,8 +300,9 @@ mpt_status mpt_batch_create(const int64_t* weights, int64_t n_chunks, int32_t ba
     // the instances' own checks and weights, on several threads when there
     // are many occurrences; the first failing instance decides the status
     mpt_status bad = MPT_OK;
-    int32_t bad_at = batch;
-    check_instances(weights, n_chunks, batch, inst_requests, req_offsets, chunk_ids, c->flags.data(), &bad, &bad_at);
+    c->chunks.reset(new int32_t[(size_t)std::max<int64_t>(occ_total, 1)]);
+    check_instances(weights, n_chunks, batch, inst_requests, req_offsets, chunk_ids, c->chunks.get(),
+                    c->flags.data(), &bad);
     if (bad != MPT_OK) {
       delete c;
       return bad;
@@ -337,7 +342,6 @@ mpt_status mpt_batch_create(const int64_t* weights, int64_t n_chunks, int32_t ba
     c->w.assign(weights, weights + n_chunks);
     c->inst_req.assign(inst_requests, inst_requests + batch + 1);
     c->req_off.assign(req_offsets, req_offsets + R + 1);
-    if (occ_total) c->chunks.assign(chunk_ids, chunk_ids + occ_total);
   } catch (...) {
     delete c;
     return MPT_ERR_OUT_OF_MEMORY;
@@ -383,7 +387,7 @@ mpt_status mpt_batch_solve(mpt_batch* b, void* d_workspace, size_t workspace_byt
   try {
     b->opt.resize(B);
     b->status.resize(B);
-    b->perm.resize((size_t)b->occurrences);
+    if (!b->perm) b->perm.reset(new int32_t[(size_t)std::max<int64_t>(b->occurrences, 1)]);
     b->dfs.resize((size_t)b->requests);
   } catch (...) {
     return MPT_ERR_OUT_OF_MEMORY;
@@ -398,7 +402,7 @@ mpt_status mpt_batch_solve(mpt_batch* b, void* d_workspace, size_t workspace_byt
   h2d(c.weights, b->w.data(), (size_t)b->n * 8);
   h2d(c.inst_req, b->inst_req.data(), (B + 1) * 8);
   h2d(c.req_off, b->req_off.data(), ((size_t)b->requests + 1) * 8);
-  h2d(c.chunks, b->chunks.data(), (size_t)b->occurrences * 8);
+  h2d(c.chunks, b->chunks.get(), (size_t)b->occurrences * 4);
   h2d(c.tab_off, b->tab_off.data(), (B + 1) * 8);
   h2d(c.inst_list, b->inst_list.data(), B * 4);
   h2d(c.flags, b->flags.data(), B);
@@ -440,7 +444,7 @@ mpt_status mpt_batch_solve(mpt_batch* b, void* d_workspace, size_t workspace_byt
   }
   d2h(b->opt.data(), c.opt, B * 8);
   d2h(b->status.data(), c.status, B * 4);
-  d2h(b->perm.data(), c.perm, (size_t)b->occurrences * 8);
+  d2h(b->perm.get(), c.perm, (size_t)b->occurrences * 4);
   d2h(b->dfs.data(), c.dfs, (size_t)b->requests * 4);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? MPT_ERR_OUT_OF_MEMORY : MPT_ERR_CUDA;
@@ -456,7 +460,7 @@ mpt_status mpt_batch_results(const mpt_batch* b, int64_t* opt, int64_t* perm_chu
   if (!b) return MPT_ERR_INVALID_ARG;
   if (!b->solved) return MPT_ERR_NOT_SOLVED;
   if (opt) std::memcpy(opt, b->opt.data(), b->opt.size() * 8);
-  if (perm_chunks && !b->perm.empty()) std::memcpy(perm_chunks, b->perm.data(), b->perm.size() * 8);
+  if (perm_chunks) std::copy(b->perm.get(), b->perm.get() + b->occurrences, perm_chunks);
   if (dfs_order && !b->dfs.empty()) std::memcpy(dfs_order, b->dfs.data(), b->dfs.size() * 4);
   return MPT_OK;
 }
