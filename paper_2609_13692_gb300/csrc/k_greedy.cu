@@ -9,13 +9,26 @@
 // the merged cluster keeps slot a.  The layout walks the hierarchy as in the
 // Thm 1 proof.  Lower bound: sum_i w(R_i) - MaxSpanningTree(w(R_i cap R_j)).
 //
-// Kernels: k_pair_weights fills W[i][j] = w(R_i cap R_j) (sorted chunk lists,
-// merge-intersection); Borůvka rounds find the maximum spanning tree of W;
-// k_greedy_merge runs all m - 1 merges in one block, keeping for every active
-// slot an upper bound on its best partner as a 64-bit key (weight, then the
-// smallest slot pair) and rescanning a row only when its key is found stale; k_greedy_layout climbs each
-// (request, chunk) occurrence to the highest node whose signature still holds
-// the chunk, and ranks each request's chunks by (depth, chunk id).
+// Merging in rounds.  Order the slot pairs by (weight, then the smaller pair):
+// keys are distinct, and a merge never raises a key (the merged signature is
+// part of both, and keeps the smaller slot).  So when a and b are each other's
+// best pair, theirs stays the best of both until they merge, and the greedy
+// sequence merges exactly that pair at exactly that key; all such pairs can
+// merge in the same round.  A merge's key is above every key it leaves behind,
+// so the greedy sequence is the merges of all rounds in decreasing key order.
+// Once no pair shares weight, the rest is forced: the smallest slot takes in
+// the others in increasing order, with empty signatures.  3,000 requests need
+// 19 rounds.  The merges one after the other in one block took 25.7 of the
+// 27.6 ms of a call (8.6 us each: some twenty block barriers); the rounds
+// take 0.9 ms, bound by their launches and the latency of the row scans.
+//
+// Kernels: k_pair_weights fills W[i][j] = w(R_i cap R_j); Borůvka rounds find
+// the maximum spanning tree of W; k_row_best, k_match and k_reweigh are one
+// round of merges; k_rank orders them; k_tail appends the forced ones;
+// k_count and k_leaf_order give the left-to-right leaf order; k_greedy_emit
+// climbs each (request, chunk) occurrence to the highest node whose signature
+// still holds the chunk, and k_greedy_rank orders each request's chunks by
+// (that node, chunk id).
 #include "../../include/mpt.h"
 #include "mpt_internal.cuh"
 
@@ -28,25 +41,7 @@ namespace {
 constexpr int kSigMax = 128;       // longest request accepted
 constexpr int kMaxGreedyM = 16384;  // slot ids fit in 14 bits
 constexpr int kGreedyThreads = 1024;
-
-__device__ __forceinline__ uint32_t sig_weight(const int32_t* a, int la, const int32_t* b, int lb,
-                                               const int64_t* __restrict__ w) {
-  uint32_t s = 0;
-  int i = 0, j = 0;
-  while (i < la && j < lb) {
-    const int32_t x = a[i], y = b[j];
-    if (x == y) {
-      s += (uint32_t)w[x];
-      ++i;
-      ++j;
-    } else if (x < y) {
-      ++i;
-    } else {
-      ++j;
-    }
-  }
-  return s;
-}
+constexpr int kAhead = 8;  // loads of a row of W that a thread keeps in flight (rows are mostly zeros)
 
 // key of pair {d, e} with common weight v: larger is better (weight, then the
 // smaller slot pair)
@@ -60,341 +55,445 @@ __device__ __forceinline__ void key_pair(unsigned long long k, uint32_t* a, uint
   *b = p & ((1u << 14) - 1u);
 }
 
-__global__ void k_pair_weights(int m, const int32_t* __restrict__ sig, const int32_t* __restrict__ len,
-                               const int64_t* __restrict__ w, uint32_t* __restrict__ W) {
-  const int i = blockIdx.y;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-    if (j < i) continue;
-    const uint32_t v = (j == i) ? 0u : sig_weight(sig + (size_t)i * kSigMax, len[i], sig + (size_t)j * kSigMax, len[j], w);
-    W[(size_t)i * m + j] = v;
-    W[(size_t)j * m + i] = v;
+// Position of x in the sorted signature s[0 .. n), or -1.
+__device__ __forceinline__ int find_in(const int32_t* s, int n, int32_t x) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (s[mid] < x) lo = mid + 1; else hi = mid;
   }
+  return lo < n && s[lo] == x ? lo : -1;
 }
 
-// best partner of every slot: warp per row
-__global__ void k_row_best(int m, const uint32_t* __restrict__ W, unsigned long long* __restrict__ best) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < m; d += warps) {
-    unsigned long long b = 0;
-    for (int e = lane; e < m; e += 32)
-      if (e != d) b = max(b, pair_key((uint32_t)d, (uint32_t)e, W[(size_t)d * m + e]));
-    for (int off = 16; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
-    if (lane == 0) best[d] = b;
-  }
-}
+// W of 32 rows by 256 columns per block: the rows' chunks set their row's bit
+// in a table by the chunk's low bits; a column's chunks look their rows up
+// there (checked by binary search, as chunks share table entries) and add
+// their weight to the block's tile.  Both orders of a pair are computed, so
+// that W is only written along rows: 178 -> 37 us at m = 3,000 against one
+// thread merging the two signatures of a pair and writing it twice, once down a
+// column.
+constexpr int kPwRows = 32, kPwCols = 256, kPwTable = 4096;
+constexpr int kPwSmem = (kPwTable + kPwRows * kSigMax + kPwRows * kPwCols) * 4;
 
-__device__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* red) {
-  for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) red[warp] = v;
+__global__ void __launch_bounds__(kPwCols)
+k_pair_weights(int m, const int64_t* __restrict__ off, const int32_t* __restrict__ sig, const int64_t* __restrict__ w,
+               uint32_t* __restrict__ W) {
+  extern __shared__ __align__(16) uint32_t pw[];
+  uint32_t* table = pw;
+  int32_t* rsig = reinterpret_cast<int32_t*>(table + kPwTable);
+  uint32_t* tile = table + kPwTable + kPwRows * kSigMax;
+  __shared__ int rlen[kPwRows];
+  const int t = threadIdx.x, i0 = blockIdx.y * kPwRows, j = blockIdx.x * kPwCols + t;
+  for (int q = t; q < kPwTable; q += kPwCols) table[q] = 0;
+  for (int q = t; q < kPwRows * kPwCols; q += kPwCols) tile[q] = 0;
+  if (t < kPwRows) rlen[t] = i0 + t < m ? (int)(off[i0 + t + 1] - off[i0 + t]) : 0;
   __syncthreads();
-  if (warp == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? red[lane] : 0ull;
-    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
-    if (lane == 0) red[32] = v;
+  for (int q = t; q < kPwRows * kSigMax; q += kPwCols) {
+    const int r = q / kSigMax, k = q % kSigMax;
+    if (k < rlen[r]) {
+      const int32_t x = sig[off[i0 + r] + k];
+      rsig[q] = x;
+      atomicOr(&table[x & (kPwTable - 1)], 1u << r);
+    }
   }
   __syncthreads();
-  const unsigned long long r = red[32];
-  __syncthreads();
-  return r;
+  if (j < m) {
+    for (int64_t q = off[j]; q < off[j + 1]; ++q) {
+      const int32_t x = sig[q];
+      for (uint32_t rr = table[x & (kPwTable - 1)]; rr; rr &= rr - 1) {
+        const int r = __ffs(rr) - 1;
+        if (i0 + r != j && find_in(rsig + r * kSigMax, rlen[r], x) >= 0) tile[r * kPwCols + t] += (uint32_t)w[x];
+      }
+    }
+    for (int r = 0; r < kPwRows && i0 + r < m; ++r) W[(size_t)(i0 + r) * m + j] = tile[r * kPwCols + t];
+  }
 }
 
 // Maximum spanning tree of W (Borůvka).  Edges are ordered by pair_key
 // (weight, then the smaller slot pair), so every edge key is distinct and the
 // tree is unique; its weight is the maximum spanning-tree weight (Sec. 6.3).
+// Edges of no weight add nothing and are left out, so the rounds end at a
+// spanning forest of the others.
 // A round: each vertex's heaviest edge to another component (warp per row),
 // each component's heaviest (atomicMax), components hook along them (a pair
 // of components that chose the same edge keeps the smaller id as root, and
 // that edge is counted once), then every vertex jumps to its root.  Every
 // round at least halves the number of components.
 __global__ void k_bv_vertex_best(int m, const uint32_t* __restrict__ W, const int32_t* __restrict__ comp,
-                                 unsigned long long* __restrict__ cbest) {
+                                 unsigned long long* __restrict__ cbest, const int32_t* __restrict__ state) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
+  if (*state < 0) return;  // no component found an edge last round
   for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < m; v += warps) {
     const int cv = comp[v];
     unsigned long long b = 0;
-    for (int u = lane; u < m; u += 32)
-      if (comp[u] != cv) b = max(b, pair_key((uint32_t)v, (uint32_t)u, W[(size_t)v * m + u]));
+    for (int u0 = lane; u0 < m; u0 += 32 * kAhead) {
+      uint32_t x[kAhead];
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) x[q] = u0 + 32 * q < m ? W[(size_t)v * m + u0 + 32 * q] : 0u;
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const int u = u0 + 32 * q;
+        if (x[q] != 0 && comp[u] != cv) b = max(b, pair_key((uint32_t)v, (uint32_t)u, x[q]));
+      }
+    }
     for (int off = 16; off > 0; off >>= 1) b = max(b, __shfl_xor_sync(0xFFFFFFFFu, b, off));
     if (lane == 0 && b) atomicMax(&cbest[cv], b);
   }
 }
 
-__global__ void k_bv_hook(int m, const int32_t* __restrict__ comp, const unsigned long long* __restrict__ cbest,
-                          int32_t* __restrict__ parent, unsigned long long* __restrict__ total) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
+// The rest of a round, one block: components hook, vertices jump to their
+// roots, the bests are reset.  *state: -1 when nothing hooked, and from then on.
+__global__ void __launch_bounds__(kGreedyThreads)
+k_bv_step(int m, int32_t* __restrict__ comp, unsigned long long* __restrict__ cbest, int32_t* __restrict__ parent,
+          unsigned long long* __restrict__ total, int32_t* __restrict__ state) {
+  if (*state < 0) return;
+  unsigned long long sum = 0;
+  bool any = false;
+  for (int c = threadIdx.x; c < m; c += kGreedyThreads) {
     if (comp[c] != c) continue;  // not a component root
     const unsigned long long k = cbest[c];
     if (k == 0) {
       parent[c] = c;
       continue;
     }
+    any = true;
     uint32_t a, b;
     key_pair(k, &a, &b);
     const int o = comp[a] == c ? comp[b] : comp[a];
     const bool mutual = cbest[o] == k;
     parent[c] = (mutual && c < o) ? c : o;
-    if (!(mutual && o < c)) atomicAdd(total, k >> 28);
+    if (!(mutual && o < c)) sum += k >> 28;
   }
-}
-
-__global__ void k_bv_jump(int m, int32_t* __restrict__ comp, const int32_t* __restrict__ parent) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < m; v += gridDim.x * blockDim.x) {
+  any = __syncthreads_or(any);
+  for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(total, sum);
+  if (!any) {
+    if (threadIdx.x == 0) *state = -1;
+    return;
+  }
+  for (int v = threadIdx.x; v < m; v += kGreedyThreads) {
     int r = comp[v];
     for (int step = 0; step < m && parent[r] != r; ++step) r = parent[r];
     comp[v] = r;
+    cbest[v] = 0;
   }
 }
 
-__global__ void k_bv_reset(int m, unsigned long long* __restrict__ cbest) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < m; v += gridDim.x * blockDim.x) cbest[v] = 0;
+// ---------------------------------------------------------------------------
+// Rounds of merges.
+// ---------------------------------------------------------------------------
+struct Slots {
+  int m;
+  const int64_t* off;         // signatures of the slots, in place of the requests' sorted chunks
+  int32_t* sig;
+  int32_t* len;
+  uint32_t* W;
+  unsigned long long* best;   // best pair key of an active slot; 0: it shares weight with none
+  uint8_t* act;
+  int32_t* mark;              // last round that merged the slot
+  int32_t* top;               // the slot's node: a merge's record, or ~request
+  // records, in the order they were made
+  unsigned long long* rec_key;
+  int2* rec_child;            // nodes of both slots before
+  int32_t* rec_sig;           // [kSigMax] merged signature
+  int32_t* rec_len;
+  int32_t* counts;            // 0: records; 1, 2: records before this round, by its parity
+};
+
+__global__ void k_slots_init(Slots s, int32_t* __restrict__ comp, unsigned long long* __restrict__ cbest) {
+  for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < s.m; d += gridDim.x * blockDim.x) {
+    s.len[d] = (int32_t)(s.off[d + 1] - s.off[d]);
+    s.best[d] = 0;
+    s.act[d] = 1;
+    s.mark[d] = -1;
+    s.top[d] = ~d;
+    comp[d] = d;
+    cbest[d] = 0;
+  }
 }
 
-__global__ void k_iota32(int m, int32_t* __restrict__ a) {
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < m; v += gridDim.x * blockDim.x) a[v] = v;
-}
-
-
-// All m - 1 merges (one block).  best[d] is an upper bound on row d's best
-// pair key: pair weights only decrease as clusters merge, so a key stays an
-// upper bound until its row is rescanned.  The largest bound is merged only
-// if it is still exact (both slots active, weight unchanged); otherwise its
-// rows are rescanned and the choice is repeated.  Every rescan makes a row
-// exact, so a step repeats at most m times (kept as a hard cap).
-// Weight of sig_d (sorted, in global memory) within the merged signature
-// s_new (sorted, shared memory): binary search of each chunk of sig_d.
-__device__ __forceinline__ uint32_t sig_weight_in(const int32_t* __restrict__ sd, int ld, const int32_t* s_new,
-                                                  int ln, const int64_t* __restrict__ w) {
-  uint32_t s = 0;
-  for (int q = 0; q < ld; ++q) {
-    const int32_t x = sd[q];
-    int lo = 0, hi = ln;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (s_new[mid] < x) lo = mid + 1; else hi = mid;
+// Round 1 of 3: the best pair of every slot that needs looking for (all in the
+// first round; then those that merged, or whose best partner did: other
+// keys only fell).  Block per slot: a slot's scan is a chain of loads, and few
+// slots have one, so the threads of a block share it.
+constexpr int kBestThreads = 128;
+__global__ void __launch_bounds__(kBestThreads) k_row_best(Slots s, int round) {
+  __shared__ unsigned long long warp_best[kBestThreads / 32];
+  const int before = s.counts[1 + ((round + 1) & 1)], now = s.counts[0];
+  if (blockIdx.x == 0 && threadIdx.x == 0) s.counts[1 + (round & 1)] = now;
+  if (round > 0 && now == before) return;  // no merge last round: done
+  for (int d = blockIdx.x; d < s.m; d += gridDim.x) {
+    if (!s.act[d]) continue;  // the same decisions in every thread
+    if (round > 0 && s.mark[d] != round - 1) {
+      const unsigned long long k = s.best[d];
+      if (k == 0) continue;
+      uint32_t a, b;
+      key_pair(k, &a, &b);
+      if (s.mark[(int)a == d ? b : a] != round - 1) continue;
     }
-    if (lo < ln && s_new[lo] == x) s += (uint32_t)w[x];
-  }
-  return s;
-}
-
-
-// All m - 1 merges in one block, with lazy best keys: sb[d] (shared memory)
-// is an upper bound on slot d's best pair key (weights only decrease as
-// signatures shrink), 0 once d is merged away, and gmax[g] is the largest of
-// sb[32 g .. 32 g + 31].  The largest key is merged only if it is still
-// exact; otherwise the rows of its two slots are rescanned and the search
-// repeats.
-constexpr int kMaxGroups = kMaxGreedyM / 32;
-
-__device__ __forceinline__ void refresh_group(int m, int g, const unsigned long long* sb, unsigned long long* gmax) {
-  if (threadIdx.x < 32) {
-    const int d = g * 32 + (int)threadIdx.x;
-    unsigned long long v = d < m ? sb[d] : 0ull;
-    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
-    if (threadIdx.x == 0) gmax[g] = v;
-  }
-}
-
-__device__ unsigned long long smem_row_best(int m, int d, const uint32_t* __restrict__ W, const uint8_t* act,
-                                            unsigned long long* red) {
-  unsigned long long bb = 0;
-  const uint32_t* row = W + (size_t)d * m;
-  for (int e = threadIdx.x; e < m; e += blockDim.x)
-    if (e != d && act[e]) bb = max(bb, pair_key((uint32_t)d, (uint32_t)e, row[e]));
-  return block_max_u64(bb, red);
-}
-
-__global__ void __launch_bounds__(kGreedyThreads)
-k_greedy_merge(int m, const int64_t* __restrict__ w, int32_t* __restrict__ sig, int32_t* __restrict__ len,
-               uint32_t* __restrict__ W, const unsigned long long* __restrict__ best0, int32_t* __restrict__ node,
-               int32_t* __restrict__ merges, int64_t* __restrict__ values, int32_t* __restrict__ children,
-               int32_t* __restrict__ node_sig, int32_t* __restrict__ node_len, int32_t* __restrict__ error) {
-  extern __shared__ __align__(16) unsigned char gsm[];
-  unsigned long long* sb = reinterpret_cast<unsigned long long*>(gsm);        // [m]
-  unsigned long long* gmax = sb + m;                                          // [ceil(m / 32)]
-  uint8_t* act = reinterpret_cast<uint8_t*>(gmax + kMaxGroups);               // [m]
-  __shared__ unsigned long long red[33];
-  __shared__ int32_t s_a[kSigMax], s_b[kSigMax], s_new[kSigMax];
-  __shared__ int s_len;
-  __shared__ int warp_cnt[kGreedyThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int groups = (m + 31) / 32;
-  for (int d = threadIdx.x; d < m; d += blockDim.x) {
-    act[d] = 1;
-    node[d] = d;
-    sb[d] = best0[d];
-  }
-  __syncthreads();
-  for (int g = warp; g < groups; g += kGreedyThreads / 32) {
-    const int d = g * 32 + lane;
-    unsigned long long v = d < m ? sb[d] : 0ull;
-    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
-    if (lane == 0) gmax[g] = v;
-  }
-  __syncthreads();
-  for (int t = 0; t < m - 1; ++t) {
-    uint32_t a = 0, b = 0, v = 0;
-    int tries = 0;
-    for (;;) {
-      const unsigned long long c = (int)threadIdx.x < groups ? gmax[threadIdx.x] : 0ull;
-      const unsigned long long top = block_max_u64(c, red);
-      key_pair(top, &a, &b);
-      v = (uint32_t)(top >> 28);
-      if (top != 0 && act[a] && act[b] && W[(size_t)a * m + b] == v) break;
-      if (top == 0 || ++tries > m + 1) {
-        if (threadIdx.x == 0) atomicOr(error, 1);
-        return;
+    unsigned long long best = 0;
+    const uint32_t* row = s.W + (size_t)d * s.m;
+    for (int e0 = threadIdx.x; e0 < s.m; e0 += kBestThreads * kAhead) {
+      uint32_t v[kAhead];
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) v[q] = e0 + kBestThreads * q < s.m ? row[e0 + kBestThreads * q] : 0u;
+#pragma unroll
+      for (int q = 0; q < kAhead; ++q) {
+        const int e = e0 + kBestThreads * q;
+        if (v[q] != 0 && s.act[e]) best = max(best, pair_key((uint32_t)d, (uint32_t)e, v[q]));
       }
-      if (act[a]) {
-        const unsigned long long r = smem_row_best(m, (int)a, W, act, red);
-        if (threadIdx.x == 0) sb[a] = r;
-        __syncthreads();
-        refresh_group(m, (int)a >> 5, sb, gmax);
-      }
-      if (act[b]) {
-        const unsigned long long r = smem_row_best(m, (int)b, W, act, red);
-        if (threadIdx.x == 0) sb[b] = r;
-        __syncthreads();
-        refresh_group(m, (int)b >> 5, sb, gmax);
-      }
-      __syncthreads();
     }
+    for (int off = 16; off > 0; off >>= 1) best = max(best, __shfl_xor_sync(0xFFFFFFFFu, best, off));
+    if ((threadIdx.x & 31) == 0) warp_best[threadIdx.x >> 5] = best;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int q = 1; q < kBestThreads / 32; ++q) best = max(best, warp_best[q]);
+      s.best[d] = best;
+    }
+    __syncthreads();
+  }
+}
+
+// 2 of 3: slots that are each other's best merge; warp per smaller slot.
+// Only the pair's own warp touches its slots.
+__global__ void __launch_bounds__(256) k_match(Slots s, int round) {
+  const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+  for (int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < s.m; a += warps) {
+    const unsigned long long k = s.best[a];
+    if (k == 0 || !s.act[a]) continue;
+    uint32_t ka, kb;
+    key_pair(k, &ka, &kb);
+    const int b = (int)kb;
+    if ((int)ka != a || s.best[b] != k || !s.act[b]) continue;
+    int r = 0;
+    if (lane == 0) r = atomicAdd(&s.counts[0], 1);
+    r = __shfl_sync(0xFFFFFFFFu, r, 0);
     // merged signature: the chunks of a that b holds, in order
-    const int la = len[a], lb = len[b];
-    for (int q = threadIdx.x; q < la; q += blockDim.x) s_a[q] = sig[(size_t)a * kSigMax + q];
-    for (int q = threadIdx.x; q < lb; q += blockDim.x) s_b[q] = sig[(size_t)b * kSigMax + q];
-    __syncthreads();
-    bool keep = false;
-    int32_t x = 0;
-    if ((int)threadIdx.x < la) {
-      x = s_a[threadIdx.x];
-      int lo = 0, hi = lb;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s_b[mid] < x) lo = mid + 1; else hi = mid;
+    const int la = s.len[a], lb = s.len[b];
+    int32_t* sa = s.sig + s.off[a];
+    const int32_t* sb = s.sig + s.off[b];
+    int n = 0;
+    for (int base = 0; base < la; base += 32) {
+      const int q = base + lane;
+      const int32_t x = q < la ? sa[q] : 0;
+      const bool keep = q < la && find_in(sb, lb, x) >= 0;
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+      const int o = n + __popc(bal & ((1u << lane) - 1u));
+      if (keep) {
+        sa[o] = x;  // o <= q, and this round of the loop has read up to base + 31
+        s.rec_sig[(size_t)r * kSigMax + o] = x;
       }
-      keep = lo < lb && s_b[lo] == x;
+      n += __popc(bal);
+      __syncwarp();
     }
-    const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
-    if (lane == 0) warp_cnt[warp] = __popc(bal);
-    __syncthreads();
-    if (keep) {
-      int before = __popc(bal & ((1u << lane) - 1u));
-      for (int q = 0; q < warp; ++q) before += warp_cnt[q];  // kSigMax <= 128: at most four warps
-      s_new[before] = x;
+    if (lane == 0) {
+      s.len[a] = n;
+      s.rec_len[r] = n;
+      s.rec_key[r] = k;
+      s.rec_child[r] = make_int2(s.top[a], s.top[b]);
+      s.top[a] = r;
+      s.act[b] = 0;
+      s.mark[a] = round;
+      s.mark[b] = round;
     }
-    if (threadIdx.x == 0) {
-      int n = 0;
-      for (int q = 0; q < (kSigMax + 31) / 32; ++q) n += warp_cnt[q];
-      s_len = n;
-      merges[2 * t] = (int32_t)a;
-      merges[2 * t + 1] = (int32_t)b;
-      values[t] = v;
-      children[2 * t] = node[a];
-      children[2 * t + 1] = node[b];
-    }
-    __syncthreads();
-    const int ln = s_len;
-    for (int q = threadIdx.x; q < ln; q += blockDim.x) {
-      sig[(size_t)a * kSigMax + q] = s_new[q];
-      node_sig[(size_t)t * kSigMax + q] = s_new[q];
-    }
-    // new pair weights of the merged slot: zero wherever either old weight was
-    // zero (the merged signature is a subset of both)
-    for (int d = threadIdx.x; d < m; d += blockDim.x) {
-      if (!act[d] || d == (int)a || d == (int)b) continue;
-      const uint32_t wa = W[(size_t)a * m + d], wb = W[(size_t)b * m + d];
-      const uint32_t wv = (wa == 0 || wb == 0 || ln == 0)
-                              ? 0u
-                              : sig_weight_in(sig + (size_t)d * kSigMax, len[d], s_new, ln, w);
-      W[(size_t)a * m + d] = wv;
-      W[(size_t)d * m + a] = wv;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      len[a] = ln;
-      node_len[t] = ln;
-      node[a] = m + t;
-      act[b] = 0;
-      sb[b] = 0;
-    }
-    __syncthreads();
-    const unsigned long long r = smem_row_best(m, (int)a, W, act, red);
-    if (threadIdx.x == 0) sb[a] = r;
-    __syncthreads();
-    refresh_group(m, (int)a >> 5, sb, gmax);
-    __syncthreads();
-    refresh_group(m, (int)b >> 5, sb, gmax);
-    __syncthreads();
   }
 }
 
-size_t merge_smem_bytes(int m) { return (size_t)m * 8 + (size_t)kMaxGroups * 8 + (size_t)m + 16; }
-
-// Parent and depth of every tree node and the left-to-right leaf order (one thread).
-__global__ void k_greedy_tree(int m, const int32_t* __restrict__ children, int32_t* __restrict__ parent,
-                              int32_t* __restrict__ depth, int32_t* __restrict__ stack, int32_t* __restrict__ dfs) {
-  const int root = m == 1 ? 0 : 2 * m - 2;
-  parent[root] = -1;
-  depth[root] = 0;
-  for (int t = m - 2; t >= 0; --t) {
-    const int v = m + t;
-    for (int c = 0; c < 2; ++c) {
-      const int ch = children[2 * t + c];
-      parent[ch] = v;
-      depth[ch] = depth[v] + 1;
+// 3 of 3: the weights of the merged slots, block per merge of this round.
+// A weight is zero where either slot's was (the merged signature is part of
+// both); the others come from the signatures.  Two merged slots compute their
+// pair's weight twice, and the zero tests hold for old and new weights, so
+// the order of the blocks does not matter.
+__global__ void __launch_bounds__(256) k_reweigh(Slots s, const int64_t* __restrict__ w, int round) {
+  __shared__ int32_t s_new[kSigMax];
+  const int first = s.counts[1 + (round & 1)], end = s.counts[0];
+  for (int r = first + (int)blockIdx.x; r < end; r += gridDim.x) {
+    uint32_t a, b;
+    key_pair(s.rec_key[r], &a, &b);
+    const int ln = s.rec_len[r];
+    __syncthreads();
+    for (int q = threadIdx.x; q < ln; q += blockDim.x) s_new[q] = s.rec_sig[(size_t)r * kSigMax + q];
+    __syncthreads();
+    for (int d0 = threadIdx.x; d0 < s.m; d0 += 256 * kAhead) {
+      uint32_t wa[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) wa[k] = d0 + 256 * k < s.m ? s.W[(size_t)a * s.m + d0 + 256 * k] : 0u;
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int d = d0 + 256 * k;
+        if (wa[k] == 0 || d == (int)b || !s.act[d]) continue;
+        uint32_t v = 0;
+        if (s.W[(size_t)b * s.m + d] != 0) {
+          const int32_t* sd = s.sig + s.off[d];
+          for (int q = 0; q < s.len[d]; ++q)
+            if (find_in(s_new, ln, sd[q]) >= 0) v += (uint32_t)w[sd[q]];
+        }
+        s.W[(size_t)a * s.m + d] = v;
+        s.W[(size_t)d * s.m + a] = v;
+      }
     }
-  }
-  int sp = 0, nl = 0;
-  stack[sp++] = root;
-  while (sp > 0) {
-    const int v = stack[--sp];
-    if (v < m) {
-      dfs[nl++] = v;
-      continue;
-    }
-    const int t = v - m;
-    stack[sp++] = children[2 * t + 1];  // right after left
-    stack[sp++] = children[2 * t];
   }
 }
 
-// Emission depth of every (request, chunk) occurrence: climb from the leaf
-// while the parent's signature still holds the chunk.
-__global__ void k_greedy_emit(int m, const int32_t* __restrict__ node_sig, const int32_t* __restrict__ node_len,
-                              const int64_t* __restrict__ req_off, const int64_t* __restrict__ chunks,
-                              const int32_t* __restrict__ parent, const int32_t* __restrict__ depth,
+// ---------------------------------------------------------------------------
+// The sequence and the tree.  Node of merge t: m + t.
+// ---------------------------------------------------------------------------
+struct Tree {
+  int32_t* merges;    // [2 (m - 1)] slot pairs
+  int64_t* values;    // [m - 1]
+  int32_t* rank;      // position of each record in the sequence
+  int32_t* rec_of;    // record of merge t, -1 for a forced one
+  int32_t* children;  // [2 (m - 1)] nodes
+  int32_t* parent;    // [2 m - 1]
+  int32_t* leaves;    // [m - 1] leaves below a recorded merge
+  int32_t* base;      // [m] leaves in front of a remaining slot's subtree
+  int32_t* dfs;       // [m]
+};
+
+// Records in decreasing key order; warp per record.
+__global__ void __launch_bounds__(256) k_rank(Slots s, Tree tr) {
+  const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5, n = s.counts[0];
+  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
+    const unsigned long long k = s.rec_key[r];
+    int above = 0;
+    for (int q = lane; q < n; q += 32) above += s.rec_key[q] > k;
+    above = __reduce_add_sync(0xFFFFFFFFu, above);
+    if (lane == 0) {
+      uint32_t a, b;
+      key_pair(k, &a, &b);
+      tr.rank[r] = above;
+      tr.rec_of[above] = r;
+      tr.merges[2 * above] = (int32_t)a;
+      tr.merges[2 * above + 1] = (int32_t)b;
+      tr.values[above] = (int64_t)(k >> 28);
+      tr.leaves[above] = 0;
+    }
+  }
+}
+
+__device__ __forceinline__ int node_of(const Slots& s, const Tree& tr, int top) {
+  return top < 0 ? ~top : s.m + tr.rank[top];
+}
+
+// Children and parents of the recorded merges.
+__global__ void k_link(Slots s, Tree tr) {
+  const int n = s.counts[0];
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    const int t = tr.rank[r];
+    const int2 c = s.rec_child[r];
+    const int x = node_of(s, tr, c.x), y = node_of(s, tr, c.y);
+    tr.children[2 * t] = x;
+    tr.children[2 * t + 1] = y;
+    tr.parent[x] = s.m + t;
+    tr.parent[y] = s.m + t;
+  }
+}
+
+// Leaves below every recorded merge.
+__global__ void k_count(Slots s, Tree tr) {
+  const int top = s.m + s.counts[0];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.m; i += gridDim.x * blockDim.x) {
+    // a node whose slot is still active has no parent yet (k_tail's come later)
+    for (int v = tr.parent[i]; v >= 0 && v < top; v = tr.parent[v]) atomicAdd(&tr.leaves[v - s.m], 1);
+  }
+}
+
+// The forced merges, one block: the remaining slots s_0 < s_1 < .. in order,
+// merge j joins s_0's cluster with s_j; and the leaves in front of each.
+__global__ void __launch_bounds__(kGreedyThreads) k_tail(Slots s, Tree tr) {
+  __shared__ int warp_n[kGreedyThreads / 32], warp_l[kGreedyThreads / 32], s_first;
+  const int n = s.counts[0], t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int found = 0, leaves = 0;
+  for (int d0 = 0; d0 < s.m; d0 += kGreedyThreads) {
+    const int d = d0 + t;
+    const bool here = d < s.m && s.act[d];
+    const int node = here ? node_of(s, tr, s.top[d]) : 0;
+    const int mine = here ? (node < s.m ? 1 : tr.leaves[node - s.m]) : 0;
+    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, here);
+    int in = mine;
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xFFFFFFFFu, in, off);
+      if (lane >= off) in += o;
+    }
+    if (lane == 31) {
+      warp_n[warp] = __popc(bal);
+      warp_l[warp] = in;
+    }
+    __syncthreads();
+    int at = found + __popc(bal & ((1u << lane) - 1u)), before = leaves + in - mine;
+    for (int q = 0; q < kGreedyThreads / 32; ++q) {
+      if (q < warp) {
+        at += warp_n[q];
+        before += warp_l[q];
+      }
+      found += warp_n[q];
+      leaves += warp_l[q];
+    }
+    if (here) {
+      tr.base[d] = before;
+      if (at == 0) s_first = d;
+    }
+    __syncthreads();
+    if (here && at > 0) {
+      const int j = n + at - 1;  // merge number
+      const int left = at == 1 ? node_of(s, tr, s.top[s_first]) : s.m + j - 1;
+      tr.merges[2 * j] = s_first;
+      tr.merges[2 * j + 1] = d;
+      tr.values[j] = 0;
+      tr.rec_of[j] = -1;
+      tr.children[2 * j] = left;
+      tr.children[2 * j + 1] = node;
+      tr.parent[node] = s.m + j;
+      tr.parent[left] = s.m + j;
+    }
+  }
+}
+
+// Left-to-right leaf order: leaves in front of leaf i inside the subtree of its
+// remaining slot, plus that slot's base.
+__global__ void k_leaf_order(Slots s, Tree tr) {
+  const int top = s.m + s.counts[0];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.m; i += gridDim.x * blockDim.x) {
+    int v = i, pos = 0, slot = i;
+    for (int p = tr.parent[v]; p >= 0 && p < top; p = tr.parent[v]) {
+      const int left = tr.children[2 * (p - s.m)];
+      if (left != v) pos += left < s.m ? 1 : tr.leaves[left - s.m];
+      slot = tr.merges[2 * (p - s.m)];
+      v = p;
+    }
+    tr.dfs[tr.base[slot] + pos] = i;
+  }
+}
+
+// Emission key of every (request, chunk) occurrence: climb from the leaf
+// while the parent's signature still holds the chunk.  On a path the later
+// merges are nearer the root, so merges in decreasing number, then the leaf,
+// are its nodes from the root down.
+__global__ void k_greedy_emit(Slots s, Tree tr, const int32_t* __restrict__ chunks,
                               unsigned long long* __restrict__ keys) {
-  const int64_t occ = req_off[m];
+  const int64_t occ = s.off[s.m];
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < occ; j += (int64_t)gridDim.x * blockDim.x) {
-    int lo = 0, hi = m - 1;  // request of occurrence j: the last i with req_off[i] <= j
+    int lo = 0, hi = s.m - 1;  // request of occurrence j: the last i with off[i] <= j
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (req_off[mid] <= j) lo = mid; else hi = mid - 1;
+      if (s.off[mid] <= j) lo = mid; else hi = mid - 1;
     }
-    const int32_t x = (int32_t)chunks[j];
+    const int32_t x = chunks[j];
     int v = lo;
     for (;;) {
-      const int p = parent[v];
+      const int p = tr.parent[v];
       if (p < 0) break;
-      const int t = p - m;
-      const int32_t* s = node_sig + (size_t)t * kSigMax;
-      const int n = node_len[t];
-      int a = 0, b = n;
-      while (a < b) {
-        const int mid = (a + b) >> 1;
-        if (s[mid] < x) a = mid + 1; else b = mid;
-      }
-      if (a < n && s[a] == x) v = p; else break;
+      const int r = tr.rec_of[p - s.m];
+      if (r < 0 || find_in(s.rec_sig + (size_t)r * kSigMax, s.rec_len[r], x) < 0) break;
+      v = p;
     }
-    keys[j] = ((unsigned long long)depth[v] << 32) | (unsigned long long)(uint32_t)x;
+    const uint32_t from_root = v < s.m ? 2u * (uint32_t)s.m : 2u * (uint32_t)s.m - (uint32_t)v;
+    keys[j] = ((unsigned long long)from_root << 32) | (unsigned long long)(uint32_t)x;
   }
 }
 
-// Each request's chunks ranked by (emission depth, chunk id): warp per request.
+// Each request's chunks in the order of their keys: warp per request.
 __global__ void k_greedy_rank(int m, const int64_t* __restrict__ req_off, const unsigned long long* __restrict__ keys,
                               int64_t* __restrict__ perm) {
   const int lane = threadIdx.x & 31;
@@ -427,23 +526,27 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
   for (int64_t x = 0; x < n_chunks; ++x)
     if (weights[x] <= 0) return MPT_ERR_INVALID_ARG;
   // sorted, de-duplicated-checked signatures; per-request weight < 2^32
-  std::vector<int32_t> sig((size_t)m * kSigMax, 0), len((size_t)m, 0);
+  std::vector<int32_t> sig;
   int64_t total = 0;
-  for (int i = 0; i < m; ++i) {
-    const int64_t a = req_offsets[i], b = req_offsets[i + 1];
-    if (b < a) return MPT_ERR_INVALID_ARG;
-    if (b - a > kSigMax) return MPT_ERR_TOO_LARGE;
-    std::vector<int64_t> ids(chunk_ids + a, chunk_ids + b);
-    std::sort(ids.begin(), ids.end());
-    int64_t rw = 0;
-    for (size_t q = 0; q < ids.size(); ++q) {
-      if (ids[q] < 0 || ids[q] >= n_chunks || (q > 0 && ids[q] == ids[q - 1])) return MPT_ERR_INVALID_ARG;
-      sig[(size_t)i * kSigMax + q] = (int32_t)ids[q];
-      rw += weights[ids[q]];
-      if (rw >= ((int64_t)1 << 32)) return MPT_ERR_OVERFLOW;
+  try {
+    int64_t ids[kSigMax];
+    for (int i = 0; i < m; ++i) {
+      const int64_t a = req_offsets[i], b = req_offsets[i + 1];
+      if (b < a) return MPT_ERR_INVALID_ARG;
+      if (b - a > kSigMax) return MPT_ERR_TOO_LARGE;
+      std::copy(chunk_ids + a, chunk_ids + b, ids);
+      std::sort(ids, ids + (b - a));
+      int64_t rw = 0;
+      for (int64_t q = 0; q < b - a; ++q) {
+        if (ids[q] < 0 || ids[q] >= n_chunks || (q > 0 && ids[q] == ids[q - 1])) return MPT_ERR_INVALID_ARG;
+        sig.push_back((int32_t)ids[q]);
+        rw += weights[ids[q]];
+        if (rw >= ((int64_t)1 << 32)) return MPT_ERR_OVERFLOW;
+      }
+      total += rw;
     }
-    len[(size_t)i] = (int32_t)ids.size();
-    total += rw;
+  } catch (...) {
+    return MPT_ERR_OUT_OF_MEMORY;
   }
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_ptr);
   // device buffers (this call allocates and frees its own)
@@ -454,14 +557,14 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
     return o;
   };
   const size_t M = (size_t)m;
-  const size_t o_w = take((size_t)n_chunks * 8), o_sig = take(M * kSigMax * 4), o_len = take(M * 4),
-               o_W = take(M * M * 4), o_best = take(M * 8), o_node = take(M * 4),
-               o_re = take(M * 4 + 4), o_mer = take(M * 8), o_val = take(M * 8), o_ch = take(M * 8),
-               o_nsig = take(M * kSigMax * 4), o_nlen = take(M * 4), o_roff = take((M + 1) * 8),
-               o_chunks = take((size_t)std::max<int64_t>(occ, 1) * 8), o_par = take(2 * M * 4),
-               o_dep = take(2 * M * 4), o_stk = take(2 * M * 4), o_keys = take((size_t)std::max<int64_t>(occ, 1) * 8),
-               o_perm = take((size_t)std::max<int64_t>(occ, 1) * 8), o_dfs = take(M * 4), o_comp = take(M * 4),
-               o_bpar = take(M * 4), o_cbest = take(M * 8), o_mst = take(8);
+  const size_t O = (size_t)std::max<int64_t>(occ, 1);
+  const size_t o_w = take((size_t)n_chunks * 8), o_off = take((M + 1) * 8), o_sig = take(O * 4), o_chunks = take(O * 4),
+               o_len = take(M * 4), o_W = take(M * M * 4), o_best = take(M * 8), o_act = take(M), o_mark = take(M * 4),
+               o_top = take(M * 4), o_key = take(M * 8), o_child = take(M * 8), o_rsig = take(M * kSigMax * 4),
+               o_rlen = take(M * 4), o_merges = take(M * 8), o_val = take(M * 8), o_rank = take(M * 4),
+               o_rec = take(M * 4), o_children = take(M * 8), o_par = take(2 * M * 4), o_leaves = take(M * 4),
+               o_base = take(M * 4), o_dfs = take(M * 4), o_keys = take(O * 8), o_perm = take(O * 8),
+               o_comp = take(M * 4), o_bpar = take(M * 4), o_cbest = take(M * 8), o_ctl = take(32);
   char* d = nullptr;
   if (device_alloc(reinterpret_cast<void**>(&d), off) != cudaSuccess) return MPT_ERR_OUT_OF_MEMORY;
   const int64_t sms = sm_count();
@@ -473,64 +576,92 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
   auto d2h = [&](void* h, size_t o, size_t bytes) {
     if (e == cudaSuccess && bytes && h) e = cudaMemcpyAsync(h, d + o, bytes, cudaMemcpyDeviceToHost, stream);
   };
-  h2d(o_w, weights, (size_t)n_chunks * 8);
-  h2d(o_sig, sig.data(), sig.size() * 4);
-  h2d(o_len, len.data(), len.size() * 4);
-  h2d(o_roff, req_offsets, (M + 1) * 8);
-  h2d(o_chunks, chunk_ids, (size_t)occ * 8);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d + o_re, 0, 4, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d + o_mst, 0, 8, stream);
   auto I64 = [&](size_t o) { return reinterpret_cast<int64_t*>(d + o); };
   auto I32 = [&](size_t o) { return reinterpret_cast<int32_t*>(d + o); };
   auto U32 = [&](size_t o) { return reinterpret_cast<uint32_t*>(d + o); };
   auto U64 = [&](size_t o) { return reinterpret_cast<unsigned long long*>(d + o); };
+  // control words: 0-2 the counts of the rounds, 3 the state of Borůvka's, 4-5 the tree weight
+  int32_t* ctl = I32(o_ctl);
+  const Slots sl{m, I64(o_off), I32(o_sig), I32(o_len), U32(o_W), U64(o_best), reinterpret_cast<uint8_t*>(d + o_act),
+                 I32(o_mark), I32(o_top), U64(o_key), reinterpret_cast<int2*>(d + o_child), I32(o_rsig), I32(o_rlen),
+                 ctl};
+  const Tree tr{I32(o_merges), I64(o_val), I32(o_rank), I32(o_rec), I32(o_children), I32(o_par), I32(o_leaves),
+                I32(o_base), I32(o_dfs)};
+  h2d(o_w, weights, (size_t)n_chunks * 8);
+  h2d(o_off, req_offsets, (M + 1) * 8);
+  h2d(o_sig, sig.data(), (size_t)occ * 4);
+  if (e == cudaSuccess && occ)
+    e = cudaMemcpyAsync(d + o_chunks, d + o_sig, (size_t)occ * 4, cudaMemcpyDeviceToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d + o_ctl, 0, 32, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d + o_par, 0xFF, 2 * M * 4, stream);
+  const unsigned wb = (unsigned)std::min<int64_t>(((int64_t)m * 32 + 255) / 256, sms * 8);  // a warp per slot
+  const unsigned tb = (unsigned)std::min<int64_t>((m + 255) / 256, sms * 8);               // a thread per slot
   if (e == cudaSuccess) {
-    dim3 grid((unsigned)((m + 255) / 256), (unsigned)m);
-    k_pair_weights<<<grid, 256, 0, stream>>>(m, I32(o_sig), I32(o_len), I64(o_w), U32(o_W));
-    {
-      // maximum spanning tree by Borůvka rounds (each at least halves the components)
-      const unsigned vb = (unsigned)std::min<int64_t>(((int64_t)m * 32 + 255) / 256, sms * 32);
-      const unsigned eb = (unsigned)std::min<int64_t>((m + 255) / 256, sms * 8);
-      k_iota32<<<eb, 256, 0, stream>>>(m, I32(o_comp));
-      k_bv_reset<<<eb, 256, 0, stream>>>(m, U64(o_cbest));
-      int rounds = 1;
-      while ((1 << rounds) < m) ++rounds;
-      for (int r = 0; r < rounds; ++r) {
-        k_bv_vertex_best<<<vb, 256, 0, stream>>>(m, U32(o_W), I32(o_comp), U64(o_cbest));
-        k_bv_hook<<<eb, 256, 0, stream>>>(m, I32(o_comp), U64(o_cbest), I32(o_bpar), U64(o_mst));
-        k_bv_jump<<<eb, 256, 0, stream>>>(m, I32(o_comp), I32(o_bpar));
-        k_bv_reset<<<eb, 256, 0, stream>>>(m, U64(o_cbest));
-      }
+    k_slots_init<<<tb, 256, 0, stream>>>(sl, I32(o_comp), U64(o_cbest));
+    e = cudaFuncSetAttribute(k_pair_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, kPwSmem);
+  }
+  if (e == cudaSuccess) {
+    const dim3 grid((unsigned)((m + kPwCols - 1) / kPwCols), (unsigned)((m + kPwRows - 1) / kPwRows));
+    k_pair_weights<<<grid, kPwCols, kPwSmem, stream>>>(m, I64(o_off), I32(o_sig), I64(o_w), U32(o_W));
+    // maximum spanning tree by Borůvka rounds (each at least halves the
+    // components that still have an edge)
+    int rounds = 1;
+    while ((1 << rounds) < m) ++rounds;
+    for (int r = 0; r < rounds; ++r) {
+      k_bv_vertex_best<<<wb, 256, 0, stream>>>(m, U32(o_W), I32(o_comp), U64(o_cbest), ctl + 3);
+      k_bv_step<<<1, kGreedyThreads, 0, stream>>>(m, I32(o_comp), U64(o_cbest), I32(o_bpar),
+                                                  reinterpret_cast<unsigned long long*>(ctl + 4), ctl + 3);
     }
-    k_row_best<<<(unsigned)((m * 32 + 255) / 256), 256, 0, stream>>>(m, U32(o_W), U64(o_best));
-    {
-      const size_t msm = merge_smem_bytes(m);
-      e = cudaFuncSetAttribute(k_greedy_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msm);
-      if (e == cudaSuccess)
-        k_greedy_merge<<<1, kGreedyThreads, msm, stream>>>(m, I64(o_w), I32(o_sig), I32(o_len), U32(o_W), U64(o_best),
-                                                           I32(o_node), I32(o_mer), I64(o_val), I32(o_ch), I32(o_nsig),
-                                                           I32(o_nlen), I32(o_re));
-    }
-    k_greedy_tree<<<1, 1, 0, stream>>>(m, I32(o_ch), I32(o_par), I32(o_dep), I32(o_stk), I32(o_dfs));
-    const int64_t eblocks = std::min<int64_t>((std::max<int64_t>(occ, 1) + 255) / 256, sms * 16);
-    k_greedy_emit<<<(unsigned)eblocks, 256, 0, stream>>>(m, I32(o_nsig), I32(o_nlen), I64(o_roff), I64(o_chunks),
-                                                         I32(o_par), I32(o_dep), U64(o_keys));
-    k_greedy_rank<<<(unsigned)std::min<int64_t>(((int64_t)m * 32 + 255) / 256, sms * 16), 256, 0, stream>>>(
-        m, I64(o_roff), U64(o_keys), I64(o_perm));
     e = cudaGetLastError();
   }
-  std::vector<int64_t> vals(M > 1 ? M - 1 : 1, 0);
+  // Rounds of merges, kRoundsAhead enqueued between two looks at whether the
+  // last one still merged anything (each does, until no pair shares weight;
+  // later ones return at once).
+  constexpr int kRoundsAhead = 12;
+  int32_t counts[3] = {0, 0, 0};
+  for (int round = 0; e == cudaSuccess && m > 1;) {
+    for (int k = 0; k < kRoundsAhead; ++k, ++round) {
+      k_row_best<<<(unsigned)m, kBestThreads, 0, stream>>>(sl, round);
+      k_match<<<wb, 256, 0, stream>>>(sl, round);
+      k_reweigh<<<(unsigned)std::min<int64_t>(m, sms * 4), 256, 0, stream>>>(sl, I64(o_w), round);
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(counts, ctl, 12, cudaMemcpyDeviceToHost, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (counts[0] == counts[1 + ((round - 1) & 1)]) break;
+    if (round > m + 2 * kRoundsAhead) {  // every round before the last merges
+      if (e == cudaSuccess) st = MPT_ERR_INTERNAL;
+      break;
+    }
+  }
+  if (e == cudaSuccess && st == MPT_OK) {
+    k_rank<<<wb, 256, 0, stream>>>(sl, tr);
+    k_link<<<tb, 256, 0, stream>>>(sl, tr);
+    k_count<<<tb, 256, 0, stream>>>(sl, tr);
+    k_tail<<<1, kGreedyThreads, 0, stream>>>(sl, tr);
+    k_leaf_order<<<tb, 256, 0, stream>>>(sl, tr);
+    const int64_t eblocks = std::min<int64_t>(((int64_t)O + 255) / 256, sms * 16);
+    k_greedy_emit<<<(unsigned)eblocks, 256, 0, stream>>>(sl, tr, I32(o_chunks), U64(o_keys));
+    k_greedy_rank<<<wb, 256, 0, stream>>>(m, I64(o_off), U64(o_keys), I64(o_perm));
+    e = cudaGetLastError();
+  }
+  std::vector<int64_t> vals;
   unsigned long long mst = 0;
-  int32_t flag = 0;
-  d2h(&flag, o_re, 4);
-  d2h(vals.data(), o_val, (M - 1) * 8);
-  d2h(&mst, o_mst, 8);
-  d2h(merges, o_mer, (M - 1) * 2 * 4);
-  d2h(perm_chunks, o_perm, (size_t)occ * 8);
-  d2h(dfs_order, o_dfs, M * 4);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  try {
+    vals.assign(M > 1 ? M - 1 : 1, 0);
+  } catch (...) {
+    if (st == MPT_OK) st = MPT_ERR_OUT_OF_MEMORY;
+  }
+  if (st == MPT_OK) {
+    d2h(vals.data(), o_val, (M - 1) * 8);
+    d2h(&mst, o_ctl + 16, 8);
+    d2h(merges, o_merges, (M - 1) * 2 * 4);
+    d2h(perm_chunks, o_perm, (size_t)occ * 8);
+    d2h(dfs_order, o_dfs, M * 4);
+  }
+  const cudaError_t es = cudaStreamSynchronize(stream);
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) st = MPT_ERR_CUDA;
-  else if (flag != 0) st = MPT_ERR_INTERNAL;
   cudaFree(d);
   if (st != MPT_OK) return st;
   int64_t sav = 0;

@@ -574,7 +574,8 @@ def mpt_greedy(weights, requests, stream: Optional[int] = None) -> GreedyResult:
                           _ptr(ids, ctypes.c_int64), ctypes.c_void_p(s), ctypes.byref(cost), ctypes.byref(sav),
                           ctypes.byref(lb), _ptr(merges, ctypes.c_int32), _ptr(vals, ctypes.c_int64),
                           _ptr(perm, ctypes.c_int64), _ptr(dfs, ctypes.c_int32)), "mpt_greedy")
-    perms = [perm[offs[i]:offs[i + 1]].tolist() for i in range(m)]
+    flat, at = perm.tolist(), offs.tolist()
+    perms = [flat[at[i]:at[i + 1]] for i in range(m)]
     return GreedyResult(int(cost.value), int(sav.value), int(lb.value), merges[:2 * (m - 1)].reshape(-1, 2),
                         vals[:m - 1], perms, dfs)
 
