@@ -3,7 +3,7 @@
 //
 // Strings are laid-out requests (chunk ids).  Everything here starts from
 // their lexicographic order (a string before its extensions), built by a
-// stable least-significant-digit radix sort over string positions:
+// merge sort whose keys are the strings' first chunks:
 //   * Thm 7's serving order is that order (the DFS order of the trie), or,
 //     with a bounded reorder window, that order inside each window;
 //   * the trie of eq. (1): in lexicographic order, string x shares exactly
@@ -22,8 +22,11 @@
 //     depth q of request t, last touched by request j < t,
 //         d = sum over r in (j, t) of w(nodes of r's path not touched again before t)
 //           + w(ancestors-or-self of v whose last touch before t is j).
+#include <algorithm>
 #include <climits>
 #include <cstring>
+#include <memory>
+#include <utility>
 #include <vector>
 
 #include "../../include/mpt.h"
@@ -31,78 +34,6 @@
 
 namespace mpt {
 namespace {
-
-// ---------------------------------------------------------------------------
-// Stable LSD radix sort of (uint32 key, uint32 value) pairs, 8 bits a pass.
-// A tile of 2048 keys per block; pass = digit histogram per tile, exclusive
-// scan of the digit-major [256][tiles] counts, stable scatter.
-// ---------------------------------------------------------------------------
-constexpr int kRsThreads = 256;
-constexpr int kRsRounds = 8;
-constexpr int kRsTile = kRsThreads * kRsRounds;
-constexpr int kRsBins = 256;
-constexpr int kRsWarps = kRsThreads / 32;
-
-__global__ void __launch_bounds__(kRsThreads)
-k_rs_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, uint32_t* __restrict__ hist, int tiles) {
-  __shared__ uint32_t h[kRsBins];
-  h[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t start = (int64_t)blockIdx.x * kRsTile;
-  for (int i = threadIdx.x; i < kRsTile; i += kRsThreads) {
-    const int64_t idx = start + i;
-    if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 0xFFu], 1u);
-  }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kRsThreads)
-k_rs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-             uint32_t* __restrict__ vout, int64_t n, int shift, const uint32_t* __restrict__ offs, int tiles) {
-  __shared__ uint32_t base[kRsBins];
-  __shared__ uint32_t tot[kRsBins];
-  __shared__ uint32_t wcnt[kRsWarps][kRsBins];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  base[tid] = offs[(int64_t)tid * tiles + blockIdx.x];
-  const int64_t start = (int64_t)blockIdx.x * kRsTile;
-  const uint32_t lt = (1u << lane) - 1u;
-  for (int round = 0; round < kRsRounds; ++round) {
-#pragma unroll
-    for (int w = 0; w < kRsWarps; ++w) wcnt[w][tid] = 0;
-    __syncthreads();
-    const int64_t idx = start + (int64_t)round * kRsThreads + tid;
-    const bool valid = idx < n;
-    uint32_t key = 0, val = 0, digit = 0xFFFFu;  // 0xFFFF: no key (never a digit)
-    if (valid) {
-      key = kin[idx];
-      val = vin[idx];
-      digit = (key >> shift) & 0xFFu;
-    }
-    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, digit);
-    const uint32_t rank = __popc(peers & lt);
-    if (valid && rank == 0) wcnt[warp][digit] = __popc(peers);
-    __syncthreads();
-    {
-      uint32_t run = 0;
-#pragma unroll
-      for (int w = 0; w < kRsWarps; ++w) {
-        const uint32_t c = wcnt[w][tid];
-        wcnt[w][tid] = run;
-        run += c;
-      }
-      tot[tid] = run;
-    }
-    __syncthreads();
-    if (valid) {
-      const uint32_t pos = base[digit] + wcnt[warp][digit] + rank;
-      kout[pos] = key;
-      vout[pos] = val;
-    }
-    __syncthreads();
-    base[tid] += tot[tid];
-  }
-}
 
 // Exclusive prefix sum of uint32 values in place (n <= 2048 * 16384).
 constexpr int kScanThreads = 256;
@@ -200,40 +131,151 @@ cudaError_t exclusive_scan(uint32_t* a, int64_t n, uint32_t* sums, cudaStream_t 
   return cudaGetLastError();
 }
 
-int64_t rs_tiles(int64_t n) { return (n + kRsTile - 1) / kRsTile; }
+// ---------------------------------------------------------------------------
+// Merge sort of (uint64 key, uint32 id) by key, then by a rule on the ids that
+// leaves no two equal.  Tiles of kSortTile pairs are sorted in shared memory
+// (bitonic); a pass then joins four runs at a time, every pair finding its
+// place by a binary search in the other three.  It replaces a stable radix sort
+// per 8 key bits and string position, 88 launches of 2 to 8 us for 2,921
+// strings of 8 chunks and 128 for 100,000: two launches here up to 4,096 pairs,
+// five up to 262,144.  Tiles of 4,096 took 52 us each, 78 steps of one block,
+// where four smaller ones and a pass take 21 us.  The searches of a pass are its time (a chain of
+// log2(run) reads from L2), so four runs a pass: two would double the passes,
+// eight more than double the reads of each.
+// ---------------------------------------------------------------------------
+constexpr int kSortTile = 1024;
+constexpr int kSortThreads = 512;
 
-// Scratch of a radix sort of n pairs: second key/value buffers, the digit
-// counts and the scan's tile sums.
-struct SortScratch {
-  uint32_t* k2;
-  uint32_t* v2;
-  uint32_t* hist;
-  uint32_t* sums;
+// Keys that are all different.
+struct ByKey {
+  __device__ __forceinline__ bool less_tie(uint32_t a, uint32_t b) const { return a < b; }
 };
 
-// Sort (*keys, *vals) by key bits [0, bits); the sorted arrays end up in
-// *keys / *vals (the pointers may be swapped with the scratch buffers).
-cudaError_t radix_sort(uint32_t** keys, uint32_t** vals, SortScratch& s, int64_t n, int bits, cudaStream_t st,
-                       int* launches) {
-  if (n <= 1 || bits <= 0) return cudaSuccess;
-  const int tiles = (int)rs_tiles(n);
-  for (int shift = 0; shift < bits; shift += 8) {
-    k_rs_hist<<<tiles, kRsThreads, 0, st>>>(*keys, n, shift, s.hist, tiles);
-    ++*launches;
-    cudaError_t e = exclusive_scan(s.hist, (int64_t)kRsBins * tiles, s.sums, st, launches);
-    if (e != cudaSuccess) return e;
-    k_rs_scatter<<<tiles, kRsThreads, 0, st>>>(*keys, *vals, s.k2, s.v2, n, shift, s.hist, tiles);
-    ++*launches;
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    uint32_t* t = *keys;
-    *keys = s.k2;
-    s.k2 = t;
-    t = *vals;
-    *vals = s.v2;
-    s.v2 = t;
+// Strings whose first `packed` chunks are equal (they are the key): by the
+// rest, a string before its extensions, then by index.
+struct ByString {
+  const int64_t* off;
+  const int32_t* chunk;
+  int64_t packed;
+  __device__ __forceinline__ bool less_tie(uint32_t a, uint32_t b) const {
+    if (a == b || a == 0xFFFFFFFFu || b == 0xFFFFFFFFu) return a < b;  // the last: padding of a tile
+    const int64_t ba = off[a], la = off[a + 1] - ba, bb = off[b], lb = off[b + 1] - bb;
+    const int64_t lim = la < lb ? la : lb;
+    for (int64_t s = packed; s < lim; ++s) {
+      const int32_t x = chunk[ba + s], y = chunk[bb + s];
+      if (x != y) return x < y;
+    }
+    return la != lb && (la > packed || lb > packed) ? la < lb : a < b;
   }
-  return cudaSuccess;
+};
+
+template <typename Rule>
+__device__ __forceinline__ bool pair_less(unsigned long long ka, uint32_t a, unsigned long long kb, uint32_t b,
+                                          const Rule& rule) {
+  return ka != kb ? ka < kb : rule.less_tie(a, b);
+}
+
+template <typename Rule>
+__global__ void __launch_bounds__(kSortThreads)
+k_sort_tiles(unsigned long long* __restrict__ keys, uint32_t* __restrict__ ids, int64_t n, Rule rule) {
+  extern __shared__ __align__(16) unsigned long long sk[];
+  uint32_t* si = reinterpret_cast<uint32_t*>(sk + kSortTile);
+  const int64_t start = (int64_t)blockIdx.x * kSortTile;
+  const int count = (int)(n - start < kSortTile ? n - start : kSortTile);
+  int size = 64;  // power of two that holds the tile
+  while (size < count) size <<= 1;
+  for (int i = threadIdx.x; i < size; i += kSortThreads) {
+    sk[i] = i < count ? keys[start + i] : ~0ull;
+    si[i] = i < count ? ids[start + i] : 0xFFFFFFFFu;
+  }
+  for (int width = 2; width <= size; width <<= 1) {
+    for (int step = width >> 1; step > 0; step >>= 1) {
+      __syncthreads();
+      for (int p = threadIdx.x; p < size / 2; p += kSortThreads) {
+        const int i = ((p & ~(step - 1)) << 1) | (p & (step - 1)), j = i | step;
+        const unsigned long long ki = sk[i], kj = sk[j];
+        const uint32_t a = si[i], c = si[j];
+        const bool up = (i & width) == 0;
+        if (pair_less(kj, c, ki, a, rule) == up) {
+          sk[i] = kj;
+          sk[j] = ki;
+          si[i] = c;
+          si[j] = a;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < count; i += kSortThreads) {
+    keys[start + i] = sk[i];
+    ids[start + i] = si[i];
+  }
+}
+
+// Joins runs 4g .. 4g + 3 of `run` sorted pairs into one.
+template <typename Rule>
+__global__ void __launch_bounds__(256)
+k_sort_merge(const unsigned long long* __restrict__ keys, const uint32_t* __restrict__ ids,
+             unsigned long long* __restrict__ kout, uint32_t* __restrict__ iout, int64_t n, int64_t run, Rule rule) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long k = keys[i];
+    const uint32_t id = ids[i];
+    const int64_t own = i / run, first = own & ~(int64_t)3;
+    int64_t lo[3], hi[3], rank = i - own * run;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int64_t other = first + (q < (int)(own - first) ? q : q + 1);
+      lo[q] = other * run < n ? other * run : n;
+      hi[q] = (other + 1) * run < n ? (other + 1) * run : n;
+      rank -= lo[q];
+    }
+    // pairs of the other runs that come before this one, the three searches in step
+    while (lo[0] < hi[0] || lo[1] < hi[1] || lo[2] < hi[2]) {
+      int64_t mid[3];
+      unsigned long long km[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        mid[q] = (lo[q] + hi[q]) >> 1;
+        km[q] = lo[q] < hi[q] ? keys[mid[q]] : 0ull;
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (lo[q] < hi[q]) {
+          if (km[q] != k ? km[q] < k : rule.less_tie(ids[mid[q]], id))
+            lo[q] = mid[q] + 1;
+          else
+            hi[q] = mid[q];
+        }
+      }
+    }
+    const int64_t to = first * run + rank + lo[0] + lo[1] + lo[2];
+    kout[to] = k;
+    iout[to] = id;
+  }
+}
+
+// Sorts (*keys, *ids); the sorted arrays end up in *keys / *ids (the pointers
+// may be swapped with the second buffers).
+template <typename Rule>
+cudaError_t merge_sort(unsigned long long** keys, uint32_t** ids, unsigned long long** k2, uint32_t** i2, int64_t n,
+                       const Rule& rule, cudaStream_t st, int* launches) {
+  if (n <= 1) return cudaSuccess;
+  constexpr int kBytes = kSortTile * 12;
+  auto tiles = k_sort_tiles<Rule>;
+  cudaError_t e = cudaFuncSetAttribute(tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+  if (e != cudaSuccess) return e;
+  tiles<<<(unsigned)((n + kSortTile - 1) / kSortTile), kSortThreads, kBytes, st>>>(*keys, *ids, n, rule);
+  ++*launches;
+  for (int64_t run = kSortTile; run < n; run *= 4) {
+    int64_t blocks = (n + 255) / 256;
+    const int64_t cap = sm_count() * 64;
+    if (blocks > cap) blocks = cap;
+    k_sort_merge<<<(unsigned)blocks, 256, 0, st>>>(*keys, *ids, *k2, *i2, n, run, rule);
+    ++*launches;
+    std::swap(*keys, *k2);
+    std::swap(*ids, *i2);
+  }
+  return cudaGetLastError();
 }
 
 int bits_for(uint64_t max_value) {
@@ -255,18 +297,19 @@ unsigned grid_for(int64_t n, int64_t per_sm = 32) {
   return (unsigned)(b < 1 ? 1 : b);
 }
 
-__global__ void k_iota(uint32_t* __restrict__ a, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    a[i] = (uint32_t)i;
-}
-
-// key of the string at sorted position i for position s: chunk + 1, or 0 past its end
-__global__ void k_lex_keys(const uint32_t* __restrict__ ord, int64_t m, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ chunk, int s, uint32_t* __restrict__ keys) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t r = ord[i];
+// Sort key of every string: its window (arrival position / window; window 0:
+// none), then its first `packed` chunks + 1 at `bits` bits each, 0 past its
+// end.  arrival (may be null: 0, 1, ..) lists the requests as they arrive.
+__global__ void k_lex_keys(int64_t m, const int64_t* __restrict__ off, const int32_t* __restrict__ chunk,
+                           const int32_t* __restrict__ arrival, int64_t window, int packed, int bits,
+                           unsigned long long* __restrict__ keys, uint32_t* __restrict__ ids) {
+  for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = arrival ? arrival[a] : a;
     const int64_t b = off[r], len = off[r + 1] - b;
-    keys[i] = s < len ? (uint32_t)chunk[b + s] + 1u : 0u;
+    unsigned long long k = window > 0 ? (unsigned long long)(a / window) : 0ull;
+    for (int s = 0; s < packed; ++s) k = (k << bits) | (s < len ? (unsigned long long)chunk[b + s] + 1ull : 0ull);
+    keys[a] = k;
+    ids[a] = (uint32_t)r;
   }
 }
 
@@ -303,14 +346,17 @@ k_lcp_cost(const uint32_t* __restrict__ ord, int64_t m, const int64_t* __restric
 // ---------------------------------------------------------------------------
 // Trie nodes and the per-access recency distance.
 // ---------------------------------------------------------------------------
-// st[k][i] = min lcp[i - 2^k + 1 .. i]  (k = 1 .. K-1; level 0 is lcp itself)
+// st[k][i] = min lcp[i - 8^k + 1 .. i] (k = 1 .. K-1; level 0 is lcp itself)
 __global__ void k_sparse_level(int32_t* __restrict__ st, int64_t m, int k) {
-  const int64_t half = (int64_t)1 << (k - 1);
+  const int64_t part = (int64_t)1 << (3 * (k - 1));
   const int32_t* prev = st + (int64_t)(k - 1) * m;
   int32_t* cur = st + (int64_t)k * m;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t a = prev[i];
-    cur[i] = i >= half ? min(a, prev[i - half]) : a;
+    int32_t v = prev[i];
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+      if (i >= q * part) v = min(v, prev[i - q * part]);
+    cur[i] = v;
   }
 }
 
@@ -319,8 +365,8 @@ __device__ __forceinline__ int64_t node_owner(const int32_t* __restrict__ st, in
   if (st[x] <= s) return x;
   int64_t p = x;  // every lcp in [p, x] is > s
   for (int k = K - 1; k >= 0; --k) {
-    const int64_t len = (int64_t)1 << k;
-    if (p - len >= 0 && st[(int64_t)k * m + (p - 1)] > s) p -= len;
+    const int64_t len = (int64_t)1 << (3 * k);
+    while (p - len >= 0 && st[(int64_t)k * m + (p - 1)] > s) p -= len;  // at most seven times
   }
   return p - 1;
 }
@@ -334,13 +380,25 @@ __global__ void k_new_nodes(const uint32_t* __restrict__ ord, int64_t m, const i
   }
 }
 
+// order[t] = t without a given one, and len[t] = length of the string served
+// at t (len[m] = 0): scanned, the accesses' first positions.
+__global__ void k_served(bool given, int64_t m, const int64_t* __restrict__ off, int32_t* __restrict__ order,
+                         uint32_t* __restrict__ len) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t <= m; t += (int64_t)gridDim.x * blockDim.x) {
+    if (t < m && !given) order[t] = (int32_t)t;
+    const int64_t r = t < m && given ? order[t] : t;
+    len[t] = t < m ? (uint32_t)(off[r + 1] - off[r]) : 0u;
+  }
+}
+
 // Per access (served position t, depth s), laid out at aoff[t] + s: its trie
-// node, its chunk weight, its request's served position.
+// node (with its own number, as a sort key), its chunk weight, its request's
+// served position.
 __global__ void __launch_bounds__(kThreads)
 k_accesses(const int32_t* __restrict__ order, int64_t m, const int64_t* __restrict__ off,
            const int32_t* __restrict__ chunk, const int64_t* __restrict__ w, const int32_t* __restrict__ lexpos,
            const int32_t* __restrict__ st, int K, const uint32_t* __restrict__ node_base,
-           const int64_t* __restrict__ aoff, uint32_t* __restrict__ node, uint32_t* __restrict__ acc_id,
+           const uint32_t* __restrict__ aoff, unsigned long long* __restrict__ node, uint32_t* __restrict__ acc_id,
            int64_t* __restrict__ aw, int64_t* __restrict__ asuf, int32_t* __restrict__ aowner) {
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
     const int32_t r = order[t];
@@ -362,13 +420,14 @@ k_accesses(const int32_t* __restrict__ order, int64_t m, const int64_t* __restri
   }
 }
 
-// After a stable sort of accesses by node (input in served order), neighbours
+// After a sort of the accesses by node, then number (served order), neighbours
 // with the same node are consecutive touches of it.
-__global__ void k_prev_next(const uint32_t* __restrict__ skey, const uint32_t* __restrict__ sacc, int64_t N,
+__global__ void k_prev_next(const unsigned long long* __restrict__ skey, const uint32_t* __restrict__ sacc, int64_t N,
                             const int32_t* __restrict__ aowner, int32_t* __restrict__ prev_t,
                             int32_t* __restrict__ next_t) {
   for (int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; z < N; z += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t a = sacc[z], k = skey[z];
+    const uint32_t a = sacc[z];
+    const unsigned long long k = skey[z];
     prev_t[a] = (z > 0 && skey[z - 1] == k) ? aowner[sacc[z - 1]] : -1;
     next_t[a] = (z + 1 < N && skey[z + 1] == k) ? aowner[sacc[z + 1]] : INT_MAX;
   }
@@ -388,10 +447,10 @@ __global__ void k_scan_limit(const int64_t* __restrict__ caps, int n_caps, const
 }
 
 // weight of the nodes of served request r's path not touched again before t
-__device__ __forceinline__ int64_t untouched_suffix(const int64_t* __restrict__ aoff, const int32_t* __restrict__ next_t,
+__device__ __forceinline__ int64_t untouched_suffix(const uint32_t* __restrict__ aoff, const int32_t* __restrict__ next_t,
                                                     const int64_t* __restrict__ asuf, int64_t r, int64_t t) {
   const int64_t b = aoff[r];
-  int64_t lo = 0, hi = aoff[r + 1] - b;  // next_t is nondecreasing along a path
+  int64_t lo = 0, hi = (int64_t)aoff[r + 1] - b;  // next_t is nondecreasing along a path
   const int64_t len = hi;
   while (lo < hi) {
     const int64_t mid = (lo + hi) >> 1;
@@ -409,14 +468,14 @@ constexpr int kDistThreads = 256;
 // path.  dist = INT64_MAX for a first touch (a miss at every capacity),
 // limit + 1 when it exceeds the largest capacity of interest.
 __global__ void __launch_bounds__(kDistThreads)
-k_distance(int64_t m, const int64_t* __restrict__ aoff, const int32_t* __restrict__ prev_t,
+k_distance(int64_t m, const uint32_t* __restrict__ aoff, const int32_t* __restrict__ prev_t,
            const int32_t* __restrict__ next_t, const int64_t* __restrict__ aw, const int64_t* __restrict__ asuf,
            const int64_t* __restrict__ limit_p, int64_t* __restrict__ dist) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (kDistThreads / 32);
   const int64_t limit = *limit_p;
   for (int64_t t = (int64_t)blockIdx.x * (kDistThreads / 32) + (threadIdx.x >> 5); t < m; t += warps) {
-    const int64_t b = aoff[t], len = aoff[t + 1] - b;
+    const int64_t b = aoff[t], len = (int64_t)aoff[t + 1] - b;
     int64_t scanned = t;  // requests [scanned, t) are summed
     int64_t sum = 0;
     bool over = limit < 0;
@@ -454,46 +513,43 @@ k_distance(int64_t m, const int64_t* __restrict__ aoff, const int32_t* __restric
 
 constexpr int kMaxCaps = 1024;
 
+// Weight of the accesses by how many of the sorted capacities they miss at:
+// bins[j] = sum of w over accesses with caps[j - 1] < dist <= caps[j].  Each
+// block keeps `copies` bins per value, a lane's own where they fit, so that
+// lanes do not queue for one; an add per capacity and access on one counter each
+// took 41 us at 23,368 accesses and 10 capacities, 165 us at 800,000.
+constexpr int kBinWords = 4096;  // uint64 bins of a block
+
 __global__ void __launch_bounds__(kThreads)
 k_cache_costs(const int64_t* __restrict__ dist, const int64_t* __restrict__ aw, int64_t N,
-              const int64_t* __restrict__ caps, int n_caps, unsigned long long* __restrict__ costs,
+              const int64_t* __restrict__ caps, int n_caps, int copies, unsigned long long* __restrict__ bins,
               unsigned long long* __restrict__ compulsory) {
-  __shared__ unsigned long long acc[kMaxCaps];
+  __shared__ unsigned long long acc[kBinWords];
   __shared__ int64_t cap_s[kMaxCaps];
-  for (int i = threadIdx.x; i < n_caps; i += blockDim.x) {
-    acc[i] = 0;
-    cap_s[i] = caps[i];
-  }
+  for (int i = threadIdx.x; i < n_caps; i += blockDim.x) cap_s[i] = caps[i];
+  for (int i = threadIdx.x; i < (n_caps + 1) * copies; i += blockDim.x) acc[i] = 0;
   __syncthreads();
+  const int copy = (int)threadIdx.x & (copies - 1);
   unsigned long long first = 0;
   for (int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; a < N; a += (int64_t)gridDim.x * blockDim.x) {
     const int64_t d = dist[a];
     const unsigned long long wa = (unsigned long long)aw[a];
     if (d == LLONG_MAX) first += wa;
-    for (int i = 0; i < n_caps; ++i)
-      if (d > cap_s[i]) atomicAdd(&acc[i], wa);
+    int lo = 0, hi = n_caps;  // capacities below d
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (cap_s[mid] < d) lo = mid + 1; else hi = mid;
+    }
+    atomicAdd(&acc[lo * copies + copy], wa);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) first += __shfl_xor_sync(0xFFFFFFFFu, first, o);
   if ((threadIdx.x & 31) == 0 && first) atomicAdd(compulsory, first);
   __syncthreads();
-  for (int i = threadIdx.x; i < n_caps; i += blockDim.x)
-    if (acc[i]) atomicAdd(&costs[i], acc[i]);
-}
-
-// order[z] = arrival[vals[z]]
-__global__ void k_gather_order(const uint32_t* __restrict__ vals, const int32_t* __restrict__ arrival, int64_t m,
-                               int32_t* __restrict__ order) {
-  for (int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; z < m; z += (int64_t)gridDim.x * blockDim.x)
-    order[z] = arrival[vals[z]];
-}
-
-__global__ void k_window_keys(const uint32_t* __restrict__ vals, const int32_t* __restrict__ arrival,
-                              const int32_t* __restrict__ lexpos, int64_t m, int64_t window, int pass,
-                              uint32_t* __restrict__ keys) {
-  for (int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; z < m; z += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t a = vals[z];
-    keys[z] = pass == 0 ? (uint32_t)lexpos[arrival[a]] : (uint32_t)((int64_t)a / window);
+  for (int i = threadIdx.x; i <= n_caps; i += blockDim.x) {
+    unsigned long long v = 0;
+    for (int q = 0; q < copies; ++q) v += acc[i * copies + q];
+    if (v) atomicAdd(&bins[i], v);
   }
 }
 
@@ -517,7 +573,7 @@ struct Arena {
 
 struct Strings {
   int64_t m = 0, total = 0, maxlen = 0;
-  std::vector<int32_t> chunk;
+  std::unique_ptr<int32_t[]> chunk;  // not initialised first
 };
 
 mpt_status check_strings(int64_t n_chunks, int64_t m, const int64_t* offsets, const int64_t* chunks, Strings* out) {
@@ -537,15 +593,18 @@ mpt_status check_strings(int64_t n_chunks, int64_t m, const int64_t* offsets, co
   out->total = total;
   out->maxlen = maxlen;
   try {
-    out->chunk.resize((size_t)(total > 0 ? total : 1));
+    out->chunk.reset(new int32_t[(size_t)(total > 0 ? total : 1)]);
   } catch (...) {
     return MPT_ERR_OUT_OF_MEMORY;
   }
+  // one pass without branches: an id in range is below n_chunks as an unsigned number
+  int32_t* to = out->chunk.get();
+  uint64_t outside = 0;
   for (int64_t p = 0; p < total; ++p) {
-    if (chunks[p] < 0 || chunks[p] >= n_chunks) return MPT_ERR_INVALID_ARG;
-    out->chunk[(size_t)p] = (int32_t)chunks[p];
+    outside |= (uint64_t)chunks[p] >= (uint64_t)n_chunks;
+    to[p] = (int32_t)chunks[p];
   }
-  return MPT_OK;
+  return outside ? MPT_ERR_INVALID_ARG : MPT_OK;
 }
 
 mpt_status check_weights(const int64_t* weights, int64_t n_chunks) {
@@ -569,9 +628,8 @@ struct LexBuffers {
   int64_t* off;
   int32_t* chunk;
   int64_t* w;
-  uint32_t* keys;
-  uint32_t* ord;
-  SortScratch sort;
+  unsigned long long *keys, *keys2;
+  uint32_t *ord, *ord2;
   int32_t* lexpos;
   int32_t* lcp;  // level 0 of the sparse table when the cache is simulated
   unsigned long long* trie;
@@ -582,37 +640,35 @@ void carve_lex(Arena& a, const Strings& s, int64_t n_chunks, int64_t sparse_leve
   b->off = a.take<int64_t>(m + 1);
   b->chunk = a.take<int32_t>(s.total);
   b->w = weights ? a.take<int64_t>(n_chunks) : nullptr;
-  b->keys = a.take<uint32_t>(m);
+  b->keys = a.take<unsigned long long>(m);
+  b->keys2 = a.take<unsigned long long>(m);
   b->ord = a.take<uint32_t>(m);
-  b->sort.k2 = a.take<uint32_t>(m);
-  b->sort.v2 = a.take<uint32_t>(m);
-  b->sort.hist = a.take<uint32_t>((int64_t)kRsBins * rs_tiles(m));
-  b->sort.sums = a.take<uint32_t>(scan_tiles((int64_t)kRsBins * rs_tiles(m)));
+  b->ord2 = a.take<uint32_t>(m);
   b->lexpos = a.take<int32_t>(m);
   b->lcp = a.take<int32_t>(m * (sparse_levels > 0 ? sparse_levels : 1));
   b->trie = a.take<unsigned long long>(1);
 }
 
-// Sorts the strings (b->ord = string at each sorted position, b->lexpos its
-// inverse); with weights, also lcp and the trie weight.
-cudaError_t run_lex(const Strings& s, LexBuffers* b, int n_bits, bool with_cost, cudaStream_t st, int* launches) {
+// Sorts the strings (b->ord = string at each sorted position), first by window
+// when there are any (window > 0; arrival on the device or null).  With
+// `with_cost`, also the inverse b->lexpos, lcp and the trie weight.
+cudaError_t run_lex(const Strings& s, LexBuffers* b, int64_t n_chunks, const int32_t* d_arrival, int64_t window,
+                    bool with_cost, cudaStream_t st, int* launches) {
   const int64_t m = s.m;
-  k_iota<<<grid_for(m), kThreads, 0, st>>>(b->ord, m);
+  // chunk + 1 takes at most 31 bits and a window number 22, so at least one chunk is packed
+  const int bits = bits_for((uint64_t)n_chunks), wbits = window > 0 ? bits_for((uint64_t)((m - 1) / window)) : 0;
+  const int fit = (64 - wbits) / bits;
+  const int packed = (int)(s.maxlen < fit ? s.maxlen : fit);
+  k_lex_keys<<<grid_for(m), kThreads, 0, st>>>(m, b->off, b->chunk, d_arrival, window, packed, bits, b->keys, b->ord);
   ++*launches;
-  for (int64_t pos = s.maxlen - 1; pos >= 0; --pos) {
-    k_lex_keys<<<grid_for(m), kThreads, 0, st>>>(b->ord, m, b->off, b->chunk, (int)pos, b->keys);
-    ++*launches;
-    cudaError_t e = radix_sort(&b->keys, &b->ord, b->sort, m, n_bits, st, launches);
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = merge_sort(&b->keys, &b->ord, &b->keys2, &b->ord2, m, ByString{b->off, b->chunk, packed}, st,
+                             launches);
+  if (e != cudaSuccess || !with_cost) return e;
   k_inverse<<<grid_for(m), kThreads, 0, st>>>(b->ord, m, b->lexpos);
   ++*launches;
-  if (with_cost) {
-    cudaError_t e = cudaMemsetAsync(b->trie, 0, sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
-    k_lcp_cost<<<grid_for(m), kThreads, 0, st>>>(b->ord, m, b->off, b->chunk, b->w, b->lcp, b->trie);
-    ++*launches;
-  }
+  if ((e = cudaMemsetAsync(b->trie, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
+  k_lcp_cost<<<grid_for(m), kThreads, 0, st>>>(b->ord, m, b->off, b->chunk, b->w, b->lcp, b->trie);
+  ++*launches;
   return cudaGetLastError();
 }
 
@@ -620,7 +676,7 @@ cudaError_t upload_strings(const Strings& s, const int64_t* offsets, const int64
                            LexBuffers* b, cudaStream_t st) {
   cudaError_t e = cudaMemcpyAsync(b->off, offsets, (size_t)(s.m + 1) * 8, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && s.total > 0)
-    e = cudaMemcpyAsync(b->chunk, s.chunk.data(), (size_t)s.total * 4, cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(b->chunk, s.chunk.get(), (size_t)s.total * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && b->w) e = cudaMemcpyAsync(b->w, weights, (size_t)n_chunks * 8, cudaMemcpyHostToDevice, st);
   return e;
 }
@@ -632,8 +688,8 @@ mpt_status cuda_status(cudaError_t e) {
 
 int sparse_levels_for(int64_t m) {
   int K = 1;
-  while (((int64_t)1 << K) <= m) ++K;
-  return K;  // 2^K > m
+  while (((int64_t)1 << (3 * K)) <= m) ++K;
+  return K;  // 8^K > m
 }
 
 }  // namespace
@@ -656,7 +712,7 @@ mpt_status trie_cost_lex(const int64_t* weights, int64_t n_chunks, int64_t m, co
   int launches = 0;
   unsigned long long h = 0;
   e = upload_strings(s, offsets, weights, n_chunks, &b, st);
-  if (e == cudaSuccess) e = run_lex(s, &b, bits_for((uint64_t)n_chunks), true, st, &launches);
+  if (e == cudaSuccess) e = run_lex(s, &b, n_chunks, nullptr, 0, true, st, &launches);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, b.trie, 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(mem);
@@ -684,46 +740,22 @@ mpt_status mpt_serve_order(int64_t n_chunks, int32_t m, const int64_t* seq_offse
   Arena a;
   LexBuffers b{};
   carve_lex(a, s, n_chunks, 1, false, &b);
-  int32_t* d_arrival = a.take<int32_t>(m);
-  int32_t* d_order = a.take<int32_t>(m);
+  // arrival positions matter only to windows
+  int32_t* d_arrival = windowed && arrival ? a.take<int32_t>(m) : nullptr;
   char* mem = nullptr;
   cudaError_t e = device_alloc(reinterpret_cast<void**>(&mem), a.off);
   if (e != cudaSuccess) return cuda_status(e);
   Arena a2{mem, 0};
   carve_lex(a2, s, n_chunks, 1, false, &b);
-  d_arrival = a2.take<int32_t>(m);
-  d_order = a2.take<int32_t>(m);
+  if (windowed && arrival) d_arrival = a2.take<int32_t>(m);
 
-  std::vector<int32_t> ident;
-  const int32_t* arr = arrival;
-  if (!arr) {
-    ident.resize((size_t)m);
-    for (int32_t i = 0; i < m; ++i) ident[(size_t)i] = i;
-    arr = ident.data();
-  }
   int launches = 0;
   e = upload_strings(s, seq_offsets, nullptr, n_chunks, &b, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_arrival, arr, (size_t)m * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = run_lex(s, &b, bits_for((uint64_t)n_chunks), false, st, &launches);
-  if (e == cudaSuccess) {
-    if (!windowed) {
-      e = cudaMemcpyAsync(d_order, b.ord, (size_t)m * 4, cudaMemcpyDeviceToDevice, st);
-    } else {
-      // sort arrival positions by (window index, lexicographic position)
-      uint32_t* keys = b.keys;
-      uint32_t* vals = b.ord;
-      k_iota<<<grid_for(m), kThreads, 0, st>>>(vals, m);
-      for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
-        k_window_keys<<<grid_for(m), kThreads, 0, st>>>(vals, d_arrival, b.lexpos, m, window, pass, keys);
-        const int nb = pass == 0 ? bits_for((uint64_t)m) : bits_for((uint64_t)((m - 1) / window));
-        e = radix_sort(&keys, &vals, b.sort, m, nb, st, &launches);
-      }
-      if (e == cudaSuccess) k_gather_order<<<grid_for(m), kThreads, 0, st>>>(vals, d_arrival, m, d_order);
-      if (e == cudaSuccess) e = cudaGetLastError();
-    }
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(order, d_order, (size_t)m * 4, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && d_arrival) e = cudaMemcpyAsync(d_arrival, arrival, (size_t)m * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = run_lex(s, &b, n_chunks, d_arrival, windowed ? window : 0, false, st, &launches);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(order, b.ord, (size_t)m * 4, cudaMemcpyDeviceToHost, st);
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
   cudaFree(mem);
   return cuda_status(e);
 }
@@ -740,7 +772,9 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
   if (ms != MPT_OK) return ms;
   if ((ms = check_weights(weights, n_chunks)) != MPT_OK) return ms;
   if (order && (ms = check_permutation(order, m)) != MPT_OK) return ms;
-  {
+  int64_t heaviest = 0;
+  for (int64_t x = 0; x < n_chunks; ++x) heaviest = weights[x] > heaviest ? weights[x] : heaviest;
+  if (heaviest > ((int64_t)1 << 62) / (s.total > 0 ? s.total : 1)) {
     // distances and costs are sums of distinct node weights: bounded by the
     // total string weight
     int64_t total_w = 0;
@@ -754,29 +788,20 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
   const int64_t N = s.total;
   const int K = sparse_levels_for(m);
 
-  std::vector<int32_t> h_order((size_t)m);
-  std::vector<int64_t> h_aoff((size_t)m + 1);
-  for (int32_t t = 0; t < m; ++t) h_order[(size_t)t] = order ? order[t] : t;
-  h_aoff[0] = 0;
-  for (int32_t t = 0; t < m; ++t) {
-    const int32_t r = h_order[(size_t)t];
-    h_aoff[(size_t)t + 1] = h_aoff[(size_t)t] + (seq_offsets[r + 1] - seq_offsets[r]);
-  }
-
-  auto carve = [&](Arena& a, LexBuffers* b, int32_t** d_order, int64_t** d_aoff, uint32_t** node_base,
-                   uint32_t** node, uint32_t** acc_id, SortScratch* as, int64_t** aw, int64_t** asuf,
+  auto carve = [&](Arena& a, LexBuffers* b, int32_t** d_order, uint32_t** d_aoff, uint32_t** node_base,
+                   unsigned long long** node, unsigned long long** node2, uint32_t** acc_id, uint32_t** acc2,
+                   uint32_t** sums, int64_t** aw, int64_t** asuf,
                    int32_t** aowner, int32_t** prev_t, int32_t** next_t, int64_t** dist, int64_t** d_caps,
-                   int64_t** limit, unsigned long long** d_costs, unsigned long long** compulsory) {
+                   int64_t** limit, unsigned long long** d_bins, unsigned long long** compulsory) {
     carve_lex(a, s, n_chunks, K, true, b);
     *d_order = a.take<int32_t>(m);
-    *d_aoff = a.take<int64_t>(m + 1);
+    *d_aoff = a.take<uint32_t>(m + 1);
     *node_base = a.take<uint32_t>(m);
-    *node = a.take<uint32_t>(N);
+    *node = a.take<unsigned long long>(N);
+    *node2 = a.take<unsigned long long>(N);
     *acc_id = a.take<uint32_t>(N);
-    as->k2 = a.take<uint32_t>(N);
-    as->v2 = a.take<uint32_t>(N);
-    as->hist = a.take<uint32_t>((int64_t)kRsBins * rs_tiles(N));
-    as->sums = a.take<uint32_t>(scan_tiles((int64_t)kRsBins * rs_tiles(N)) + scan_tiles(m));
+    *acc2 = a.take<uint32_t>(N);
+    *sums = a.take<uint32_t>(scan_tiles((int64_t)m + 1));
     *aw = a.take<int64_t>(N);
     *asuf = a.take<int64_t>(N);
     *aowner = a.take<int32_t>(N);
@@ -785,55 +810,65 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
     *dist = a.take<int64_t>(N);
     *d_caps = a.take<int64_t>(n_caps);
     *limit = a.take<int64_t>(1);
-    *d_costs = a.take<unsigned long long>(n_caps);
+    *d_bins = a.take<unsigned long long>(n_caps + 1);
     *compulsory = a.take<unsigned long long>(1);
   };
   LexBuffers b{};
   int32_t* d_order;
-  int64_t *d_aoff, *aw, *asuf, *dist, *d_caps, *limit;
-  uint32_t *node_base, *node, *acc_id;
-  SortScratch as{};
+  int64_t *aw, *asuf, *dist, *d_caps, *limit;
+  uint32_t *d_aoff, *node_base, *acc_id, *acc2, *sums;
   int32_t *aowner, *prev_t, *next_t;
-  unsigned long long *d_costs, *compulsory;
+  unsigned long long *node, *node2, *d_bins, *compulsory;
   Arena a;
-  carve(a, &b, &d_order, &d_aoff, &node_base, &node, &acc_id, &as, &aw, &asuf, &aowner, &prev_t, &next_t, &dist,
-        &d_caps, &limit, &d_costs, &compulsory);
+  carve(a, &b, &d_order, &d_aoff, &node_base, &node, &node2, &acc_id, &acc2, &sums, &aw, &asuf, &aowner, &prev_t,
+        &next_t, &dist, &d_caps, &limit, &d_bins, &compulsory);
   char* mem = nullptr;
   cudaError_t e = device_alloc(reinterpret_cast<void**>(&mem), a.off);
   if (e != cudaSuccess) return cuda_status(e);
   Arena a2{mem, 0};
-  carve(a2, &b, &d_order, &d_aoff, &node_base, &node, &acc_id, &as, &aw, &asuf, &aowner, &prev_t, &next_t, &dist,
-        &d_caps, &limit, &d_costs, &compulsory);
+  carve(a2, &b, &d_order, &d_aoff, &node_base, &node, &node2, &acc_id, &acc2, &sums, &aw, &asuf, &aowner, &prev_t,
+        &next_t, &dist, &d_caps, &limit, &d_bins, &compulsory);
 
   int launches = 0;
   unsigned long long h_trie = 0, h_first = 0;
-  std::vector<unsigned long long> h_costs((size_t)(n_caps > 0 ? n_caps : 1));
+  std::vector<unsigned long long> h_bins((size_t)n_caps + 1);
+  // the capacities in increasing order
+  std::vector<int32_t> by_cap((size_t)n_caps);
+  std::vector<int64_t> h_caps((size_t)n_caps);
+  for (int32_t i = 0; i < n_caps; ++i) by_cap[(size_t)i] = i;
+  std::sort(by_cap.begin(), by_cap.end(), [&](int32_t x, int32_t y) { return capacities[x] < capacities[y]; });
+  for (int32_t i = 0; i < n_caps; ++i) h_caps[(size_t)i] = capacities[by_cap[(size_t)i]];
+  int copies = 32;
+  while (copies > 1 && copies * (n_caps + 1) > kBinWords) copies >>= 1;
   e = upload_strings(s, seq_offsets, weights, n_chunks, &b, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_order, h_order.data(), (size_t)m * 4, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_aoff, h_aoff.data(), (size_t)(m + 1) * 8, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && order) e = cudaMemcpyAsync(d_order, order, (size_t)m * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    // served position -> first access: the lengths in served order, summed
+    k_served<<<grid_for(m + 1), kThreads, 0, st>>>(order != nullptr, m, b.off, d_order, d_aoff);
+    ++launches;
+    e = exclusive_scan(d_aoff, m + 1, sums, st, &launches);
+  }
   if (e == cudaSuccess && n_caps > 0)
-    e = cudaMemcpyAsync(d_caps, capacities, (size_t)n_caps * 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_costs, 0, (size_t)(n_caps > 0 ? n_caps : 1) * 8, st);
+    e = cudaMemcpyAsync(d_caps, h_caps.data(), (size_t)n_caps * 8, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_bins, 0, ((size_t)n_caps + 1) * 8, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(compulsory, 0, 8, st);
-  if (e == cudaSuccess) e = run_lex(s, &b, bits_for((uint64_t)n_chunks), true, st, &launches);
+  if (e == cudaSuccess) e = run_lex(s, &b, n_chunks, nullptr, 0, true, st, &launches);
   if (e == cudaSuccess && N > 0) {
     for (int k = 1; k < K; ++k) k_sparse_level<<<grid_for(m), kThreads, 0, st>>>(b.lcp, m, k);
     k_new_nodes<<<grid_for(m), kThreads, 0, st>>>(b.ord, m, b.off, b.lcp, node_base);
     launches += K;
-    e = exclusive_scan(node_base, m, as.sums, st, &launches);
+    e = exclusive_scan(node_base, m, sums, st, &launches);
     if (e == cudaSuccess) {
       k_accesses<<<grid_for(m), kThreads, 0, st>>>(d_order, m, b.off, b.chunk, b.w, b.lexpos, b.lcp, K, node_base,
                                                    d_aoff, node, acc_id, aw, asuf, aowner);
       ++launches;
-      uint32_t* keys = node;
-      uint32_t* vals = acc_id;
-      e = radix_sort(&keys, &vals, as, N, bits_for((uint64_t)N), st, &launches);
+      e = merge_sort(&node, &acc_id, &node2, &acc2, N, ByKey{}, st, &launches);
       if (e == cudaSuccess) {
-        k_prev_next<<<grid_for(N), kThreads, 0, st>>>(keys, vals, N, aowner, prev_t, next_t);
+        k_prev_next<<<grid_for(N), kThreads, 0, st>>>(node, acc_id, N, aowner, prev_t, next_t);
         k_scan_limit<<<1, 32, 0, st>>>(d_caps, n_caps, b.trie, limit);
         k_distance<<<grid_for(m * 32, 64), kDistThreads, 0, st>>>(m, d_aoff, prev_t, next_t, aw, asuf, limit,
                                                                          dist);
-        k_cache_costs<<<grid_for(N, 8), kThreads, 0, st>>>(dist, aw, N, d_caps, n_caps, d_costs, compulsory);
+        k_cache_costs<<<grid_for(N, 4), kThreads, 0, st>>>(dist, aw, N, d_caps, n_caps, copies, d_bins, compulsory);
         launches += 4;
         e = cudaGetLastError();
       }
@@ -841,14 +876,18 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h_trie, b.trie, 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h_first, compulsory, 8, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && n_caps > 0)
-    e = cudaMemcpyAsync(h_costs.data(), d_costs, (size_t)n_caps * 8, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h_bins.data(), d_bins, ((size_t)n_caps + 1) * 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFree(mem);
   if (e != cudaSuccess) return cuda_status(e);
   // every trie node is first touched exactly once
   if (h_first != h_trie) return MPT_ERR_INTERNAL;
-  for (int32_t i = 0; i < n_caps; ++i) costs[i] = (int64_t)h_costs[(size_t)i];
+  unsigned long long missed = 0;  // by the accesses beyond the i-th capacity
+  for (int32_t i = n_caps - 1; i >= 0; --i) {
+    missed += h_bins[(size_t)i + 1];
+    costs[by_cap[(size_t)i]] = (int64_t)missed;
+  }
   if (unbounded) *unbounded = (int64_t)h_trie;
   return MPT_OK;
 }
