@@ -936,6 +936,8 @@ cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cud
 }
 
 cudaError_t launch_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
+  const cudaError_t e = blocked_attributes(true);  // step 1 has no pairs before it
+  if (e != cudaSuccess) return e;
   launch_tiles(s, ws, kh, ws.prune_info, stream);
   ++*launches;
   return cudaGetLastError();

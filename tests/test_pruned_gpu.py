@@ -9,6 +9,10 @@ requests, ties, a universal chunk, instances that must stay with the full
 recurrence.
 """
 
+import subprocess
+import sys
+from pathlib import Path
+
 import numpy as np
 import pytest
 
@@ -110,6 +114,21 @@ def test_wide_many_members(mpt):
     Fa, wa, sa = mpt.mpt_tables(a.ctx)
     Fb, wb, sb = mpt.mpt_tables(b.ctx)
     assert torch.equal(Fa, Fb << 21) and torch.equal(wa, wb << 21) and torch.equal(sa, sb)
+
+
+@pytest.mark.parametrize("scale", [1, 1 << 21])
+def test_long_lists_in_a_fresh_process(mpt, scale):
+    """The first solve of a process meets a tile with a long list in step 1,
+    before any launch that raises the kernels' shared-memory limits."""
+    code = ("import numpy as np; from tests.test_pruned_gpu import _from_supports, _mask\n"
+            "from paper_2609_13692_gb300 import mpt\n"
+            "inst = _from_supports(20, [_mask(*range(0, 20, 2)), _mask(*range(3, 20)), _mask(0, 1), _mask(1, 19)], 6)\n"
+            f"print(mpt.solve(inst.weights * {scale}, inst.bits).opt // {scale})")
+    root = Path(__file__).resolve().parent.parent
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    inst = _from_supports(20, [_mask(*range(0, 20, 2)), _mask(*range(3, 20)), _mask(0, 1), _mask(1, 19)], 6)
+    assert int(r.stdout) == mpt.solve(inst.weights, inst.bits, mode="blocked").opt
 
 
 def test_route(mpt):
