@@ -39,12 +39,13 @@
 // k_dp_pruned is bound by the integer ALU pipe where a popular passage gives
 // long a1 lists: 55 % of the pipe busy in the heaviest layers of the first 26
 // of the 28 requests, a sixth of it on the bookkeeping per pair, the rest of
-// the time lost to the barrier per pair (the warps of a block have 1, 2 or 4
+// the time lost to the barrier per pair (the warps of a group have 1, 2 or 4
 // rows of work each).  Also measured there (tile stage at m = 28, seed 1,
-// 15.6 ms): three slots and three blocks per SM 16.8 ms, two slots and three
-// blocks 16.7, two blocks 21.9; the members evaluated one by one instead of by
-// rows 242 ms; the inner bits in natural order 69.9 ms; the warps' row groups
-// dealt in turn per SM instead of by a hash 16.2 ms.
+// 13.1 ms): a block per tile, four to an SM, with the row groups dealt by a
+// hash of the block 15.5 ms, in turn per SM 16.2; three such blocks with three
+// slots 16.8, with two slots 16.7, two blocks with four 21.9; the members
+// evaluated one by one instead of by rows 242 ms; the inner bits in natural
+// order 69.9 ms.
 #include "mpt_internal.cuh"
 
 namespace mpt {
@@ -72,15 +73,28 @@ struct PrunedCfg {
   static constexpr int kLogWarps = kPB - kRB - 5;
   // rows kept per Ta: those of a short list, or all (64-bit keys have no other kernel for a long one)
   static constexpr int kKept = sizeof(Key) == 4 ? kPruneRows : kRows;
-  static constexpr int kBlocks = sizeof(Key) == 4 ? 4 : 2;  // per SM
+  static constexpr int kGroups = sizeof(Key) == 4 ? 4 : 1;  // per block, at most
   static constexpr int kSlots = 2;
   static constexpr int kSlotBytes = (kRows + kPruneRows) * kRowBytes;  // Y window, X rows
   static constexpr int kTileBytes = kRows * (kRow + 1) * (int)sizeof(Key);  // a tile's keys, rows kRow + 1 apart
   static constexpr int kSeqStride = kRows + 2;  // so that a row's entries lie in different banks
   static constexpr int kSeqBytes = kRow * kSeqStride * 2;
-  static constexpr int kSmem = kSlots * kSlotBytes + kSeqBytes + kPQueue * 4;
+  static constexpr int kSharedAt = kSlots * kSlotBytes + kSeqBytes + kPQueue * 4;
   static_assert(kSlotBytes >= kTileBytes, "a tile's keys fit a slot");
-  static_assert((kSmem + 3072) * kBlocks <= 228 * 1024, "blocks per SM");
+  static constexpr int kGroupBytes = (kSharedAt + 4096 + 127) / 128 * 128;
+  static_assert(kGroupBytes * kGroups <= 227 * 1024, "one block fits an SM");
+};
+
+// What a group of k_dp_pruned shares beside its windows and queue.
+template <typename Key>
+struct PrunedShared {
+  // listed entries of the tile T: F << b, split, Ua, row of the list; by level, levels' sizes
+  Key f[kPruneSelf];
+  uint2 rows[PrunedCfg<Key>::kSlots][kPruneRows];  // (a1 | rows << 16, mask) of the staged pairs
+  uint32_t sp[kPruneSelf], start[kPB + 2], warp_n[PrunedCfg<Key>::kRows / 32];
+  uint32_t last, any, unit;
+  uint16_t u[kPruneSelf];
+  uint8_t k[kPruneSelf], order[kPruneSelf];
 };
 
 // w(I(T, .)) and the row list of every T, one block per tile at a time, from
@@ -261,15 +275,6 @@ __device__ __forceinline__ unsigned long long min_keep(unsigned long long a, uns
   *keep = a <= b;
   return *keep ? a : b;
 }
-__device__ __forceinline__ uint32_t warp_min(uint32_t v) { return __reduce_min_sync(0xFFFFFFFFu, v); }
-__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
-  for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, v, off);
-    v = o < v ? o : v;
-  }
-  return v;
-}
-
 __device__ __forceinline__ void pcopy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -332,8 +337,10 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
   }
 }
 
-// One tile T with |T| = kh >= 1 per block, or `items` blocks per tile that
-// each take every items-th pair.  Thread = row s1 of the tile, with its
+// One tile T with |T| = kh >= 1 per group of threads, or `items` groups per tile
+// that each take every items-th pair; a block of up to kGroups groups stays on
+// an SM and its groups take the next unit of the layer as they finish (*next).
+// Thread = row s1 of the tile, with its
 // kRow outputs' best keys in registers and, in shared memory, the numbers of
 // their pairs in the queue (written only on a strict improvement, the pairs
 // coming in increasing Ta).  Per pair the complement window Y and the listed
@@ -344,20 +351,21 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 // The inner bits are stored in an order (perm) that puts those of the request
 // sets that cost most first into a2, where a listed row is then one register
 // convolution without idle lanes, and next into the bits that tell the warps
-// apart.  The warps are dealt the row groups in an order that varies with
-// the block: rows with more of a list's a1 bits take longer, and the blocks
-// of one SM then load its four sub-partitions about alike.
-// Blocks of one tile, rounds of one block beyond the queue and, with
+// apart.  Rows with more of a list's a1 bits take longer (1, 2, 2 and 4 rows of
+// work for the four warps of a group, say), so the groups deal their warps the
+// row groups in rotated orders and each sub-partition has one of each kind.
+// Groups of one tile, rounds of one group beyond the queue and, with
 // long_lists, the pair kernel's minima meet in `partial` ((key << 32 | Ta); for
 // 64-bit keys, one block per tile and no pair kernel, the key, and Ta in
-// partial_ta).  The block that finishes last (done[]) goes on to the tile's
+// partial_ta).  The group that finishes last (done[]) goes on to the tile's
 // entries.
 template <typename Key, typename Tab>
-__global__ void __launch_bounds__(PrunedCfg<Key>::kRows, PrunedCfg<Key>::kBlocks)
+__global__ void __launch_bounds__(PrunedCfg<Key>::kRows * (sizeof(Key) == 4 ? PrunedCfg<Key>::kGroups : 1),
+                                  sizeof(Key) == 4 ? 1 : 2)
 k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
             const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
             const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* partial_ta,
-            uint32_t* __restrict__ done, Key* Gp,
+            uint32_t* __restrict__ done, uint32_t* __restrict__ next, Key* Gp,
             Key* Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
   using C = PrunedCfg<Key>;
   constexpr int kRB = C::kRB, kRow = C::kRow, NT = C::kRows, kWarps = NT / 32;
@@ -365,20 +373,30 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   constexpr Key kNone = ~(Key)0;
   constexpr uint32_t kSelf = 0xFFFFu, kListed = 0x8000u;  // pair numbers of the self pair and of listed entries
   static_assert(kPQueue <= 0x8000, "pair numbers fit beside the two marks");
-  extern __shared__ __align__(16) char psm[];
+  extern __shared__ __align__(16) char block_sm[];
+  const uint32_t group = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid & 31u, warp = tid >> 5;
+  char* psm = block_sm + group * C::kGroupBytes;
   Key* skey = reinterpret_cast<Key*>(psm + C::kSlotBytes);  // after the pairs: keys, rows kRow + 1 apart
   uint16_t* seq = reinterpret_cast<uint16_t*>(psm + C::kSlots * C::kSlotBytes);  // [in-row entry][thread]
   uint32_t* queue = reinterpret_cast<uint32_t*>(psm + C::kSlots * C::kSlotBytes + C::kSeqBytes);
-  __shared__ uint32_t warp_n[kWarps];
-  __shared__ uint2 s_rows[C::kSlots][kPruneRows];  // (a1 | rows << 16, mask)
-  // listed entries of T: F << b, split, Ua, row of the list; by level, levels' sizes
-  __shared__ Key s_f[kPruneSelf];
-  __shared__ uint32_t s_sp[kPruneSelf], s_start[kPB + 2];
-  __shared__ uint16_t s_u[kPruneSelf];
-  __shared__ uint8_t s_k[kPruneSelf], s_order[kPruneSelf];
-  __shared__ uint32_t s_last;
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-  const uint32_t tiles = gridDim.x / items, tile = blockIdx.x % tiles, item = blockIdx.x / tiles;
+  PrunedShared<Key>& sh = *reinterpret_cast<PrunedShared<Key>*>(psm + C::kSharedAt);
+  auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + group), "n"(NT) : "memory"); };  // of this group
+  // The warps of one sub-partition (number mod 4) get row groups of every kind:
+  // those of the groups rotated, or of a group of eight warps mirrored.
+  auto rows_of = [&](uint32_t w) { return kWarps == 4 ? (w + group) & 3u : (w < 4 ? w : 11u - w); };
+  auto warp_of = [&](uint32_t rg) { return kWarps == 4 ? (rg - group) & 3u : (rg < 4 ? rg : 11u - rg); };
+  const uint32_t s1 = lane | (rows_of(warp) << 5);
+  auto key_at = [&](uint32_t U) -> Key& { return skey[U + (U >> kRB)]; };
+  auto seq_at = [&](uint32_t U) -> uint16_t& {  // in the column of the thread that has the row
+    const uint32_t r = U >> kRB;
+    return seq[(U & (kRow - 1)) * C::kSeqStride + ((r & 31u) | (warp_of(r >> 5) << 5))];
+  };
+  const uint32_t tiles = (uint32_t)c_binom.v[L][kh];
+
+  // One unit: a tile, or one of `items` parts of it.  Every thread of the
+  // group takes the same way out.
+  auto run = [&](uint32_t unit) {
+  const uint32_t tile = unit % tiles, item = unit / tiles;
   const uint32_t T = colex_unrank((unsigned long long)tile, kh, L);
   if (MPT_BAD(flags, T < (1u << L) && __popc(T) == kh)) return;
   const uint32_t iT = info[T];
@@ -390,15 +408,6 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   const uint32_t cT = (iT >> kMembersShift) & 0x1FFFu;
   const int l = __ffs(T) - 1;
   const uint32_t low = 1u << l, rest = T ^ low;
-  // (the blocks of one SM differ by a multiple of 4, hence the hash)
-  const uint32_t rot = (blockIdx.x * 2654435761u) >> (32 - C::kLogWarps);
-  const uint32_t s1 = lane | (((warp + rot) & (kWarps - 1)) << 5);
-  auto key_at = [&](uint32_t U) -> Key& { return skey[U + (U >> kRB)]; };
-  auto seq_at = [&](uint32_t U) -> uint16_t& {  // in the column of the thread that has the row
-    const uint32_t r = U >> kRB;
-    return seq[(U & (kRow - 1)) * C::kSeqStride + ((r & 31u) | ((((r >> 5) + kWarps - rot) & (kWarps - 1)) << 5))];
-  };
-
   Key bk[kRow];
 #pragma unroll
   for (int i = 0; i < kRow; ++i) {
@@ -437,7 +446,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     for (int j = 0; j < kHeld; ++j) {
       const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
       if (r < n && r < (uint32_t)kPruneRows) {
-        if (col == 0) s_rows[s][r] = make_uint2(held[j].x | (n << 16), held[j].y);
+        if (col == 0) sh.rows[s][r] = make_uint2(held[j].x | (n << 16), held[j].y);
         pcopy16(slot + (NT + r) * kRowBytes + col, x + held[j].x * kRowBytes + col);
       }
     }
@@ -467,23 +476,23 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       for (int k = 0; k < kScan; ++k) n += candidate(base + (uint32_t)(k * NT)) != 0;
     }
     n = __reduce_add_sync(0xFFFFFFFFu, n);
-    if (lane == 0) warp_n[warp] = n;
-    __syncthreads();
+    if (lane == 0) sh.warp_n[warp] = n;
+    sync();
     n = 0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) n += warp_n[w];
+    for (int w = 0; w < kWarps; ++w) n += sh.warp_n[w];
     parts = min(items, max(1u, n / (uint32_t)kPruneMinPairs));
     if (item >= parts) return;
-    __syncthreads();
+    sync();
   }
 
   // Keys and Ta's of the round to shared memory; from here thread tid has the
   // outputs tid, tid + NT, ..
   auto dump = [&]() {
-    __syncthreads();
+    sync();
 #pragma unroll
     for (int i = 0; i < kRow; ++i) skey[s1 * (kRow + 1) + i] = bk[i];
-    __syncthreads();
+    sync();
   };
   unsigned long long* pt = partial + ((size_t)tile << kPB);
   uint32_t* pt_ta = partial_ta + ((size_t)tile << kPB);  // 64-bit keys
@@ -516,7 +525,11 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         any = any || ((Ta & ~T) == 0 && Ta != T);
       }
     }
-    met = __syncthreads_or(any) || met || long_tile;
+    if (tid == 0) sh.any = 0;
+    sync();
+    if (any) sh.any = 1;
+    sync();
+    met = sh.any != 0 || met || long_tile;
   }
   // phase 0: the pairs; phase 1: the self pair, Ta = T over the tile's own
   // members, B = (0, U \ Ua) in tile 0
@@ -532,14 +545,14 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           bal[k] = __ballot_sync(0xFFFFFFFFu, Ta[k] != 0);
           mine += (uint32_t)__popc(bal[k]);
         }
-        __syncthreads();
-        if (lane == 0) warp_n[warp] = mine;
-        __syncthreads();
+        sync();
+        if (lane == 0) sh.warp_n[warp] = mine;
+        sync();
         uint32_t at = found, sum = 0;
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
-          at += (uint32_t)w < warp ? warp_n[w] : 0u;
-          sum += warp_n[w];
+          at += (uint32_t)w < warp ? sh.warp_n[w] : 0u;
+          sum += sh.warp_n[w];
         }
         // this block's pairs are the found ones numbered item, item + parts, ..
         const uint32_t q0 = (found + parts - 1 - item) / parts, q1 = (found + sum + parts - 1 - item) / parts;
@@ -553,7 +566,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         found += sum;
         qn += q1 - q0;
       }
-      __syncthreads();
+      sync();
       // the first kSlots - 1 pairs; a group is committed for each slot, also
       // without a pair, so that the waits below can count them
 #pragma unroll
@@ -573,7 +586,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       stage_window(psm, Gc);
       asm volatile("cp.async.commit_group;" ::: "memory");
       const uint32_t n = iT & kRowsMask;  // at most kPruneRows
-      if (tid <= (uint32_t)kPB + 1) s_start[tid] = 0;
+      if (tid <= (uint32_t)kPB + 1) sh.start[tid] = 0;
       if (warp == 0) {
         static_assert(kPruneRows <= 32, "one list row per lane");
         const uint2 own = lane < n ? rows[(size_t)T * C::kKept + lane] : make_uint2(0u, 0u);
@@ -582,27 +595,27 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           const uint2 e = make_uint2(__shfl_sync(0xFFFFFFFFu, own.x, k), __shfl_sync(0xFFFFFFFFu, own.y, k));
           if (e.y >> lane & 1u) {
             const uint32_t i = at + __popc(e.y & ((1u << lane) - 1u));
-            s_u[i] = (uint16_t)((e.x << kRB) | lane);
-            s_k[i] = (uint8_t)k;
+            sh.u[i] = (uint16_t)((e.x << kRB) | lane);
+            sh.k[i] = (uint8_t)k;
           }
-          if (lane == 0) s_rows[0][k] = make_uint2(e.x | (n << 16), e.y);
+          if (lane == 0) sh.rows[0][k] = make_uint2(e.x | (n << 16), e.y);
           at += __popc(e.y);
         }
       }
-      __syncthreads();
+      sync();
       static_assert(kPruneSelf <= NT, "one thread per listed entry");
       const bool mine = tid < cT;
-      const uint32_t u = mine ? s_u[tid] : 0u;
+      const uint32_t u = mine ? sh.u[tid] : 0u;
       const uint32_t level = mine ? (uint32_t)__popc(u) : 32u;
       const Key w = mine ? (Key)wIr[((size_t)T << kPB) | u] : (Key)0;
       uint32_t rank = 0;
       for (uint32_t j = 0; j < cT; ++j) {
-        const uint32_t lj = (uint32_t)__popc(s_u[j]);
+        const uint32_t lj = (uint32_t)__popc(sh.u[j]);
         rank += lj < level || (lj == level && j < tid);
       }
       if (mine) {
-        s_order[rank] = (uint8_t)tid;
-        atomicAdd(&s_start[level + 1], 1u);
+        sh.order[rank] = (uint8_t)tid;
+        atomicAdd(&sh.start[level + 1], 1u);
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       Key best = mine && kh >= 2 ? key_at(u) : kNone;
@@ -615,16 +628,16 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
             f = (best >> kPB) - w;
             A = (((uint32_t)(best & kPMask) + perm.nat(u) - kPMask) << L) | ta;
           }
-          s_f[tid] = f << kPB;
-          s_sp[tid] = A;
-          *reinterpret_cast<Key*>(psm + (NT + s_k[tid]) * kRowBytes + (u & (kRow - 1)) * sizeof(Key)) = f << kPB;
+          sh.f[tid] = f << kPB;
+          sh.sp[tid] = A;
+          *reinterpret_cast<Key*>(psm + (NT + sh.k[tid]) * kRowBytes + (u & (kRow - 1)) * sizeof(Key)) = f << kPB;
         }
-        __syncthreads();
-        for (const uint32_t end = k + s_start[lv + 1]; k < end; ++k) {
-          const uint32_t j = s_order[k], uj = s_u[j], v = u ^ uj;
+        sync();
+        for (const uint32_t end = k + sh.start[lv + 1]; k < end; ++k) {
+          const uint32_t j = sh.order[k], uj = sh.u[j], v = u ^ uj;
           if (mine && level > lv && (uj & ~u) == 0) {
             const uint32_t r = v >> kRB, off = (v & (kRow - 1)) * (uint32_t)sizeof(Key);
-            const Key c = s_f[j] + *reinterpret_cast<const Key*>(psm + r * kRowBytes + (off ^ ((r & 7u) * 16u)));
+            const Key c = sh.f[j] + *reinterpret_cast<const Key*>(psm + r * kRowBytes + (off ^ ((r & 7u) * 16u)));
             if (c < best) {  // equal: the smaller Ta stays
               best = c;
               ta = T;
@@ -637,7 +650,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       // pair p's copies have landed; behind the barrier every thread is done
       // with pair p - 1, whose slot takes the next pair to be copied
       asm volatile("cp.async.wait_group %0;" ::"n"(C::kSlots - 2) : "memory");
-      __syncthreads();
+      sync();
       if (phase == 0) {
         const uint32_t q = p + (uint32_t)(C::kSlots - 1);
         if (q < qn) stage(q, s == 0 ? C::kSlots - 1 : s - 1);
@@ -645,7 +658,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         if (q + 1 < qn) hold(q + 1);
       }
       const char* slot = psm + s * C::kSlotBytes;
-      const uint2* list = s_rows[s];
+      const uint2* list = sh.rows[s];
       const uint32_t n = list[0].x >> 16;
       Key acc[kRow];
 #pragma unroll
@@ -690,7 +703,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         to_partial();
         if (base < total) {  // a further round
           met = true;
-          __syncthreads();
+          sync();
 #pragma unroll
           for (int i = 0; i < kRow; ++i) {
             bk[i] = kNone;
@@ -700,22 +713,22 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         }
         if (long_tile) return;  // the row kernel goes on from there
         __threadfence();
-        __syncthreads();
+        sync();
         if (parts > 1) {
           if (tid == 0) {
             const uint32_t before = atomicAdd(&done[tile], 1u);
-            s_last = before == parts - 1;
-            if (s_last) done[tile] = 0;  // for the next layer
+            sh.last = before == parts - 1;
+            if (sh.last) done[tile] = 0;  // for the next layer
           }
-          __syncthreads();
-          if (!s_last) return;
+          sync();
+          if (!sh.last) return;
           __threadfence();
         }
         for (uint32_t U = tid; U <= kPMask; U += NT) {
           const unsigned long long v = __ldcg(&pt[U]);
           key_at(U) = (Key)(v >> 32);
         }
-        __syncthreads();
+        sync();
 #pragma unroll
         for (int i = 0; i < kRow; ++i) bk[i] = skey[s1 * (kRow + 1) + i];
       }
@@ -733,7 +746,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           }
         }
         met = true;
-        __syncthreads();
+        sync();
         if (base < total) {
 #pragma unroll
           for (int i = 0; i < kRow; ++i) {
@@ -744,7 +757,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
         }
         if (long_tile && long_lists) return;
         for (uint32_t U = tid; U <= kPMask; U += NT) key_at(U) = pt[U];
-        __syncthreads();
+        sync();
 #pragma unroll
         for (int i = 0; i < kRow; ++i) bk[i] = skey[s1 * (kRow + 1) + i];
       }
@@ -760,10 +773,10 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   // w(I(T, U)) = 0 outside the tile's list; the listed entries replace theirs
   if (cT != 0) {
     for (uint32_t i = tid; i < cT; i += NT) {
-      key_at(s_u[i]) = s_f[i];
-      seq_at(s_u[i]) = (uint16_t)(kListed | i);
+      key_at(sh.u[i]) = sh.f[i];
+      seq_at(sh.u[i]) = (uint16_t)(kListed | i);
     }
-    __syncthreads();
+    sync();
   }
   const size_t tbase = (size_t)T << kPB;
   const uint32_t nat_lo = perm.nat(tid);
@@ -773,7 +786,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     const uint32_t number = cT != 0 ? seq_at(U) : 0u;
     uint32_t A;
     if ((number & kListed) && number != kSelf) {
-      A = s_sp[number & ~kListed];
+      A = sh.sp[number & ~kListed];
     } else {
       A = (((uint32_t)(key & kPMask) + nat - kPMask) << L) | (number == kSelf ? T : ta_at(U));
       key &= ~(Key)kPMask;  // F << b
@@ -782,6 +795,17 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     Gp[tbase | U] = key;
     Gc[tbase | U] = key | (Key)(~nat & kPMask);
     split_rot[tbase | U] = A;
+  }
+  };
+  // the first unit of a group is its own number, the others come from *next
+  const uint32_t units = tiles * items, own = gridDim.x * (blockDim.x / NT);
+  for (uint32_t unit = blockIdx.x + gridDim.x * group; unit < units;) {
+    run(unit);
+    if (own >= units) break;
+    sync();  // every thread is done with the unit's shared memory
+    if (tid == 0) sh.unit = own + atomicAdd(next, 1u);
+    sync();
+    unit = sh.unit;
   }
 }
 
@@ -799,12 +823,19 @@ template <typename Key, typename Tab>
 cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, uint32_t items,
                   unsigned long long* partial, Key* Gp, Key* Gc, cudaStream_t stream, int* launches) {
   using C = PrunedCfg<Key>;
+  static_assert(sizeof(PrunedShared<Key>) <= 4096, "a group's shared values");
   auto k = k_dp_pruned<Key, Tab>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kGroupBytes * C::kGroups);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)(h_binom.v[s.L][kh] * items), C::kRows, C::kSmem, stream>>>(
-      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long, ws.prune_n, partial, ws.partial_ta, ws.prune_done, Gp, Gc,
-      ws.split_rot, ws.counters + 1);
+  // a block per SM, and in it as many groups as there are units for; 64-bit
+  // groups, whose eight warps are balanced by themselves, as blocks of one
+  // (m = 24, weights x 4096: 0.41 ms of tile stage, 0.44 with two to a block)
+  const unsigned long long units = h_binom.v[s.L][kh] * items, sms = (unsigned long long)sm_count();
+  const int groups = sizeof(Key) == 8 ? 1 : units >= sms * C::kGroups ? C::kGroups : (int)((units + sms - 1) / sms);
+  k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
+      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long,
+      ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc, ws.split_rot,
+      ws.counters + 1);
   ++*launches;
   return cudaGetLastError();
 }
@@ -812,7 +843,7 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
 }  // namespace
 
 cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
-  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, kPruneSplitTiles * 4, stream);
+  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, (kPruneSplitTiles + kMaxMembersL) * 4, stream);
   if (e != cudaSuccess) return e;
   auto* lean = reinterpret_cast<unsigned int*>(ws.fw_rot);
   auto* full = reinterpret_cast<unsigned long long*>(ws.wI_rot);

@@ -93,8 +93,9 @@ constexpr size_t kMaxSupports = 8192;
 //     j-th of N_T contributes 2^(L - 1 - e_j) (3/2)^(requests of N_T above it)
 //     over all choices of the others.
 // A pair whose list lies in N_U alone takes 3^|N_U| 2^(b - |N_U|) of the 3^b
-// splits of a full pair, at about a third of its rate.  The pruned form is
-// taken when the pairs' times so estimated are below 0.6 of the full
+// splits of a full pair, at about half its rate (26 requests of 40 passages:
+// 0.39 of a full pair's time at |N_U| = 8, where 2 (2/3)^4 = 0.395).  The pruned
+// form is taken when the pairs' times so estimated are below 0.7 of the full
 // recurrence's, or when there is no long list.  Leave-one-out requests (every
 // N_x all but one) stay with the full form.
 void prune_shape(mpt_ctx* c) {
@@ -119,15 +120,15 @@ void prune_shape(mpt_ctx* c) {
       above *= 1.5;
       above2 *= 2.0;
     }
-    // of a full pair's time: the inner splits, at a third of its rate
-    double inner = 3.0;
+    // of a full pair's time: the inner splits, at half its rate
+    double inner = 2.0;
     for (int u = __builtin_popcount(U); u < s.b; ++u) inner *= 2.0 / 3.0;
     time += here * (inner + 0.05 < 1.0 ? inner + 0.05 : 1.0);
   }
   for (int l = 0; l < s.L; ++l)
     s.prune_long = s.prune_long || members[l] > (double)mpt::kPruneSelf || rows[l] > (double)mpt::kPruneRows;
   s.prune_most = *std::max_element(tas, tas + s.L);
-  s.pruned = !s.prune_long || time < 0.6 * full;
+  s.pruned = !s.prune_long || time < 0.7 * full;
   if (!s.pruned) return;
   // Stored order of the inner bits: those of the N_x whose members cost most
   // (pairs times inner splits) first.  The first five are the in-row bits,
@@ -267,7 +268,7 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
     ws->prune_short = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_long = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_n = reinterpret_cast<uint32_t*>(take(2 * mpt::kMaxMembersL * 4));
-    ws->prune_done = reinterpret_cast<uint32_t*>(take(mpt::kPruneSplitTiles * 4));
+    ws->prune_done = reinterpret_cast<uint32_t*>(take((mpt::kPruneSplitTiles + mpt::kMaxMembersL) * 4));
   }
   return off;
 }

@@ -240,7 +240,7 @@ struct Workspace {
   uint32_t* prune_short;  // [2^L] Ta's with a short list, by lowest request
   uint32_t* prune_long;   // [2^L] Ta's with a long list, by lowest request
   uint32_t* prune_n;      // [2 * kMaxMembersL] their numbers per lowest request
-  uint32_t* prune_done;   // [kPruneSplitTiles] finished blocks of each tile of a layer
+  uint32_t* prune_done;   // [kPruneSplitTiles] finished parts of each tile of a layer; [kMaxMembersL] units taken per layer
   // layout
   unsigned long long* keys;  // [slots]
   int64_t* perm_offsets;     // [m + 1]
