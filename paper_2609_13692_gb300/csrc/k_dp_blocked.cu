@@ -789,11 +789,18 @@ constexpr unsigned long long kItemOverheadPairs = 2;
 // about kItemOverheadPairs pairs more (its first window copy and its final
 // merge).  The layer then takes ceil(blocks / SMs) waves of (pairs per item +
 // overhead); take the item count that minimises that, fewer blocks on ties.
-// Items keep at least kMinPairsPerItem pairs; at most max_items per tile.
+// Items keep at least kMinPairsPerItem pairs unless the layer is too short to
+// fill the SMs with those; at most max_items per tile.  Leave-one-out, m = 20
+// (8 tile layers of at most 70 tiles): pair stage 0.47 -> 0.28 ms.
 void choose_items(unsigned long long tiles, uint32_t P, int sms, unsigned long long max_items,
                   unsigned long long* items_out, uint32_t* ppi_out) {
   const unsigned long long waves_of = sms > 0 ? (unsigned long long)sms : 1ull;
   unsigned long long cap = (P + kMinPairsPerItem - 1) / kMinPairsPerItem;
+  // a layer with fewer blocks than that would leave SMs empty: shorter items,
+  // as many as two waves of blocks hold
+  unsigned long long spread = 2 * waves_of / tiles;
+  if (spread > P) spread = P;
+  if (cap < spread) cap = spread;
   if (cap > max_items) cap = max_items;
   if (cap < 1) cap = 1;
   if (cap > 8192) cap = 8192;
