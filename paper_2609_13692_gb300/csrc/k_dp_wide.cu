@@ -25,9 +25,9 @@
 // writes its 4096 bests to a slot of its own: no atomics in global memory.
 //
 // Tile kernel (|T| >= 1; tile 0 is k_dp_tile0.cu's).  One block per tile
-// finishes all 4096 entries level by level in |U|: the self pair
-// (A = (T, Ua), B = (0, U \ Ua)) by lanes per subset, then the lexicographic
-// (key, Ta) minimum with the tile's pair slots.
+// finishes all 4096 entries by rows of 16, level by level in the row bits: the
+// self pair (A = (T, Ua), B = (0, U \ Ua)) and the lexicographic (key, Ta)
+// minimum with the tile's pair slots.
 #include "mpt_internal.cuh"
 
 namespace mpt {
@@ -45,8 +45,9 @@ constexpr int kWWin = kWRows * kWRowStride;
 constexpr int kWThreads = 256;
 constexpr int kWOwned = (1 << kWB) / kWThreads;  // 16 outputs folded per thread
 constexpr int kWSmemBytes = (2 * 2 * kWWin + 2 * (1 << kWB)) * (int)sizeof(u64);
-constexpr int kWTileThreads = 512;
-constexpr int kWTileSmemBytes = 2 * (1 << kWB) * (int)sizeof(u64) + (1 << kWB) * (int)sizeof(uint16_t);
+constexpr int kWTileThreads = 288;
+constexpr int kWBestWords = (1 << kWB) + kWRows;  // per-output arrays, rows 17 words apart
+constexpr int kWTileSmemBytes = (2 * kWWin + kWBestWords) * (int)sizeof(u64) + kWBestWords * (int)sizeof(uint32_t);
 constexpr int kWChunks = 1645;
 constexpr int kWLong = 109;               // threads with 7 chunks; the others take 6
 
@@ -131,36 +132,6 @@ constexpr WidePlan make_wide_plan() {
 constexpr WidePlan kWidePlanHost = make_wide_plan();
 static_assert(kWidePlanHost.nchunk == kWChunks && kWidePlanHost.total == kWChunks, "chunk plan");
 static __constant__ WidePlan c_wplan = make_wide_plan();
-
-// The 4096 subsets of 12 inner bits sorted by size, then colex rank: the order
-// in which the tile kernel finishes them.  The same for every tile, so it is
-// a static table (global memory, read with coalesced loads) rather than being
-// recomputed per block from the binomial table, whose per-thread indices the
-// constant cache would serve one by one.
-struct OrderTable {
-  uint16_t v[1 << kWB];
-};
-
-constexpr OrderTable make_order12() {
-  OrderTable t{};
-  uint32_t start[kWB + 2] = {};
-  for (int p = 0; p <= kWB; ++p) start[p + 1] = start[p] + (uint32_t)h_binom.v[kWB][p];
-  for (uint32_t u = 0; u < (1u << kWB); ++u) {
-    uint32_t r = 0, s = u;
-    int k = 1;
-    while (s) {
-      int pos = 0;
-      while (!((s >> pos) & 1u)) ++pos;
-      r += (uint32_t)h_binom.v[pos][k];
-      ++k;
-      s &= s - 1;
-    }
-    t.v[start[popc8(u)] + r] = (uint16_t)u;
-  }
-  return t;
-}
-
-static __device__ const OrderTable g_order12 = make_order12();
 
 // Row placement: the low 3 row bits XOR-ed with higher ones; linear over GF(2).
 __device__ __forceinline__ uint32_t row_pos_w(uint32_t r) { return r ^ (((r >> 3) ^ (r >> 6)) & 7u); }
@@ -349,118 +320,214 @@ __device__ __forceinline__ int64_t load_wI_w(const Tab* p) {
   return (int64_t)__ldg(p);
 }
 
-// Tile kernel (any |T| = kh, any b <= 12): finishes the tile's 2^b entries.
+// Folds a tile's `items` slots into its first one: the lexicographic
+// (key, Ta) minimum of each output.  A block takes 32 outputs with 8 warps
+// that share the slots; it reads and writes only its own outputs.
+__global__ void __launch_bounds__(256)
+k_fold_slots_w(u64* __restrict__ pkey, uint32_t* __restrict__ pta, uint32_t items) {
+  __shared__ u64 sk[8][32];
+  __shared__ uint32_t st[8][32];
+  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+  const size_t first = ((size_t)(blockIdx.x >> (kWB - 5)) * items << kWB) | ((blockIdx.x & ((1u << (kWB - 5)) - 1u)) << 5) | lane;
+  u64 best = ~0ull;
+  uint32_t ta = ~0u;
+#pragma unroll 4
+  for (uint32_t it = w; it < items; it += 8) {
+    const u64 k = pkey[first + ((size_t)it << kWB)];
+    const uint32_t t = pta[first + ((size_t)it << kWB)];
+    if (k < best || (k == best && t < ta)) {
+      best = k;
+      ta = t;
+    }
+  }
+  sk[w][lane] = best;
+  st[w][lane] = ta;
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int i = 1; i < 8; ++i) {
+      const u64 k = sk[i][lane];
+      const uint32_t t = st[i][lane];
+      if (k < best || (k == best && t < ta)) {
+        best = k;
+        ta = t;
+      }
+    }
+    pkey[first] = best;
+    pta[first] = ta;
+  }
+}
+
+// Word of output U = (s1, s2) in a per-output array: rows are 17 words apart,
+// so threads that hold different rows and the same s2 hit different banks.
+__device__ __forceinline__ uint32_t best_word_w(uint32_t U) { return U + (U >> kWB2); }
+
+// Tile kernel, |T| = kh >= 1, 12 inner bits: the tile's rows of 16 level by
+// level in |s1|, as k_dp_tile_rows does with 32-bit keys.  Candidates of
+// U = (s1, s2) with Ua = (a1, a2), a proper subset of U:
+//   * a1 a proper subset of s1: rows of this tile finished at earlier levels
+//     against whole rows of tile 0, by the pair kernel's register convolution;
+//   * a1 = s1: a 4-bit recurrence inside the row, in registers.
+// Layers are short where this kernel matters (the pair kernel's work grows
+// with 2^|T|, this one's does not), so a tile gets a block of 9 warps, which
+// bound its chain: at the widest level 70 rows by 4 lanes.  A lane per few
+// submasks with two dependent shared loads each, and a block barrier per size
+// of U, took 565 us for one tile (m = 13); this form takes 75 us.
 template <typename Tab>
 __global__ void __launch_bounds__(kWTileThreads)
-k_dp_tile_w(int L, int b, int kh, const Tab* __restrict__ wIr, const u64* __restrict__ pkey,
-            const uint32_t* __restrict__ pta, uint32_t items, u64* __restrict__ Gp, u64* __restrict__ Gc,
-            uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags, const uint32_t* __restrict__ info, InnerPerm perm) {
+k_dp_tile_w(int L, int kh, const Tab* __restrict__ wIr, const u64* __restrict__ pkey, const uint32_t* __restrict__ pta,
+            uint32_t items, uint32_t stride, u64* __restrict__ Gp, u64* __restrict__ Gc, uint32_t* __restrict__ split_rot,
+            int32_t* __restrict__ flags, const uint32_t* __restrict__ info, InnerPerm perm) {
   extern __shared__ __align__(16) u64 tsm[];
-  u64* cur = tsm;                       // this tile, F << b
-  u64* oc = tsm + (1 << kWB);           // complement form of tile 0
-  uint16_t* order = reinterpret_cast<uint16_t*>(tsm + 2 * (1 << kWB));  // subsets by size, then colex
+  u64* cur = tsm;              // this tile, F << 12, padded rows
+  u64* zc = cur + kWWin;       // tile 0, complement form, padded rows
+  u64* bkey = zc + kWWin;      // best key per output so far
+  uint32_t* bsplit = reinterpret_cast<uint32_t*>(bkey + kWBestWords);  // its Ta; after finishing, the split A
+  constexpr uint32_t kMask = (1u << kWB) - 1u;
 
   const uint32_t tile = blockIdx.x;
   const uint32_t T = colex_unrank(tile, kh, L);
+  const size_t tbase = (size_t)T << kWB;
+  if (MPT_BAD(flags, tile < c_binom.v[L][kh] && T < (1u << L) && __popc(T) == kh)) return;
   if (info && !(info[T] & kTileLong)) return;  // finished by k_dp_pruned
-  const int size = 1 << b;
-  const uint32_t mask = (uint32_t)size - 1u;
 
-  for (int u = threadIdx.x; u < size; u += kWTileThreads) {
-    order[u] = g_order12.v[u];
-    oc[u] = Gc[u];
+  for (int c = threadIdx.x; c < (1 << (kWB - 1)); c += kWTileThreads) {
+    const int row = c >> (kWB2 - 1), k = c & ((1 << (kWB2 - 1)) - 1);
+    *reinterpret_cast<ulonglong2*>(zc + row_pos_w((uint32_t)row) * kWRowStride + 2 * k) =
+        *reinterpret_cast<const ulonglong2*>(Gc + 2 * c);
   }
-  __syncthreads();
-
-  uint32_t start = 0;
-  for (int p = 0; p <= b; ++p) {
-    const int cnt = (int)c_binom.v[b][p];
-    const int g = p > 3 ? min(p - 3, 5) : 0;  // log2(lanes per output)
-    const int G = 1 << g;
-    const int groups = kWTileThreads >> g;
-    for (int base = 0; base < cnt; base += groups) {
-      const int gi = base + (int)(threadIdx.x >> g);
-      const uint32_t r = threadIdx.x & (uint32_t)(G - 1);
-      const bool active = gi < cnt;
-      u64 best = ~0ull;
-      uint32_t U = 0;
-      bool single = false;
-      if (active) {
-        U = order[start + gi];
-        const uint32_t nreq = (uint32_t)p + (uint32_t)kh;
-        single = nreq == 1;
-        if (nreq >= 2 && U != 0) {
-          // Ua: a proper subset of U (Ta = T)
-          const uint32_t emask = U;
-          uint32_t hi = 0, rr = emask;
-          for (int t = 0; t < g; ++t) {
-            const uint32_t top = 1u << (31 - __clz(rr));
-            hi |= top;
-            rr ^= top;
-          }
-          const uint32_t freem = emask ^ hi;
-          const uint32_t fixed = deposit_bits(r, hi);
-          uint32_t s = 0;
-          do {
-            const uint32_t part = fixed | s;
-            if (part != emask) {
-              const uint32_t Ua = part;
-              const u64 key = cur[Ua] + oc[U ^ Ua];
-              best = key < best ? key : best;
-            }
-            s = (s - freem) & freem;
-          } while (s != 0);
-        }
-      }
-      // the self pair's candidates carry Ta = T; the pair
-      // kernel's slots of this tile, one per block, are spread over the G
-      // lanes of the output; then the lexicographic (key, Ta) minimum of the
-      // group, in which the self pair wins ties only against larger Ta
-      uint32_t ta = T;
-      if (active && kh >= 2) {
-        for (uint32_t it = r; it < items; it += (uint32_t)G) {
-          const size_t w = ((size_t)(tile * items + it) << b) | U;
-          const u64 k2 = pkey[w];
-          const uint32_t t2 = pta[w];
-          if (k2 < best || (k2 == best && t2 < ta)) {
-            best = k2;
-            ta = t2;
-          }
-        }
-      }
-      for (int off = G >> 1; off > 0; off >>= 1) {
-        const u64 o = __shfl_xor_sync(0xFFFFFFFFu, best, off);
-        const uint32_t ot = __shfl_xor_sync(0xFFFFFFFFu, ta, off);
-        if (o < best || (o == best && ot < ta)) {
-          best = o;
-          ta = ot;
-        }
-      }
-      if (active && r == 0) {
-        const size_t idx = ((size_t)T << b) | U;
-        int64_t f;
-        uint32_t A;
-        const uint32_t nat = info ? perm.nat(U) : U;  // stored order undone (pruned recurrence)
-        if (single) {
-          f = load_wI_w(wIr + idx);
-          A = 0;
-        } else {
-          const uint32_t Ua = (uint32_t)(best & mask) + nat - mask;
-          f = (int64_t)(best >> b) - load_wI_w(wIr + idx);
-          A = (Ua << L) | ta;
-        }
-        const u64 gp = (u64)f << b;
-        const u64 gc = gp | (u64)(~nat & mask);
-        cur[U] = gp;
-        if (!MPT_BAD(flags, idx < ((size_t)1 << (L + b)) && valid_split(T | (nat << L), A))) {
-          Gp[idx] = gp;
-          Gc[idx] = gc;
-          split_rot[idx] = A;
+  for (int u = threadIdx.x; u < (1 << kWB); u += kWTileThreads) {
+    u64 best = ~0ull;
+    uint32_t ta = T;
+    if (kh >= 2) {
+      const size_t slot = ((size_t)tile * stride << kWB) | (uint32_t)u;
+      best = pkey[slot];
+      ta = pta[slot];
+      for (uint32_t it = 1; it < items; ++it) {
+        const u64 k = pkey[slot + ((size_t)it << kWB)];
+        const uint32_t t = pta[slot + ((size_t)it << kWB)];
+        if (k < best || (k == best && t < ta)) {
+          best = k;
+          ta = t;
         }
       }
     }
-    start += (uint32_t)cnt;
+    bkey[best_word_w((uint32_t)u)] = best;
+    bsplit[best_word_w((uint32_t)u)] = ta;
+  }
+  __syncthreads();
+
+  for (int p1 = 0; p1 <= kWB1; ++p1) {
+    const int rows = (int)c_binom.v[kWB1][p1];
+    // the threads that finish this level's rows fetch their w(I(S)) now
+    int64_t wv[kWRow];
+    const bool finisher = (int)threadIdx.x < rows;
+    const uint32_t s1f = finisher ? colex_unrank((unsigned long long)threadIdx.x, p1, kWB1) : 0u;
+    if (finisher) {
+#pragma unroll
+      for (int i = 0; i < kWRow; ++i) wv[i] = load_wI_w(wIr + (tbase | (s1f << kWB2) | (uint32_t)i));
+    }
+    if (p1 >= 1) {
+      int g = p1 < 5 ? p1 : 5;  // log2(lanes per row)
+      while ((rows << g) > kWTileThreads) --g;
+      const int G = 1 << g;
+      const int ri = (int)(threadIdx.x >> g);
+      const uint32_t r = threadIdx.x & (uint32_t)(G - 1);
+      const bool active = ri < rows;
+      u64 acc[kWRow];
+#pragma unroll
+      for (int i = 0; i < kWRow; ++i) acc[i] = ~0ull;
+      uint32_t s1 = 0;
+      if (active) {
+        s1 = colex_unrank((unsigned long long)ri, p1, kWB1);
+        uint32_t hi = 0, rr = s1;
+        for (int t = 0; t < g; ++t) {
+          const uint32_t top = 1u << (31 - __clz(rr));
+          hi |= top;
+          rr ^= top;
+        }
+        const uint32_t freem = s1 ^ hi;
+        const uint32_t fixed = deposit_bits(r, hi);
+        uint32_t sub = 0;
+        do {
+          const uint32_t a1 = fixed | sub;
+          if (a1 != s1) {
+            u64 x[kWRow], y[kWRow];
+            load_row_w(x, cur + row_pos_w(a1) * kWRowStride);
+            load_row_w(y, zc + row_pos_w(s1 ^ a1) * kWRowStride);
+            conv16(acc, x, y);
+          }
+          sub = (sub - freem) & freem;
+        } while (sub != 0);
+      }
+      for (int off = G >> 1; off > 0; off >>= 1) {
+#pragma unroll
+        for (int i = 0; i < kWRow; ++i) {
+          const u64 o = __shfl_xor_sync(0xFFFFFFFFu, acc[i], off);
+          acc[i] = o < acc[i] ? o : acc[i];
+        }
+      }
+      if (active && r == 0) {
+#pragma unroll
+        for (int i = 0; i < kWRow; ++i) {
+          const uint32_t o = best_word_w((s1 << kWB2) | (uint32_t)i);
+          if (acc[i] < bkey[o]) {
+            bkey[o] = acc[i];
+            bsplit[o] = T;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (finisher) {
+      const uint32_t nat_s1 = info ? perm.nat(s1f << kWB2) : s1f << kWB2;  // stored order undone (pruned recurrence)
+      u64 z[kWRow], c[kWRow];
+      load_row_w(z, zc);  // row 0 is at position 0
+#pragma unroll
+      for (int s2 = 0; s2 < kWRow; ++s2) {
+        u64 key = ~0ull;
+#pragma unroll
+        for (int a2 = 0; a2 < kWRow; ++a2) {
+          if ((a2 & s2) == a2 && a2 != s2) {
+            const u64 k = c[a2] + z[s2 ^ a2];
+            key = k < key ? k : key;
+          }
+        }
+        const uint32_t U = (s1f << kWB2) | (uint32_t)s2;
+        u64 bk = bkey[best_word_w(U)];
+        uint32_t bt = bsplit[best_word_w(U)];
+        if (key < bk) {  // ties keep the smaller Ta, a proper part of T
+          bk = key;
+          bt = T;
+        }
+        int64_t f;
+        uint32_t A;
+        if (kh == 1 && U == 0) {  // S = T, a single request
+          f = wv[s2];
+          A = 0;
+        } else {
+          const uint32_t Ua = (uint32_t)(bk & kMask) + (nat_s1 | (info ? perm.nat((uint32_t)s2) : (uint32_t)s2)) - kMask;
+          f = (int64_t)(bk >> kWB) - wv[s2];
+          A = (Ua << L) | bt;
+        }
+        c[s2] = (u64)f << kWB;
+        bsplit[best_word_w(U)] = A;
+      }
+      ulonglong2* dst = reinterpret_cast<ulonglong2*>(cur + row_pos_w(s1f) * kWRowStride);
+#pragma unroll
+      for (int q = 0; q < kWRow / 2; ++q) dst[q] = make_ulonglong2(c[2 * q], c[2 * q + 1]);
+    }
     __syncthreads();
+  }
+
+  for (int u = threadIdx.x; u < (1 << kWB); u += kWTileThreads) {
+    const u64 gp = cur[row_pos_w((uint32_t)u >> kWB2) * kWRowStride + (u & (kWRow - 1))];
+    const uint32_t A = bsplit[best_word_w((uint32_t)u)];
+    const uint32_t nat = info ? perm.nat((uint32_t)u) : (uint32_t)u;
+    if (MPT_BAD(flags, valid_split(T | (nat << L), A))) continue;
+    Gp[tbase | (uint32_t)u] = gp;
+    Gc[tbase | (uint32_t)u] = gp | (u64)(~nat & kMask);
+    split_rot[tbase | (uint32_t)u] = A;
   }
 }
 
@@ -476,19 +543,31 @@ int64_t wide_partial_slots(int m, int b) {
 
 namespace {
 
+// More slots of a tile than this are folded by a kernel of their own: one
+// block reading the 304 slots of the last tile would take as long as the tile.
+constexpr uint32_t kWInlineSlots = 4;
+
 // The tiles of step kh >= 1, with `items` slots each (info: the pruned
 // recurrence's lists, or null).
 void launch_wide_tiles(const Shape& s, const Workspace& ws, int kh, uint32_t items, const uint32_t* info,
-                       cudaStream_t stream) {
+                       cudaStream_t stream, int* launches) {
   const unsigned tiles = (unsigned)h_binom.v[s.L][kh];
+  uint32_t stride = items;
+  if (kh >= 2 && items > kWInlineSlots) {
+    k_fold_slots_w<<<tiles << (kWB - 5), 256, 0, stream>>>(ws.partial, ws.partial_ta, items);
+    ++*launches;
+    items = 1;
+  }
+  auto run = [&](auto kernel, const auto* wI) {
+    kernel<<<tiles, kWTileThreads, kWTileSmemBytes, stream>>>(s.L, kh, wI, ws.partial, ws.partial_ta, items, stride,
+                                                              ws.Gp64, ws.Gc64, ws.split_rot, ws.counters + 1, info,
+                                                              s.perm);
+    ++*launches;
+  };
   if (s.lean)
-    k_dp_tile_w<<<tiles, kWTileThreads, kWTileSmemBytes, stream>>>(s.L, s.b, kh, ws.fw_rot, ws.partial, ws.partial_ta,
-                                                                   items, ws.Gp64, ws.Gc64, ws.split_rot,
-                                                                   ws.counters + 1, info, s.perm);
+    run(k_dp_tile_w<int32_t>, ws.fw_rot);
   else
-    k_dp_tile_w<<<tiles, kWTileThreads, kWTileSmemBytes, stream>>>(s.L, s.b, kh, ws.wI_rot, ws.partial, ws.partial_ta,
-                                                                   items, ws.Gp64, ws.Gc64, ws.split_rot,
-                                                                   ws.counters + 1, info, s.perm);
+    run(k_dp_tile_w<int64_t>, ws.wI_rot);
 }
 
 cudaError_t wide_tile_attributes() {
@@ -503,8 +582,7 @@ cudaError_t wide_tile_attributes() {
 cudaError_t launch_wide_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
   const cudaError_t e = wide_tile_attributes();
   if (e != cudaSuccess) return e;
-  launch_wide_tiles(s, ws, kh, 1u, ws.prune_info, stream);
-  ++*launches;
+  launch_wide_tiles(s, ws, kh, 1u, ws.prune_info, stream, launches);
   return cudaGetLastError();
 }
 
@@ -541,14 +619,15 @@ cudaError_t launch_dp_wide(const Shape& s, const Workspace& ws, cudaStream_t str
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches], stream);
-    if (kh == 0)
+    if (kh == 0) {
       e = launch_tile0(s, ws, stream);
-    else
-      launch_wide_tiles(s, ws, kh, (uint32_t)items, nullptr, stream);
+      ++*launches;
+    } else {
+      launch_wide_tiles(s, ws, kh, (uint32_t)items, nullptr, stream, launches);
+    }
     if (e != cudaSuccess) return e;
     if (timing && timing->tile_ev) cudaEventRecord(timing->tile_ev[2 * timing->tile_launches + 1], stream);
     if (timing) timing->tile_launches++;
-    ++*launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -110,6 +110,13 @@ def _scaled_equal(mpt, inst, c):
     return narrow, wide
 
 
+@pytest.mark.parametrize("m", [14, 16, 20])
+def test_wide_slots_and_rows(mpt, m):
+    """Leave-one-out families, whose splits all tie: tiles with one slot
+    (m = 14), a few (m = 16), and up to 127 that are folded first (m = 20)."""
+    _scaled_equal(mpt, I.leave_one_out(m), 1 << 21)
+
+
 def test_wide_scaled_rag_m24(mpt):
     """The RAG-shaped m = 24 workload at 4096x its weights against the 32-bit path."""
     _scaled_equal(mpt, I.config(3), 4096)
