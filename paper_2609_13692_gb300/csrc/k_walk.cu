@@ -24,6 +24,9 @@ namespace {
 constexpr int kWalkThreads = 256;
 constexpr int kMaxM = 32;
 
+// One block, bound by its chains: the walk's splits, one dependent read per
+// level of the hierarchy instead of one per node (m = 28: 45 -> 27 us).
+// opt: OPT, then the eight counters as int32.
 __global__ void __launch_bounds__(kWalkThreads)
 k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F, const int32_t* __restrict__ F32,
        const uint32_t* __restrict__ Gp, const unsigned long long* __restrict__ Gp64,
@@ -32,81 +35,104 @@ k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F,
        unsigned long long* __restrict__ keys, int64_t* __restrict__ perm_offsets, int64_t* __restrict__ perm_chunks,
        int32_t* __restrict__ dfs, int64_t* __restrict__ opt) {
   __shared__ uint32_t anc[kMaxM][kMaxM];  // anc[i][d]: the depth-d node on request i's path
+  __shared__ uint32_t nodes[2][kMaxM];    // a level's nodes, and where their leaves start in dfs order
+  __shared__ int starts[2][kMaxM];
   __shared__ int leaf_depth[kMaxM];
   __shared__ int cnt[kMaxM];
   __shared__ int fill[kMaxM];
   __shared__ long long offs[kMaxM + 1];
   __shared__ int bad;
 
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t full = (m >= 32) ? 0xFFFFFFFFu : ((1u << m) - 1u);
   if (tid < kMaxM) {
     cnt[tid] = 0;
     fill[tid] = 0;
     leaf_depth[tid] = 0;
   }
-  if (tid == 0) {
-    bad = 0;
-    const uint32_t full = (m >= 32) ? 0xFFFFFFFFu : ((1u << m) - 1u);
-    uint32_t stk[2 * kMaxM];
-    int stk_d[2 * kMaxM];
-    int sp = 0, nleaf = 0;
-    stk[sp] = full;
-    stk_d[sp] = 0;
-    ++sp;
-    while (sp > 0 && !bad) {
-      --sp;
-      const uint32_t S = stk[sp];
-      const int d = stk_d[sp];
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  if (warp == 0) {
+    // level by level, a lane per node: a level's nodes are disjoint, so there
+    // are at most m of them, and those at a level are looked up together
+    if (lane == 0) {
+      nodes[0][0] = full;
+      starts[0][0] = 0;
+    }
+    int live = 1;
+    bool wrong = false;
+    for (int d = 0; live > 0; ++d) {
+      __syncwarp();
+      const bool has = lane < live;
+      const uint32_t S = has ? nodes[d & 1][lane] : 0u;
+      const int at = has ? starts[d & 1][lane] : 0;
+      const bool inner = (S & (S - 1)) != 0;
       for (uint32_t r = S; r; r &= r - 1) anc[__ffs(r) - 1][d] = S;
-      if ((S & (S - 1)) == 0) {
+      if (has && !inner) {
         const int i = __ffs(S) - 1;
         leaf_depth[i] = d;
-        dfs[nleaf++] = i;
-        continue;
+        dfs[at] = i;
       }
       // blocked path: split and F (as F << b in Gp) in rotated order
-      const uint32_t A = (Gp || Gp64) ? split[rot_index(S, L, b, perm)] : split[S];
-      if (A == 0 || (A & ~S) != 0 || A == S || sp + 2 > 2 * kMaxM) {
-        bad = 1;
-        break;
+      uint32_t A = 0;
+      if (inner) A = (Gp || Gp64) ? split[rot_index(S, L, b, perm)] : split[S];
+      wrong = __any_sync(0xFFFFFFFFu, inner && (A == 0 || (A & ~S) != 0 || A == S));
+      if (wrong) break;
+      const uint32_t inners = __ballot_sync(0xFFFFFFFFu, inner);
+      if (inner) {
+        const int to = 2 * __popc(inners & ((1u << lane) - 1u));
+        nodes[(d + 1) & 1][to] = A;
+        starts[(d + 1) & 1][to] = at;
+        nodes[(d + 1) & 1][to + 1] = S ^ A;  // right child, its leaves after the left subtree's
+        starts[(d + 1) & 1][to + 1] = at + __popc(A);
       }
-      stk[sp] = S ^ A;  // right child, visited after the left subtree
-      stk_d[sp] = d + 1;
-      ++sp;
-      stk[sp] = A;
-      stk_d[sp] = d + 1;
-      ++sp;
+      live = 2 * __popc(inners);
     }
-    if (bad) atomicOr(&counters[1], kErrBadSplit);
+    if (wrong && lane == 0) {
+      bad = 1;
+      atomicOr(&counters[1], kErrBadSplit);
+    }
+  } else if (warp == 1) {
     int64_t pi_all = 0;
     if (priv) {
-      for (int i = 0; i < m; ++i) pi_all += (int64_t)priv[i];
+      pi_all = lane < m ? (int64_t)priv[lane] : 0;
+      for (int off = 16; off > 0; off >>= 1) pi_all += __shfl_xor_sync(0xFFFFFFFFu, pi_all, off);
       pi_all += (int64_t)priv[kUniversalSlot];
     }
-    *opt = Gp64 ? (int64_t)(Gp64[rot_index(full, L, b, perm)] >> b) + pi_all
-           : Gp ? (int64_t)(Gp[rot_index(full, L, b, perm)] >> b) + pi_all
-                : (F ? F[full] : (int64_t)F32[full]);
+    if (lane == 0)
+      *opt = Gp64 ? (int64_t)(Gp64[rot_index(full, L, b, perm)] >> b) + pi_all
+             : Gp ? (int64_t)(Gp[rot_index(full, L, b, perm)] >> b) + pi_all
+                  : (F ? F[full] : (int64_t)F32[full]);
+  }
+  int used = counters[0];
+  if (used > slots) used = (int)slots;
+  if (warp >= 2)
+    for (int t = tid - 64; t < used; t += kWalkThreads - 64)
+      for (uint32_t r = used_N[t]; r; r &= r - 1) atomicAdd(&cnt[__ffs(r) - 1], 1);
+  __syncthreads();
+  if (warp == 0) {
+    const int own = lane < m ? cnt[lane] : 0;
+    long long acc = own;
+    for (int off = 1; off < 32; off <<= 1) {
+      const long long o = __shfl_up_sync(0xFFFFFFFFu, acc, off);
+      if (lane >= off) acc += o;
+    }
+    if (lane < m) {
+      offs[lane] = acc - own;
+      perm_offsets[lane] = acc - own;
+    }
+    if (lane == m - 1) {
+      offs[m] = acc;
+      perm_offsets[m] = acc;
+      if (acc != slots) atomicOr(&counters[1], kErrLayoutCount);
+    }
+    __syncwarp();
+    // the counters leave with the results, in one copy (they changed in this
+    // kernel, so they are read past L1)
+    if (lane < 8) reinterpret_cast<int32_t*>(opt)[2 + lane] = __ldcg(counters + lane);
   }
   __syncthreads();
   if (bad) return;
-
-  int used = counters[0];
-  if (used > slots) used = (int)slots;
-  for (int t = tid; t < used; t += kWalkThreads)
-    for (uint32_t r = used_N[t]; r; r &= r - 1) atomicAdd(&cnt[__ffs(r) - 1], 1);
-  __syncthreads();
-  if (tid == 0) {
-    long long acc = 0;
-    for (int i = 0; i < m; ++i) {
-      offs[i] = acc;
-      perm_offsets[i] = acc;
-      acc += cnt[i];
-    }
-    offs[m] = acc;
-    perm_offsets[m] = acc;
-    if (acc != slots) atomicOr(&counters[1], kErrLayoutCount);
-  }
-  __syncthreads();
 
   for (int t = tid; t < used; t += kWalkThreads) {
     const uint32_t N = used_N[t];
@@ -121,7 +147,6 @@ k_walk(int m, const uint32_t* __restrict__ split, const int64_t* __restrict__ F,
   }
   __syncthreads();
 
-  const int lane = tid & 31, warp = tid >> 5;
   for (int i = warp; i < m; i += kWalkThreads / 32) {
     const long long base = offs[i];
     const int len = cnt[i];

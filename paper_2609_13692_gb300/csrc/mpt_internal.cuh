@@ -246,7 +246,7 @@ struct Workspace {
   int64_t* perm_offsets;     // [m + 1]
   int64_t* perm_chunks;      // [slots]
   int32_t* dfs;              // [m]
-  int64_t* opt;              // [1]
+  int64_t* opt;              // [1], then the eight counters (int32)
 };
 
 // Order in which the blocked tables keep the inner bits U of a subset: bit j
@@ -363,6 +363,7 @@ int64_t wide_partial_slots(int m, int b);
 cudaError_t launch_dp_wide(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                            BlockedTiming* timing, int step_begin = 0, int step_end = -1);
 
+constexpr size_t kOptBytes = 8 + 8 * 4;  // OPT, and the counters beside it
 cudaError_t launch_walk(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches);
 
 // Natural-order tables from the blocked path's rotated ones (k_tables.cu):
