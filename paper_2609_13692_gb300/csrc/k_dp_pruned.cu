@@ -117,7 +117,7 @@ template <typename Key, typename G>
 __global__ void __launch_bounds__(256)
 k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N, const unsigned long long* __restrict__ w,
               G* __restrict__ wIr, uint32_t* __restrict__ info, uint2* __restrict__ rows,
-              const int32_t* __restrict__ counters) {
+              int32_t* __restrict__ counters) {
   using C = PrunedCfg<Key>;
   constexpr int kThreads = 256, kPer = 16 / (int)sizeof(G);
   __shared__ __align__(16) G s[1 << kPB];
@@ -194,6 +194,7 @@ k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N,
     if (tid == 0) {
       const bool many = nr > (uint32_t)kPruneRows;
       const bool is_long = sizeof(Key) == 4 && (many || (long_ok && nc > kLongSteps));
+      if (is_long && !long_ok) atomicOr(counters + 1, kErrWorkspace);  // against the host's bound
       info[T] = nr == 0 ? 0u
                         : nr | (nm << kMembersShift) | (is_long ? kListLong : 0u) |
                               (is_long || many || nm > (uint32_t)kPruneSelf ? kTileLong : 0u);
@@ -362,7 +363,7 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 template <typename Key, typename Tab>
 __global__ void __launch_bounds__(PrunedCfg<Key>::kRows * (sizeof(Key) == 4 ? PrunedCfg<Key>::kGroups : 1),
                                   sizeof(Key) == 4 ? 1 : 2)
-k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
+k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
             const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
             const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* partial_ta,
             uint32_t* __restrict__ done, uint32_t* __restrict__ next, Key* Gp,
@@ -402,7 +403,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
   const uint32_t iT = info[T];
   const bool long_tile = (iT & kTileLong) != 0;
   if (long_tile && kh == 1) {  // no pairs: the row kernel does it all
-    if (!long_lists && tid == 0) atomicOr(flags, kErrWorkspace);
+    if (!long_tiles && tid == 0) atomicOr(flags, kErrWorkspace);
     return;
   }
   const uint32_t cT = (iT >> kMembersShift) & 0x1FFFu;
@@ -529,8 +530,9 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
     sync();
     if (any) sh.any = 1;
     sync();
-    met = sh.any != 0 || met || long_tile;
+    met = met || sh.any != 0;
   }
+  if (sizeof(Key) == 4 && kh >= 2) met = met || long_tile;
   // phase 0: the pairs; phase 1: the self pair, Ta = T over the tile's own
   // members, B = (0, U \ Ua) in tile 0
   for (int phase = kh >= 2 ? 0 : 1; phase < 2;) {
@@ -755,7 +757,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
           }
           continue;
         }
-        if (long_tile && long_lists) return;
+        if (long_tile && long_tiles) return;
         for (uint32_t U = tid; U <= kPMask; U += NT) key_at(U) = pt[U];
         sync();
 #pragma unroll
@@ -763,7 +765,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_lists, InnerPerm perm, cons
       }
     }
     if (long_tile) {
-      // only with the pair and row kernels around (the host's bound)
+      // only with the row kernel around (the host's bound)
       if (tid == 0) atomicOr(flags, kErrWorkspace);
       return;
     }
@@ -813,7 +815,7 @@ template <typename Key, typename G>
 cudaError_t tables(const Shape& s, const Workspace& ws, G* wIr, cudaStream_t stream, int* launches) {
   const int64_t tiles = (int64_t)1 << s.L, most = sm_count() * 8 * 8;
   k_prune_tiles<Key><<<(unsigned)(tiles < most ? tiles : most), 256, 0, stream>>>(
-      s.L, s.prune_long, s.n_shared, ws.shared_N, ws.shared_w, wIr, ws.prune_info, ws.prune_rows, ws.counters);
+      s.L, s.prune_pairs, s.n_shared, ws.shared_N, ws.shared_w, wIr, ws.prune_info, ws.prune_rows, ws.counters);
   k_prune_members<<<(unsigned)s.L, 1024, 0, stream>>>(s.L, ws.prune_info, ws.prune_short, ws.prune_long, ws.prune_n);
   *launches += 2;
   return cudaGetLastError();
@@ -833,14 +835,55 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
   const unsigned long long units = h_binom.v[s.L][kh] * items, sms = (unsigned long long)sm_count();
   const int groups = sizeof(Key) == 8 ? 1 : units >= sms * C::kGroups ? C::kGroups : (int)((units + sms - 1) / sms);
   k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
-      s.L, kh, items, s.prune_long, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long,
+      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long,
       ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc, ws.split_rot,
       ws.counters + 1);
   ++*launches;
   return cudaGetLastError();
 }
 
+// The members of each single request's list by k_prune_tiles' rules: the
+// listed rows, members and cost of {l} bound those of every T that holds l.
+template <typename Key>
+void singles(int L, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs) {
+  using C = PrunedCfg<Key>;
+  *tiles = *pairs = false;
+  for (int l = 0; l < L && !(*tiles && (*pairs || sizeof(Key) == 8)); ++l) {
+    uint32_t row[C::kRows] = {1u};
+    for (size_t i = 0; i < n; ++i)
+      if (supports[i] >> l & 1u) {
+        const uint32_t v = perm.stored(supports[i] >> L);
+        row[v >> C::kRB] |= 1u << (v & (C::kRow - 1));
+      }
+    static constexpr uint32_t kWithout[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
+    for (int j = 0; j < C::kRB; ++j)
+      for (uint32_t& r : row) r |= r >> (1 << j) & kWithout[j];
+    for (uint32_t bit = 1; bit < (uint32_t)C::kRows; bit <<= 1)
+      for (uint32_t r = 0; r < (uint32_t)C::kRows; ++r)
+        if (!(r & bit)) row[r] |= row[r | bit];
+    uint32_t rows = 0, members = 0, cost = 0;
+    for (uint32_t r = 0; r < (uint32_t)C::kRows; ++r) {
+      if (row[r] == 0) continue;
+      uint32_t steps = 0;
+      for (uint32_t a = row[r]; a; a &= a - 1) steps += (uint32_t)C::kRow >> __builtin_popcount(__builtin_ctz(a));
+      ++rows;
+      members += (uint32_t)__builtin_popcount(row[r]);
+      cost += (steps + kUnitSteps) << (C::kLogWarps - __builtin_popcount(r >> 5));
+    }
+    const bool many = rows > (uint32_t)kPruneRows, is_long = sizeof(Key) == 4 && (many || cost > kLongSteps);
+    *pairs = *pairs || is_long;
+    *tiles = *tiles || is_long || many || members > (uint32_t)kPruneSelf;
+  }
+}
+
 }  // namespace
+
+void prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs) {
+  if (s.wide)
+    singles<unsigned long long>(s.L, perm, supports, n, tiles, pairs);
+  else
+    singles<uint32_t>(s.L, perm, supports, n, tiles, pairs);
+}
 
 cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
   cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, (kPruneSplitTiles + kMaxMembersL) * 4, stream);
@@ -883,7 +926,7 @@ cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t s
     const uint32_t items = pruned_items(s, kh);
     if (pruned_meet(s, kh, items))
       e = cudaMemsetAsync(ws.partial, 0xFF, (size_t)(h_binom.v[s.L][kh] << kPB) * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess && kh >= 2 && s.prune_long && !s.wide) {
+    if (e == cudaSuccess && kh >= 2 && s.prune_pairs) {
       if (timing) mark(timing->pair_ev, 2 * timing->pair_launches);
       e = launch_listed_pairs(s, ws, kh, stream, launches);
       if (timing) mark(timing->pair_ev, 2 * timing->pair_launches++ + 1);

@@ -283,7 +283,8 @@ struct Shape {
   bool pruned;      // one-shot solves run the pruned recurrence (k_dp_pruned.cu)
   int n_shared;       // chunks that some (two or more) but not all requests share
   double prune_most;  // the host's bound on the pairs of one tile
-  bool prune_long;  // some list may be long
+  bool prune_long;  // some list may be long, or some tile left to the row kernel
+  bool prune_pairs; // some list may be long (32-bit keys)
 };
 
 // Pruned recurrence (k_dp_pruned.cu): rows of a short list, members of a tile
@@ -337,6 +338,10 @@ int blocked_max_launches(const Shape& s);  // upper bound on pair + tile launche
 cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                               BlockedTiming* timing, int step_begin = 0, int step_end = -1);
 // The same over the members only (k_dp_pruned.cu): lists, then every step.
+// Whether the lists of the single tile requests, which hold those of all other
+// Ta's, leave any tile to the row kernel (*tiles) or any list to the pair
+// kernel (*pairs).
+void prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs);
 cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                              BlockedTiming* timing);
 // w(I) (instead of K2) and the lists; needs K1's list of shared chunks.

@@ -140,6 +140,19 @@ def test_route(mpt):
     assert p["launches_pairs"] == 3 and p["splits_pairs"] > 0
 
 
+@pytest.mark.parametrize("inner,launches", [(7, 0), (8, 0), (10, 5)])
+def test_kernels_for_long_lists(mpt, inner, launches):
+    """Three sets with the same inner requests: their bounds add up to long
+    lists, their lists are one of 128 members, of 256 members in 8 rows (the
+    row kernel alone), of 1,024 members in 32 rows (the pair kernel too)."""
+    top = _mask(*range(6, 6 + inner))
+    inst = _from_supports(18, [top | _mask(0), top | _mask(0, 1), top | _mask(0, 2), _mask(3, 17)], inner)
+    test_equals_the_full_recurrence(mpt, inst)
+    test_wide_equals_the_full_recurrence(mpt, inst)
+    r = mpt.solve(inst.weights, inst.bits, profile=True)
+    assert mpt.mpt_get_profile(r.ctx)["launches_pairs"] == launches
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2])
 def test_m24_equals_the_full_recurrence(mpt, seed):
     inst = I.config(3, seed=seed)
