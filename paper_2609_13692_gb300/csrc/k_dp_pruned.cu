@@ -100,11 +100,11 @@ struct PrunedShared {
 // w(I(T, .)) and the row list of every T, one block per tile at a time, from
 // the sets N_x of the chunks that some but not all requests share (N: stored
 // rotated index, w: weight; K1's list): w(I(S)) = sum of w over N containing
-// S.  Few tiles lie within any N_x, so most are a write of zeros, and the
-// others a superset sum over the 2^12 inner sets in shared memory: the table
-// is written once and never read, where the general transform (K2) reads and
-// writes it once per 8 to 12 request bits after a clear.
-// m = 28: 0.29 + 2.0 ms of clear and transform (HBM-bound) -> 0.29 ms (7.5 TB/s written).
+// S.  Few tiles lie within any N_x; they are a superset sum over the 2^12
+// inner sets in shared memory, and the others are left unwritten: their readers
+// know from info that they are 0.  The general transform (K2) reads and writes
+// the table once per 8 to 12 request bits after a clear.  m = 28: 0.29 + 2.0 ms
+// of clear and transform (HBM-bound) -> 0.06 ms (0.29 with the zeros written).
 // The row list: threads = rows, the mask of a row from its non-zero entries.
 // info: 0 when T has no member, else rows | members << kMembersShift |
 // kListLong (32-bit keys) when they are more than kPruneRows or, where the pair
@@ -141,7 +141,10 @@ k_prune_tiles(int L, bool long_ok, int n_shared, const uint32_t* __restrict__ N,
     }
     G* out = wIr + ((size_t)T << kPB);
     if (!clear) {
-      for (uint32_t v = tid; v < (1u << kPB) / kPer; v += kThreads) reinterpret_cast<uint4*>(out)[v] = make_uint4(0, 0, 0, 0);
+      // no member: 0 to every reader, which goes by info, but in tile 0 and
+      // beside a single request's listed entry
+      if (T == 0 || single)
+        for (uint32_t v = tid; v < (1u << kPB) / kPer; v += kThreads) reinterpret_cast<uint4*>(out)[v] = make_uint4(0, 0, 0, 0);
       if (tid == 0) {
         info[T] = single ? 1u | (1u << kMembersShift) : 0u;  // a single request is always listed
         if (single) rows[(size_t)T * C::kKept] = make_uint2(0u, 1u);

@@ -707,6 +707,7 @@ mpt_status mpt_solve_end(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes
   if ((st = run_back(c, c->shape, ws, reinterpret_cast<cudaStream_t>(stream_ptr), &launches, nullptr, &opt)) != MPT_OK) return st;
   c->ws = ws;
   c->solved_shape = c->shape;
+  c->solved_shape.pruned = false;  // staged solves run the full recurrence
   c->opt = opt;
   c->staged_next = -1;
   std::memset(&c->prof, 0, sizeof(c->prof));
@@ -742,10 +743,11 @@ mpt_status ensure_natural(mpt_ctx* c) {
   if (e == cudaSuccess && s.wide)
     e = mpt::unrotate_tables_wide(s, ws.split_rot, reinterpret_cast<uint32_t*>(ws.Gc64), ws.wI_rot,
                                   s.lean ? nullptr : ws.wI, ws.Gp64, s.lean ? nullptr : ws.F, s.lean ? ws.fw : nullptr,
-                                  ws.priv, c->conv_stream);
+                                  ws.priv, c->conv_stream, s.pruned ? ws.prune_info : nullptr);
   else if (e == cudaSuccess)
     e = mpt::unrotate_tables(s, ws.split_rot, ws.Gc, ws.wI_rot, s.lean ? nullptr : ws.wI, ws.Gp,
-                             s.lean ? nullptr : ws.F, s.lean ? ws.fw : nullptr, ws.priv, c->conv_stream);
+                             s.lean ? nullptr : ws.F, s.lean ? ws.fw : nullptr, ws.priv, c->conv_stream,
+                             s.pruned ? ws.prune_info : nullptr);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->conv_stream);
   if (e != cudaSuccess) st = cuda_fail(c, e, "natural-order tables");
   cudaSetDevice(prev);

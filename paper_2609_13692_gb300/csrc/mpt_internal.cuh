@@ -377,14 +377,16 @@ cudaError_t launch_walk(const Shape& s, const Workspace& ws, cudaStream_t stream
 // F32_nat[S] = (Gp[idx(S)] >> b) + sum_{i in S} pi_i + u (S non-empty).
 // priv (the kOffsetSlots offsets on the device) may be null: no offsets.  Null destinations are skipped; they run
 // in this order, so a destination may be the source of an earlier conversion.
+// info: the pruned recurrence's lists, or null (w(I) is written, and read, only
+// in tiles with a member).
 cudaError_t unrotate_tables(const Shape& s, const uint32_t* split_rot, uint32_t* split_nat, const int64_t* wI_rot,
                             int64_t* wI_nat, const uint32_t* Gp, int64_t* F_nat, int32_t* F32_nat,
-                            const unsigned long long* priv, cudaStream_t stream);
+                            const unsigned long long* priv, cudaStream_t stream, const uint32_t* info = nullptr);
 // The same for the wide path (F from the uint64 Gp table).
 cudaError_t unrotate_tables_wide(const Shape& s, const uint32_t* split_rot, uint32_t* split_nat,
                                  const int64_t* wI_rot, int64_t* wI_nat, const unsigned long long* Gp64,
                                  int64_t* F_nat, int32_t* F32_nat, const unsigned long long* priv,
-                                 cudaStream_t stream);
+                                 cudaStream_t stream, const uint32_t* info = nullptr);
 // eq. (1) for any number of strings by lexicographic sorting (k_sched.cu)
 mpt_status trie_cost_lex(const int64_t* weights, int64_t n_chunks, int64_t m, const int64_t* offsets,
                          const int64_t* chunks, cudaStream_t st, int64_t* cost);

@@ -153,6 +153,28 @@ def test_kernels_for_long_lists(mpt, inner, launches):
     assert mpt.mpt_get_profile(r.ctx)["launches_pairs"] == launches
 
 
+@pytest.mark.parametrize("m", [13, 16, 17, 20])
+@pytest.mark.parametrize("scale", [1, 1 << 21])
+def test_tables_from_a_used_workspace(mpt, m, scale):
+    """w(I) is written only in tiles with a member: what lay in the workspace
+    before must not show in the tables, at one, 16 and 32 tile parts or more."""
+    inst = I.rag_pools(m, 3000, 5, 40, 8, 1.1, seed=m)
+    w = inst.weights * scale
+    ref = mpt.solve(w, inst.bits, mode="blocked" if scale == 1 else "wide")
+    for kind in ("int64", "lean") if scale == 1 else ("int64",):
+        ctx = mpt.mpt_create(w, inst.bits)
+        mpt.mpt_set_tables(ctx, kind)
+        ws = torch.full((mpt.mpt_workspace_bytes(ctx),), 0xA5, dtype=torch.uint8, device="cuda")
+        assert mpt.mpt_solve(ctx, ws) == ref.opt
+        F, wI, split = mpt.mpt_tables(ref.ctx)
+        if kind == "int64":
+            for x, y in zip(mpt.mpt_tables(ctx), (F, wI, split)):
+                assert torch.equal(x, y)
+        else:
+            F32, split32 = mpt.mpt_tables32(ctx)
+            assert torch.equal(F32.long(), F) and torch.equal(split32, split)
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2])
 def test_m24_equals_the_full_recurrence(mpt, seed):
     inst = I.config(3, seed=seed)
