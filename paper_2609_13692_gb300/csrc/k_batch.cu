@@ -1,6 +1,8 @@
-// Batched exact solve of many small instances (m <= 15 requests each), one
-// block per instance with its tables in shared memory: the row-blocked
-// kernel for packed keys (m >= 6), the per-subset kernel otherwise.
+// Batched exact solve of many small instances (m <= 16 requests each), one
+// block per instance with its tables in shared memory: for packed keys the
+// row-blocked kernel (m >= 6) and, before it, a kernel for the instances of
+// 14 requests and more that have few splits to look at; the per-subset kernel
+// otherwise.
 //
 // This is the paper's own use of the exact recurrence (Sec. 6.2: 72 synthetic
 // groups of 10-15 requests; Sec. 7: real request groups of at most 13): many
@@ -624,6 +626,315 @@ __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put
   return true;
 }
 
+// ---------------------------------------------------------------------------
+// The same recurrence over members for m = 14..16, in a kernel of its own: it
+// needs few registers, so a block has as many threads as the SM's shared
+// memory leaves room for.  A set U is kept at the reverse V of its bits
+// (request j at bit m-1-j), where the sets of one lowest request are one
+// range and the ranges are finished in increasing order, 32 consecutive sets
+// per warp; phys XORs V's top five bits into its low five, so that warps over
+// consecutive V and over consecutive U both read 32 banks.  T holds w(I(S)),
+// then F(S) << m; sp the split.
+// kHalf (m = 16): 2^16 words do not fit shared memory, but the sets with
+// request 0 are no other set's B, and only as members are they its A.  T holds
+// the sets without it; the members with it are listed first, from a superset
+// sum of their own, and their F and split are kept in the block's scratch
+// slot; the other sets with it are finished as they are written out.
+// An instance with too many members is left to k_batch_rows, marked in its
+// split table, where {0} has no split.
+// Bound by the list loops' shared loads.  1,000 groups of 14-16 requests, with
+// the members in k_batch_rows (256 threads, m = 16 in global memory) and here:
+// kernels of m = 16, 15 and 14 1.72, 0.66 and 0.27 ms -> 0.42, 0.26 and 0.12 ms,
+// a solve 2.05 -> 0.71 ms.  For m = 12 and 13 the same kernel and the empty launch
+// behind it take 0.24 and 0.49 ms where k_batch_rows takes 0.25 and 0.51.
+constexpr int kMembersM = 14;
+constexpr uint32_t kLeftToRows = 0xFFFFFFFFu;
+
+struct MembersShape {
+  int list_cap;
+  size_t smem;
+};
+constexpr int members_threads(int m) { return m <= 14 ? 512 : 1024; }
+// list_cap 0: the occurrences leave no room for the lists
+inline MembersShape members_shape(int m, int occ_cap) {
+  const bool half = m >= 16;
+  const size_t H = (size_t)1 << (half ? m - 1 : m);
+  const size_t fixed = H * 6 + (half ? H / 8 : 0) + (size_t)occ_cap * 24, room = 220 * 1024;
+  const size_t want = m <= 14 ? 1024 : 4096;  // m = 14: two blocks to an SM
+  if (fixed + 1024 * 8 > room) return {0, 0};
+  const size_t cap = (room - fixed) / 8 < want ? (room - fixed) / 8 : want;
+  return {(int)cap, fixed + cap * 8};
+}
+
+template <int TPI, bool kHalf>
+__global__ void __launch_bounds__(TPI, TPI == 512 ? 2 : 1)
+k_batch_members(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
+                const int64_t* __restrict__ req_off, const int32_t* __restrict__ chunks,
+                const int64_t* __restrict__ tab_off, const int32_t* __restrict__ inst_list,
+                const uint8_t* __restrict__ flags, int occ_cap, int list_cap, int mm, int64_t* __restrict__ opt_out,
+                int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
+                int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int inst = inst_list[blockIdx.x];
+  const int64_t r0 = inst_req[inst], r1 = inst_req[inst + 1];
+  const int m = (int)(r1 - r0);  // == mm
+  const int64_t o0 = req_off[r0], o1 = req_off[r1];
+  const int occ = (int)(o1 - o0);
+  const int hb = kHalf ? mm - 1 : mm;
+  const uint32_t H = 1u << hb, N = 1u << mm, mask = N - 1u;
+  const int64_t tb = tab_off[inst];
+  uint32_t* gsp = split_out + tb;
+
+  uint32_t* T = reinterpret_cast<uint32_t*>(smem_raw);                         // [H]
+  uint16_t* sp = reinterpret_cast<uint16_t*>(T + H);                           // [H]
+  uint32_t* with0 = reinterpret_cast<uint32_t*>(sp + H);                       // kHalf: [H / 32] members with request 0
+  uint2* list = reinterpret_cast<uint2*>(with0 + (kHalf ? H / 32 : 0));        // [list_cap]
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(list + list_cap);  // [occ_cap]
+  int32_t* cx = reinterpret_cast<int32_t*>(keys + occ_cap);                    // [occ_cap]
+  uint32_t* cN = reinterpret_cast<uint32_t*>(cx + occ_cap);                    // [occ_cap]
+  uint32_t* tmask = cN + occ_cap;                                              // [2 * occ_cap] hash-table masks
+  // kHalf: F << m and split of the members with request 0, by the other requests
+  uint32_t* f0 = kHalf ? rows_scratch + (size_t)blockIdx.x * ((size_t)(1 << (mm - 5)) * kBRowStride) : nullptr;
+  __shared__ int ndistinct, most, use, cnt[kBMaxRowsM], start[kBMaxRowsM + 1];
+  __shared__ int roff[17];
+  __shared__ unsigned long long off[kBatchOffsets];
+  __shared__ long long hi_off[(1 << kBMaxRowsM) / 1024];
+  __shared__ uint32_t w_single;
+  __shared__ int32_t bflags;
+  const int t = threadIdx.x;
+  if (MPT_BAD(&bflags, m == mm && occ <= occ_cap && (!kHalf || rows_scratch))) {
+    if (t == 0) status[inst] = kErrBounds;
+    return;
+  }
+  if (t == 0) {
+    bflags = 0;
+    most = 1;
+  }
+  if (t < kBMaxRowsM) cnt[t] = 1;
+  if (t < kBatchOffsets) off[t] = 0;
+  const int nd = batch_gather<TPI>(m, r0, o0, occ, occ_cap, req_off, chunks, reinterpret_cast<int32_t*>(keys), tmask,
+                                   cx, cN, roff, &ndistinct, &bflags);
+  const bool use_off = (flags[inst] & kFlagOffsets) != 0;
+  auto rev = [&](uint32_t U) { return __brev(U) >> (32 - mm); };
+  auto phys = [&](uint32_t V) { return V ^ (V >> (hb - 5)); };
+
+  // w(I(.)) of the sets without request 0 (all sets, unless kHalf), or of
+  // those with it (with: kHalf)
+  auto tables = [&](bool with, bool first) {
+    for (uint32_t v = t; v < H; v += TPI) T[v] = 0;
+    __syncthreads();
+    for (int u = t; u < nd; u += TPI) {
+      const uint32_t Nx = cN[u];
+      const unsigned long long wx = (unsigned long long)weights[cx[u]];
+      if (use_off && (Nx & (Nx - 1)) == 0) {
+        if (first) atomicAdd(&off[__ffs(Nx) - 1], wx);
+      } else if (use_off && Nx == mask) {
+        if (first) atomicAdd(&off[kBatchUniv], wx);
+      } else if (!with || (Nx & 1u)) {
+        atomicAdd(&T[phys(rev(Nx) & (H - 1u))], (uint32_t)wx);
+      }
+    }
+    __syncthreads();
+    for (int j = 0; j < hb; j += 3) {
+      if (j + 3 <= hb) {
+        const uint32_t d0 = phys(1u << j), d1 = phys(2u << j), d2 = phys(4u << j);
+        for (uint32_t p = t; p < (H >> 3); p += TPI) {
+          // lanes over bits that phys takes to different banks
+          const bool top = j + 3 <= hb - 5;
+          const uint32_t q = top ? p >> 5 : p;
+          const uint32_t V = ((q >> j) << (j + 3)) | (q & ((1u << j) - 1u)) | (top ? (p & 31u) << (hb - 5) : 0u);
+          uint32_t* x = T;
+          const uint32_t i0 = phys(V);
+          const uint32_t i1 = i0 ^ d0, i2 = i0 ^ d1, i3 = i1 ^ d1, i4 = i0 ^ d2, i5 = i1 ^ d2, i6 = i2 ^ d2, i7 = i3 ^ d2;
+          uint32_t v0 = x[i0], v1 = x[i1], v2 = x[i2], v3 = x[i3], v4 = x[i4], v5 = x[i5], v6 = x[i6];
+          const uint32_t v7 = x[i7];
+          v0 += v1, v2 += v3, v4 += v5, v6 += v7;
+          v0 += v2, v1 += v3, v4 += v6, v5 += v7;
+          v0 += v4, v1 += v5, v2 += v6, v3 += v7;
+          x[i0] = v0, x[i1] = v1, x[i2] = v2, x[i3] = v3, x[i4] = v4, x[i5] = v5, x[i6] = v6;
+        }
+        __syncthreads();
+      } else {
+        for (int k = j; k < hb; ++k) {
+          const uint32_t d = phys(1u << k);
+          for (uint32_t p = t; p < (H >> 1); p += TPI) {
+            const uint32_t V = ((p >> k) << (k + 1)) | (p & ((1u << k) - 1u));
+            T[phys(V)] += T[phys(V) ^ d];
+          }
+          __syncthreads();
+        }
+      }
+    }
+  };
+
+  uint32_t wall = 0;
+  if constexpr (kHalf) {
+    for (uint32_t v = t; v < H / 32; v += TPI) with0[v] = 0;
+    tables(true, true);
+    wall = T[phys(H - 1u)];
+    for (uint32_t V = t; V < H; V += TPI) {
+      const uint32_t w = T[phys(V)], U = rev(V | H);
+      if (V == 0) {
+        w_single = w;
+        f0[0] = w << m;
+      } else if (w > wall) {
+        const int e = atomicAdd(&cnt[0], 1);
+        if (e < list_cap) list[e] = make_uint2(U, w);
+        atomicOr(&with0[U >> 6], 1u << (U >> 1 & 31u));
+        atomicMax(&most, __popc(U));
+      }
+    }
+    __syncthreads();
+  }
+  tables(false, !kHalf);
+  if constexpr (!kHalf) wall = T[phys(H - 1u)];
+  for (uint32_t V = t; V < H; V += TPI) {
+    const uint32_t U = rev(V);
+    if ((U & (U - 1u)) != 0 && T[phys(V)] > wall) {
+      atomicAdd(&cnt[__ffs(U) - 1], 1);
+      atomicMax(&most, __popc(U));
+    }
+  }
+  __syncthreads();
+  if (t == 0) {
+    unsigned long long tests = 0, splits = 1;
+    int at = 0;
+    for (int l = 0; l < m; ++l) {
+      start[l] = at;
+      at += cnt[l];
+      tests += (unsigned long long)cnt[l] << (m - 1 - l);
+      splits *= 3;
+      if (!(kHalf && l == 0)) cnt[l] = 1;
+    }
+    start[m] = at;
+    use = at <= list_cap && 2 * tests < splits / 2;
+    if (!use) gsp[1] = kLeftToRows;
+  }
+  __syncthreads();
+  if (!use) return;
+  for (uint32_t V = t; V < H; V += TPI) {
+    const uint32_t U = rev(V), v = T[phys(V)];
+    if ((U & (U - 1u)) == 0) {
+      T[phys(V)] = U ? v << m : 0u;
+      sp[phys(V)] = 0;
+      if (U) list[start[__ffs(U) - 1]] = make_uint2(U, (v << m) + U);
+    } else if (v > wall) {
+      const int l = __ffs(U) - 1;
+      list[start[l] + atomicAdd(&cnt[l], 1)] = make_uint2(U, v);
+    }
+  }
+  if (kHalf && t == 0) list[0] = make_uint2(1u, (w_single << m) + 1u);
+  const int total = start[m];
+  // the members, size by size, each over its own parts (members or single)
+  for (int p = 2; p <= most; ++p) {
+    __syncthreads();
+    for (int e = t; e < total; e += TPI) {
+      const uint32_t A = list[e].x;
+      if (__popc(A) != p) continue;
+      const uint32_t low = A & (~A + 1u), rest = A ^ low;
+      const bool in0 = kHalf && low == 1u;
+      uint32_t key = 0xFFFFFFFFu;
+      for (uint32_t sub = 0; sub != rest; sub = (sub - rest) & rest) {
+        const uint32_t a = low | sub;
+        const uint32_t fa = in0 ? f0[sub >> 1] : T[phys(rev(a))];
+        key = min(key, fa + a + T[phys(rev(A ^ a))]);
+      }
+      const uint32_t f = ((key >> m) - list[e].y) << m;
+      list[e].y = f + A;
+      if (in0) {
+        f0[A >> 1] = f;
+        f0[H + (A >> 1)] = key & mask;
+      } else {
+        T[phys(rev(A))] = f;
+        sp[phys(rev(A))] = (uint16_t)(key & mask);
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = t; e < total; e += TPI) {
+    const uint32_t V = rev(list[e].x) & (H - 1u);
+    list[e].x = V | (phys(V) << 16);
+  }
+  // the other sets, by lowest request from the highest down
+  for (int l = m - 2; l >= (kHalf ? 1 : 0); --l) {
+    __syncthreads();
+    const int b0 = start[l], b1 = start[l + 1];
+    const uint32_t own = 1u << (m - 1 - l);
+    for (uint32_t h = t; h < own; h += TPI) {
+      const uint32_t V = own | h, at = phys(V);
+      // only an unfinished set still has w* here (as in batch_members)
+      if (h == 0 || T[at] != wall) continue;
+      const uint32_t warp_all = V | 31u;  // holds every V of the warp
+      uint32_t key = 0xFFFFFFFFu;
+      for (int e = b0; e < b1; ++e) {
+        const uint2 a = list[e];
+        const uint32_t va = a.x & 0xFFFFu;
+        if ((va & ~warp_all) != 0) continue;
+        if ((va & ~V) == 0) key = min(key, a.y + T[at ^ (a.x >> 16)]);
+      }
+      T[at] = ((key >> m) - wall) << m;
+      sp[at] = (uint16_t)(key & mask);
+    }
+  }
+  // outputs; kHalf: the sets with request 0 beside those without
+  const int per = kHalf ? 1 : 0;  // requests left of the thread's own
+  for (uint32_t i = t; i < (H + TPI - 1) / TPI; i += TPI) {
+    long long v = use_off ? (long long)off[kBatchUniv] : 0;
+    for (uint32_t r = i * TPI; r; r &= r - 1) v += use_off ? (long long)off[__ffs(r) - 1 + per] : 0;
+    hi_off[i] = v;
+  }
+  __syncthreads();
+  int64_t lo = 0;
+  if (use_off)
+    for (uint32_t r = (uint32_t)t; r; r &= r - 1) lo += (int64_t)off[__ffs(r) - 1 + per];
+  for (uint32_t i = t; i < H; i += TPI) {
+    const uint32_t V = __brev(i) >> (32 - hb), at = phys(V);
+    const uint32_t A = sp[at];
+    const int64_t add = lo + hi_off[i / TPI];
+    const int64_t F = (int64_t)(T[at] >> m) + (i != 0 ? add : 0);
+    (void)MPT_BAD(&bflags, valid_split(i << per, A));
+    if constexpr (!kHalf) {
+      F_out[tb + i] = F;
+      gsp[i] = A;
+      if (i == mask) opt_out[inst] = F;
+    } else {
+      uint32_t f, A1;
+      if (i == 0) {
+        f = w_single;
+        A1 = 0;
+      } else if (with0[i >> 5] >> (i & 31u) & 1u) {
+        f = f0[i] >> m;
+        A1 = f0[H + i];
+      } else {
+        const uint32_t warp_all = i | 31u;
+        uint32_t key = 0xFFFFFFFFu;
+        for (int e = 0; e < start[1]; ++e) {
+          const uint2 a = list[e];
+          const uint32_t an = (a.y & mask) >> 1;
+          if ((an & ~warp_all) != 0) continue;
+          if ((an & ~i) == 0) key = min(key, a.y + T[at ^ (a.x >> 16)]);
+        }
+        f = (key >> m) - wall;
+        A1 = key & mask;
+      }
+      const int64_t F1 = (int64_t)f + add + (use_off ? (int64_t)off[0] : 0);
+      (void)MPT_BAD(&bflags, valid_split(2u * i + 1u, A1));
+      F_out[tb + 2 * i] = F;
+      F_out[tb + 2 * i + 1] = F1;
+      gsp[2 * i] = A;
+      gsp[2 * i + 1] = A1;
+      if (i == H - 1u) opt_out[inst] = F1;
+    }
+  }
+  __syncthreads();
+  batch_walk<TPI>(inst, m, r0, o0, roff, static_cast<const uint32_t*>(gsp), keys, cx, cN, nd, perm_out, dfs_out,
+                  status);
+  if (kBoundsChecked) {
+    __syncthreads();
+    if (t == 0 && bflags) status[inst] = bflags;
+  }
+}
+
 template <int TPI, bool kGRows = false>
 __global__ void __launch_bounds__(TPI, TPI >= 256 ? 3 : (TPI == 128 ? 6 : 12))  // 12 warps or more per SM
 k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
@@ -631,9 +942,11 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
              const int64_t* __restrict__ tab_off, const int32_t* __restrict__ inst_list,
              const uint8_t* __restrict__ flags, int occ_cap, int mm, int64_t* __restrict__ opt_out,
              int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
-             int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch) {
+             int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch,
+             bool members_ran) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int inst = inst_list[blockIdx.x];
+  if (members_ran && split_out[tab_off[inst] + 1] != kLeftToRows) return;  // finished by k_batch_members
   const int64_t r0 = inst_req[inst], r1 = inst_req[inst + 1];
   const int m = (int)(r1 - r0);  // == mm
   const int64_t o0 = req_off[r0], o1 = req_off[r1];
@@ -719,7 +1032,7 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
     __syncthreads();
   }
 
-  if (!batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
+  if (members_ran || !batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
                           [&](uint32_t U, uint32_t A) { put_split(U, A, &bflags); })) {
   // level 0: row 0, the recurrence on the five low requests
   if (t == 0) {
@@ -935,11 +1248,30 @@ cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weig
   const size_t smem = batch_rows_smem_bytes(m, occ_cap);
   const int tpi = batch_rows_threads(m);
   cudaError_t e = cudaSuccess;
+  const MembersShape ms = m >= kMembersM ? members_shape(m, occ_cap) : MembersShape{0, 0};
+  const bool members = ms.list_cap > 0;
+  if (members) {
+    auto first = [&](auto kernel) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms.smem);
+      if (e == cudaSuccess)
+        kernel<<<(unsigned)count, members_threads(m), ms.smem, stream>>>(
+            weights, inst_req, req_off, chunks, tab_off, inst_list, flags, occ_cap, ms.list_cap, m, opt, F, split, perm,
+            dfs, status, rows_scratch);
+    };
+    if (m >= 16)
+      first(k_batch_members<1024, true>);
+    else if (m == 15)
+      first(k_batch_members<1024, false>);
+    else
+      first(k_batch_members<512, false>);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   auto go = [&](auto kernel) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
       kernel<<<(unsigned)count, tpi, smem, stream>>>(weights, inst_req, req_off, chunks, tab_off, inst_list, flags,
-                                                      occ_cap, m, opt, F, split, perm, dfs, status, rows_scratch);
+                                                      occ_cap, m, opt, F, split, perm, dfs, status, rows_scratch, members);
   };
   if (m >= kBGlobalRowsM)
     go(k_batch_rows<256, true>);

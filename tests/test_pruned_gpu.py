@@ -215,3 +215,28 @@ def test_batch_equals_single_solves(mpt, scale):
         tF, _, ts = mpt.mpt_tables(one.ctx)
         assert opt[i] == one.opt and perms[i] == one.permutations() and orders[i] == one.dfs_order.tolist(), i
         assert torch.equal(F[offs[i]:offs[i + 1]], tF) and torch.equal(split[offs[i]:offs[i + 1]], ts), i
+
+
+@pytest.mark.parametrize("m", [14, 15, 16])
+def test_batch_members_and_rows(mpt, m):
+    """From 14 requests on, groups of few members are solved by a kernel of
+    their own and the others left to the row form: both kinds in one call, with
+    and without heavy private and common chunks, and requests so long that the
+    lists find no room."""
+    rng = np.random.default_rng(m)
+    w = np.concatenate([rng.integers(1, 9, size=600), np.full(m + 1, 1 << 26)]).astype(np.int64)
+    loo = [[x for x in range(m) if x != i] for i in range(m)]
+    groups = [loo]
+    for g in range(5):
+        pool = rng.choice(np.arange(m, 600), size=40 + 20 * g, replace=False)
+        groups.append([sorted(rng.choice(pool, size=int(rng.integers(0, 6)), replace=False).tolist()) for _ in range(m)])
+    groups += [[r + [600, 601 + i] for i, r in enumerate(g)] for g in groups[:3]]
+    groups.append([[]] * m)
+    for more in ([], [[sorted(rng.choice(600, size=int(rng.integers(45, 60)), replace=False).tolist()) for _ in range(m)]]):
+        opt, perms, orders, b = mpt.solve_batch(w, groups + more)
+        F, split, offs = mpt.mpt_batch_tables(b)
+        for i, g in enumerate(groups + more):
+            one = mpt.solve(w, I.pack_requests(g, len(w)), mode="blocked")
+            tF, _, ts = mpt.mpt_tables(one.ctx)
+            assert opt[i] == one.opt and perms[i] == one.permutations() and orders[i] == one.dfs_order.tolist(), i
+            assert torch.equal(F[offs[i]:offs[i + 1]], tF) and torch.equal(split[offs[i]:offs[i + 1]], ts), i
