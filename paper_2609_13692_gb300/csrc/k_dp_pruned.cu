@@ -65,7 +65,7 @@ constexpr int kPruneMinPairs = 16;     // pairs that a further block of a tile h
 
 // Shape of the kernel for 32-bit keys (rows of 32) and 64-bit keys (rows of
 // 16): one thread per row.
-template <typename Key>
+template <typename Key, int kSlots_ = 2>
 struct PrunedCfg {
   static constexpr int kRB = sizeof(Key) == 4 ? 5 : 4;
   static constexpr int kRow = 1 << kRB;
@@ -73,24 +73,25 @@ struct PrunedCfg {
   static constexpr int kLogWarps = kPB - kRB - 5;
   // rows kept per Ta: those of a short list, or all (64-bit keys have no other kernel for a long one)
   static constexpr int kKept = sizeof(Key) == 4 ? kPruneRows : kRows;
-  static constexpr int kGroups = sizeof(Key) == 4 ? 4 : 1;  // per block, at most
-  static constexpr int kSlots = 2;
+  static constexpr int kSlots = kSlots_;  // windows of pairs: one in use, the others being copied
+  static constexpr int kGroups = sizeof(Key) == 8 ? 1 : kSlots == 2 ? 4 : kSlots <= 4 ? 2 : 1;  // per block, at most
   static constexpr int kSlotBytes = (kRows + kPruneRows) * kRowBytes;  // Y window, X rows
   static constexpr int kTileBytes = kRows * (kRow + 1) * (int)sizeof(Key);  // a tile's keys, rows kRow + 1 apart
   static constexpr int kSeqStride = kRows + 2;  // so that a row's entries lie in different banks
   static constexpr int kSeqBytes = kRow * kSeqStride * 2;
   static constexpr int kSharedAt = kSlots * kSlotBytes + kSeqBytes + kPQueue * 4;
   static_assert(kSlotBytes >= kTileBytes, "a tile's keys fit a slot");
-  static constexpr int kGroupBytes = (kSharedAt + 4096 + 127) / 128 * 128;
+  static constexpr int kSharedBytes = 3072 + kSlots * 512;
+  static constexpr int kGroupBytes = (kSharedAt + kSharedBytes + 127) / 128 * 128;
   static_assert(kGroupBytes * kGroups <= 227 * 1024, "one block fits an SM");
 };
 
 // What a group of k_dp_pruned shares beside its windows and queue.
-template <typename Key>
+template <typename Key, int kSlots_>
 struct PrunedShared {
   // listed entries of the tile T: F << b, split, Ua, row of the list; by level, levels' sizes
   Key f[kPruneSelf];
-  uint2 rows[PrunedCfg<Key>::kSlots][kPruneRows];  // (a1 | rows << 16, mask) of the staged pairs
+  uint2 rows[2 * kSlots_][kPruneRows];  // lists of the pairs in use, staged and to be staged next: (a1, mask)
   uint32_t sp[kPruneSelf], start[kPB + 2], warp_n[PrunedCfg<Key>::kRows / 32];
   uint32_t last, any, unit;
   uint16_t u[kPruneSelf];
@@ -348,7 +349,9 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 // kRow outputs' best keys in registers and, in shared memory, the numbers of
 // their pairs in the queue (written only on a strict improvement, the pairs
 // coming in increasing Ta).  Per pair the complement window Y and the listed
-// rows of X are copied to shared memory, kSlots - 1 pairs ahead of the steps;
+// rows of X are copied to shared memory, kSlots - 1 pairs ahead of the steps
+// and the lists as far ahead of those (read into registers one pair ahead
+// instead: 1 % slower where all four groups run);
 // one barrier per pair.  Every lane of a warp runs the same (a1, mask) at a
 // time, with those lanes idle whose row does not hold a1, so that X is read
 // by broadcast.
@@ -363,15 +366,15 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 // 64-bit keys, one block per tile and no pair kernel, the key, and Ta in
 // partial_ta).  The group that finishes last (done[]) goes on to the tile's
 // entries.
-template <typename Key, typename Tab>
-__global__ void __launch_bounds__(PrunedCfg<Key>::kRows * (sizeof(Key) == 4 ? PrunedCfg<Key>::kGroups : 1),
-                                  sizeof(Key) == 4 ? 1 : 2)
+template <typename Key, typename Tab, int kSlots_>
+__global__ void __launch_bounds__(PrunedCfg<Key, kSlots_>::kRows * PrunedCfg<Key, kSlots_>::kGroups,
+                                  sizeof(Key) == 8 && kSlots_ == 2 ? 2 : 1)
 k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
             const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
             const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* partial_ta,
             uint32_t* __restrict__ done, uint32_t* __restrict__ next, Key* Gp,
             Key* Gc, uint32_t* __restrict__ split_rot, int32_t* __restrict__ flags) {
-  using C = PrunedCfg<Key>;
+  using C = PrunedCfg<Key, kSlots_>;
   constexpr int kRB = C::kRB, kRow = C::kRow, NT = C::kRows, kWarps = NT / 32;
   constexpr uint32_t kFull = 0xFFFFFFFFu >> (32 - kRow);
   constexpr Key kNone = ~(Key)0;
@@ -383,7 +386,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   Key* skey = reinterpret_cast<Key*>(psm + C::kSlotBytes);  // after the pairs: keys, rows kRow + 1 apart
   uint16_t* seq = reinterpret_cast<uint16_t*>(psm + C::kSlots * C::kSlotBytes);  // [in-row entry][thread]
   uint32_t* queue = reinterpret_cast<uint32_t*>(psm + C::kSlots * C::kSlotBytes + C::kSeqBytes);
-  PrunedShared<Key>& sh = *reinterpret_cast<PrunedShared<Key>*>(psm + C::kSharedAt);
+  auto& sh = *reinterpret_cast<PrunedShared<Key, kSlots_>*>(psm + C::kSharedAt);
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + group), "n"(NT) : "memory"); };  // of this group
   // The warps of one sub-partition (number mod 4) get row groups of every kind:
   // those of the groups rotated, or of a group of eight warps mirrored.
@@ -428,32 +431,20 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
       pcopy16(slot + r * kRowBytes + swz, y + r * kRowBytes + col);
     }
   };
-  // The row list of queued pair p: rows tid / 8 and tid / 8 + NT / 8 (at most
-  // kPruneRows in all) of this thread's copies, read one pair ahead of them.
-  constexpr int kHeld = (kPruneRows * 8 + NT - 1) / NT;
-  uint2 held[kHeld];
-  auto hold = [&](uint32_t p) {
-    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = queue[p] >> kQueueShift;
-#pragma unroll
-    for (int j = 0; j < kHeld; ++j) {
-      const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
-      if (r < n && r < (uint32_t)kPruneRows) held[j] = rows[(size_t)Tp * C::kKept + r];
-    }
+  // The row list of queued pair p, copied kSlots - 1 pairs ahead of its windows.
+  constexpr int kRing = 2 * C::kSlots;
+  auto stage_list = [&](uint32_t p) {
+    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = min(queue[p] >> kQueueShift, (uint32_t)kPruneRows);
+    if (2 * tid < n) pcopy16(&sh.rows[p % kRing][2 * tid], rows + (size_t)Tp * C::kKept + 2 * tid);
   };
   auto stage = [&](uint32_t p, uint32_t s) {
-    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = queue[p] >> kQueueShift;
+    const uint32_t Tp = queue[p] & ((1u << kQueueShift) - 1u), n = min(queue[p] >> kQueueShift, (uint32_t)kPruneRows);
     char* slot = psm + s * C::kSlotBytes;
     const uint32_t col = (tid & 7u) * 16u;
     const char* x = reinterpret_cast<const char*>(Gp + ((size_t)Tp << kPB));
     stage_window(slot, Gc + ((size_t)(T ^ Tp) << kPB));
-#pragma unroll
-    for (int j = 0; j < kHeld; ++j) {
-      const uint32_t r = (tid >> 3) + (uint32_t)(j * (NT / 8));
-      if (r < n && r < (uint32_t)kPruneRows) {
-        if (col == 0) sh.rows[s][r] = make_uint2(held[j].x | (n << 16), held[j].y);
-        pcopy16(slot + (NT + r) * kRowBytes + col, x + held[j].x * kRowBytes + col);
-      }
-    }
+    for (uint32_t r = tid >> 3; r < n; r += NT / 8)
+      pcopy16(slot + (NT + r) * kRowBytes + col, x + sh.rows[p % kRing][r].x * kRowBytes + col);
   };
   // Candidates: the short lists of lowest request l, or the proper parts of T
   // holding it when those are fewer; both in increasing order.  A queue entry,
@@ -572,17 +563,19 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
         qn += q1 - q0;
       }
       sync();
-      // the first kSlots - 1 pairs; a group is committed for each slot, also
-      // without a pair, so that the waits below can count them
+      // the first lists, then the first kSlots - 1 pairs; a group is committed
+      // for each slot, also without a pair, so that the waits below can count them
+#pragma unroll
+      for (uint32_t p = 0; p < (uint32_t)kRing - 2; ++p)
+        if (p < qn) stage_list(p);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      sync();
 #pragma unroll
       for (int p = 0; p < C::kSlots - 1; ++p) {
-        if ((uint32_t)p < qn) {
-          hold(p);
-          stage(p, p);
-        }
+        if ((uint32_t)p < qn) stage(p, p);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      if ((uint32_t)(C::kSlots - 1) < qn) hold(C::kSlots - 1);
     } else {
       if (cT == 0) break;
       // The listed entries themselves first, one thread each, level by level
@@ -603,7 +596,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
             sh.u[i] = (uint16_t)((e.x << kRB) | lane);
             sh.k[i] = (uint8_t)k;
           }
-          if (lane == 0) sh.rows[0][k] = make_uint2(e.x | (n << 16), e.y);
+          if (lane == 0) sh.rows[0][k] = e;
           at += __popc(e.y);
         }
       }
@@ -659,17 +652,17 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
       if (phase == 0) {
         const uint32_t q = p + (uint32_t)(C::kSlots - 1);
         if (q < qn) stage(q, s == 0 ? C::kSlots - 1 : s - 1);
+        if (q + C::kSlots - 1 < qn) stage_list(q + C::kSlots - 1);
         asm volatile("cp.async.commit_group;" ::: "memory");
-        if (q + 1 < qn) hold(q + 1);
       }
       const char* slot = psm + s * C::kSlotBytes;
-      const uint2* list = sh.rows[s];
-      const uint32_t n = list[0].x >> 16;
+      const uint2* list = sh.rows[p % kRing];
+      const uint32_t n = phase == 0 ? queue[p] >> kQueueShift : iT & kRowsMask;
       Key acc[kRow];
 #pragma unroll
       for (int i = 0; i < kRow; ++i) acc[i] = kNone;
       for (uint32_t k = 0; k < min(n, (uint32_t)kPruneRows); ++k) {
-        const uint32_t a1 = list[k].x & 0xFFFFu, mask = list[k].y;
+        const uint32_t a1 = list[k].x, mask = list[k].y;
         if ((a1 & ~s1) != 0) continue;
         Key y[kRow];
         const uint32_t r = s1 ^ a1;
@@ -824,25 +817,42 @@ cudaError_t tables(const Shape& s, const Workspace& ws, G* wIr, cudaStream_t str
   return cudaGetLastError();
 }
 
+template <typename Key, typename Tab, int kSlots_>
+cudaError_t launch_layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, uint32_t items, int groups,
+                         unsigned long long units, unsigned long long* partial, Key* Gp, Key* Gc, cudaStream_t stream) {
+  using C = PrunedCfg<Key, kSlots_>;
+  static_assert(sizeof(PrunedShared<Key, kSlots_>) <= C::kSharedBytes, "a group's shared values");
+  auto k = k_dp_pruned<Key, Tab, kSlots_>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kGroupBytes * C::kGroups);
+  if (e != cudaSuccess) return e;
+  const unsigned long long sms = (unsigned long long)sm_count();
+  k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
+      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short,
+      ws.prune_long, ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc,
+      ws.split_rot, ws.counters + 1);
+  return cudaGetLastError();
+}
+
 template <typename Key, typename Tab>
 cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, uint32_t items,
                   unsigned long long* partial, Key* Gp, Key* Gc, cudaStream_t stream, int* launches) {
-  using C = PrunedCfg<Key>;
-  static_assert(sizeof(PrunedShared<Key>) <= 4096, "a group's shared values");
-  auto k = k_dp_pruned<Key, Tab>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kGroupBytes * C::kGroups);
-  if (e != cudaSuccess) return e;
   // a block per SM, and in it as many groups as there are units for; 64-bit
   // groups, whose eight warps are balanced by themselves, as blocks of one
-  // (m = 24, weights x 4096: 0.41 ms of tile stage, 0.44 with two to a block)
+  // (m = 24, weights x 4096: 0.41 ms of tile stage, 0.44 with two to a block).
+  // Where a group has an SM, or half of one, to itself, nothing but copies
+  // further ahead hides their latency: 23 requests of 40 passages, six of whose
+  // eleven steps are of that size, 1.01 -> 0.93 ms from create to tables.
   const unsigned long long units = h_binom.v[s.L][kh] * items, sms = (unsigned long long)sm_count();
-  const int groups = sizeof(Key) == 8 ? 1 : units >= sms * C::kGroups ? C::kGroups : (int)((units + sms - 1) / sms);
-  k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
-      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short, ws.prune_long,
-      ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc, ws.split_rot,
-      ws.counters + 1);
   ++*launches;
-  return cudaGetLastError();
+  if (units <= sms)
+    return launch_layer<Key, Tab, sizeof(Key) == 8 ? 4 : 6>(s, ws, wIr, kh, items, 1, units, partial, Gp, Gc, stream);
+  if constexpr (sizeof(Key) == 8) {
+    return launch_layer<Key, Tab, 2>(s, ws, wIr, kh, items, 1, units, partial, Gp, Gc, stream);
+  } else {
+    if (units <= 2 * sms) return launch_layer<Key, Tab, 4>(s, ws, wIr, kh, items, 2, units, partial, Gp, Gc, stream);
+    const int groups = units >= sms * 4 ? 4 : (int)((units + sms - 1) / sms);
+    return launch_layer<Key, Tab, 2>(s, ws, wIr, kh, items, groups, units, partial, Gp, Gc, stream);
+  }
 }
 
 // The members of each single request's list by k_prune_tiles' rules: the
