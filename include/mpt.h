@@ -61,8 +61,12 @@ typedef struct mpt_ctx mpt_ctx;
  * recurrence on F(S) - sum_{i in S} pi_i - u and add it back in every output.
  * AUTO picks BLOCKED whenever W < 2^(32 - b), b = min(m, 12) tile bits
  * (2^20 from m = 12 on; its 32-bit packed keys are then exact), else WIDE
- * while W < 2^51 (64-bit packed keys), else GENERAL.  All of them return the
- * same tables, OPT and layout. */
+ * while W < 2^51 (64-bit packed keys), else GENERAL.  Under AUTO mpt_solve
+ * leaves out the splits that cannot be the reported one (their named part has
+ * two requests or more and no chunk common to all of them that not every
+ * request needs) where the requests share few enough chunks for that to be
+ * cheaper; BLOCKED and WIDE look at every split.  All of them return the same
+ * tables, OPT and layout. */
 typedef enum mpt_dp_mode {
   MPT_DP_AUTO = 0,
   MPT_DP_BLOCKED = 1, /* shared-memory tiled min-plus; needs W < 2^(32 - min(m, 12)) */
@@ -81,7 +85,8 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
 
 /* Bytes of device workspace mpt_solve needs for this context: the input
  * copies, the intersection-weight table wI int64[2^m], F int64[2^m],
- * split uint32[2^m], the blocked DP's working tables and the layout buffers. */
+ * split uint32[2^m], the blocked DP's working tables, the layout buffers and,
+ * under AUTO, the lists of the splits that are looked at. */
 mpt_status mpt_workspace_bytes(const mpt_ctx* ctx, size_t* bytes);
 
 /* Choose the DP kernels (default MPT_DP_AUTO).  BLOCKED is refused with
@@ -109,6 +114,7 @@ mpt_status mpt_solve(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes, vo
  * each depend only on earlier ones (Sec. 3.1 layers: one step per tile layer
  * |T| = 0 .. m - b of the blocked kernels, or the singletons and one step per
  * subset size of the general kernels); mpt_solve_steps gives their number.
+ * Staged solves look at every split, under AUTO too.
  *   mpt_solve_begin:  input copies, K1, K2 and step 0;
  *   mpt_solve_layers: the next `count` steps (fewer at the end); *next_step
  *                     (may be NULL) receives the index of the next step;
@@ -205,7 +211,7 @@ typedef struct mpt_profile {
   double ms_dp_general; /* general DP: all launches */
   double ms_walk;       /* hierarchy walk -> layout */
   double ms_d2h;        /* result copies */
-  double splits_pairs;  /* splits evaluated by the pair kernel */
+  double splits_pairs;  /* splits evaluated by the pair kernel (under AUTO: 0 where it was not needed) */
   double splits_total;  /* (3^m + 1)/2 - 2^m */
   int64_t launches_pairs;
   int64_t launches_total; /* kernels launched by the last solve (memsets excluded) */
@@ -223,7 +229,8 @@ mpt_status mpt_get_profile(const mpt_ctx* ctx, mpt_profile* out);
  * Every instance shares one chunk universe and weight array; instance b owns
  * requests inst_requests[b] .. inst_requests[b+1]-1, request r the chunk ids
  * chunk_ids[req_offsets[r] .. req_offsets[r+1]).  One CUDA block solves one
- * instance with all of its tables in shared memory; results follow the same
+ * instance with its tables in shared memory (partly in the workspace at 16
+ * requests); results follow the same
  * conventions as mpt_solve / mpt_layout for each instance on its own (request
  * bit i = the instance's i-th request).
  * ------------------------------------------------------------------------- */

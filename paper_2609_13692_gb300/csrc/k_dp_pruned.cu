@@ -32,10 +32,10 @@
 // kPruneRows are read from the table as they come.
 //
 // Measured on one GB300 (whole solve with layout and tables, full recurrence
-// before, pruned after): 28 requests of 20 passages 673 -> 7.6 .. 23 ms by
+// before, pruned after): 28 requests of 20 passages 673 -> 4.7 .. 16.2 ms by
 // seed (a passage held by 12 to 17 of the 28 decides it), 24 requests of 10
-// passages 11.1 -> 0.9 ms and with 64-bit keys 80 -> 1.0 ms, 26 requests of 40
-// passages 81 -> 17 .. 29 ms.
+// passages 11.1 -> 0.8 ms and with 64-bit keys 80 -> 0.9 ms, 26 requests of 40
+// passages 81 -> 14.6 .. 31.7 ms.
 // k_dp_pruned is bound by the integer ALU pipe where a popular passage gives
 // long a1 lists: 55 % of the pipe busy in the heaviest layers of the first 26
 // of the 28 requests, a sixth of it on the bookkeeping per pair, the rest of
