@@ -33,6 +33,8 @@
 // the least Ua; across proper pairs, taken in increasing Ta with strict
 // improvement, the least Ta; then the self pair (largest Ta = T).  That is the
 // lexicographic order on (value, A) as an integer, since A = Ua * 2^L + Ta.
+#include <type_traits>
+
 #include "mpt_internal.cuh"
 
 namespace mpt {
@@ -603,15 +605,22 @@ __device__ __forceinline__ int64_t load_wI(const Tab* p) {
 //     the row, in registers, in increasing s2 (every proper subset of s2 is
 //     smaller than s2).
 // Rows are finished level by level in |s1|, so every row read is final.
-constexpr int kRowsThreads = 96;
+//
+// Layers with no more tiles than SMs are as long as one tile's chain: their
+// blocks have 288 threads, at least one lane per row pair up to |s1| = 3 and at
+// most four pairs per lane above, and w(I) in shared memory from the start.
+// Leave-one-out, m = 20 (8 such layers): solve 738 -> 693 us.  Longer layers have
+// three or four blocks of 96 threads per SM instead (m = 28 with 192 threads
+// to all: 8.7 ms of tile stage, 8.4 with 96; with 384: 15.2).
+constexpr int kRowsThreads = 96, kRowsThreadsShort = 288;
 constexpr int kBestWords = (1 << kB) + kRows;  // per-output arrays, rows 33 words apart
 // With kZcGlobal, tile 0's complement rows are read from global memory (the
 // same 16 KB for every block, so they stay in L1) instead of a shared copy:
 // 52 KB of shared memory per block instead of 70, four blocks per SM instead
 // of three.  That pays on long layers (m >= 26: 7.95 vs 8.37 ms of tile
 // stage at m = 28) but not on short ones (m = 24: 1.22 vs 1.19 ms).
-constexpr int rows_smem_bytes(bool zc_global) {
-  return ((zc_global ? 1 : 2) * kWin + 2 * kBestWords) * (int)sizeof(uint32_t);
+constexpr int rows_smem_bytes(bool zc_global, bool w_shared) {
+  return ((zc_global ? 1 : 2) * kWin + (w_shared ? 3 : 2) * kBestWords) * (int)sizeof(uint32_t);
 }
 constexpr int kZcGlobalMinL = 14;
 
@@ -639,8 +648,8 @@ __device__ __forceinline__ void load_zrow(uint32_t (&v)[kRow], const uint32_t* z
   }
 }
 
-template <typename Tab, bool kZcGlobal>
-__global__ void __launch_bounds__(kRowsThreads)
+template <typename Tab, bool kZcGlobal, int kThreads>
+__global__ void __launch_bounds__(kThreads)
 k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long long* __restrict__ partial,
                uint32_t* __restrict__ Gp, uint32_t* __restrict__ Gc, uint32_t* __restrict__ split_rot,
                int32_t* __restrict__ flags, const uint32_t* __restrict__ info, InnerPerm perm) {
@@ -649,6 +658,8 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
   uint32_t* zc = smem + kWin;                             // tile 0, complement form, padded rows (shared copy)
   uint32_t* bkey = smem + (kZcGlobal ? 1 : 2) * kWin;     // best key per output so far
   uint32_t* bsplit = bkey + kBestWords;                   // its Ta; after finishing, the split A
+  constexpr bool kShort = kThreads > kRowsThreads;
+  uint32_t* ws = bsplit + kBestWords;                     // kShort: the tile's w(I)
   constexpr uint32_t kMask = (1u << kB) - 1u;
 
   const uint32_t tile = blockIdx.x;
@@ -658,16 +669,17 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
   if (info && !(info[T] & kTileLong)) return;  // finished by k_dp_pruned
 
   if constexpr (!kZcGlobal) {
-    for (int c = threadIdx.x; c < (1 << (kB - 2)); c += kRowsThreads) {
+    for (int c = threadIdx.x; c < (1 << (kB - 2)); c += kThreads) {
       const int row = c >> (kB2 - 2), k = c & ((1 << (kB2 - 2)) - 1);
       *reinterpret_cast<uint4*>(zc + row_pos((uint32_t)row) * kRowStride + 4 * k) =
           *reinterpret_cast<const uint4*>(Gc + 4 * c);
     }
   }
-  for (int u = threadIdx.x; u < (1 << kB); u += kRowsThreads) {
+  for (int u = threadIdx.x; u < (1 << kB); u += kThreads) {
     const unsigned long long pv = kh >= 2 ? partial[((size_t)tile << kB) | (uint32_t)u] : ~0ull;
     bkey[best_word((uint32_t)u)] = (uint32_t)(pv >> 32);
     bsplit[best_word((uint32_t)u)] = (uint32_t)pv;
+    if (kShort) ws[best_word((uint32_t)u)] = (uint32_t)load_wI(wIr + (tbase | (uint32_t)u));
   }
   __syncthreads();
 
@@ -679,13 +691,18 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
     uint32_t wv[kRow];
     const bool finisher = (int)threadIdx.x < rows;
     const uint32_t s1f = finisher ? colex_unrank((unsigned long long)threadIdx.x, p1, kB1) : 0u;
-    if (finisher) {
+    if (finisher && !kShort) {
 #pragma unroll
       for (int i = 0; i < kRow; ++i) wv[i] = (uint32_t)load_wI(wIr + (tbase | (s1f << kB2) | (uint32_t)i));
     }
     if (p1 >= 1) {
-      // lanes per row chosen so that each lane runs at most 8 row pairs
-      const int g = p1 > 3 ? p1 - 3 : 0;
+      // lanes per row chosen so that each lane runs at most 8 row pairs, or as
+      // many as the block has
+      int g = p1 > 3 ? p1 - 3 : 0;
+      if (kShort) {
+        g = p1 < 5 ? p1 : 5;
+        while ((rows << g) > kThreads) --g;
+      }
       const int G = 1 << g;
       const int ri = (int)(threadIdx.x >> g);
       const uint32_t r = threadIdx.x & (uint32_t)(G - 1);
@@ -752,11 +769,11 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
         }
         uint32_t f, A;
         if (kh == 1 && U == 0) {  // S = T, a single request
-          f = wv[s2];
+          f = kShort ? ws[best_word(U)] : wv[s2];
           A = 0;
         } else {
           const uint32_t Ua = (bk & kMask) + (nat_s1 | (info ? perm.nat((uint32_t)s2) : (uint32_t)s2)) - kMask;
-          f = (bk >> kB) - wv[s2];
+          f = (bk >> kB) - (kShort ? ws[best_word(U)] : wv[s2]);
           A = (Ua << L) | bt;
         }
         c[s2] = f << kB;
@@ -769,7 +786,7 @@ k_dp_tile_rows(int L, int kh, const Tab* __restrict__ wIr, const unsigned long l
     __syncthreads();
   }
 
-  for (int u = threadIdx.x; u < (1 << kB); u += kRowsThreads) {
+  for (int u = threadIdx.x; u < (1 << kB); u += kThreads) {
     const uint32_t gp = cur[row_pos((uint32_t)u >> kB2) * kRowStride + (u & (kRow - 1))];
     const uint32_t A = bsplit[best_word((uint32_t)u)];
     const uint32_t nat = info ? perm.nat((uint32_t)u) : (uint32_t)u;
@@ -844,14 +861,16 @@ cudaError_t blocked_attributes(bool listed) {
                                                 kListedSmemBytes)
                          : cudaFuncSetAttribute(k_dp_pairs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 kPairSmemBytes);
-  auto rows = [&](auto kernel, bool zc_global) {
+  auto rows = [&](auto kernel, bool zc_global, bool w_shared = false) {
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem_bytes(zc_global));
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem_bytes(zc_global, w_shared));
   };
-  rows(k_dp_tile_rows<int64_t, false>, false);
-  rows(k_dp_tile_rows<int32_t, false>, false);
-  rows(k_dp_tile_rows<int64_t, true>, true);
-  rows(k_dp_tile_rows<int32_t, true>, true);
+  rows(k_dp_tile_rows<int64_t, false, kRowsThreads>, false);
+  rows(k_dp_tile_rows<int32_t, false, kRowsThreads>, false);
+  rows(k_dp_tile_rows<int64_t, true, kRowsThreads>, true);
+  rows(k_dp_tile_rows<int32_t, true, kRowsThreads>, true);
+  rows(k_dp_tile_rows<int64_t, false, kRowsThreadsShort>, false, true);
+  rows(k_dp_tile_rows<int32_t, false, kRowsThreadsShort>, false, true);
   return e;
 }
 
@@ -860,16 +879,23 @@ void launch_tiles(const Shape& s, const Workspace& ws, int kh, const uint32_t* i
   const unsigned long long tiles = h_binom.v[s.L][kh];
   const unsigned long long* part = kh >= 2 ? ws.partial : nullptr;
   const bool zg = s.L >= kZcGlobalMinL;
-  const int sm_bytes = rows_smem_bytes(zg);
-  if (s.lean) {
-    auto k = zg ? k_dp_tile_rows<int32_t, true> : k_dp_tile_rows<int32_t, false>;
-    k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(s.L, kh, ws.fw_rot, part, ws.Gp, ws.Gc, ws.split_rot,
-                                                           ws.counters + 1, info, s.perm);
-  } else {
-    auto k = zg ? k_dp_tile_rows<int64_t, true> : k_dp_tile_rows<int64_t, false>;
-    k<<<(unsigned)tiles, kRowsThreads, sm_bytes, stream>>>(s.L, kh, ws.wI_rot, part, ws.Gp, ws.Gc, ws.split_rot,
-                                                           ws.counters + 1, info, s.perm);
-  }
+  auto run = [&](auto kernel, const auto* wI, int threads, bool zc_global) {
+    kernel<<<(unsigned)tiles, threads, rows_smem_bytes(zc_global, threads > kRowsThreads), stream>>>(
+        s.L, kh, wI, part, ws.Gp, ws.Gc, ws.split_rot, ws.counters + 1, info, s.perm);
+  };
+  auto pick = [&](const auto* wI) {
+    using Tab = std::remove_const_t<std::remove_pointer_t<decltype(wI)>>;
+    if (tiles <= (unsigned long long)sm_count())
+      run(k_dp_tile_rows<Tab, false, kRowsThreadsShort>, wI, kRowsThreadsShort, false);
+    else if (zg)
+      run(k_dp_tile_rows<Tab, true, kRowsThreads>, wI, kRowsThreads, true);
+    else
+      run(k_dp_tile_rows<Tab, false, kRowsThreads>, wI, kRowsThreads, false);
+  };
+  if (s.lean)
+    pick(static_cast<const int32_t*>(ws.fw_rot));
+  else
+    pick(static_cast<const int64_t*>(ws.wI_rot));
 }
 
 }  // namespace
