@@ -275,6 +275,48 @@ k_prune_members(int L, const uint32_t* __restrict__ info, uint32_t* __restrict__
   }
 }
 
+// The tiles of a layer differ in work by two orders of magnitude (those within
+// a popular passage's N_x have all their parts for members), and a heavy one
+// taken last leaves the other SMs waiting: SMs were busy for 80 % of the heavy
+// layers' time.  Tiles are dealt from the most work to the least, by classes of
+// sqrt(2) of an estimate: over the N_x that hold T's lowest request, their
+// common parts with T times the inner splits.  m = 28: solves
+// of 3.05, 3.61, 8.47 and 14.41 ms by seed -> 2.85, 3.38, 8.34 and 14.11 ms, with
+// two launches of 13 us each; so only where the host's estimate of the pairs is
+// above kPruneSortPairs (some 0.5 ms).
+__device__ __forceinline__ int work_class(uint32_t T, int n, const uint32_t* __restrict__ N) {
+  float work = 1.0f;
+  const uint32_t low = T & (~T + 1u);
+  for (int i = 0; i < n; ++i) {
+    const uint32_t Ni = N[i], NT = Ni >> kPB;
+    if (NT & low) work += exp2f((float)(__popc(NT & T) - 1) + 0.585f * (float)__popc(Ni & kPMask));
+  }
+  const int c = (int)(2.0f * log2f(work));
+  return kPruneClasses - 1 - min(c, kPruneClasses - 1);  // the most work first
+}
+
+__global__ void __launch_bounds__(256)
+k_prune_classes(int L, int n_shared, const uint32_t* __restrict__ N, const int32_t* __restrict__ counters,
+                uint32_t* __restrict__ hist) {
+  const int n = min(counters[3], n_shared);
+  for (uint32_t T = 1 + blockIdx.x * blockDim.x + threadIdx.x; T < (1u << L); T += gridDim.x * blockDim.x)
+    atomicAdd(&hist[__popc(T) * kPruneClasses + work_class(T, n, N)], 1u);
+}
+
+__global__ void __launch_bounds__(256)
+k_prune_order(int L, int n_shared, const uint32_t* __restrict__ N, const int32_t* __restrict__ counters,
+              const uint32_t* __restrict__ hist, uint32_t* __restrict__ placed, uint32_t* __restrict__ order) {
+  const int n = min(counters[3], n_shared);
+  for (uint32_t T = 1 + blockIdx.x * blockDim.x + threadIdx.x; T < (1u << L); T += gridDim.x * blockDim.x) {
+    const int kh = __popc(T), c = work_class(T, n, N);
+    uint32_t at = 0;
+    for (int k = 0; k < kh; ++k) at += (uint32_t)c_binom.v[L][k];
+    for (int q = 0; q < c; ++q) at += hist[kh * kPruneClasses + q];
+    at += atomicAdd(&placed[kh * kPruneClasses + c], 1u);
+    order[at] = colex_rank(T);
+  }
+}
+
 __device__ __forceinline__ uint32_t min_keep(uint32_t a, uint32_t b, bool* keep) { return __vibmin_u32(a, b, keep); }
 __device__ __forceinline__ unsigned long long min_keep(unsigned long long a, unsigned long long b, bool* keep) {
   *keep = a <= b;
@@ -369,7 +411,8 @@ __device__ __forceinline__ void pconv(Key (&acc)[kRow], const char* x, const Key
 template <typename Key, typename Tab, int kSlots_>
 __global__ void __launch_bounds__(PrunedCfg<Key, kSlots_>::kRows * PrunedCfg<Key, kSlots_>::kGroups,
                                   sizeof(Key) == 8 && kSlots_ == 2 ? 2 : 1)
-k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, InnerPerm perm, const Tab* __restrict__ wIr,
+k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, InnerPerm perm,
+            const uint32_t* __restrict__ order, const Tab* __restrict__ wIr,
             const uint32_t* __restrict__ info, const uint2* __restrict__ rows, const uint32_t* __restrict__ short_ta,
             const uint32_t* __restrict__ long_ta, const uint32_t* __restrict__ member_n, unsigned long long* partial, uint32_t* partial_ta,
             uint32_t* __restrict__ done, uint32_t* __restrict__ next, Key* Gp,
@@ -403,7 +446,8 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   // One unit: a tile, or one of `items` parts of it.  Every thread of the
   // group takes the same way out.
   auto run = [&](uint32_t unit) {
-  const uint32_t tile = unit % tiles, item = unit / tiles;
+  const uint32_t item = unit / tiles, tile = order ? order[unit % tiles] : unit % tiles;
+  if (MPT_BAD(flags, tile < tiles)) return;
   const uint32_t T = colex_unrank((unsigned long long)tile, kh, L);
   if (MPT_BAD(flags, T < (1u << L) && __popc(T) == kh)) return;
   const uint32_t iT = info[T];
@@ -814,6 +858,14 @@ cudaError_t tables(const Shape& s, const Workspace& ws, G* wIr, cudaStream_t str
       s.L, s.prune_pairs, s.n_shared, ws.shared_N, ws.shared_w, wIr, ws.prune_info, ws.prune_rows, ws.counters);
   k_prune_members<<<(unsigned)s.L, 1024, 0, stream>>>(s.L, ws.prune_info, ws.prune_short, ws.prune_long, ws.prune_n);
   *launches += 2;
+  if (s.prune_sort) {
+    const unsigned blocks = (unsigned)(tiles / 256 + 1 < sm_count() * 4 ? tiles / 256 + 1 : sm_count() * 4);
+    uint32_t* placed = ws.prune_hist + kMaxMembersL * kPruneClasses;
+    k_prune_classes<<<blocks, 256, 0, stream>>>(s.L, s.n_shared, ws.shared_N, ws.counters, ws.prune_hist);
+    k_prune_order<<<blocks, 256, 0, stream>>>(s.L, s.n_shared, ws.shared_N, ws.counters, ws.prune_hist, placed,
+                                              ws.prune_order);
+    *launches += 2;
+  }
   return cudaGetLastError();
 }
 
@@ -826,8 +878,14 @@ cudaError_t launch_layer(const Shape& s, const Workspace& ws, const Tab* wIr, in
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kGroupBytes * C::kGroups);
   if (e != cudaSuccess) return e;
   const unsigned long long sms = (unsigned long long)sm_count();
+  const uint32_t* order = nullptr;
+  if (s.prune_sort) {
+    unsigned long long before = 0;
+    for (int q = 0; q < kh; ++q) before += h_binom.v[s.L][q];
+    order = ws.prune_order + before;
+  }
   k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
-      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, wIr, ws.prune_info, ws.prune_rows, ws.prune_short,
+      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, order, wIr, ws.prune_info, ws.prune_rows, ws.prune_short,
       ws.prune_long, ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc,
       ws.split_rot, ws.counters + 1);
   return cudaGetLastError();
@@ -899,7 +957,8 @@ void prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* suppor
 }
 
 cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
-  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, (kPruneSplitTiles + kMaxMembersL) * 4, stream);
+  const size_t cleared = kPruneSplitTiles + kMaxMembersL + 2 * kMaxMembersL * kPruneClasses;
+  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, cleared * 4, stream);
   if (e != cudaSuccess) return e;
   auto* lean = reinterpret_cast<unsigned int*>(ws.fw_rot);
   auto* full = reinterpret_cast<unsigned long long*>(ws.wI_rot);

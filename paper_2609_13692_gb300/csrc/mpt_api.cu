@@ -102,7 +102,7 @@ constexpr size_t kMaxSupports = 8192;
 void prune_shape(mpt_ctx* c) {
   mpt::Shape& s = c->shape;
   c->perm = mpt::InnerPerm{};
-  s.pruned = s.prune_long = s.prune_pairs = false;
+  s.pruned = s.prune_long = s.prune_pairs = s.prune_sort = false;
   if (c->mode != MPT_DP_AUTO || !s.blocked || s.L < 1 || c->many_supports) return;
   double members[32], rows[32], tas[32];
   for (int l = 0; l < s.L; ++l) members[l] = rows[l] = tas[l] = 1.0;
@@ -131,6 +131,7 @@ void prune_shape(mpt_ctx* c) {
   s.prune_most = *std::max_element(tas, tas + s.L);
   s.pruned = !s.prune_long || time < 0.7 * full;
   s.prune_pairs = s.prune_long && !s.wide;
+  s.prune_sort = time > mpt::kPruneSortPairs;
   if (!s.pruned) return;
   // Stored order of the inner bits: those of the N_x whose members cost most
   // (pairs times inner splits) first.  The first five are the in-row bits,
@@ -261,7 +262,7 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
   ws->dfs = reinterpret_cast<int32_t*>(take((size_t)s.m * 4));
   ws->opt = reinterpret_cast<int64_t*>(take(mpt::kOptBytes));
   // after everything else, so that the rest sits where it does without them
-  ws->prune_info = ws->prune_short = ws->prune_long = ws->prune_n = ws->prune_done = nullptr;
+  ws->prune_info = ws->prune_short = ws->prune_long = ws->prune_n = ws->prune_done = ws->prune_hist = ws->prune_order = nullptr;
   ws->prune_rows = nullptr;
   ws->shared_N = nullptr;
   ws->shared_w = nullptr;
@@ -275,7 +276,10 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
     ws->prune_short = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_long = reinterpret_cast<uint32_t*>(take(P * 4));
     ws->prune_n = reinterpret_cast<uint32_t*>(take(2 * mpt::kMaxMembersL * 4));
-    ws->prune_done = reinterpret_cast<uint32_t*>(take((mpt::kPruneSplitTiles + mpt::kMaxMembersL) * 4));
+    const size_t hist = 2 * (size_t)mpt::kMaxMembersL * mpt::kPruneClasses;
+    ws->prune_done = reinterpret_cast<uint32_t*>(take((mpt::kPruneSplitTiles + mpt::kMaxMembersL + hist) * 4));
+    ws->prune_hist = ws->prune_done ? ws->prune_done + mpt::kPruneSplitTiles + mpt::kMaxMembersL : nullptr;
+    ws->prune_order = reinterpret_cast<uint32_t*>(take(P * 4));
   }
   return off;
 }

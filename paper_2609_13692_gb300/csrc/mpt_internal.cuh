@@ -241,6 +241,8 @@ struct Workspace {
   uint32_t* prune_long;   // [2^L] Ta's with a long list, by lowest request
   uint32_t* prune_n;      // [2 * kMaxMembersL] their numbers per lowest request
   uint32_t* prune_done;   // [kPruneSplitTiles] finished parts of each tile of a layer; [kMaxMembersL] units taken per layer
+  uint32_t* prune_hist;   // [2 * kMaxMembersL * kPruneClasses] tiles per layer and class of work, and those placed
+  uint32_t* prune_order;  // [2^L] by layer, its tiles from the most work to the least
   // layout
   unsigned long long* keys;  // [slots]
   int64_t* perm_offsets;     // [m + 1]
@@ -285,6 +287,7 @@ struct Shape {
   double prune_most;  // the host's bound on the pairs of one tile
   bool prune_long;  // some list may be long, or some tile left to the row kernel
   bool prune_pairs; // some list may be long (32-bit keys)
+  bool prune_sort;  // a layer's tiles are taken from the most work to the least
 };
 
 // Pruned recurrence (k_dp_pruned.cu): rows of a short list, members of a tile
@@ -294,6 +297,8 @@ constexpr int kPruneRows = 32;
 constexpr int kPruneSelf = 128;
 constexpr int kPruneSplitTiles = 16384;
 constexpr int kMaxMembersL = 32;
+constexpr int kPruneClasses = 64;
+constexpr double kPruneSortPairs = 16000;  // estimated full pairs from which a solve sorts its tiles (k_dp_pruned.cu)
 constexpr uint32_t kListLong = 1u << 30;
 constexpr uint32_t kTileLong = 1u << 31;
 

@@ -175,6 +175,23 @@ def test_tables_from_a_used_workspace(mpt, m, scale):
             assert torch.equal(F32.long(), F) and torch.equal(split32, split)
 
 
+@pytest.mark.parametrize("scale", [1, 1 << 12])
+def test_sorted_tiles(mpt, scale):
+    """Enough pairs that the tiles of a layer are taken from the most work to
+    the least (two launches more), tile bits and classes of several sizes."""
+    top = _mask(*range(12, 20))
+    inst = _from_supports(23, [top | _mask(*range(0, 8)), top | _mask(*range(1, 9)), top | _mask(0, *range(2, 9)),
+                               _mask(0, 10, 21), _mask(9, 10, 11)], 23, 400)
+    w = inst.weights * scale
+    a, b = mpt.solve(w, inst.bits), mpt.solve(w, inst.bits, mode="blocked" if scale == 1 else "wide")
+    assert a.opt == b.opt
+    for x, y in zip(mpt.mpt_tables(a.ctx), mpt.mpt_tables(b.ctx)):
+        assert torch.equal(x, y)
+    # K1, lists (2), sort (2), tile 0, 11 layers of tiles, long ones (11), pairs, walk
+    p = mpt.mpt_get_profile(mpt.solve(w, inst.bits, profile=True).ctx)
+    assert p["launches_total"] == 7 + 11 + 11 + p["launches_pairs"]
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2])
 def test_m24_equals_the_full_recurrence(mpt, seed):
     inst = I.config(3, seed=seed)
