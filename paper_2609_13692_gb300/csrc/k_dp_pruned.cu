@@ -422,6 +422,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   constexpr uint32_t kFull = 0xFFFFFFFFu >> (32 - kRow);
   constexpr Key kNone = ~(Key)0;
   constexpr uint32_t kSelf = 0xFFFFu, kListed = 0x8000u;  // pair numbers of the self pair and of listed entries
+  constexpr int kMeet = 8;
   static_assert(kPQueue <= 0x8000, "pair numbers fit beside the two marks");
   extern __shared__ __align__(16) char block_sm[];
   const uint32_t group = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid & 31u, warp = tid >> 5;
@@ -446,7 +447,9 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   // One unit: a tile, or one of `items` parts of it.  Every thread of the
   // group takes the same way out.
   auto run = [&](uint32_t unit) {
-  const uint32_t item = unit / tiles, tile = order ? order[unit % tiles] : unit % tiles;
+  // sorted: the parts of one tile one after the other, the heavy tiles' first
+  // (all tiles' first parts, then all second ones: 2 to 8 % longer solves)
+  const uint32_t item = order ? unit % items : unit / tiles, tile = order ? order[unit / items] : unit % tiles;
   if (MPT_BAD(flags, tile < tiles)) return;
   const uint32_t T = colex_unrank((unsigned long long)tile, kh, L);
   if (MPT_BAD(flags, T < (1u << L) && __popc(T) == kh)) return;
@@ -543,10 +546,21 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
     return sizeof(Key) == 4 ? (uint32_t)__ldcg(&pt[U]) : pt_ta[U];
   };
   auto to_partial = [&]() {
-    for (uint32_t U = tid; U <= kPMask; U += NT) {
-      const unsigned long long own =
-          ((unsigned long long)key_at(U) << 32) | (queue[seq_at(U)] & ((1u << kQueueShift) - 1u));
-      if (own < __ldcg(&pt[U])) atomicMin(&pt[U], own);
+    // kMeet reads in flight at a time, here, where the minima are read back and
+    // in the last pass over the tile: one at a time, each of a thread's 32 waited
+    // for L2 (m = 28 by seed: 2.59, 3.34, 8.08 and 13.68 -> 2.34, 3.08, 7.49 and
+    // 12.91 ms per solve)
+    for (uint32_t U0 = tid; U0 <= kPMask; U0 += kMeet * NT) {
+      unsigned long long there[kMeet];
+#pragma unroll
+      for (int q = 0; q < kMeet; ++q) there[q] = __ldcg(&pt[U0 + (uint32_t)(q * NT)]);
+#pragma unroll
+      for (int q = 0; q < kMeet; ++q) {
+        const uint32_t U = U0 + (uint32_t)(q * NT);
+        const unsigned long long own =
+            ((unsigned long long)key_at(U) << 32) | (queue[seq_at(U)] & ((1u << kQueueShift) - 1u));
+        if (own < there[q]) atomicMin(&pt[U], own);
+      }
     }
   };
 
@@ -766,9 +780,12 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
           if (!sh.last) return;
           __threadfence();
         }
-        for (uint32_t U = tid; U <= kPMask; U += NT) {
-          const unsigned long long v = __ldcg(&pt[U]);
-          key_at(U) = (Key)(v >> 32);
+        for (uint32_t U0 = tid; U0 <= kPMask; U0 += kMeet * NT) {
+          unsigned long long there[kMeet];
+#pragma unroll
+          for (int q = 0; q < kMeet; ++q) there[q] = __ldcg(&pt[U0 + (uint32_t)(q * NT)]);
+#pragma unroll
+          for (int q = 0; q < kMeet; ++q) key_at(U0 + (uint32_t)(q * NT)) = (Key)(there[q] >> 32);
         }
         sync();
 #pragma unroll
@@ -822,7 +839,16 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   }
   const size_t tbase = (size_t)T << kPB;
   const uint32_t nat_lo = perm.nat(tid);
-  for (uint32_t U0 = 0; U0 <= kPMask; U0 += NT) {
+  for (uint32_t UB = 0; UB <= kPMask; UB += kMeet * NT) {
+  uint32_t ta_of[kMeet];
+#pragma unroll
+  for (int q = 0; q < kMeet; ++q) {
+    const uint32_t U = (UB + (uint32_t)(q * NT)) | tid;
+    ta_of[q] = !met && (seq_at(U) & kListed) ? 0u : ta_at(U);  // kListed, kSelf: no number of a queued pair
+  }
+#pragma unroll
+  for (int q = 0; q < kMeet; ++q) {
+    const uint32_t U0 = UB + (uint32_t)(q * NT);
     const uint32_t U = U0 | tid, nat = nat_lo | perm.nat(U0);
     Key key = key_at(U);
     const uint32_t number = cT != 0 ? seq_at(U) : 0u;
@@ -830,13 +856,14 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
     if ((number & kListed) && number != kSelf) {
       A = sh.sp[number & ~kListed];
     } else {
-      A = (((uint32_t)(key & kPMask) + nat - kPMask) << L) | (number == kSelf ? T : ta_at(U));
+      A = (((uint32_t)(key & kPMask) + nat - kPMask) << L) | (number == kSelf ? T : ta_of[q]);
       key &= ~(Key)kPMask;  // F << b
     }
     if (MPT_BAD(flags, valid_split(T | (nat << L), A))) continue;
     Gp[tbase | U] = key;
     Gc[tbase | U] = key | (Key)(~nat & kPMask);
     split_rot[tbase | U] = A;
+  }
   }
   };
   // the first unit of a group is its own number, the others come from *next
