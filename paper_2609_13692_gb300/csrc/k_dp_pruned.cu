@@ -444,6 +444,15 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
   };
   const uint32_t tiles = (uint32_t)c_binom.v[L][kh];
 
+  // The layer before may still run (launch_layer): what it and earlier ones
+  // wrote is read only behind earlier().
+  bool waited = false;
+  auto earlier = [&]() {
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    waited = true;
+  };
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
   // One unit: a tile, or one of `items` parts of it.  Every thread of the
   // group takes the same way out.
   auto run = [&](uint32_t unit) {
@@ -629,12 +638,14 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
       asm volatile("cp.async.commit_group;" ::: "memory");
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       sync();
+      earlier();
 #pragma unroll
       for (int p = 0; p < C::kSlots - 1; ++p) {
         if ((uint32_t)p < qn) stage(p, p);
         asm volatile("cp.async.commit_group;" ::: "memory");
       }
     } else {
+      earlier();
       if (cT == 0) break;
       // The listed entries themselves first, one thread each, level by level
       // in |Ua| (a member Ua' within Ua has a lower level): a level's entries
@@ -876,6 +887,7 @@ k_dp_pruned(int L, int kh, uint32_t items, bool long_tiles, bool long_lists, Inn
     sync();
     unit = sh.unit;
   }
+  earlier();  // a layer is finished only behind the one before
 }
 
 template <typename Key, typename G>
@@ -911,11 +923,24 @@ cudaError_t launch_layer(const Shape& s, const Workspace& ws, const Tab* wIr, in
     for (int q = 0; q < kh; ++q) before += h_binom.v[s.L][q];
     order = ws.prune_order + before;
   }
-  k<<<(unsigned)(sizeof(Key) == 8 || units < sms ? units : sms), C::kRows * groups, C::kGroupBytes * groups, stream>>>(
-      s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, order, wIr, ws.prune_info, ws.prune_rows, ws.prune_short,
-      ws.prune_long, ws.prune_n, partial, ws.partial_ta, ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc,
-      ws.split_rot, ws.counters + 1);
-  return cudaGetLastError();
+  // The layer may start while the one before runs out of blocks: its first
+  // units' candidates, queues and lists do not depend on it.  24 requests of 10
+  // passages, 12 layers: 0.40 -> 0.33 ms per solve; 23 of 40: 0.73 -> 0.67 ms.
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(sizeof(Key) == 8 || units < sms ? units : sms));
+  cfg.blockDim = dim3((unsigned)(C::kRows * groups));
+  cfg.dynamicSmemBytes = (size_t)(C::kGroupBytes * groups);
+  cfg.stream = stream;
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, s.L, kh, items, s.prune_long, s.prune_pairs, s.perm, order, wIr,
+                            (const uint32_t*)ws.prune_info, (const uint2*)ws.prune_rows, (const uint32_t*)ws.prune_short,
+                            (const uint32_t*)ws.prune_long, (const uint32_t*)ws.prune_n, partial, ws.partial_ta,
+                            ws.prune_done, ws.prune_done + kPruneSplitTiles + kh, Gp, Gc, ws.split_rot,
+                            ws.counters + 1);
 }
 
 template <typename Key, typename Tab>

@@ -124,6 +124,7 @@ k_dp_tile0(int L, int b, InnerPerm perm, const Tab* __restrict__ wIr, Key* __res
   Key* ws = cur + C::kRows * C::kStride;    // w(I), then split
   Key* amin = ws + C::kRows * (kRow + 1);   // phase A minima of a level's rows
   const int t = threadIdx.x, nb = b - kRB;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // k_dp_pruned's first layer gets ready meanwhile
   const uint32_t mask = (1u << b) - 1u;
   for (uint32_t v = t; v <= mask; v += kT0Threads) {
     const uint32_t U = perm.nat(v);
