@@ -104,8 +104,8 @@ void prune_shape(mpt_ctx* c) {
   c->perm = mpt::InnerPerm{};
   s.pruned = s.prune_long = s.prune_pairs = s.prune_sort = false;
   if (c->mode != MPT_DP_AUTO || !s.blocked || s.L < 1 || c->many_supports) return;
-  double members[32], rows[32], tas[32];
-  for (int l = 0; l < s.L; ++l) members[l] = rows[l] = tas[l] = 1.0;
+  double members[32], tas[32];
+  for (int l = 0; l < s.L; ++l) members[l] = tas[l] = 1.0;
   double time = 0.05 * (double)(1ull << s.L);
   double full = 0.5;
   for (int l = 0; l < s.L; ++l) full *= 3.0;
@@ -115,7 +115,6 @@ void prune_shape(mpt_ctx* c) {
     for (int l = s.L - 1; l >= 0; --l) {
       if (!((T >> l) & 1u)) continue;
       members[l] += (double)(1ull << __builtin_popcount(U));
-      rows[l] += (double)(1ull << __builtin_popcount(U >> (s.wide ? 4 : 5)));
       here += (double)(1ull << (s.L - 1 - l)) * above;
       tas[l] += above2;
       above *= 1.5;
@@ -126,13 +125,10 @@ void prune_shape(mpt_ctx* c) {
     for (int u = __builtin_popcount(U); u < s.b; ++u) inner *= 2.0 / 3.0;
     time += here * (inner + 0.05 < 1.0 ? inner + 0.05 : 1.0);
   }
-  for (int l = 0; l < s.L; ++l)
-    s.prune_long = s.prune_long || members[l] > (double)mpt::kPruneSelf || rows[l] > (double)mpt::kPruneRows;
+  const bool cheap = time < 0.7 * full;
+  const bool few = *std::max_element(members, members + s.L) <= (double)mpt::kPruneSelf;
+  if (!cheap && !few) return;
   s.prune_most = *std::max_element(tas, tas + s.L);
-  s.pruned = !s.prune_long || time < 0.7 * full;
-  s.prune_pairs = s.prune_long && !s.wide;
-  s.prune_sort = time > mpt::kPruneSortPairs;
-  if (!s.pruned) return;
   // Stored order of the inner bits: those of the N_x whose members cost most
   // (pairs times inner splits) first.  The first five are the in-row bits,
   // the next two tell the warps of a block apart, the last five its lanes.
@@ -149,8 +145,9 @@ void prune_shape(mpt_ctx* c) {
       for (int u = __builtin_popcount(U); u > 0; --u) sum *= 1.5;
       cost.emplace_back(-sum, U);
     }
+    cost.emplace_back(0.0, (1u << s.b) - 1u);
   } catch (...) {
-    return;  // the natural order
+    cost.clear();  // the natural order
   }
   std::sort(cost.begin(), cost.end());
   // (64-bit keys: rows of 16, so four, three and five)
@@ -159,17 +156,30 @@ void prune_shape(mpt_ctx* c) {
   const uint8_t* place = s.wide ? place64 : place32;
   uint32_t left = (1u << s.b) - 1u;
   int n = 0;
-  cost.emplace_back(0.0, left);
   for (const auto& e : cost)
     for (uint32_t r = e.second & left; r; r &= r - 1) {
       c->perm.to_nat[place[n++]] = (uint8_t)__builtin_ctz(r);
       left &= ~(r & (~r + 1u));
     }
-  // The sums above count a member once per N_x that holds it.  The lists of the
-  // single requests, counted exactly, say whether the pair and row kernels have
+  // Rows are counted in that order.  These sums count a member once per N_x that
+  // holds it; the lists of the single requests, counted exactly, say whether the pair and row kernels have
   // anything to do: 23 requests of 40 passages, whose lists are all short, spent
   // 0.2 ms of 1.0 on launches of the two that found nothing.
-  if (s.prune_long) mpt::prune_singles(s, c->perm, c->supports.data(), c->supports.size(), &s.prune_long, &s.prune_pairs);
+  double rows[32];
+  for (int l = 0; l < s.L; ++l) rows[l] = 1.0;
+  for (uint32_t N : c->supports) {
+    const double r = (double)(1ull << __builtin_popcount(c->perm.stored(N >> s.L) >> (s.wide ? 4 : 5)));
+    for (int l = 0; l < s.L; ++l)
+      if ((N >> l) & 1u) rows[l] += r;
+  }
+  if (!few || *std::max_element(rows, rows + s.L) > (double)mpt::kPruneRows)
+    mpt::prune_singles(s, c->perm, c->supports.data(), c->supports.size(), &s.prune_long, &s.prune_pairs);
+  s.pruned = !s.prune_long || cheap;
+  s.prune_sort = time > mpt::kPruneSortPairs;
+  if (!s.pruned) {
+    s.prune_long = s.prune_pairs = s.prune_sort = false;
+    c->perm = mpt::InnerPerm{};
+  }
 }
 
 void refresh_shape(mpt_ctx* c) {

@@ -175,6 +175,20 @@ def test_tables_from_a_used_workspace(mpt, m, scale):
             assert torch.equal(F32.long(), F) and torch.equal(split32, split)
 
 
+@pytest.mark.parametrize("scale", [1, 1 << 21])
+@pytest.mark.parametrize("inner", [5, 6])
+def test_rows_counted_in_stored_order(mpt, scale, inner):
+    """A list of 2^inner members in one or two rows by the natural order of the
+    inner bits, and in 2^inner rows by the stored one, which has the bits of
+    costlier sets in front."""
+    inst = _from_supports(18, [_mask(1, 2, 3, 4, *range(12, 16)), _mask(1, 2, 3, 4, 16, 17),
+                               _mask(5, *range(6, 6 + inner))], inner)
+    if scale == 1:
+        test_equals_the_full_recurrence(mpt, inst)
+    else:
+        test_wide_equals_the_full_recurrence(mpt, inst)
+
+
 @pytest.mark.parametrize("scale", [1, 1 << 12])
 def test_sorted_tiles(mpt, scale):
     """Enough pairs that the tiles of a layer are taken from the most work to
