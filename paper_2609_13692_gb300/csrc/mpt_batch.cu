@@ -196,14 +196,18 @@ void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, co
                      const int64_t* req_offsets, const int64_t* chunk_ids, int32_t* ids32, uint8_t* flags,
                      mpt_status* bad) {
   const int64_t occ = req_offsets[inst_requests[batch]];
-  const int64_t cores = std::max<int64_t>(1, (int64_t)std::thread::hardware_concurrency());
+  const int64_t cores = occ >> 15 ? std::max<int64_t>(1, (int64_t)std::thread::hardware_concurrency()) : 1;
   const int64_t ranges = std::min<int64_t>({8, cores, 1 + (occ >> 15), batch});
+  int64_t most = 8, slots = 16;  // of the largest instance
+  for (int32_t b = 0; b < batch; ++b)
+    most = std::max<int64_t>(most, req_offsets[inst_requests[b + 1]] - req_offsets[inst_requests[b]]);
+  while (slots < 2 * std::min<int64_t>(most, kBatchMaxOcc)) slots <<= 1;
   struct Range {
     std::vector<ChunkSlot> table;
     mpt_status status = MPT_OK;
   };
   std::vector<Range> out((size_t)ranges);
-  for (Range& r : out) r.table.resize(2 * kBatchMaxOcc);  // here, so that a thread has nothing that throws
+  for (Range& r : out) r.table.resize((size_t)slots);  // here, so that a thread has nothing that throws
   auto work = [&](int64_t k) {
     Range& r = out[(size_t)k];
     const int32_t end = (int32_t)(batch * (k + 1) / ranges);
