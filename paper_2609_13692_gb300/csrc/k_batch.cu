@@ -935,6 +935,10 @@ k_batch_members(const int64_t* __restrict__ weights, const int64_t* __restrict__
   }
 }
 
+// What k_batch_rows does about the members: tries them first, takes what
+// k_batch_members left, or leaves them out.
+enum class Members { kTry, kRan, kNone };
+
 template <int TPI, bool kGRows = false>
 __global__ void __launch_bounds__(TPI, TPI >= 256 ? 3 : (TPI == 128 ? 6 : 12))  // 12 warps or more per SM
 k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
@@ -943,10 +947,10 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
              const uint8_t* __restrict__ flags, int occ_cap, int mm, int64_t* __restrict__ opt_out,
              int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
              int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch,
-             bool members_ran) {
+             Members members) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int inst = inst_list[blockIdx.x];
-  if (members_ran && split_out[tab_off[inst] + 1] != kLeftToRows) return;  // finished by k_batch_members
+  if (members == Members::kRan && split_out[tab_off[inst] + 1] != kLeftToRows) return;  // finished by k_batch_members
   const int64_t r0 = inst_req[inst], r1 = inst_req[inst + 1];
   const int m = (int)(r1 - r0);  // == mm
   const int64_t o0 = req_off[r0], o1 = req_off[r1];
@@ -1032,7 +1036,7 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
     __syncthreads();
   }
 
-  if (members_ran || !batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
+  if (members != Members::kTry || !batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
                           [&](uint32_t U, uint32_t A) { put_split(U, A, &bflags); })) {
   // level 0: row 0, the recurrence on the five low requests
   if (t == 0) {
@@ -1249,8 +1253,15 @@ cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weig
   const int tpi = batch_rows_threads(m);
   cudaError_t e = cudaSuccess;
   const MembersShape ms = m >= kMembersM ? members_shape(m, occ_cap) : MembersShape{0, 0};
-  const bool members = ms.list_cap > 0;
-  if (members) {
+  // Looking at members only is less work but a longer chain per instance, so
+  // below 14 requests it waits for enough blocks to hide that (13 requests:
+  // 10 instances 123 us per solve against 111, 1,200 324 against 302, 2,400 485
+  // against 509, 9,600 1.54 ms against 1.69; 9 requests: 1,200 123 against 126 us,
+  // 9,600 324 against 396).
+  const Members members = ms.list_cap > 0 ? Members::kRan
+                          : m >= kMembersM || count >= 12 * sm_count() ? Members::kTry
+                                                                       : Members::kNone;
+  if (members == Members::kRan) {
     auto first = [&](auto kernel) {
       e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms.smem);
       if (e == cudaSuccess)

@@ -617,7 +617,7 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
   // Rounds of merges, `ahead` enqueued between two looks at whether the last one
   // still merged anything (each does, until no pair shares weight; later ones
   // return at once).  Few requests need few: with 12 for all, 20 requests took
-  // 501 us, now GR20.
+  // 501 us, now 445.
   int ahead = 2;
   while (ahead < 12 && (4 << ahead) < 4 * 4 * m) ++ahead;  // 2 + log2(m), at most 12
   if (ahead > m) ahead = m;

@@ -271,3 +271,22 @@ def test_batch_members_and_rows(mpt, m):
             tF, _, ts = mpt.mpt_tables(one.ctx)
             assert opt[i] == one.opt and perms[i] == one.permutations() and orders[i] == one.dfs_order.tolist(), i
             assert torch.equal(F[offs[i]:offs[i + 1]], tF) and torch.equal(split[offs[i]:offs[i + 1]], ts), i
+
+
+@pytest.mark.parametrize("m", [6, 9, 11, 12, 13])
+def test_batch_members_of_many_groups(mpt, m):
+    """Below 14 requests the members are tried from some two thousand groups of
+    one size on: one call of 2,400 against three of 800."""
+    rng = np.random.default_rng(100 + m)
+    w = rng.integers(1, 9, size=400).astype(np.int64)
+    groups = []
+    for _ in range(2400):
+        pool = rng.choice(400, size=int(rng.integers(8, 60)), replace=False)
+        groups.append([rng.choice(pool, size=int(rng.integers(0, 7)), replace=False).tolist() for _ in range(m)])
+    opt, perms, orders, b = mpt.solve_batch(w, groups)
+    F, split, _ = mpt.mpt_batch_tables(b)
+    for k in range(0, 2400, 800):
+        o, p, d, part = mpt.solve_batch(w, groups[k:k + 800])
+        pF, ps, _ = mpt.mpt_batch_tables(part)
+        assert list(o) == list(opt[k:k + 800]) and p == perms[k:k + 800] and d == orders[k:k + 800]
+        assert torch.equal(pF, F[k << m:(k + 800) << m]) and torch.equal(ps, split[k << m:(k + 800) << m])
