@@ -13,16 +13,94 @@
 #include "../../include/mpt.h"
 #include "mpt_internal.cuh"
 
+namespace mpt {
+
+constexpr int kMaxShared = 8192;  // chunks that some but not all requests share, in a pruned solve
+
+// The request sets N_x of the chunks that some but not all requests share, and
+// the bounds on a pruned solve (k_dp_pruned.cu) that follow set by set.  Its
+// members are the parts of some N_x, so with N = (N_T, N_U) the tile and inner
+// bits of N_x:
+//   * the members (Ta, Ua) of one Ta number at most the sum over N_T containing
+//     Ta of 2^|N_U|, and no Ta has more than the single request in it;
+//   * the pairs with a member Ta are, over all tiles T, at most
+//     sum over N of sum over Ta within N_T of 2^(L - 1 - lowest(Ta) - (|Ta| - 1)),
+//     plus one per T for the single request.  A Ta whose lowest request is the
+//     j-th of N_T contributes 2^(L - 1 - e_j) (3/2)^(requests of N_T above it)
+//     over all choices of the others.
+// A pair whose list lies in N_U alone takes 3^|N_U| 2^(b - |N_U|) of the 3^b
+// splits of a full pair, at about half its rate (26 requests of 40 passages:
+// 0.39 of a full pair's time at |N_U| = 8, where 2 (2/3)^4 = 0.395).
+// The bounds only grow, so the sets of an instance far from the pruned form are
+// given up after the first few: all 8,000 chunks of 14 to 20 requests that share
+// half or a third of them, taken bit by bit and sorted, cost mpt_create 0.7 to
+// 1.1 ms (0.06 to 0.1 without them; a solve takes 0.25 to 0.7).
+struct Overlap {
+  int L = 0;                    // tile bits; 0: nothing to collect
+  int n_shared = 0;             // chunks whose sets were taken
+  bool out = false;             // the pruned form is not for this instance
+  std::vector<uint32_t> sets;   // distinct sets, in the order found
+  std::vector<uint32_t> table;  // open addressing, 0 = free
+  double members[32], tas[32], most_members = 1.0, time = 0.0, full = 0.0;
+
+  void begin(int m) {
+    L = m - blocked_tile_bits(m);
+    full = 0.5;
+    for (int l = 0; l < L; ++l) {
+      members[l] = tas[l] = 1.0;
+      full *= 3.0;
+    }
+    time = 0.05 * (double)(1ull << L);
+  }
+  bool cheap() const { return time < 0.7 * full; }
+  bool few() const { return most_members <= (double)kPruneSelf; }
+
+  // One more chunk with request set N (two requests or more, not all).
+  void add(uint32_t N) {
+    if (out || ++n_shared > kMaxShared) {
+      out = true;
+      return;
+    }
+    if (table.empty()) table.assign(2 * kMaxShared, 0u);
+    uint32_t h = (N * 2654435761u) >> 18;
+    static_assert(2 * kMaxShared == 1 << (32 - 18), "hash bits");
+    for (; table[h] != 0; h = (h + 1u) & (2u * kMaxShared - 1u))
+      if (table[h] == N) return;
+    table[h] = N;
+    sets.push_back(N);
+    const uint32_t T = N & ((1u << L) - 1u);
+    const int inner_bits = __builtin_popcount(N >> L);
+    double above = 1.0, above2 = 1.0, here = 0.0;
+    for (int l = L - 1; l >= 0; --l) {
+      if (!((T >> l) & 1u)) continue;
+      members[l] += (double)(1ull << inner_bits);
+      if (members[l] > most_members) most_members = members[l];
+      here += (double)(1ull << (L - 1 - l)) * above;
+      tas[l] += above2;
+      above *= 1.5;
+      above2 *= 2.0;
+    }
+    // of a full pair's time: the inner splits, at half its rate
+    double inner = 2.0;
+    for (int u = inner_bits; u < 12; ++u) inner *= 2.0 / 3.0;
+    time += here * (inner + 0.05 < 1.0 ? inner + 0.05 : 1.0);
+    out = !cheap() && !few();
+  }
+  void done() {
+    table = std::vector<uint32_t>();
+    if (out) sets = std::vector<uint32_t>();
+  }
+};
+
+}  // namespace mpt
+
 struct mpt_ctx {
   mpt::Shape shape{};
   std::vector<int64_t> w;
   std::vector<uint64_t> bits;
   int64_t sum_w = 0;     // sum_i w(R_i)
   int64_t shared_w = 0;  // the same less the chunks one or every request needs
-  // distinct request sets N_x of the other chunks, when there are at most
-  // kMaxSupports of those chunks (many_supports otherwise)
-  std::vector<uint32_t> supports;
-  bool many_supports = false;
+  mpt::Overlap overlap;         // of the other chunks' request sets
   mpt::InnerPerm perm;          // stored order of the inner bits in the pruned recurrence
   mpt::Shape solved_shape{};    // of the last solve: as `shape`, with the order its tables have
   int32_t mode = MPT_DP_AUTO;
@@ -78,63 +156,27 @@ bool use_wide(const mpt_ctx* c) {
   return c->mode == MPT_DP_AUTO && !blocked_feasible(c) && wide_feasible(c);
 }
 
-constexpr size_t kMaxSupports = 8192;
-
-// Whether a one-shot AUTO solve takes the pruned recurrence
-// (k_dp_pruned.cu), from the sets N_x alone.  Its members are the parts of
-// some N_x, so with N = (N_T, N_U) the tile and inner bits of N_x:
-//   * the members (Ta, Ua) of one Ta number at most sum over N_T containing
-//     Ta of 2^|N_U|, their rows at most the sum of 2^|row bits of N_U|, and no
-//     Ta has more than the single request in it.  When no request's sums
-//     exceed the limits of a short list, there is no long one and the pair
-//     and row kernels are not launched at all;
-//   * the pairs with a member Ta are, over all tiles T, at most
-//     sum over N of sum over Ta within N_T of 2^(L - 1 - lowest(Ta) - (|Ta| - 1)),
-//     plus one per T for the single request.  A Ta whose lowest request is the
-//     j-th of N_T contributes 2^(L - 1 - e_j) (3/2)^(requests of N_T above it)
-//     over all choices of the others.
-// A pair whose list lies in N_U alone takes 3^|N_U| 2^(b - |N_U|) of the 3^b
-// splits of a full pair, at about half its rate (26 requests of 40 passages:
-// 0.39 of a full pair's time at |N_U| = 8, where 2 (2/3)^4 = 0.395).  The pruned
-// form is taken when the pairs' times so estimated are below 0.7 of the full
-// recurrence's, or when there is no long list.  Leave-one-out requests (every
-// N_x all but one) stay with the full form.
+// Whether a one-shot AUTO solve takes the pruned recurrence (k_dp_pruned.cu),
+// from the sets N_x alone: where the pairs' times estimated by Overlap are
+// below 0.7 of the full recurrence's, or no request's members exceed the
+// limits of a short list, so that the pair and row kernels are not launched
+// at all.  Leave-one-out requests (every N_x all but one) stay with the full
+// form.
 void prune_shape(mpt_ctx* c) {
   mpt::Shape& s = c->shape;
+  const mpt::Overlap& o = c->overlap;
   c->perm = mpt::InnerPerm{};
   s.pruned = s.prune_long = s.prune_pairs = s.prune_sort = false;
-  if (c->mode != MPT_DP_AUTO || !s.blocked || s.L < 1 || c->many_supports) return;
-  double members[32], tas[32];
-  for (int l = 0; l < s.L; ++l) members[l] = tas[l] = 1.0;
-  double time = 0.05 * (double)(1ull << s.L);
-  double full = 0.5;
-  for (int l = 0; l < s.L; ++l) full *= 3.0;
-  for (uint32_t N : c->supports) {
-    const uint32_t T = N & ((1u << s.L) - 1u), U = N >> s.L;
-    double above = 1.0, above2 = 1.0, here = 0.0;
-    for (int l = s.L - 1; l >= 0; --l) {
-      if (!((T >> l) & 1u)) continue;
-      members[l] += (double)(1ull << __builtin_popcount(U));
-      here += (double)(1ull << (s.L - 1 - l)) * above;
-      tas[l] += above2;
-      above *= 1.5;
-      above2 *= 2.0;
-    }
-    // of a full pair's time: the inner splits, at half its rate
-    double inner = 2.0;
-    for (int u = __builtin_popcount(U); u < s.b; ++u) inner *= 2.0 / 3.0;
-    time += here * (inner + 0.05 < 1.0 ? inner + 0.05 : 1.0);
-  }
-  const bool cheap = time < 0.7 * full;
-  const bool few = *std::max_element(members, members + s.L) <= (double)mpt::kPruneSelf;
-  if (!cheap && !few) return;
-  s.prune_most = *std::max_element(tas, tas + s.L);
+  if (c->mode != MPT_DP_AUTO || !s.blocked || s.L < 1 || o.out) return;
+  const bool cheap = o.cheap(), few = o.few();
+  s.n_shared = o.n_shared;
+  s.prune_most = *std::max_element(o.tas, o.tas + s.L);
   // Stored order of the inner bits: those of the N_x whose members cost most
   // (pairs times inner splits) first.  The first five are the in-row bits,
   // the next two tell the warps of a block apart, the last five its lanes.
   std::vector<std::pair<double, uint32_t>> cost;
   try {
-    for (uint32_t N : c->supports) {
+    for (uint32_t N : o.sets) {
       const uint32_t T = N & ((1u << s.L) - 1u), U = N >> s.L;
       double sum = 0.0, above = 1.0;
       for (int l = s.L - 1; l >= 0; --l)
@@ -167,15 +209,15 @@ void prune_shape(mpt_ctx* c) {
   // 0.2 ms of 1.0 on launches of the two that found nothing.
   double rows[32];
   for (int l = 0; l < s.L; ++l) rows[l] = 1.0;
-  for (uint32_t N : c->supports) {
+  for (uint32_t N : o.sets) {
     const double r = (double)(1ull << __builtin_popcount(c->perm.stored(N >> s.L) >> (s.wide ? 4 : 5)));
     for (int l = 0; l < s.L; ++l)
       if ((N >> l) & 1u) rows[l] += r;
   }
   if (!few || *std::max_element(rows, rows + s.L) > (double)mpt::kPruneRows)
-    mpt::prune_singles(s, c->perm, c->supports.data(), c->supports.size(), &s.prune_long, &s.prune_pairs);
+    mpt::prune_singles(s, c->perm, o.sets.data(), o.sets.size(), &s.prune_long, &s.prune_pairs);
   s.pruned = !s.prune_long || cheap;
-  s.prune_sort = time > mpt::kPruneSortPairs;
+  s.prune_sort = o.time > mpt::kPruneSortPairs;
   if (!s.pruned) {
     s.prune_long = s.prune_pairs = s.prune_sort = false;
     c->perm = mpt::InnerPerm{};
@@ -347,8 +389,8 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
   // exactly one request needs (per word, the bits seen once, s1, but not
   // twice, s2) and, for m >= 2, m times those that every request needs
   int64_t private_w = 0;
-  std::vector<uint32_t> supports;
-  bool many_supports = false;
+  mpt::Overlap overlap;
+  overlap.begin(m);
   for (int64_t j = 0; j < words; ++j) {
     uint64_t s1 = 0, s2 = 0, all = ~0ull;
     for (int i = 0; i < m; ++i) {
@@ -361,22 +403,20 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
     if (m >= 2)
       for (uint64_t v = all; v; v &= v - 1) private_w += (int64_t)m * weights[j * 64 + __builtin_ctzll(v)];
     // the other shared chunks' request sets (only instances with tile bits use them)
-    for (uint64_t v = s2 & ~all; v && m > mpt::blocked_tile_bits(m) && !many_supports; v &= v - 1) {
-      const int bit = __builtin_ctzll(v);
-      uint32_t N = 0;
-      for (int i = 0; i < m; ++i)
-        N |= (uint32_t)((req_bits[(size_t)i * (size_t)words + (size_t)j] >> bit) & 1u) << i;
-      try {
-        supports.push_back(N);
-      } catch (...) {
-        return MPT_ERR_OUT_OF_MEMORY;
-      }
-      many_supports = supports.size() > kMaxSupports;
+    const uint64_t shared = s2 & ~all;
+    if (shared == 0 || overlap.L < 1 || overlap.out) continue;
+    uint32_t N[64];
+    for (uint64_t v = shared; v; v &= v - 1) N[__builtin_ctzll(v)] = 0;
+    for (int i = 0; i < m; ++i)
+      for (uint64_t v = req_bits[(size_t)i * (size_t)words + (size_t)j] & shared; v; v &= v - 1)
+        N[__builtin_ctzll(v)] |= 1u << i;
+    try {
+      for (uint64_t v = shared; v; v &= v - 1) overlap.add(N[__builtin_ctzll(v)]);
+    } catch (...) {
+      return MPT_ERR_OUT_OF_MEMORY;
     }
   }
-  const int n_shared = (int)supports.size();  // (when not too many)
-  std::sort(supports.begin(), supports.end());
-  supports.erase(std::unique(supports.begin(), supports.end()), supports.end());
+  overlap.done();
   mpt_ctx* c = new (std::nothrow) mpt_ctx();
   if (!c) return MPT_ERR_OUT_OF_MEMORY;
   try {
@@ -392,9 +432,7 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
   c->shape.slots = slots;
   c->sum_w = sum;
   c->shared_w = sum - private_w;
-  c->shape.n_shared = n_shared;
-  c->supports = std::move(supports);
-  c->many_supports = many_supports;
+  c->overlap = std::move(overlap);
   refresh_shape(c);
   *out = c;
   return MPT_OK;
