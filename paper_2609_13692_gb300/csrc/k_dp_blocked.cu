@@ -950,17 +950,25 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
   return cudaSuccess;
 }
 
-cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
-  cudaError_t e = blocked_attributes(true);
-  if (e != cudaSuccess) return e;
-  const unsigned long long tiles = h_binom.v[s.L][kh], sms = (unsigned long long)sm_count();
-  const uint32_t P = (1u << (kh - 1)) - 1u;
-  // blocks for about four waves, and enough that a block's pairs fit its list
+// Blocks per tile of a layer's listed pairs: about four waves of them, and
+// enough that a block's pairs fit its list.
+unsigned long long listed_items(int L, int kh, unsigned long long sms) {
+  const unsigned long long tiles = h_binom.v[L][kh];
+  const unsigned long long P = (1ull << (kh - 1)) - 1ull;
   unsigned long long items = (4 * sms + tiles - 1) / tiles;
   const unsigned long long most = (P + kMinPairsPerItem - 1) / kMinPairsPerItem;
   const unsigned long long least = (P + kListCap - 1) / kListCap;
   if (items > most) items = most;
   if (items < least) items = least;
+  return items;
+}
+
+cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches) {
+  cudaError_t e = blocked_attributes(true);
+  if (e != cudaSuccess) return e;
+  const unsigned long long tiles = h_binom.v[s.L][kh];
+  const uint32_t P = (1u << (kh - 1)) - 1u;
+  const unsigned long long items = listed_items(s.L, kh, (unsigned long long)sm_count());
   const ListedPairs lp{ws.prune_info, ws.prune_long, ws.prune_n, reinterpret_cast<unsigned int*>(ws.counters + 2)};
   k_dp_pairs<true><<<(unsigned)(tiles * items), kPairThreads, kListedSmemBytes, stream>>>(
       ws.Gp, ws.Gc, ws.partial, s.L, kh, P, (uint32_t)items, 0u, ws.counters + 1, lp);

@@ -47,6 +47,9 @@
 // order 69.9 ms.
 #include "mpt_internal.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace mpt {
 namespace {
 
@@ -65,6 +68,7 @@ constexpr uint32_t kUnitSteps = 60;
 // ms, with 12,000 31.0, 9.9, 29.1, 34.9, 43.7, with 14,000 26.0, 9.4, 24.2, 34.9,
 // 43.6, with 17,000 25.7, 9.4, 24.2, 34.1, 50.0.
 constexpr uint32_t kLongSteps = 14000;
+constexpr double kFullPairSteps = 16600.0;
 constexpr int kPruneMinPairs = 16;     // pairs that a further block of a tile has to have
 
 // Shape of the kernel for 32-bit keys (rows of 32) and 64-bit keys (rows of
@@ -972,14 +976,14 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
 // The members of each single request's list by k_prune_tiles' rules: the
 // listed rows, members and cost of {l} bound those of every T that holds l.
 template <typename Key>
-void singles(int L, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs) {
+void singles(int L, const InnerPerm& perm, const uint32_t* sets, size_t n, bool* tiles, bool* pairs, double* costs) {
   using C = PrunedCfg<Key>;
   *tiles = *pairs = false;
-  for (int l = 0; l < L && !(*tiles && (*pairs || sizeof(Key) == 8)); ++l) {
+  for (int l = 0; l < L; ++l) {
     uint32_t row[C::kRows] = {1u};
     for (size_t i = 0; i < n; ++i)
-      if (supports[i] >> l & 1u) {
-        const uint32_t v = perm.stored(supports[i] >> L);
+      if (sets[i] >> l & 1u) {
+        const uint32_t v = perm.stored(sets[i] >> L);
         row[v >> C::kRB] |= 1u << (v & (C::kRow - 1));
       }
     static constexpr uint32_t kWithout[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
@@ -1000,28 +1004,8 @@ void singles(int L, const InnerPerm& perm, const uint32_t* supports, size_t n, b
     const bool many = rows > (uint32_t)kPruneRows, is_long = sizeof(Key) == 4 && (many || cost > kLongSteps);
     *pairs = *pairs || is_long;
     *tiles = *tiles || is_long || many || members > (uint32_t)kPruneSelf;
+    costs[l] = is_long ? kFullPairSteps : (double)cost;
   }
-}
-
-}  // namespace
-
-void prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs) {
-  if (s.wide)
-    singles<unsigned long long>(s.L, perm, supports, n, tiles, pairs);
-  else
-    singles<uint32_t>(s.L, perm, supports, n, tiles, pairs);
-}
-
-cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
-  const size_t cleared = kPruneSplitTiles + kMaxMembersL + 2 * kMaxMembersL * kPruneClasses;
-  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, cleared * 4, stream);
-  if (e != cudaSuccess) return e;
-  auto* lean = reinterpret_cast<unsigned int*>(ws.fw_rot);
-  auto* full = reinterpret_cast<unsigned long long*>(ws.wI_rot);
-  if (s.wide)
-    return s.lean ? tables<unsigned long long>(s, ws, lean, stream, launches)
-                  : tables<unsigned long long>(s, ws, full, stream, launches);
-  return s.lean ? tables<uint32_t>(s, ws, lean, stream, launches) : tables<uint32_t>(s, ws, full, stream, launches);
 }
 
 // Blocks per tile of a layer with 32-bit keys.  The pairs of a tile vary from
@@ -1035,6 +1019,142 @@ uint32_t pruned_items(const Shape& s, int kh) {
   const double P = (double)((1ull << (kh - 1)) - 1ull), most = P < s.prune_most ? P : s.prune_most;
   const double items = most / kPartPairs < kMostBlocks / tiles ? most / kPartPairs : kMostBlocks / tiles;
   return items < 1.0 ? 1u : (uint32_t)items;
+}
+
+// Whether the pruned recurrence is the faster one where some list or tile is
+// left to the pair and row kernels.  Each layer takes as long as its work over
+// all SMs or a block's part of its heaviest tile, whichever is more, in this
+// kernel and in the pair kernel, besides what the kernels of a layer take with
+// nothing to do; work in warp steps of the lists, on the 152 SMs of a GB300 (no
+// CUDA call is made here).  The lists of one Ta are the
+// sum over the sets N with Ta within N_T of the list of N alone (a product over
+// its bits, as k_prune_tiles counts it), less what the sets have in common: the
+// singles' lists are known, and with sum S and union e of those of {l}, and C
+// such that e = C (1 - exp(-S / C)), the n larger Ta's with lowest request l and
+// sum t over all of them are taken as n C (1 - exp(-t / (n C))).
+//
+// Constants (ms): fitted to solves of 2,300 instances of 13 to 28 requests whose
+// estimate matters (random sets of one density or size, few large ones, pooled
+// passages, uniform requests; both key widths): median error 0 to 6 %, 5 % to
+// 95 % of them within -27 .. +68 %.  Full solves: fitted to the same, from
+// below (m = 13 to 27: 0.13 .. 229 ms, 64-bit keys m = 13 to 24: 0.17 .. 62 ms).
+// Of the 801 of them that the pairs' estimate alone (Overlap in mpt_api.cu) would send
+// here, 240 were slower than the full form by more than 5 %, by up to 2.9 times
+// and, with 64-bit keys, which have no pair kernel for a heavy list, 14 times.
+// This rule takes 450 of them, one of which is (by 9 %), and leaves some 55
+// out that would be faster by more than 10 % (by up to 1.7 times).
+template <typename Key>
+bool pruned_pays(const Shape& s, const InnerPerm& perm, const uint32_t* sets, size_t n, const double* single,
+                 bool pairs) {
+  using C = PrunedCfg<Key>;
+  constexpr bool kWide = sizeof(Key) == 8;
+  // a warp step over all SMs and in one block, of a short list and in the pair kernel
+  constexpr double kStep[2] = {kWide ? 5e-9 : 2.4e-9, 2.4e-9}, kOwnStep[2] = {kWide ? 1.7e-6 : 7e-7, 3e-7};
+  const double per_solve = kWide ? 0.157 : pairs ? 0.077 : 0.112, per_layer = kWide ? 0.0247 : pairs ? 0.063 : 0.0302,
+               per_tile = kWide ? 1e-5 : pairs ? 2e-4 : 2.8e-5;
+  const int L = s.L;
+  double three = 1.0;
+  for (int l = 0; l < L; ++l) three *= 3.0;
+  const double full = kWide ? 0.06 + 0.11 * L + 1.08e-4 * three : 0.06 + 0.066 * L + 1.55e-5 * three;
+  auto choose = [](int a, int i) { return i < 0 || i > a ? 0.0 : (double)h_binom.v[a][i]; };
+  // sums of the sets' lists (short, long), by lowest request l of a Ta and requests of N_T above l
+  double sum[2][kMaxMembersL][kMaxMembersL] = {};
+  for (size_t q = 0; q < n; ++q) {
+    const uint32_t v = perm.stored(sets[q] >> L), row = v >> C::kRB;
+    const int in_row = __builtin_popcount(v & (C::kRow - 1)), lanes = __builtin_popcount(row & 31u),
+              warps = __builtin_popcount(row >> 5);
+    double cost = (double)C::kRow;
+    for (int i = 0; i < in_row; ++i) cost *= 1.5;
+    cost = (cost + kUnitSteps) * (double)(1u << lanes) * (double)(1u << C::kLogWarps);
+    for (int i = 0; i < warps; ++i) cost *= 1.5;
+    const bool is_long = !kWide && (lanes + warps > 5 || cost > kLongSteps);
+    int above = 0;
+    for (int l = L - 1; l >= 0; --l)
+      if (sets[q] >> l & 1u) sum[is_long][l][above++] += is_long ? kFullPairSteps : cost;
+  }
+  double layer[2][kMaxMembersL + 1] = {}, heaviest[2][kMaxMembersL + 1] = {};
+  for (int l = 0; l < L; ++l) {
+    const int A = L - 1 - l;
+    double S = 0.0;
+    for (int a = 0; a < L; ++a) S += sum[0][l][a] + sum[1][l][a];
+    const double e = single[l];
+    const bool e_long = !kWide && e >= kFullPairSteps;
+    double Cs = 0.0;  // 0: nothing in common
+    if (S > 0.0 && e < 0.999 * S) {
+      double lo = 1e-9, hi = S / e + 1.0;  // x = S / C: (1 - exp(-x)) / x falls from 1 to below e / S
+      for (int i = 0; i < 50; ++i) {
+        const double x = 0.5 * (lo + hi);
+        (-std::expm1(-x) / x > e / S ? lo : hi) = x;
+      }
+      Cs = S / lo;
+    }
+    // the lists (t[0] short, t[1] long) of `count` Ta's of i + 1 requests, at most `cap` of them above l
+    auto lists = [&](int i, int cap, double count, double* t) {
+      t[0] = t[1] = 0.0;
+      for (int a = i; a < L; ++a) {
+        const double c = choose(a < cap ? a : cap, i);
+        t[0] += sum[0][l][a] * c;
+        t[1] += sum[1][l][a] * c;
+      }
+      const double all = t[0] + t[1];
+      if (all == 0.0) return false;
+      if (Cs > 0.0 && count > 0.0) {
+        const double f = count * Cs * -std::expm1(-all / (count * Cs)) / all;
+        t[0] *= f;
+        t[1] *= f;
+      }
+      return true;
+    };
+    double t[2];
+    for (int i = 0; i <= A; ++i) {  // Ta = l and i more
+      if (i == 0) {
+        t[e_long] = e;
+        t[!e_long] = 0.0;
+      } else if (!lists(i, L, choose(A, i), t)) {
+        break;
+      }
+      for (int kh = i + 2; kh <= L && kh - 1 <= A; ++kh)
+        for (int q = 0; q < 2; ++q) layer[q][kh] += t[q] * choose(A - i, kh - 1 - i);
+    }
+    for (int kh = 2; kh - 1 <= A; ++kh) {
+      double v[2] = {e_long ? 0.0 : e, e_long ? e : 0.0};
+      for (int i = 1; i < kh - 1 && lists(i, kh - 1, choose(kh - 1, i), t); ++i) {
+        v[0] += t[0];
+        v[1] += t[1];
+      }
+      for (int q = 0; q < 2; ++q) heaviest[q][kh] = std::max(heaviest[q][kh], v[q]);
+    }
+  }
+  double ms = per_solve + per_layer * L + per_tile * (double)(1ull << L);
+  for (int kh = 2; kh <= L; ++kh) {
+    const double parts[2] = {(double)pruned_items(s, kh), (double)listed_items(L, kh, 152)};
+    for (int q = 0; q < 2; ++q) ms += std::max(kStep[q] * layer[q][kh], kOwnStep[q] * heaviest[q][kh] / parts[q]);
+  }
+  return 1.15 * ms < full;
+}
+
+}  // namespace
+
+bool prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* sets, size_t n, bool* tiles, bool* pairs) {
+  double costs[kMaxMembersL];
+  if (s.wide) {
+    singles<unsigned long long>(s.L, perm, sets, n, tiles, pairs, costs);
+    return !*tiles || pruned_pays<unsigned long long>(s, perm, sets, n, costs, *pairs);
+  }
+  singles<uint32_t>(s.L, perm, sets, n, tiles, pairs, costs);
+  return !*tiles || pruned_pays<uint32_t>(s, perm, sets, n, costs, *pairs);
+}
+
+cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches) {
+  const size_t cleared = kPruneSplitTiles + kMaxMembersL + 2 * kMaxMembersL * kPruneClasses;
+  cudaError_t e = cudaMemsetAsync(ws.prune_done, 0, cleared * 4, stream);
+  if (e != cudaSuccess) return e;
+  auto* lean = reinterpret_cast<unsigned int*>(ws.fw_rot);
+  auto* full = reinterpret_cast<unsigned long long*>(ws.wI_rot);
+  if (s.wide)
+    return s.lean ? tables<unsigned long long>(s, ws, lean, stream, launches)
+                  : tables<unsigned long long>(s, ws, full, stream, launches);
+  return s.lean ? tables<uint32_t>(s, ws, lean, stream, launches) : tables<uint32_t>(s, ws, full, stream, launches);
 }
 
 // Whether the blocks of a layer meet in `partial`.

@@ -157,11 +157,12 @@ bool use_wide(const mpt_ctx* c) {
 }
 
 // Whether a one-shot AUTO solve takes the pruned recurrence (k_dp_pruned.cu),
-// from the sets N_x alone: where the pairs' times estimated by Overlap are
-// below 0.7 of the full recurrence's, or no request's members exceed the
-// limits of a short list, so that the pair and row kernels are not launched
-// at all.  Leave-one-out requests (every N_x all but one) stay with the full
-// form.
+// from the sets N_x alone: where no list is long, so that the pair and row
+// kernels are not launched at all, and where the layers' times estimated from
+// the lists are below the full recurrence's (pruned_pays).  Instances whose
+// pairs alone, estimated by Overlap, take more than 0.7 of the full ones, and
+// whose members may exceed a short list, are not looked at any further;
+// leave-one-out requests (every N_x all but one) are among them.
 void prune_shape(mpt_ctx* c) {
   mpt::Shape& s = c->shape;
   const mpt::Overlap& o = c->overlap;
@@ -214,9 +215,10 @@ void prune_shape(mpt_ctx* c) {
     for (int l = 0; l < s.L; ++l)
       if ((N >> l) & 1u) rows[l] += r;
   }
+  s.pruned = true;
   if (!few || *std::max_element(rows, rows + s.L) > (double)mpt::kPruneRows)
-    mpt::prune_singles(s, c->perm, o.sets.data(), o.sets.size(), &s.prune_long, &s.prune_pairs);
-  s.pruned = !s.prune_long || cheap;
+    s.pruned = mpt::prune_singles(s, c->perm, o.sets.data(), o.sets.size(), &s.prune_long, &s.prune_pairs);
+  s.pruned = s.pruned && (!s.prune_long || cheap);
   s.prune_sort = o.time > mpt::kPruneSortPairs;
   if (!s.pruned) {
     s.prune_long = s.prune_pairs = s.prune_sort = false;

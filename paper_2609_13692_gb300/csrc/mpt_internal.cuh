@@ -345,8 +345,8 @@ cudaError_t launch_dp_blocked(const Shape& s, const Workspace& ws, cudaStream_t 
 // The same over the members only (k_dp_pruned.cu): lists, then every step.
 // Whether the lists of the single tile requests, which hold those of all other
 // Ta's, leave any tile to the row kernel (*tiles) or any list to the pair
-// kernel (*pairs).
-void prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* supports, size_t n, bool* tiles, bool* pairs);
+// kernel (*pairs); false when the full recurrence is then the faster one.
+bool prune_singles(const Shape& s, const InnerPerm& perm, const uint32_t* sets, size_t n, bool* tiles, bool* pairs);
 cudaError_t launch_dp_pruned(const Shape& s, const Workspace& ws, cudaStream_t stream, int* launches,
                              BlockedTiming* timing);
 // w(I) (instead of K2) and the lists; needs K1's list of shared chunks.
@@ -354,6 +354,7 @@ cudaError_t launch_prune_tables(const Shape& s, const Workspace& ws, cudaStream_
 // Step kh over its long lists only: the 32-bit pair kernel, and the row kernels
 // of either key width on tiles with a long list.
 cudaError_t launch_listed_pairs(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
+unsigned long long listed_items(int L, int kh, unsigned long long sms);  // its blocks per tile
 cudaError_t launch_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
 cudaError_t launch_wide_listed_tiles(const Shape& s, const Workspace& ws, int kh, cudaStream_t stream, int* launches);
 // Tile 0 with either key width (k_dp_tile0.cu).

@@ -290,3 +290,43 @@ def test_batch_members_of_many_groups(mpt, m):
         pF, ps, _ = mpt.mpt_batch_tables(part)
         assert list(o) == list(opt[k:k + 800]) and p == perms[k:k + 800] and d == orders[k:k + 800]
         assert torch.equal(pF, F[k << m:(k + 800) << m]) and torch.equal(ps, split[k << m:(k + 800) << m])
+
+
+def _heavy_sets(m, size, count, seed):
+    rng = np.random.default_rng(seed)
+    sets = [_mask(*(int(i) for i in rng.choice(m, size=size, replace=False))) for _ in range(count)]
+    pairs = [_mask(*(int(i) for i in rng.choice(m, size=2, replace=False))) for _ in range(30)]
+    return _from_supports(m, sets + pairs, seed)
+
+
+@pytest.mark.parametrize("m,size,count,scale", [(19, 17, 1, 1 << 12), (20, 15, 3, 1 << 12), (22, 18, 2, 1 << 12),
+                                                (20, 14, 4, 1), (21, 15, 2, 1)])
+def test_heavy_lists_stay_with_the_full_recurrence(mpt, m, size, count, scale):
+    """A few chunks that most requests hold: lists so long that the full
+    recurrence is the faster one (the pruned one took two to ten times as
+    long): AUTO launches what the full form launches."""
+    inst = _heavy_sets(m, size, count, m + size)
+    w = inst.weights * scale
+    got = [mpt.mpt_get_profile(mpt.solve(w, inst.bits, mode=mode, profile=True).ctx)
+           for mode in ("auto", "wide" if scale > 1 else "blocked")]
+    assert got[0]["launches_total"] == got[1]["launches_total"]
+    assert got[0]["splits_pairs"] == got[1]["splits_pairs"] > 0
+
+
+@pytest.mark.parametrize("scale", [1, 1 << 21])
+def test_long_lists_of_a_pruned_solve_in_a_fresh_process(mpt, scale):
+    """As test_long_lists_in_a_fresh_process, on an instance large enough that
+    its long lists do not send it to the full recurrence."""
+    sets = "_mask(*range(0, 24, 2)) | _mask(1, 3, 5, 7, 9), _mask(*range(0, 12)), _mask(2, 13), _mask(0, *range(12, 24)), _mask(3, 20)"
+    code = ("import numpy as np; from tests.test_pruned_gpu import _from_supports, _mask\n"
+            "from paper_2609_13692_gb300 import mpt\n"
+            f"inst = _from_supports(24, [{sets}], 8)\n"
+            f"r = mpt.solve(inst.weights * {scale}, inst.bits, profile=True)\n"
+            "print(r.opt, mpt.mpt_get_profile(r.ctx)['launches_total'])")
+    root = Path(__file__).resolve().parent.parent
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    opt, launches = (int(x) for x in r.stdout.split())
+    inst = _from_supports(24, eval(f"[{sets}]"), 8)
+    full = mpt.solve(inst.weights * scale, inst.bits, mode="wide" if scale > 1 else "blocked", profile=True)
+    assert opt == full.opt and launches != mpt.mpt_get_profile(full.ctx)["launches_total"]
