@@ -17,22 +17,30 @@
 // merge in the same round.  A merge's key is above every key it leaves behind,
 // so the greedy sequence is the merges of all rounds in decreasing key order.
 // Once no pair shares weight, the rest is forced: the smallest slot takes in
-// the others in increasing order, with empty signatures.  3,000 requests need
-// 19 rounds.  The merges one after the other in one block took 25.7 of the
-// 27.6 ms of a call (8.6 us each: some twenty block barriers); the rounds
-// take 0.9 ms, bound by their launches and the latency of the row scans.
+// the others in increasing order, with empty signatures.  3,000 requests of 8
+// passages from pools of 60 need 19 rounds.  The merges one after the other in
+// one block took 25.7 of the 27.6 ms of a call (8.6 us each: some twenty block
+// barriers); the rounds take 0.9 ms, bound by their launches and the latency of
+// the row scans.
+//
+// Where one passage is in every request, or weights are equal, pairs tie and the
+// slot order lets one or two merge per round: what is left then goes to one
+// block (k_merge_rest).  3,000 requests with nothing in common but one passage:
+// 96 ms in rounds alone, 14.4 so (22.9 in one block from the start); 12,000 of
+// them 1,755 and 165 ms (319).
 //
 // Kernels: k_pair_weights fills W[i][j] = w(R_i cap R_j); Borůvka rounds find
 // the maximum spanning tree of W; k_row_best, k_match and k_reweigh are one
-// round of merges; k_rank orders them; k_tail appends the forced ones;
-// k_count and k_leaf_order give the left-to-right leaf order; k_greedy_emit
-// climbs each (request, chunk) occurrence to the highest node whose signature
-// still holds the chunk, and k_greedy_rank orders each request's chunks by
-// (that node, chunk id).
+// round of merges, k_merge_rest merges one by one; k_rank orders them; k_tail
+// appends the forced ones; k_count and k_leaf_order give the left-to-right leaf
+// order; k_greedy_emit climbs each (request, chunk) occurrence to the highest
+// node whose signature still holds the chunk, and k_greedy_rank orders each
+// request's chunks by (that node, chunk id).
 #include "../../include/mpt.h"
 #include "mpt_internal.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 namespace mpt {
@@ -214,9 +222,10 @@ __global__ void k_slots_init(Slots s, int32_t* __restrict__ comp, unsigned long 
 }
 
 // Round 1 of 3: the best pair of every slot that needs looking for (all in the
-// first round; then those that merged, or whose best partner did: other
-// keys only fell).  Block per slot: a slot's scan is a chain of loads, and few
-// slots have one, so the threads of a block share it.
+// first round; then those that merged, or whose best partner did, unless it
+// kept its slot and their pair its weight: other keys only fell).  Block per
+// slot: a slot's scan is a chain of loads, and few slots have one, so the
+// threads of a block share it.
 constexpr int kBestThreads = 128;
 __global__ void __launch_bounds__(kBestThreads) k_row_best(Slots s, int round) {
   __shared__ unsigned long long warp_best[kBestThreads / 32];
@@ -230,7 +239,8 @@ __global__ void __launch_bounds__(kBestThreads) k_row_best(Slots s, int round) {
       if (k == 0) continue;
       uint32_t a, b;
       key_pair(k, &a, &b);
-      if (s.mark[(int)a == d ? b : a] != round - 1) continue;
+      const uint32_t p = (int)a == d ? b : a;
+      if (s.mark[p] != round - 1 || (s.act[p] && s.W[(size_t)d * s.m + p] == (uint32_t)(k >> 28))) continue;
     }
     unsigned long long best = 0;
     const uint32_t* row = s.W + (size_t)d * s.m;
@@ -334,6 +344,185 @@ __global__ void __launch_bounds__(256) k_reweigh(Slots s, const int64_t* __restr
       }
     }
   }
+}
+
+// The remaining merges one after the other, in one block.  best[d] is an upper
+// bound on slot d's best key (keys only fall), kept in shared memory as sb,
+// with gmax[g] the largest of sb[32 g .. 32 g + 31].  The largest key is merged
+// only if it is still exact; otherwise the rows of its two slots are scanned
+// again and the search repeats.  2 to 5 us a merge up to 3,000 requests with
+// signatures of 8 chunks, mostly barriers; with 100 chunks (nested requests) 54
+// us, 70 with a thread per other slot instead of kShare.
+constexpr int kMaxGroups = kMaxGreedyM / 32;
+constexpr int kNoRounds = 32, kFewRounds = 64;  // requests
+constexpr int kShare = 16;
+size_t rest_smem_bytes(int m) { return (size_t)m * 8 + (size_t)kMaxGroups * 8 + (size_t)m * 2 + (size_t)m; }
+
+__device__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* red) {
+  for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = lane < kGreedyThreads / 32 ? red[lane] : 0ull;
+    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+    if (lane == 0) red[32] = v;
+  }
+  __syncthreads();
+  const unsigned long long r = red[32];
+  __syncthreads();
+  return r;
+}
+
+__global__ void __launch_bounds__(kGreedyThreads) k_merge_rest(Slots s, const int64_t* __restrict__ w) {
+  extern __shared__ __align__(16) unsigned char gsm[];
+  unsigned long long* sb = reinterpret_cast<unsigned long long*>(gsm);  // [m]
+  unsigned long long* gmax = sb + s.m;                                  // [kMaxGroups]
+  uint16_t* live = reinterpret_cast<uint16_t*>(gmax + kMaxGroups);      // [m]
+  uint8_t* act = reinterpret_cast<uint8_t*>(live + s.m);                // [m]
+  __shared__ int live_n;
+  __shared__ unsigned long long red[33];
+  __shared__ int32_t s_b[kSigMax], s_new[kSigMax];
+  __shared__ int warp_n[kSigMax / 32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, m = s.m, groups = (m + 31) / 32;
+  // the largest of a group's bounds; by the first warp
+  auto refresh = [&](int g) {
+    if (t < 32) {
+      const int d = g * 32 + t;
+      unsigned long long v = d < m ? sb[d] : 0ull;
+      for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+      if (t == 0) gmax[g] = v;
+    }
+  };
+  auto rescan = [&](int d) {
+    unsigned long long best = 0;
+    const uint32_t* row = s.W + (size_t)d * m;
+    for (int e0 = t; e0 < m; e0 += kGreedyThreads * 4) {
+      uint32_t v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) v[q] = e0 + kGreedyThreads * q < m ? row[e0 + kGreedyThreads * q] : 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e = e0 + kGreedyThreads * q;
+        if (v[q] != 0 && act[e]) best = max(best, pair_key((uint32_t)d, (uint32_t)e, v[q]));
+      }
+    }
+    best = block_max_u64(best, red);
+    if (t == 0) sb[d] = best;
+    __syncthreads();
+    refresh(d >> 5);
+  };
+  for (int d = t; d < m; d += kGreedyThreads) {
+    act[d] = s.act[d];
+    sb[d] = s.act[d] ? s.best[d] : 0ull;
+  }
+  __syncthreads();
+  for (int g = warp; g < groups; g += kGreedyThreads / 32) {
+    const int d = g * 32 + lane;
+    unsigned long long v = d < m ? sb[d] : 0ull;
+    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+    if (lane == 0) gmax[g] = v;
+  }
+  __syncthreads();
+  int r = s.counts[0];
+  for (int tries = 0; r < m - 1 && tries <= m;) {  // a rescan makes a row exact: at most m between two merges
+    const unsigned long long top = block_max_u64(t < groups ? gmax[t] : 0ull, red);
+    if (top == 0) break;  // no pair shares weight
+    uint32_t a, b;
+    key_pair(top, &a, &b);
+    if (!act[a] || !act[b] || s.W[(size_t)a * m + b] != (uint32_t)(top >> 28)) {
+      ++tries;
+      if (act[a]) rescan((int)a);
+      if (act[b]) rescan((int)b);
+      __syncthreads();
+      continue;
+    }
+    tries = 0;
+    // merged signature: the chunks of a that b holds, in order
+    const int la = s.len[a], lb = s.len[b];
+    int32_t* sa = s.sig + s.off[a];
+    const int32_t x = t < la ? sa[t] : 0;
+    if (t < lb) s_b[t] = s.sig[s.off[b] + t];
+    __syncthreads();
+    const bool keep = t < la && find_in(s_b, lb, x) >= 0;
+    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+    if (lane == 0 && warp < kSigMax / 32) warp_n[warp] = __popc(bal);
+    __syncthreads();
+    int ln = 0;
+    for (int q = 0; q < kSigMax / 32; ++q) ln += warp_n[q];
+    if (keep) {
+      int o = __popc(bal & ((1u << lane) - 1u));
+      for (int q = 0; q < warp; ++q) o += warp_n[q];
+      s_new[o] = x;
+    }
+    __syncthreads();
+    if (t < ln) {
+      sa[t] = s_new[t];
+      s.rec_sig[(size_t)r * kSigMax + t] = s_new[t];
+    }
+    if (t == 0) {
+      s.len[a] = ln;
+      s.rec_len[r] = ln;
+      s.rec_key[r] = top;
+      s.rec_child[r] = make_int2(s.top[a], s.top[b]);
+      s.top[a] = r;
+      s.act[b] = act[b] = 0;
+      sb[b] = 0;
+    }
+    __syncthreads();
+    // its weights (zero where either slot's was), and its best pair on the way;
+    // with long signatures, kShare threads per other slot
+    unsigned long long best = 0;
+    auto put = [&](int d, uint32_t wa, uint32_t v) {
+      if (v != wa) {
+        s.W[(size_t)a * m + d] = v;
+        s.W[(size_t)d * m + a] = v;
+      }
+      if (v != 0) best = max(best, pair_key(a, (uint32_t)d, v));
+    };
+    auto shared_weight = [&](int d, int first, int step) {
+      const int32_t* sd = s.sig + s.off[d];
+      const int ld = s.len[d];
+      uint32_t v = 0;
+      for (int q = first; q < ld; q += step) {
+        const int32_t x = sd[q];
+        if (find_in(s_new, ln, x) >= 0) v += (uint32_t)w[x];
+      }
+      return v;
+    };
+    if (t == 0) live_n = 0;
+    __syncthreads();
+    for (int d = t; d < m; d += kGreedyThreads) {
+      const uint32_t wa = s.W[(size_t)a * m + d];
+      if (wa == 0 || !act[d]) continue;
+      if (s.W[(size_t)b * m + d] == 0)
+        put(d, wa, 0u);
+      else if (ln <= kShare)
+        put(d, wa, shared_weight(d, 0, 1));
+      else
+        live[atomicAdd(&live_n, 1)] = (uint16_t)d;
+    }
+    if (ln > kShare) {
+      __syncthreads();
+      for (int i0 = 0; i0 < live_n; i0 += kGreedyThreads / kShare) {
+        const int i = i0 + t / kShare;
+        uint32_t v = i < live_n ? shared_weight(live[i], t % kShare, kShare) : 0u;
+        for (int off = 1; off < kShare; off <<= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+        if (i < live_n && t % kShare == 0) put(live[i], s.W[(size_t)a * m + live[i]], v);
+      }
+    }
+    best = block_max_u64(best, red);
+    if (t == 0) sb[a] = best;
+    __syncthreads();
+    refresh((int)a >> 5);
+    if ((b >> 5) != (a >> 5)) {
+      __syncthreads();
+      refresh((int)b >> 5);
+    }
+    __syncthreads();
+    ++r;
+  }
+  if (t == 0) s.counts[0] = r;
 }
 
 // ---------------------------------------------------------------------------
@@ -614,27 +803,34 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
     }
     e = cudaGetLastError();
   }
-  // Rounds of merges, `ahead` enqueued between two looks at whether the last one
-  // still merged anything (each does, until no pair shares weight; later ones
-  // return at once).  Few requests need few: with 12 for all, 20 requests took
-  // 501 us, now 445.
-  int ahead = 2;
-  while (ahead < 12 && (4 << ahead) < 4 * 4 * m) ++ahead;  // 2 + log2(m), at most 12
-  if (ahead > m) ahead = m;
+  // Rounds of merges, `ahead` enqueued between two looks at what they merged
+  // (nothing, once no pair shares weight; later rounds return at once).  Where
+  // keys tie or wait for one another a round merges a pair or two, and the rest
+  // goes to one block (2 to 5 us a merge with signatures of 8 chunks, a round 9
+  // us).  Few requests go there at once, or after a few rounds without a look.
+  const int ahead = m <= kNoRounds ? 0 : m <= kFewRounds ? 4 : std::min(12, 2 + (int)std::log2((double)m));
   int32_t counts[3] = {0, 0, 0};
-  for (int round = 0; e == cudaSuccess && m > 1;) {
+  bool rest = m <= kFewRounds;
+  for (int round = 0, merged = 0; e == cudaSuccess && m > 1; merged = counts[0]) {
     for (int k = 0; k < ahead; ++k, ++round) {
       k_row_best<<<(unsigned)m, kBestThreads, 0, stream>>>(sl, round);
       k_match<<<wb, 256, 0, stream>>>(sl, round);
       k_reweigh<<<(unsigned)std::min<int64_t>(m, sms * 4), 256, 0, stream>>>(sl, I64(o_w), round);
     }
+    if (ahead == 0) k_row_best<<<(unsigned)m, kBestThreads, 0, stream>>>(sl, 0);
     e = cudaGetLastError();
+    if (rest) break;
     if (e == cudaSuccess) e = cudaMemcpyAsync(counts, ctl, 12, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (counts[0] == counts[1 + ((round - 1) & 1)]) break;
-    if (round > m + 2 * ahead) {  // every round before the last merges
-      if (e == cudaSuccess) st = MPT_ERR_INTERNAL;
-      break;
+    if (e != cudaSuccess || counts[0] == counts[1 + ((round - 1) & 1)]) break;
+    rest = 2 * (counts[0] - merged) < 5 * ahead;
+    if (rest) break;
+  }
+  if (e == cudaSuccess && rest && m > 1) {
+    e = cudaFuncSetAttribute(k_merge_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rest_smem_bytes(m));
+    if (e == cudaSuccess) {
+      k_merge_rest<<<1, kGreedyThreads, rest_smem_bytes(m), stream>>>(sl, I64(o_w));
+      e = cudaGetLastError();
     }
   }
   if (e == cudaSuccess && st == MPT_OK) {
