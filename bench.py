@@ -477,17 +477,11 @@ def run_ours(args):
             c3 = mpt.mpt_create(inst.weights, inst.bits)
             if args.tables != "int64":
                 mpt.mpt_set_tables(c3, args.tables)
-            need = mpt.mpt_workspace_bytes(c3)
-            opt = mpt.mpt_solve(c3, ws if ws.numel() >= need else auto_ws[0], stream.cuda_stream)
+            opt = mpt.mpt_solve(c3, ws, stream.cuda_stream)
             mpt.mpt_layout(c3)
             mpt.mpt_destroy(c3)
             return opt
 
-        c3 = mpt.mpt_create(inst.weights, inst.bits)
-        if args.tables != "int64":
-            mpt.mpt_set_tables(c3, args.tables)
-        auto_ws = [torch.empty(mpt.mpt_workspace_bytes(c3), dtype=torch.uint8, device=device)]
-        mpt.mpt_destroy(c3)
         for _ in range(3):
             assert auto_pass() == opts[-1]
         torch.cuda.synchronize()

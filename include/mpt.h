@@ -86,7 +86,12 @@ mpt_status mpt_create(const int64_t* weights, int64_t n_chunks, const uint64_t* 
 /* Bytes of device workspace mpt_solve needs for this context: the input
  * copies, the intersection-weight table wI int64[2^m], F int64[2^m],
  * split uint32[2^m], the blocked DP's working tables, the layout buffers and,
- * under AUTO, the lists of the splits that are looked at. */
+ * with tables in tiles (m > 12), room at the end for the lists of the splits
+ * that AUTO looks at.  The size follows from n_chunks, m, sum_i |R_i|, the key
+ * width, the table layout and whether the GENERAL kernels run, not from which
+ * chunks the requests share: requests of one shape fit one workspace.  Staged
+ * solves, mpt_solve under BLOCKED and WIDE, and under AUTO when it looks at
+ * every split, do not use that room and take a workspace without it. */
 mpt_status mpt_workspace_bytes(const mpt_ctx* ctx, size_t* bytes);
 
 /* Choose the DP kernels (default MPT_DP_AUTO).  BLOCKED is refused with

@@ -15,8 +15,6 @@
 
 namespace mpt {
 
-constexpr int kMaxShared = 8192;  // chunks that some but not all requests share, in a pruned solve
-
 // The request sets N_x of the chunks that some but not all requests share, and
 // the bounds on a pruned solve (k_dp_pruned.cu) that follow set by set.  Its
 // members are the parts of some N_x, so with N = (N_T, N_U) the tile and inner
@@ -236,6 +234,7 @@ void refresh_shape(mpt_ctx* c) {
   s.partial_entries = !s.blocked ? 0
                       : s.wide   ? (mpt::wide_partial_slots(s.m, s.b) << s.b)
                                  : mpt::blocked_partial_entries(s.m, s.b);
+  s.prune_room = s.blocked && s.L >= 1;
   prune_shape(c);
 }
 
@@ -320,9 +319,11 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
   ws->prune_rows = nullptr;
   ws->shared_N = nullptr;
   ws->shared_w = nullptr;
-  if (s.pruned) {
+  if (s.prune_room) {
+    // by the shape alone, so that requests of one shape fit one workspace,
+    // however they overlap: a shared chunk has two occurrences or more
     const size_t P = (size_t)1 << s.L;
-    const size_t ns = (size_t)(s.n_shared > 0 ? s.n_shared : 1);
+    const size_t ns = std::min(slots / 2 + 1, (size_t)mpt::kMaxShared);
     ws->shared_N = reinterpret_cast<uint32_t*>(take(ns * 4));
     ws->shared_w = reinterpret_cast<unsigned long long*>(take(ns * 8));
     ws->prune_info = reinterpret_cast<uint32_t*>(take(P * 4));
@@ -492,9 +493,12 @@ static float elapsed(cudaEvent_t a, cudaEvent_t b) {
 namespace {
 
 // Resolve the workspace of a solve (the caller's, or one the context owns)
-// and carve it.
-mpt_status bind_workspace(mpt_ctx* c, void* d_workspace, size_t workspace_bytes, mpt::Workspace* ws, char** base) {
-  const mpt::Shape& s = c->shape;
+// and carve it.  lists: the solve is a pruned one; others also take a
+// caller's workspace that ends in front of the room for its lists.
+mpt_status bind_workspace(mpt_ctx* c, bool lists, void* d_workspace, size_t workspace_bytes, mpt::Workspace* ws,
+                          char** base) {
+  mpt::Shape s = c->shape;
+  s.prune_room = s.prune_room && (lists || !d_workspace);
   const size_t need = mpt::carve_workspace(s, nullptr, ws);
   if (d_workspace) {
     if (workspace_bytes < need) return MPT_ERR_WORKSPACE_TOO_SMALL;
@@ -615,7 +619,7 @@ mpt_status mpt_solve(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes, vo
 
   mpt::Workspace ws{};
   char* base = nullptr;
-  mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
+  mpt_status st = bind_workspace(c, s.pruned, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
 
   // events: 7 stage marks + 2 per blocked-DP launch
@@ -700,7 +704,7 @@ mpt_status mpt_solve_begin(mpt_ctx* ctx, void* d_workspace, size_t workspace_byt
   c->err.clear();
   mpt::Workspace ws{};
   char* base = nullptr;
-  mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
+  mpt_status st = bind_workspace(c, false, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   int launches = 0;
   if ((st = run_front(c, c->shape, ws, false, base, stream, &launches, nullptr)) != MPT_OK) return st;
@@ -717,7 +721,7 @@ mpt_status mpt_solve_resume(mpt_ctx* ctx, void* d_workspace, size_t workspace_by
   if (next_step < 1 || next_step > mpt::dp_steps(c->shape)) return MPT_ERR_INVALID_ARG;
   mpt::Workspace ws{};
   char* base = nullptr;
-  mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
+  mpt_status st = bind_workspace(c, false, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   c->solved = false;
   c->resident = base;  // a checkpoint carries the input copies with it
@@ -733,7 +737,7 @@ mpt_status mpt_solve_layers(mpt_ctx* ctx, void* d_workspace, size_t workspace_by
   if (c->staged_next < 0) return MPT_ERR_NOT_SOLVED;
   mpt::Workspace ws{};
   char* base = nullptr;
-  mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
+  mpt_status st = bind_workspace(c, false, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   if (base != c->staged_base) return MPT_ERR_INVALID_ARG;
   const int total = mpt::dp_steps(c->shape);
@@ -753,7 +757,7 @@ mpt_status mpt_solve_end(mpt_ctx* ctx, void* d_workspace, size_t workspace_bytes
   if (c->staged_next < 0 || c->staged_next != mpt::dp_steps(c->shape)) return MPT_ERR_NOT_SOLVED;
   mpt::Workspace ws{};
   char* base = nullptr;
-  mpt_status st = bind_workspace(c, d_workspace, workspace_bytes, &ws, &base);
+  mpt_status st = bind_workspace(c, false, d_workspace, workspace_bytes, &ws, &base);
   if (st != MPT_OK) return st;
   if (base != c->staged_base) return MPT_ERR_INVALID_ARG;
   int launches = 0;

@@ -283,7 +283,8 @@ struct Shape {
   int64_t partial_entries;
   InnerPerm perm;   // of the tables of this solve
   bool pruned;      // one-shot solves run the pruned recurrence (k_dp_pruned.cu)
-  int n_shared;       // chunks that some (two or more) but not all requests share
+  bool prune_room;  // the workspace has room for its lists
+  int n_shared;       // chunks that some (two or more) but not all requests share (pruned)
   double prune_most;  // the host's bound on the pairs of one tile
   bool prune_long;  // some list may be long, or some tile left to the row kernel
   bool prune_pairs; // some list may be long (32-bit keys)
@@ -294,6 +295,7 @@ struct Shape {
 // that the pruned kernel finishes itself, the most tiles of a layer that is
 // cut into several blocks per tile, and the flags of a list.
 constexpr int kPruneRows = 32;
+constexpr int kMaxShared = 8192;  // chunks that some but not all requests share, at most
 constexpr int kPruneSelf = 128;
 constexpr int kPruneSplitTiles = 16384;
 constexpr int kMaxMembersL = 32;
