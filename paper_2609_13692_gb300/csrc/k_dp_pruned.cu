@@ -57,6 +57,7 @@ constexpr int kPB = 12;  // inner bits of a tile
 constexpr uint32_t kPMask = (1u << kPB) - 1u;
 constexpr int kPQueue = 512;     // pairs queued between two rounds of evaluation
 constexpr int kQueueShift = 20;  // queue entries: Ta below (L <= 20), rows above
+static_assert(kPruneClasses <= 256, "classes are kept in bytes");
 static_assert(256 < 1 << (32 - kQueueShift), "queue entries hold the row count");
 constexpr int kRowBytes = 128;
 constexpr int kMembersShift = 9;  // info: rows below, members above
@@ -305,18 +306,20 @@ __device__ __forceinline__ int work_class(uint32_t T, int n, const uint32_t* __r
 
 __global__ void __launch_bounds__(256)
 k_prune_classes(int L, int n_shared, const uint32_t* __restrict__ N, const int32_t* __restrict__ counters,
-                uint32_t* __restrict__ hist) {
+                uint32_t* __restrict__ hist, uint8_t* __restrict__ cls) {
   const int n = min(counters[3], n_shared);
-  for (uint32_t T = 1 + blockIdx.x * blockDim.x + threadIdx.x; T < (1u << L); T += gridDim.x * blockDim.x)
-    atomicAdd(&hist[__popc(T) * kPruneClasses + work_class(T, n, N)], 1u);
+  for (uint32_t T = 1 + blockIdx.x * blockDim.x + threadIdx.x; T < (1u << L); T += gridDim.x * blockDim.x) {
+    const int c = work_class(T, n, N);
+    cls[T] = (uint8_t)c;
+    atomicAdd(&hist[__popc(T) * kPruneClasses + c], 1u);
+  }
 }
 
 __global__ void __launch_bounds__(256)
-k_prune_order(int L, int n_shared, const uint32_t* __restrict__ N, const int32_t* __restrict__ counters,
-              const uint32_t* __restrict__ hist, uint32_t* __restrict__ placed, uint32_t* __restrict__ order) {
-  const int n = min(counters[3], n_shared);
+k_prune_order(int L, const uint8_t* __restrict__ cls, const uint32_t* __restrict__ hist,
+              uint32_t* __restrict__ placed, uint32_t* __restrict__ order) {
   for (uint32_t T = 1 + blockIdx.x * blockDim.x + threadIdx.x; T < (1u << L); T += gridDim.x * blockDim.x) {
-    const int kh = __popc(T), c = work_class(T, n, N);
+    const int kh = __popc(T), c = cls[T];  // as counted: the order is a permutation whatever the estimate
     uint32_t at = 0;
     for (int k = 0; k < kh; ++k) at += (uint32_t)c_binom.v[L][k];
     for (int q = 0; q < c; ++q) at += hist[kh * kPruneClasses + q];
@@ -908,9 +911,9 @@ cudaError_t tables(const Shape& s, const Workspace& ws, G* wIr, cudaStream_t str
   if (s.prune_sort) {
     const unsigned blocks = (unsigned)(tiles / 256 + 1 < sm_count() * 4 ? tiles / 256 + 1 : sm_count() * 4);
     uint32_t* placed = ws.prune_hist + kMaxMembersL * kPruneClasses;
-    k_prune_classes<<<blocks, 256, 0, stream>>>(s.L, s.n_shared, ws.shared_N, ws.counters, ws.prune_hist);
-    k_prune_order<<<blocks, 256, 0, stream>>>(s.L, s.n_shared, ws.shared_N, ws.counters, ws.prune_hist, placed,
-                                              ws.prune_order);
+    k_prune_classes<<<blocks, 256, 0, stream>>>(s.L, s.n_shared, ws.shared_N, ws.counters, ws.prune_hist,
+                                                ws.prune_class);
+    k_prune_order<<<blocks, 256, 0, stream>>>(s.L, ws.prune_class, ws.prune_hist, placed, ws.prune_order);
     *launches += 2;
   }
   return cudaGetLastError();

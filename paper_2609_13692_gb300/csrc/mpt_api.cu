@@ -316,6 +316,7 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
   ws->opt = reinterpret_cast<int64_t*>(take(mpt::kOptBytes));
   // after everything else, so that the rest sits where it does without them
   ws->prune_info = ws->prune_short = ws->prune_long = ws->prune_n = ws->prune_done = ws->prune_hist = ws->prune_order = nullptr;
+  ws->prune_class = nullptr;
   ws->prune_rows = nullptr;
   ws->shared_N = nullptr;
   ws->shared_w = nullptr;
@@ -335,6 +336,7 @@ size_t carve_workspace(const Shape& s, char* base, Workspace* ws) {
     ws->prune_done = reinterpret_cast<uint32_t*>(take((mpt::kPruneSplitTiles + mpt::kMaxMembersL + hist) * 4));
     ws->prune_hist = ws->prune_done ? ws->prune_done + mpt::kPruneSplitTiles + mpt::kMaxMembersL : nullptr;
     ws->prune_order = reinterpret_cast<uint32_t*>(take(P * 4));
+    ws->prune_class = reinterpret_cast<uint8_t*>(take(P));
   }
   return off;
 }

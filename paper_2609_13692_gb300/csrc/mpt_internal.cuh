@@ -242,6 +242,7 @@ struct Workspace {
   uint32_t* prune_n;      // [2 * kMaxMembersL] their numbers per lowest request
   uint32_t* prune_done;   // [kPruneSplitTiles] finished parts of each tile of a layer; [kMaxMembersL] units taken per layer
   uint32_t* prune_hist;   // [2 * kMaxMembersL * kPruneClasses] tiles per layer and class of work, and those placed
+  uint8_t* prune_class;   // [2^L] class of work of each tile
   uint32_t* prune_order;  // [2^L] by layer, its tiles from the most work to the least
   // layout
   unsigned long long* keys;  // [slots]
