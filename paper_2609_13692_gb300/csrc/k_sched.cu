@@ -146,7 +146,7 @@ cudaError_t exclusive_scan(uint32_t* a, int64_t n, uint32_t* sums, cudaStream_t 
 constexpr int kSortTile = 1024;
 constexpr int kSortThreads = 512;
 
-// Keys that are all different.
+// Keys that are all different, or hold whole strings: equal ones by index.
 struct ByKey {
   __device__ __forceinline__ bool less_tie(uint32_t a, uint32_t b) const { return a < b; }
 };
@@ -661,8 +661,10 @@ cudaError_t run_lex(const Strings& s, LexBuffers* b, int64_t n_chunks, const int
   const int packed = (int)(s.maxlen < fit ? s.maxlen : fit);
   k_lex_keys<<<grid_for(m), kThreads, 0, st>>>(m, b->off, b->chunk, d_arrival, window, packed, bits, b->keys, b->ord);
   ++*launches;
-  cudaError_t e = merge_sort(&b->keys, &b->ord, &b->keys2, &b->ord2, m, ByString{b->off, b->chunk, packed}, st,
-                             launches);
+  cudaError_t e = packed == s.maxlen
+                      ? merge_sort(&b->keys, &b->ord, &b->keys2, &b->ord2, m, ByKey{}, st, launches)
+                      : merge_sort(&b->keys, &b->ord, &b->keys2, &b->ord2, m, ByString{b->off, b->chunk, packed}, st,
+                                   launches);
   if (e != cudaSuccess || !with_cost) return e;
   k_inverse<<<grid_for(m), kThreads, 0, st>>>(b->ord, m, b->lexpos);
   ++*launches;
