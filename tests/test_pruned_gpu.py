@@ -330,3 +330,18 @@ def test_long_lists_of_a_pruned_solve_in_a_fresh_process(mpt, scale):
     inst = _from_supports(24, eval(f"[{sets}]"), 8)
     full = mpt.solve(inst.weights * scale, inst.bits, mode="wide" if scale > 1 else "blocked", profile=True)
     assert opt == full.opt and launches != mpt.mpt_get_profile(full.ctx)["launches_total"]
+
+
+def test_more_pairs_than_a_queue(mpt):
+    """32-bit keys beyond one queue of pairs: a chunk held by 12 of the 17 tile
+    requests of 29 leaves tiles of 11 requests 1,023 pairs in one group, in
+    more than one round (12,376 tiles are too many to be cut into parts); another
+    that shares most of them, and pairs around both."""
+    inst = _from_supports(29, [_mask(*range(0, 12), 20), _mask(*range(1, 13), 21, 22), _mask(0, 13, 25), _mask(5, 28)], 29, 60)
+    got = []
+    for mode in ("auto", "blocked"):
+        r = mpt.solve(inst.weights, inst.bits, mode=mode, tables="lean")
+        got.append((r.opt, r.perm_chunks.tolist(), r.dfs_order.tolist(), *mpt.mpt_tables32(r.ctx)))
+        assert (mpt.mpt_get_profile(r.ctx)["splits_pairs"] == 0) == (mode == "auto")
+    assert got[0][:3] == got[1][:3]
+    assert torch.equal(got[0][3], got[1][3]) and torch.equal(got[0][4], got[1][4])

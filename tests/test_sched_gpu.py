@@ -185,3 +185,34 @@ def test_layout_pinned_greedy(mpt):
     # t >= k pins everything: the production layout
     res = mpt.mpt_layout_pinned(w, ranked, 8, "greedy")
     assert res.strings == [list(r) for r in ranked]
+
+
+def test_serve_order_beyond_the_sort_key(mpt):
+    """More strings than a tile of the sort, whose 17-bit chunk ids share more
+    chunks than fit a key (three, two with windows): equal in five chunks and
+    then different, exact duplicates, proper prefixes of one another; shuffled
+    arrivals, windows of several sizes, and the cost of the whole set."""
+    rng = np.random.default_rng(29)
+    n = 100_000
+    heads = [[int(x) for x in rng.choice(n, 5, replace=False)] for _ in range(12)]
+    s = []
+    for i in range(9000):
+        head = heads[int(rng.integers(12))]
+        kind = i % 4
+        if kind == 0:
+            s.append(head + [int(x) for x in rng.integers(0, 40, size=int(rng.integers(0, 4)))])
+        elif kind == 1:
+            s.append(head[:int(rng.integers(0, 6))])
+        elif kind == 2:
+            s.append(list(s[int(rng.integers(len(s)))]))
+        else:
+            s.append(head + [99_999, int(rng.integers(0, 9))])
+    m = len(s)
+    assert mpt.mpt_serve_order(n, s).tolist() == O.serve_order(s)
+    arrival = [int(x) for x in rng.permutation(m)]
+    for W in (3, 1000, 1025, m - 1):
+        assert mpt.mpt_serve_order(n, s, arrival, W).tolist() == O.serve_order(s, arrival, W), W
+        assert mpt.mpt_serve_order(n, s, None, W).tolist() == O.serve_order(s, list(range(m)), W), W
+    w = rng.integers(1, 50, size=n).astype(np.int64)
+    offs, ids = mpt.to_csr(s)
+    assert mpt.mpt_trie_cost(w, offs, ids) == O.trie_cost_sorted(w, s)
