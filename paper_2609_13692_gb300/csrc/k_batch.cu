@@ -438,6 +438,8 @@ __host__ __device__ constexpr int batch_level_rows(int nb) {
   return (c + 1) & ~1;
 }
 static_assert(batch_level_rows(kBMaxRowsM - 5) == kBMaxLevelRows, "the most rows of one level (m = 16)");
+constexpr int kBMasksInMinimaM = 15;
+static_assert(2 * 2048 <= batch_level_rows(kBMasksInMinimaM - 5) * kBkStride, "the masks of 2,048 occurrences");
 
 // threads per block of the row-blocked kernel for m requests: enough lanes for
 // the busiest level (rows x lanes per row) -- 30 up to m = 11, 84 at m = 12,
@@ -973,8 +975,10 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
       reinterpret_cast<unsigned long long*>(bk + batch_level_rows(mm - 5) * kBkStride);  // [occ_cap]
   int32_t* cx = reinterpret_cast<int32_t*>(keys + occ_cap);                        // [occ_cap]
   uint32_t* cN = reinterpret_cast<uint32_t*>(cx + occ_cap);                        // [occ_cap]
-  uint32_t* tmask = cN + occ_cap;                                                  // [2 * occ_cap] hash-table masks
-  uint16_t* split = reinterpret_cast<uint16_t*>(tmask + 2 * occ_cap);              // [2^m] for the walk (m < 14)
+  // [2 * occ_cap] hash-table masks, needed before the minima: at m = 15, where
+  // 2,048 occurrences would not fit otherwise, in their place
+  uint32_t* tmask = mm == kBMasksInMinimaM ? bk : cN + occ_cap;
+  uint16_t* split = reinterpret_cast<uint16_t*>(cN + 3 * occ_cap);                 // [2^m] for the walk (m < 14)
   // from m = 14 the split table is written to its output slots directly and
   // the walk reads it there
   const bool gsplit = mm >= kBGlobalSplitM;
@@ -1232,7 +1236,7 @@ cudaError_t launch_batch(int count, int m, int occ_cap, const int64_t* weights, 
 size_t batch_rows_smem_bytes(int m, int occ_cap) {
   const size_t R = (size_t)1 << (m - 5);
   return (m >= kBGlobalRowsM ? 0 : R * kBRowStride * 4) + (size_t)batch_level_rows(m - 5) * kBkStride * 4 +
-         (size_t)occ_cap * 16 + (size_t)occ_cap * 8 + (m >= kBGlobalSplitM ? 0 : ((size_t)2 << m)) + 64;
+         (size_t)occ_cap * 16 + (m == kBMasksInMinimaM ? 0 : (size_t)occ_cap * 8) + (m >= kBGlobalSplitM ? 0 : ((size_t)2 << m)) + 64;
 }
 
 // 4-byte words of global row scratch one instance of size m needs (0 while

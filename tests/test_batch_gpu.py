@@ -189,3 +189,19 @@ def test_batch_private_and_common_weights(mpt):
     assert all(_shared_weight(w, reqs) < 1 << (32 - len(reqs)) for reqs in batch)
     assert max(sum(int(w[x]) for r in reqs for x in r) for reqs in batch) >= 1 << 40
     check_batch(mpt, w, batch)
+
+
+@pytest.mark.parametrize("occurrences", [1024, 1025, 1993, 2048])
+def test_fifteen_long_requests(mpt, occurrences):
+    """15 requests with packed keys may have 2,048 chunk occurrences."""
+    rng = np.random.default_rng(occurrences)
+    n, m = 900, 15
+    sizes = [occurrences // m + (i < occurrences % m) for i in range(m)]
+    w = np.ones(n, dtype=np.int64)
+    reqs = [sorted(rng.choice(n, size=k, replace=False).tolist()) for k in sizes]
+    opt, perms, orders, b = mpt.solve_batch(w, [reqs])
+    one = mpt.solve(w, I.pack_requests(reqs, n), mode="blocked")
+    assert opt[0] == one.opt and perms[0] == one.permutations() and orders[0] == one.dfs_order.tolist()
+    F, split, _ = mpt.mpt_batch_tables(b)
+    tF, _, ts = mpt.mpt_tables(one.ctx)
+    assert torch.equal(F, tF) and torch.equal(split, ts)
