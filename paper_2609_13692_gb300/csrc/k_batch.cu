@@ -1,6 +1,6 @@
 // Batched exact solve of many small instances (m <= 16 requests each), one
 // block per instance with its tables in shared memory: for packed keys the
-// row-blocked kernel (m >= 6) and, before it, a kernel for the instances of
+// row-blocked kernel (m >= 6) and, beside it, a kernel for the instances of
 // 14 requests and more that have few splits to look at; the per-subset kernel
 // otherwise.
 //
@@ -534,12 +534,15 @@ __device__ __forceinline__ void bconv_restricted(uint32_t (&acc)[kBRow], const u
 // request, the single request first, as (A, Gp(A)); keys hold A, so the
 // order in a list does not matter.
 // False, with Gp untouched, when there is no room for the list or its tests
-// (sum over S of its list's length) are more than half of the row form's
-// 3^m / 2 splits.  1,000 groups of 14-16 requests: 5.7 -> 2.0 ms per solve;
-// 20,000 groups of 8-13: 1.49 -> 1.30 ms, most of it copies.  With the line at
-// a quarter of the splits 2.0 and 1.42 ms, at an eighth 2.8 and 1.53, at all
-// of them 2.0 and 1.27; a test costs two to four row steps, so half is where
-// an instance near the line loses least.
+// (sum over S of its list's length) are more than 1 / kMembersLine of the 3^m
+// that the row form's splits are half of.  A test costs two to four row steps
+// and the lists are walked by few warps, so the line falls with m.  A solve of
+// 2,000 groups of 12 requests of 8 passages out of 200, 80, 60 and 40 each (tests
+// 0.038, 0.07, 0.12 and 0.21 of 3^m): rows 0.26 ms, members 0.22, 0.27, 0.38 and
+// 0.46; of 13 requests (0.028, 0.08, 0.09, 0.24): 0.46 and 0.34, 0.51, 0.58, 1.08;
+// of 10 requests (0.05, 0.15, 0.20, 0.31): 0.18 and 0.15, 0.19, 0.19, 0.19.
+__device__ constexpr int kMembersLine[14] = {0, 0, 0, 0, 0, 0, 2, 2, 3, 4, 6, 9, 14, 15};
+
 template <int TPI, typename Put>
 __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put) {
   __shared__ int cnt[kBMaxRowsM], start[kBMaxRowsM + 1], most, use;
@@ -549,11 +552,19 @@ __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put
   if (t == 0) most = 1;
   __syncthreads();
   const uint32_t wall = Gp[bidx(mask)];
+  // a thread's sets have the lowest request of its number, but for thread 0
+  int own = 0, largest = 0;
   for (uint32_t U = t; U < N; U += TPI)
     if ((U & (U - 1u)) != 0 && Gp[bidx(U)] > wall) {
-      atomicAdd(&cnt[__ffs(U) - 1], 1);
-      atomicMax(&most, __popc(U));
+      if (t != 0)
+        ++own;
+      else
+        atomicAdd(&cnt[__ffs(U) - 1], 1);
+      largest = max(largest, __popc(U));
     }
+  if (own) atomicAdd(&cnt[__ffs(t) - 1], own);
+  largest = __reduce_max_sync(0xFFFFFFFFu, largest);
+  if ((t & 31) == 0) atomicMax(&most, largest);
   __syncthreads();
   if (t == 0) {
     unsigned long long tests = 0, splits = 1;
@@ -566,7 +577,7 @@ __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put
       cnt[l] = 1;
     }
     start[m] = at;
-    use = at <= cap && 2 * tests < splits / 2;
+    use = at <= cap && tests * kMembersLine[m] < splits;
   }
   __syncthreads();
   if (!use) return false;
@@ -642,15 +653,14 @@ __device__ bool batch_members(int m, uint32_t* Gp, uint2* list, int cap, Put put
 // the sets without it; the members with it are listed first, from a superset
 // sum of their own, and their F and split are kept in the block's scratch
 // slot; the other sets with it are finished as they are written out.
-// An instance with too many members is left to k_batch_rows, marked in its
-// split table, where {0} has no split.
+// mpt_batch_create picks the instances (members_bound in mpt_batch.cu) and the
+// others go to k_batch_rows on another stream at the same time.
 // Bound by the list loops' shared loads.  1,000 groups of 14-16 requests, with
 // the members in k_batch_rows (256 threads, m = 16 in global memory) and here:
 // kernels of m = 16, 15 and 14 1.72, 0.66 and 0.27 ms -> 0.42, 0.26 and 0.12 ms,
 // a solve 2.05 -> 0.71 ms.  For m = 12 and 13 the same kernel and the empty launch
-// behind it take 0.24 and 0.49 ms where k_batch_rows takes 0.25 and 0.51.
+// behind it took 0.24 and 0.49 ms where k_batch_rows took 0.25 and 0.51.
 constexpr int kMembersM = 14;
-constexpr uint32_t kLeftToRows = 0xFFFFFFFFu;
 
 struct MembersShape {
   int list_cap;
@@ -799,18 +809,15 @@ k_batch_members(const int64_t* __restrict__ weights, const int64_t* __restrict__
   }
   __syncthreads();
   if (t == 0) {
-    unsigned long long tests = 0, splits = 1;
     int at = 0;
     for (int l = 0; l < m; ++l) {
       start[l] = at;
       at += cnt[l];
-      tests += (unsigned long long)cnt[l] << (m - 1 - l);
-      splits *= 3;
       if (!(kHalf && l == 0)) cnt[l] = 1;
     }
     start[m] = at;
-    use = at <= list_cap && 2 * tests < splits / 2;
-    if (!use) gsp[1] = kLeftToRows;
+    use = at <= list_cap;
+    if (!use) status[inst] = kErrWorkspace;  // against the host's bound
   }
   __syncthreads();
   if (!use) return;
@@ -937,10 +944,6 @@ k_batch_members(const int64_t* __restrict__ weights, const int64_t* __restrict__
   }
 }
 
-// What k_batch_rows does about the members: tries them first, takes what
-// k_batch_members left, or leaves them out.
-enum class Members { kTry, kRan, kNone };
-
 template <int TPI, bool kGRows = false>
 __global__ void __launch_bounds__(TPI, TPI >= 256 ? 3 : (TPI == 128 ? 6 : 12))  // 12 warps or more per SM
 k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ inst_req,
@@ -949,10 +952,9 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
              const uint8_t* __restrict__ flags, int occ_cap, int mm, int64_t* __restrict__ opt_out,
              int64_t* __restrict__ F_out, uint32_t* __restrict__ split_out, int32_t* __restrict__ perm_out,
              int32_t* __restrict__ dfs_out, int32_t* __restrict__ status, uint32_t* __restrict__ rows_scratch,
-             Members members) {
+             bool members) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int inst = inst_list[blockIdx.x];
-  if (members == Members::kRan && split_out[tab_off[inst] + 1] != kLeftToRows) return;  // finished by k_batch_members
   const int64_t r0 = inst_req[inst], r1 = inst_req[inst + 1];
   const int m = (int)(r1 - r0);  // == mm
   const int64_t o0 = req_off[r0], o1 = req_off[r1];
@@ -1040,7 +1042,7 @@ k_batch_rows(const int64_t* __restrict__ weights, const int64_t* __restrict__ in
     __syncthreads();
   }
 
-  if (members != Members::kTry || !batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
+  if (!members || !batch_members<TPI>(m, Gp, reinterpret_cast<uint2*>(bk), batch_level_rows(mm - 5) * kBkStride / 2,
                           [&](uint32_t U, uint32_t A) { put_split(U, A, &bflags); })) {
   // level 0: row 0, the recurrence on the five low requests
   if (t == 0) {
@@ -1245,6 +1247,35 @@ size_t batch_rows_scratch_words(int m) {
   return m >= kBGlobalRowsM ? ((size_t)1 << (m - 5)) * kBRowStride : 0;
 }
 
+// Members that k_batch_members has room for beside the occurrences (0: none).
+int batch_members_cap(int m, int occ_cap) { return m >= kMembersM ? members_shape(m, occ_cap).list_cap : 0; }
+
+// k_batch_members over `count` instances of size m >= 14, whose members fit.
+cudaError_t launch_batch_members(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
+                                 const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
+                                 const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
+                                 uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status,
+                                 uint32_t* rows_scratch, cudaStream_t stream) {
+  const MembersShape ms = members_shape(m, occ_cap);
+  if (m < kMembersM || m > kBMaxRowsM || ms.list_cap == 0 || (m >= kBGlobalRowsM && !rows_scratch))
+    return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
+  auto go = [&](auto kernel) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms.smem);
+    if (e == cudaSuccess)
+      kernel<<<(unsigned)count, members_threads(m), ms.smem, stream>>>(weights, inst_req, req_off, chunks, tab_off,
+                                                                       inst_list, flags, occ_cap, ms.list_cap, m, opt,
+                                                                       F, split, perm, dfs, status, rows_scratch);
+  };
+  if (m >= 16)
+    go(k_batch_members<1024, true>);
+  else if (m == 15)
+    go(k_batch_members<1024, false>);
+  else
+    go(k_batch_members<512, false>);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // One grid of the row-blocked kernel over `count` instances of size m >= 6
 // whose request weights allow packed keys.
 cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
@@ -1256,32 +1287,12 @@ cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weig
   const size_t smem = batch_rows_smem_bytes(m, occ_cap);
   const int tpi = batch_rows_threads(m);
   cudaError_t e = cudaSuccess;
-  const MembersShape ms = m >= kMembersM ? members_shape(m, occ_cap) : MembersShape{0, 0};
   // Looking at members only is less work but a longer chain per instance, so
   // below 14 requests it waits for enough blocks to hide that (13 requests:
   // 10 instances 123 us per solve against 111, 1,200 324 against 302, 2,400 485
   // against 509, 9,600 1.54 ms against 1.69; 9 requests: 1,200 123 against 126 us,
   // 9,600 324 against 396).
-  const Members members = ms.list_cap > 0 ? Members::kRan
-                          : m >= kMembersM || count >= 12 * sm_count() ? Members::kTry
-                                                                       : Members::kNone;
-  if (members == Members::kRan) {
-    auto first = [&](auto kernel) {
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms.smem);
-      if (e == cudaSuccess)
-        kernel<<<(unsigned)count, members_threads(m), ms.smem, stream>>>(
-            weights, inst_req, req_off, chunks, tab_off, inst_list, flags, occ_cap, ms.list_cap, m, opt, F, split, perm,
-            dfs, status, rows_scratch);
-    };
-    if (m >= 16)
-      first(k_batch_members<1024, true>);
-    else if (m == 15)
-      first(k_batch_members<1024, false>);
-    else
-      first(k_batch_members<512, false>);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  const bool members = m < kMembersM && count >= 12 * sm_count();
   auto go = [&](auto kernel) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)

@@ -26,6 +26,12 @@ cudaError_t launch_batch_rows(int count, int m, int occ_cap, const int64_t* weig
                               const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
                               uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status, uint32_t* rows_scratch,
                               cudaStream_t stream);
+int batch_members_cap(int m, int occ_cap);
+cudaError_t launch_batch_members(int count, int m, int occ_cap, const int64_t* weights, const int64_t* inst_req,
+                                 const int64_t* req_off, const int32_t* chunks, const int64_t* tab_off,
+                                 const int32_t* inst_list, const uint8_t* flags, int64_t* opt, int64_t* F,
+                                 uint32_t* split, int32_t* perm, int32_t* dfs, int32_t* status,
+                                 uint32_t* rows_scratch, cudaStream_t stream);
 }  // namespace mpt
 
 struct mpt_batch {
@@ -36,11 +42,13 @@ struct mpt_batch {
   // chunk ids fit 32 bits (n < 2^31); not initialised, written by mpt_batch_create's threads
   std::unique_ptr<int32_t[]> chunks;
   // instances grouped by size m: inst_list[group_start[m] .. group_start[m+1]),
-  // those for the row-blocked kernel (m >= 6, packed keys) first, up to
-  // group_rows_end[m]; each part with its own occurrence cap
+  // those for the kernel over the members (m >= 14, packed keys, few members)
+  // first, up to group_members_end[m], then those for the row-blocked kernel
+  // (m >= 6, packed keys), up to group_rows_end[m]; each part with its own
+  // occurrence cap
   std::vector<int32_t> inst_list;
-  std::vector<int64_t> group_start, group_rows_end;
-  std::vector<int> group_occ_cap_rows, group_occ_cap;
+  std::vector<int64_t> group_start, group_members_end, group_rows_end;
+  std::vector<int> group_occ_cap_members, group_occ_cap_rows, group_occ_cap;
   // per instance: kFlagPacked when the shared weight is below 2^(32 - m)
   // (32-bit keys), kFlagOffsets when sum_i w(R_i) is not (private and
   // universal chunks kept out of the kernels' values, k_batch.cu)
@@ -126,13 +134,51 @@ constexpr int64_t kBatchSumLimit = (int64_t)1 << 62;
 // 43 of the 45 ms of a pass over 20,000 groups of 8-13 requests.
 struct ChunkSlot {
   int64_t inst = -1;  // the instance that filled the slot
-  int64_t last = -1;  // the last request that held the chunk
-  int32_t chunk = 0, count = 0;
+  int32_t chunk = 0;
+  uint32_t mask = 0;  // the instance's requests that hold the chunk
 };
+
+// Members of an instance (k_batch.cu: requests that share a chunk which not
+// all share), at most, from the sets of requests that share one; 0 where
+// k_batch_rows is the faster kernel or the smaller ones have no other.  Pairs
+// are counted as they are, larger members once for every set that holds them.
+// The line is on the tests of the lists, sum over the members A of
+// 2^(m - 1 - lowest(A)), against the 3^m that the row form's splits are half of:
+// it lies where the heaviest of some hundred instances, two to an SM, takes what
+// the rows take.  m = 14, 300 groups of 8 passages out of 100, 60, 50 and 40 each
+// (tests 0.044, 0.07, 0.11 and 0.22 of 3^m): rows 0.24 ms, members 0.18, 0.23, 0.31 and
+// 0.37; m = 15 (0.03, 0.06, 0.10, 0.15): 0.54 and 0.28, 0.36, 0.53, 0.90; m = 16 (0.02,
+// 0.05, 0.09, 0.13): 3.8 and 0.53, 0.64, 1.0, 1.7.
+constexpr int kMembersFromM = 14;
+
+int members_bound(int m, const uint16_t* sets, int n) {
+  static constexpr unsigned long long kLine[3] = {10, 8, 4};
+  uint32_t pairs[16] = {};
+  unsigned long long larger[16] = {}, tests = 0, splits = 1, members = 0;
+  for (int k = 0; k < n; ++k) {
+    const uint32_t N = sets[k];
+    int above = 0;
+    for (int l = m - 1; l >= 0; --l)
+      if (N >> l & 1u) {
+        pairs[l] |= N >> l >> 1;
+        larger[l] += (1ull << above) - 1ull - (unsigned long long)above;
+        ++above;
+      }
+  }
+  for (int l = 0; l < m; ++l) {
+    const unsigned long long most = 1ull << (m - 1 - l);
+    const unsigned long long here =
+        std::min(most, 1ull + (unsigned long long)__builtin_popcount(pairs[l]) + larger[l]);  // 1: the single request
+    tests += here * most;
+    members += here;
+    splits *= 3;
+  }
+  return tests * kLine[m - kMembersFromM] < splits ? (int)members : 0;
+}
 
 mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, int64_t r0, int64_t r1,
                           const int64_t* req_offsets, const int64_t* chunk_ids, ChunkSlot* table, int32_t* ids32,
-                          uint8_t* flags) {
+                          uint8_t* flags, int32_t* members) {
   const int m = (int)(r1 - r0);
   const int64_t occ = req_offsets[r1] - req_offsets[r0];
   if (occ > kBatchMaxOcc) return MPT_ERR_TOO_LARGE;
@@ -152,27 +198,29 @@ mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, i
       if (e.inst != b) {
         e.inst = b;
         e.chunk = (int32_t)x;
-        e.count = 0;
+        e.mask = 0;
         used[distinct++] = (uint16_t)h;
-      } else if (e.last == r) {
+      } else if (e.mask >> (r - r0) & 1u) {
         return MPT_ERR_INVALID_ARG;  // twice in one request
       }
-      e.last = r;
-      ++e.count;
+      e.mask |= 1u << (r - r0);
     }
   }
   // sum_i w(R_i) (below 2^62) and the shared weight W (below 2^31): the
   // request weight less the chunks that one or all m >= 2 requests hold,
   // which the kernels keep out of their 32-bit values (k_batch.cu)
   int64_t sum = 0, shared = 0;
+  uint16_t sets[kBatchMaxOcc / 2];
+  int n_sets = 0;
   for (int k = 0; k < distinct; ++k) {
     const ChunkSlot& e = table[used[k]];
-    const int64_t cnt = e.count, wx = weights[e.chunk];
+    const int64_t cnt = __builtin_popcount(e.mask), wx = weights[e.chunk];
     if (wx > (kBatchSumLimit - 1 - sum) / cnt) return MPT_ERR_OVERFLOW;
     sum += cnt * wx;
     if (cnt >= 2 && cnt < m) {
       shared += cnt * wx;
       if (shared >= ((int64_t)1 << 31)) return MPT_ERR_OVERFLOW;
+      sets[n_sets++] = (uint16_t)e.mask;  // two occurrences or more each
     }
   }
   *flags = (uint8_t)((shared < ((int64_t)1 << (32 - m)) ? mpt::kFlagPacked : 0) |
@@ -186,6 +234,11 @@ mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, i
   const bool rows = m >= 6 && (*flags & mpt::kFlagPacked);
   if ((rows ? mpt::batch_rows_smem_bytes(m, cap) : mpt::batch_smem_bytes(m, cap)) > kBatchMaxSmem)
     return MPT_ERR_TOO_LARGE;
+  *members = 0;
+  if (rows && m >= kMembersFromM) {
+    std::sort(sets, sets + n_sets);
+    *members = members_bound(m, sets, (int)(std::unique(sets, sets + n_sets) - sets));
+  }
   return MPT_OK;
 }
 
@@ -194,7 +247,7 @@ mpt_status check_instance(const int64_t* weights, int64_t n_chunks, int64_t b, i
 // occurrences); a thread that cannot be started has its range done here.
 void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, const int64_t* inst_requests,
                      const int64_t* req_offsets, const int64_t* chunk_ids, int32_t* ids32, uint8_t* flags,
-                     mpt_status* bad) {
+                     int32_t* members, mpt_status* bad) {
   const int64_t occ = req_offsets[inst_requests[batch]];
   const int64_t cores = occ >> 15 ? std::max<int64_t>(1, (int64_t)std::thread::hardware_concurrency()) : 1;
   const int64_t ranges = std::min<int64_t>({8, cores, 1 + (occ >> 15), batch});
@@ -213,7 +266,7 @@ void check_instances(const int64_t* weights, int64_t n_chunks, int32_t batch, co
     const int32_t end = (int32_t)(batch * (k + 1) / ranges);
     for (int32_t b = (int32_t)(batch * k / ranges); b < end && r.status == MPT_OK; ++b) {
       r.status = check_instance(weights, n_chunks, b, inst_requests[b], inst_requests[b + 1], req_offsets, chunk_ids,
-                                r.table.data(), ids32, flags + b);
+                                r.table.data(), ids32, flags + b, members + b);
     }
   };
   std::vector<std::thread> threads;
@@ -301,12 +354,13 @@ mpt_status mpt_batch_create(const int64_t* weights, int64_t n_chunks, int32_t ba
     c->tab_off.resize((size_t)batch + 1);
     c->flags.assign((size_t)batch, 0);
     std::vector<int> inst_occ((size_t)batch);
+    std::vector<int32_t> members((size_t)batch);
     // the instances' own checks and weights, on several threads when there
     // are many occurrences; the first failing instance decides the status
     mpt_status bad = MPT_OK;
     c->chunks.reset(new int32_t[(size_t)std::max<int64_t>(occ_total, 1)]);
     check_instances(weights, n_chunks, batch, inst_requests, req_offsets, chunk_ids, c->chunks.get(),
-                    c->flags.data(), &bad);
+                    c->flags.data(), members.data(), &bad);
     if (bad != MPT_OK) {
       delete c;
       return bad;
@@ -328,19 +382,32 @@ mpt_status mpt_batch_create(const int64_t* weights, int64_t n_chunks, int32_t ba
     for (int32_t b = 0; b < batch; ++b) ++c->group_start[(size_t)(inst_requests[b + 1] - inst_requests[b]) + 1];
     for (int m = 1; m <= kBatchMaxM + 1; ++m) c->group_start[(size_t)m] += c->group_start[(size_t)m - 1];
     c->inst_list.resize((size_t)batch);
+    c->group_occ_cap_members.assign(kBatchMaxM + 1, 1);
     c->group_occ_cap_rows.assign(kBatchMaxM + 1, 1);
     c->group_occ_cap.assign(kBatchMaxM + 1, 1);
+    // the members have to fit beside the most occurrences of their part
+    for (int32_t b = 0; b < batch; ++b) {
+      const int m = (int)(inst_requests[b + 1] - inst_requests[b]);
+      int cap = c->group_occ_cap_members[(size_t)m];
+      while (members[(size_t)b] > 0 && cap < inst_occ[(size_t)b]) cap <<= 1;
+      if (mpt::batch_members_cap(m, cap) == 0) members[(size_t)b] = 0;
+      if (members[(size_t)b] > 0) c->group_occ_cap_members[(size_t)m] = cap;
+    }
     std::vector<int64_t> fill(c->group_start.begin(), c->group_start.end());
-    for (int pass = 0; pass < 2; ++pass) {
+    for (int pass = 0; pass < 3; ++pass) {
       for (int32_t b = 0; b < batch; ++b) {
         const int m = (int)(inst_requests[b + 1] - inst_requests[b]);
         const bool rows = m >= 6 && (c->flags[(size_t)b] & mpt::kFlagPacked);
-        if (rows != (pass == 0)) continue;
+        const bool few = members[(size_t)b] > 0 &&
+                         members[(size_t)b] <= mpt::batch_members_cap(m, c->group_occ_cap_members[(size_t)m]);
+        if ((few ? 0 : rows ? 1 : 2) != pass) continue;
         c->inst_list[(size_t)fill[(size_t)m]++] = b;
+        if (few) continue;
         int& cap = rows ? c->group_occ_cap_rows[(size_t)m] : c->group_occ_cap[(size_t)m];
         while (cap < inst_occ[(size_t)b]) cap <<= 1;
       }
-      if (pass == 0) c->group_rows_end.assign(fill.begin(), fill.end());
+      if (pass == 0) c->group_members_end.assign(fill.begin(), fill.end());
+      if (pass == 1) c->group_rows_end.assign(fill.begin(), fill.end());
     }
     c->table_entries = tab;
     c->w.assign(weights, weights + n_chunks);
@@ -421,14 +488,21 @@ mpt_status mpt_batch_solve(mpt_batch* b, void* d_workspace, size_t workspace_byt
   }
   int next_side = 0;
   for (int m = kBatchMaxM; m >= 1 && e == cudaSuccess; --m) {
-    const int64_t g0 = b->group_start[(size_t)m], gr = b->group_rows_end[(size_t)m],
-                  g1 = b->group_start[(size_t)m + 1];
+    const int64_t g0 = b->group_start[(size_t)m], gm = b->group_members_end[(size_t)m],
+                  gr = b->group_rows_end[(size_t)m], g1 = b->group_start[(size_t)m + 1];
     if (g1 == g0) continue;
-    cudaStream_t st = forked ? b->side[(size_t)(next_side++ % kBatchSideStreams)] : stream;
-    if (gr > g0)
-      e = mpt::launch_batch_rows((int)(gr - g0), m, b->group_occ_cap_rows[(size_t)m], c.weights, c.inst_req, c.req_off,
-                                 c.chunks, c.tab_off, c.inst_list + g0, c.flags, c.opt, c.F, c.split, c.perm, c.dfs,
-                                 c.status, c.rows_scratch, st);
+    auto side = [&]() { return forked ? b->side[(size_t)(next_side++ % kBatchSideStreams)] : stream; };
+    // the parts of a size run at the same time: each block has its own slot of the scratch rows
+    uint32_t* after = c.rows_scratch ? c.rows_scratch + (size_t)(gm - g0) * mpt::batch_rows_scratch_words(m) : nullptr;
+    cudaStream_t st = side();
+    if (gr > gm)
+      e = mpt::launch_batch_rows((int)(gr - gm), m, b->group_occ_cap_rows[(size_t)m], c.weights, c.inst_req, c.req_off,
+                                 c.chunks, c.tab_off, c.inst_list + gm, c.flags, c.opt, c.F, c.split, c.perm, c.dfs,
+                                 c.status, after, st);
+    if (e == cudaSuccess && gm > g0)
+      e = mpt::launch_batch_members((int)(gm - g0), m, b->group_occ_cap_members[(size_t)m], c.weights, c.inst_req,
+                                    c.req_off, c.chunks, c.tab_off, c.inst_list + g0, c.flags, c.opt, c.F, c.split,
+                                    c.perm, c.dfs, c.status, c.rows_scratch, gr > gm ? side() : st);
     if (e == cudaSuccess && g1 > gr)
       e = mpt::launch_batch((int)(g1 - gr), m, b->group_occ_cap[(size_t)m], c.weights, c.inst_req, c.req_off,
                             c.chunks, c.tab_off, c.inst_list + gr, c.flags, c.opt, c.F, c.split, c.perm, c.dfs,

@@ -205,3 +205,52 @@ def test_fifteen_long_requests(mpt, occurrences):
     F, split, _ = mpt.mpt_batch_tables(b)
     tF, _, ts = mpt.mpt_tables(one.ctx)
     assert torch.equal(F, tF) and torch.equal(split, ts)
+
+
+def _solve_seconds(mpt, m, groups):
+    import time
+
+    b = mpt.mpt_batch_create(np.ones(400, dtype=np.int64), *mpt.pack_batch(groups))
+    ws = torch.empty(mpt.mpt_batch_workspace_bytes(b), dtype=torch.uint8, device="cuda")
+    best = 1.0
+    for _ in range(8):
+        t = time.perf_counter()
+        mpt.mpt_batch_solve(b, ws)
+        best = min(best, time.perf_counter() - t)
+    return best
+
+
+@pytest.mark.parametrize("m,count,k,pool", [(12, 2000, 8, 40), (13, 2000, 8, 40), (14, 100, 10, 40), (14, 300, 10, 40),
+                                            (15, 100, 10, 40), (15, 300, 12, 40), (16, 100, 12, 40)])
+def test_half_dense_groups_take_no_longer_than_dense_ones(mpt, m, count, k, pool):
+    """Groups with too many members for the recurrence over the members to pay,
+    few enough that it was tried: not slower than leave-one-out groups, which
+    the row form solves (they took 1.24 to 1.78 times as long)."""
+    rng = np.random.default_rng(m * count)
+    half = []
+    for _ in range(count):
+        p = rng.choice(400, size=pool, replace=False)
+        half.append([rng.choice(p, size=k, replace=False).tolist() for _ in range(m)])
+    dense = [[[x for x in range(m) if x != i] for i in range(m)]] * count
+    assert _solve_seconds(mpt, m, half) < 1.25 * _solve_seconds(mpt, m, dense)
+
+
+@pytest.mark.parametrize("m", [14, 15, 16])
+def test_members_and_rows_at_once(mpt, m):
+    """Groups of one size on both sides of the line between the kernels, some
+    with so many occurrences that the lists have no room."""
+    rng = np.random.default_rng(m + 50)
+    w = rng.integers(1, 4, size=400).astype(np.int64)
+    groups = []
+    for i in range(24):
+        k, pool = [(8, 200), (8, 60), (8, 40), (10, 40), (14, 24), (100, 400)][i % 6]
+        p = rng.choice(400, size=pool, replace=False)
+        groups.append([rng.choice(p, size=k, replace=False).tolist() for _ in range(m)])
+    order = rng.permutation(24)
+    opt, perms, orders, b = mpt.solve_batch(w, [groups[i] for i in order])
+    F, split, offs = mpt.mpt_batch_tables(b)
+    for at, i in enumerate(order):
+        one = mpt.solve(w, I.pack_requests(groups[i], 400), mode="blocked")
+        tF, _, ts = mpt.mpt_tables(one.ctx)
+        assert opt[at] == one.opt and perms[at] == one.permutations() and orders[at] == one.dfs_order.tolist(), i
+        assert torch.equal(F[offs[at]:offs[at + 1]], tF) and torch.equal(split[offs[at]:offs[at + 1]], ts), i
