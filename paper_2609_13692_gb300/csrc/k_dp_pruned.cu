@@ -48,7 +48,6 @@
 #include "mpt_internal.cuh"
 
 #include <algorithm>
-#include <cmath>
 
 namespace mpt {
 namespace {
@@ -978,9 +977,22 @@ cudaError_t layer(const Shape& s, const Workspace& ws, const Tab* wIr, int kh, u
 
 // The members of each single request's list by k_prune_tiles' rules: the
 // listed rows, members and cost of {l} bound those of every T that holds l.
+struct ByteSums {
+  uint8_t bits[256] = {}, eighths[256] = {};  // set bits; sum over them of 8 >> bits of their number
+};
+constexpr ByteSums make_byte_sums() {
+  ByteSums t{};
+  for (int v = 1; v < 256; ++v) t.bits[v] = (uint8_t)(t.bits[v >> 1] + (v & 1));
+  for (int v = 0; v < 256; ++v)
+    for (int i = 0; i < 8; ++i)
+      if (v >> i & 1) t.eighths[v] = (uint8_t)(t.eighths[v] + (8 >> t.bits[i]));
+  return t;
+}
+
 template <typename Key>
 void singles(int L, const InnerPerm& perm, const uint32_t* sets, size_t n, bool* tiles, bool* pairs, double* costs) {
   using C = PrunedCfg<Key>;
+  static constexpr ByteSums kByte = make_byte_sums();
   *tiles = *pairs = false;
   for (int l = 0; l < L; ++l) {
     uint32_t row[C::kRows] = {1u};
@@ -999,10 +1011,13 @@ void singles(int L, const InnerPerm& perm, const uint32_t* sets, size_t n, bool*
     for (uint32_t r = 0; r < (uint32_t)C::kRows; ++r) {
       if (row[r] == 0) continue;
       uint32_t steps = 0;
-      for (uint32_t a = row[r]; a; a &= a - 1) steps += (uint32_t)C::kRow >> __builtin_popcount(__builtin_ctz(a));
+      for (int q = 0; q < C::kRow / 8; ++q) {
+        const uint32_t v = row[r] >> (8 * q) & 255u;
+        steps += kByte.eighths[v] * ((uint32_t)C::kRow / 8) >> kByte.bits[q];  // q: the members' bits above the byte
+        members += kByte.bits[v];
+      }
       ++rows;
-      members += (uint32_t)__builtin_popcount(row[r]);
-      cost += (steps + kUnitSteps) << (C::kLogWarps - __builtin_popcount(r >> 5));
+      cost += (steps + kUnitSteps) << (C::kLogWarps - kByte.bits[r >> 5]);
     }
     const bool many = rows > (uint32_t)kPruneRows, is_long = sizeof(Key) == 4 && (many || cost > kLongSteps);
     *pairs = *pairs || is_long;
@@ -1029,22 +1044,22 @@ uint32_t pruned_items(const Shape& s, int kh) {
 // all SMs or a block's part of its heaviest tile, whichever is more, in this
 // kernel and in the pair kernel, besides what the kernels of a layer take with
 // nothing to do; work in warp steps of the lists, on the 152 SMs of a GB300 (no
-// CUDA call is made here).  The lists of one Ta are the
-// sum over the sets N with Ta within N_T of the list of N alone (a product over
-// its bits, as k_prune_tiles counts it), less what the sets have in common: the
-// singles' lists are known, and with sum S and union e of those of {l}, and C
-// such that e = C (1 - exp(-S / C)), the n larger Ta's with lowest request l and
-// sum t over all of them are taken as n C (1 - exp(-t / (n C))).
+// CUDA call is made here).  The lists of one Ta are the sum over the sets N with
+// Ta within N_T of the list of N alone (a product over its bits, as
+// k_prune_tiles counts it), less what the sets have in common: the singles'
+// lists are known, and with sum S and union e of those of {l}, and C such that
+// e = S / (1 + S / C), the n larger Ta's with lowest request l and sum t over all
+// of them are taken as t / (1 + t / (n C)).
 //
 // Constants (ms): fitted to solves of 2,300 instances of 13 to 28 requests whose
 // estimate matters (random sets of one density or size, few large ones, pooled
 // passages, uniform requests; both key widths): median error 0 to 6 %, 5 % to
-// 95 % of them within -27 .. +68 %.  Full solves: fitted to the same, from
+// 95 % of them within -24 .. +50 %.  Full solves: fitted to the same, from
 // below (m = 13 to 27: 0.13 .. 229 ms, 64-bit keys m = 13 to 24: 0.17 .. 62 ms).
-// Of the 801 of them that the pairs' estimate alone (Overlap in mpt_api.cu) would send
-// here, 240 were slower than the full form by more than 5 %, by up to 2.9 times
-// and, with 64-bit keys, which have no pair kernel for a heavy list, 14 times.
-// This rule takes 450 of them, one of which is (by 9 %), and leaves some 55
+// Of the 801 of them that the pairs' estimate alone (Overlap in mpt_api.cu) would
+// send here, 240 were slower than the full form by more than 5 %, by up to 2.9
+// times and, with 64-bit keys, which have no pair kernel for a heavy list, 14
+// times.  This rule takes 466 of them, one of which is (by 9 %), and leaves 41
 // out that would be faster by more than 10 % (by up to 1.7 times).
 template <typename Key>
 bool pruned_pays(const Shape& s, const InnerPerm& perm, const uint32_t* sets, size_t n, const double* single,
@@ -1079,30 +1094,27 @@ bool pruned_pays(const Shape& s, const InnerPerm& perm, const uint32_t* sets, si
   for (int l = 0; l < L; ++l) {
     const int A = L - 1 - l;
     double S = 0.0;
-    for (int a = 0; a < L; ++a) S += sum[0][l][a] + sum[1][l][a];
+    int used[kMaxMembersL], n_used = 0;  // the a that occur
+    for (int a = 0; a < L; ++a) {
+      const double here = sum[0][l][a] + sum[1][l][a];
+      S += here;
+      if (here > 0.0) used[n_used++] = a;
+    }
     const double e = single[l];
     const bool e_long = !kWide && e >= kFullPairSteps;
-    double Cs = 0.0;  // 0: nothing in common
-    if (S > 0.0 && e < 0.999 * S) {
-      double lo = 1e-9, hi = S / e + 1.0;  // x = S / C: (1 - exp(-x)) / x falls from 1 to below e / S
-      for (int i = 0; i < 50; ++i) {
-        const double x = 0.5 * (lo + hi);
-        (-std::expm1(-x) / x > e / S ? lo : hi) = x;
-      }
-      Cs = S / lo;
-    }
+    const double Cs = S > 0.0 && e < 0.999 * S ? e * S / (S - e) : 0.0;  // 0: nothing in common
     // the lists (t[0] short, t[1] long) of `count` Ta's of i + 1 requests, at most `cap` of them above l
     auto lists = [&](int i, int cap, double count, double* t) {
       t[0] = t[1] = 0.0;
-      for (int a = i; a < L; ++a) {
-        const double c = choose(a < cap ? a : cap, i);
-        t[0] += sum[0][l][a] * c;
-        t[1] += sum[1][l][a] * c;
+      for (int q = n_used - 1; q >= 0 && used[q] >= i; --q) {
+        const double c = choose(used[q] < cap ? used[q] : cap, i);
+        t[0] += sum[0][l][used[q]] * c;
+        t[1] += sum[1][l][used[q]] * c;
       }
       const double all = t[0] + t[1];
       if (all == 0.0) return false;
       if (Cs > 0.0 && count > 0.0) {
-        const double f = count * Cs * -std::expm1(-all / (count * Cs)) / all;
+        const double f = count * Cs / (count * Cs + all);
         t[0] *= f;
         t[1] *= f;
       }
@@ -1133,7 +1145,7 @@ bool pruned_pays(const Shape& s, const InnerPerm& perm, const uint32_t* sets, si
     const double parts[2] = {(double)pruned_items(s, kh), (double)listed_items(L, kh, 152)};
     for (int q = 0; q < 2; ++q) ms += std::max(kStep[q] * layer[q][kh], kOwnStep[q] * heaviest[q][kh] / parts[q]);
   }
-  return 1.15 * ms < full;
+  return (pairs ? 1.15 : 1.1) * ms < full;
 }
 
 }  // namespace
