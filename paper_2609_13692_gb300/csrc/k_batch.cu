@@ -540,7 +540,10 @@ __device__ __forceinline__ void bconv_restricted(uint32_t (&acc)[kBRow], const u
 // 2,000 groups of 12 requests of 8 passages out of 200, 80, 60 and 40 each (tests
 // 0.038, 0.07, 0.12 and 0.21 of 3^m): rows 0.26 ms, members 0.22, 0.27, 0.38 and
 // 0.46; of 13 requests (0.028, 0.08, 0.09, 0.24): 0.46 and 0.34, 0.51, 0.58, 1.08;
-// of 10 requests (0.05, 0.15, 0.20, 0.31): 0.18 and 0.15, 0.19, 0.19, 0.19.
+// of 10 requests (0.05, 0.15, 0.20, 0.31): 0.18 and 0.15, 0.19, 0.19, 0.19.  With
+// sizes of 8 to 13 in one call the SMs are shared and members pay a little
+// further up: 20,000 groups 1.20 ms with this line, 1.28 with 3, 4, 6, 9, 14, 15 from
+// m = 8 on.
 __device__ constexpr int kMembersLine[14] = {0, 0, 0, 0, 0, 0, 4, 4, 4, 4, 5, 6, 8, 10};
 
 template <int TPI, typename Put>

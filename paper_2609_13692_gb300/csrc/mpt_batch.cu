@@ -148,7 +148,8 @@ struct ChunkSlot {
 // the rows take.  m = 14, 300 groups of 8 passages out of 100, 60, 50 and 40 each
 // (tests 0.044, 0.07, 0.11 and 0.22 of 3^m): rows 0.24 ms, members 0.18, 0.23, 0.31 and
 // 0.37; m = 15 (0.03, 0.06, 0.10, 0.15): 0.54 and 0.28, 0.36, 0.53, 0.90; m = 16 (0.02,
-// 0.05, 0.09, 0.13): 3.8 and 0.53, 0.64, 1.0, 1.7.
+// 0.05, 0.08, 0.12, 0.26, the heaviest of them twice that): 3.8 and 0.42, 0.64, 1.0,
+// 1.8, 2.1, where one group of the rows' alone takes 1.7.
 constexpr int kMembersFromM = 14;
 
 // A set's larger members by its bytes, so that the loop has no branch on its
@@ -177,7 +178,7 @@ constexpr ByteSums make_byte_sums() {
 
 int members_bound(int m, const uint16_t* sets, int n) {
   static constexpr ByteSums kByte = make_byte_sums();
-  static constexpr uint64_t kLine[3] = {10, 8, 4};
+  static constexpr uint64_t kLine[3] = {10, 8, 2};
   uint16_t pairs[16] = {};
   uint16_t seen[32] = {};  // sets, by a hash: one met again is mostly left out
   uint64_t tests = 0, splits = 1, members = 0;
