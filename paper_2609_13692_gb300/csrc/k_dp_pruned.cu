@@ -31,20 +31,20 @@
 // 64-bit keys have no pair kernel for long lists: their rows beyond the first
 // kPruneRows are read from the table as they come.
 //
-// Measured on one GB300 (whole solve with layout and tables, full recurrence
-// before, pruned after): 28 requests of 20 passages 673 -> 3.9 .. 14.6 ms by
-// seed (a passage held by 12 to 17 of the 28 decides it), 24 requests of 10
-// passages 11.1 -> 0.7 ms and with 64-bit keys 80 -> 0.8 .. 0.9 ms, 26 requests of
-// 40 passages 81 -> 13.5 .. 30.6 ms.
+// Measured on one GB300 (create, solve, layout and tables; full recurrence before,
+// pruned after, by seed): 28 requests of 20 passages 673 -> 3.9 .. 17 ms (a passage
+// held by 12 to 17 of the 28 decides it), 24 requests of 10 passages 11.1 -> 0.7 .. 0.8
+// ms and with 64-bit keys 80 -> 0.7 .. 1.0 ms, 26 requests of 40 passages, lean tables,
+// 81 -> 5 .. 58 ms.
 // k_dp_pruned is bound by the integer ALU pipe where a popular passage gives
 // long a1 lists: 83 % of the pipe busy over the heaviest layers of 26 requests of
 // 40 passages, 57 to 75 % with 20 passages, the rest of the time lost to the
 // barrier per pair (the warps of a group have 1, 2 or 4 rows of work each).  Also
-// measured (tile stage at m = 28, seed 1, when the kernel took 13.1 ms): a block per tile, four to an SM, with the row groups dealt by a
-// hash of the block 15.5 ms, in turn per SM 16.2; three such blocks with three
-// slots 16.8, with two slots 16.7, two blocks with four 21.9; the members
-// evaluated one by one instead of by rows 242 ms; the inner bits in natural
-// order 69.9 ms.
+// measured (tile stage at m = 28, seed 1, when the kernel took 13.1 ms): a block
+// per tile, four to an SM, with the row groups dealt by a hash of the block 15.5
+// ms, in turn per SM 16.2; three such blocks with three slots 16.8, with two slots
+// 16.7, two blocks with four 21.9; the members evaluated one by one instead of by
+// rows 242 ms; the inner bits in natural order 69.9 ms.
 #include "mpt_internal.cuh"
 
 #include <algorithm>
@@ -66,7 +66,9 @@ constexpr uint32_t kUnitSteps = 60;
 // steps of a warp.  Lists dearer than this go there.  26 requests of 40
 // passages, seeds 9, 11, 12, 13 and 14: with 9,000 42.7, 17.5, 43.0, 55.6 and 43.7
 // ms, with 12,000 31.0, 9.9, 29.1, 34.9, 43.7, with 14,000 26.0, 9.4, 24.2, 34.9,
-// 43.6, with 17,000 25.7, 9.4, 24.2, 34.1, 50.0.
+// 43.6, with 17,000 25.7, 9.4, 24.2, 34.1, 50.0.  Over 60 instances of 21 to 28
+// requests (pooled passages, random sets, few large sets, uniform requests) 10,000
+// takes 3.5 % longer on the average and up to 1.9 times, 20,000 as long (0.91 to 1.05).
 constexpr uint32_t kLongSteps = 14000;
 constexpr double kFullPairSteps = 16600.0;
 constexpr int kPruneMinPairs = 16;     // pairs that a further block of a tile has to have
