@@ -40,7 +40,6 @@
 #include "mpt_internal.cuh"
 
 #include <algorithm>
-#include <cmath>
 #include <vector>
 
 namespace mpt {
@@ -808,7 +807,9 @@ extern "C" mpt_status mpt_greedy(const int64_t* weights, int64_t n_chunks, int32
   // keys tie or wait for one another a round merges a pair or two, and the rest
   // goes to one block (2 to 5 us a merge with signatures of 8 chunks, a round 9
   // us).  Few requests go there at once, or after a few rounds without a look.
-  const int ahead = m <= kNoRounds ? 0 : m <= kFewRounds ? 4 : std::min(12, 2 + (int)std::log2((double)m));
+  int ahead = 2;
+  while (ahead < 12 && (1 << ahead) < 4 * m) ++ahead;  // 2 + log2(m), rounded up
+  if (m <= kFewRounds) ahead = m <= kNoRounds ? 0 : 4;
   int32_t counts[3] = {0, 0, 0};
   bool rest = m <= kFewRounds;
   for (int round = 0, merged = 0; e == cudaSuccess && m > 1; merged = counts[0]) {
