@@ -615,7 +615,12 @@ mpt_status check_weights(const int64_t* weights, int64_t n_chunks) {
 }
 
 mpt_status check_permutation(const int32_t* p, int64_t m) {
-  std::vector<char> seen((size_t)m, 0);
+  std::vector<char> seen;
+  try {
+    seen.assign((size_t)m, 0);
+  } catch (...) {
+    return MPT_ERR_OUT_OF_MEMORY;
+  }
   for (int64_t i = 0; i < m; ++i) {
     if (p[i] < 0 || p[i] >= m || seen[(size_t)p[i]]) return MPT_ERR_INVALID_ARG;
     seen[(size_t)p[i]] = 1;
@@ -786,6 +791,16 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
       total_w += wx;
     }
   }
+  std::vector<unsigned long long> h_bins;
+  std::vector<int32_t> by_cap;
+  std::vector<int64_t> h_caps;
+  try {
+    h_bins.resize((size_t)n_caps + 1);
+    by_cap.resize((size_t)n_caps);
+    h_caps.resize((size_t)n_caps);
+  } catch (...) {
+    return MPT_ERR_OUT_OF_MEMORY;
+  }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int64_t N = s.total;
   const int K = sparse_levels_for(m);
@@ -833,10 +848,7 @@ mpt_status mpt_cache_costs(const int64_t* weights, int64_t n_chunks, int32_t m, 
 
   int launches = 0;
   unsigned long long h_trie = 0, h_first = 0;
-  std::vector<unsigned long long> h_bins((size_t)n_caps + 1);
   // the capacities in increasing order
-  std::vector<int32_t> by_cap((size_t)n_caps);
-  std::vector<int64_t> h_caps((size_t)n_caps);
   for (int32_t i = 0; i < n_caps; ++i) by_cap[(size_t)i] = i;
   std::sort(by_cap.begin(), by_cap.end(), [&](int32_t x, int32_t y) { return capacities[x] < capacities[y]; });
   for (int32_t i = 0; i < n_caps; ++i) h_caps[(size_t)i] = capacities[by_cap[(size_t)i]];
@@ -909,18 +921,28 @@ mpt_status mpt_layout_pinned(const int64_t* weights, int64_t n_chunks, int32_t m
   for (int64_t p = 0; p < total; ++p)
     if (ranked_chunks[p] < 0 || ranked_chunks[p] >= n_chunks) return MPT_ERR_INVALID_ARG;
   // free part of request i: its ranked list after the first t entries
-  std::vector<int64_t> foff((size_t)m + 1, 0), fchunks, seq((size_t)(total > 0 ? total : 1));
-  for (int32_t i = 0; i < m; ++i) {
-    const int64_t a = ranked_offsets[i], b = ranked_offsets[i + 1];
-    const int64_t pin = b - a < t ? b - a : t;
-    for (int64_t p = a + pin; p < b; ++p) fchunks.push_back(ranked_chunks[p]);
-    foff[(size_t)i + 1] = (int64_t)fchunks.size();
+  std::vector<int64_t> foff, fchunks, seq, fperm, poff;
+  std::vector<uint64_t> bits;
+  const int64_t words = (n_chunks + 63) / 64;
+  try {
+    foff.assign((size_t)m + 1, 0);
+    seq.resize((size_t)(total > 0 ? total : 1));
+    for (int32_t i = 0; i < m; ++i) {
+      const int64_t a = ranked_offsets[i], b = ranked_offsets[i + 1];
+      const int64_t pin = b - a < t ? b - a : t;
+      for (int64_t p = a + pin; p < b; ++p) fchunks.push_back(ranked_chunks[p]);
+      foff[(size_t)i + 1] = (int64_t)fchunks.size();
+    }
+    fperm.resize(fchunks.size() > 0 ? fchunks.size() : 1);
+    if (method == MPT_PIN_EXACT) {
+      bits.assign((size_t)m * (size_t)words, 0);
+      poff.resize((size_t)m + 1);
+    }
+  } catch (...) {
+    return MPT_ERR_OUT_OF_MEMORY;
   }
-  std::vector<int64_t> fperm(fchunks.size() > 0 ? fchunks.size() : 1);
   mpt_status ms;
   if (method == MPT_PIN_EXACT) {
-    const int64_t words = (n_chunks + 63) / 64;
-    std::vector<uint64_t> bits((size_t)m * (size_t)words, 0);
     for (int32_t i = 0; i < m; ++i)
       for (int64_t p = foff[(size_t)i]; p < foff[(size_t)i + 1]; ++p) {
         const int64_t x = fchunks[(size_t)p];
@@ -931,7 +953,6 @@ mpt_status mpt_layout_pinned(const int64_t* weights, int64_t n_chunks, int32_t m
     mpt_ctx* ctx = nullptr;
     if ((ms = mpt_create(weights, n_chunks, bits.data(), m, &ctx)) != MPT_OK) return ms;
     int64_t opt = 0;
-    std::vector<int64_t> poff((size_t)m + 1);
     ms = mpt_solve(ctx, nullptr, 0, stream, &opt);
     if (ms == MPT_OK) ms = mpt_layout(ctx, poff.data(), fperm.data(), nullptr);
     mpt_destroy(ctx);
